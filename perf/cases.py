@@ -267,10 +267,11 @@ def prepare(case, seed):
         s["rows"] = {f: getattr(store, f)[:n].clone() for f in ("px", "py", "pz", "type")}
     s["store"], s["n"] = store, n
     if k != "plan":
-        s["child"] = {f: torch.zeros(store.capacity - n, device="cuda",
-                                     dtype=getattr(store, f).dtype)
-                      for f in qed.FLOAT_FIELDS + ("id", "type")}
-        s["order"] = torch.empty(store.capacity - n, device="cuda", dtype=torch.int64)
+        room = store.capacity - n
+        s["child"] = {"id": torch.zeros(room, device="cuda", dtype=torch.int64),
+                      "type": torch.zeros(room, device="cuda", dtype=torch.uint8),
+                      "fields": torch.zeros(len(qed.FLOAT_FIELDS), room, device="cuda")}
+        s["order"] = torch.empty(room, device="cuda", dtype=torch.int64)
     if k == "host":
         h = qed.HostStore(store.capacity)
         for f in qed.FLOAT_FIELDS + ("id", "type"):
@@ -294,9 +295,10 @@ def _out(s, stats):
     out = {f: getattr(store, f)[:n] for f in ("px", "py", "pz", "type")}
     order = s["order"][:m - n]
     torch.sort(store.id[n:m].cuda(non_blocking=True), out=(child["id"][:m - n], order))
-    for f in qed.FLOAT_FIELDS + ("type",):
-        torch.index_select(getattr(store, f)[n:m].cuda(non_blocking=True), 0, order,
-                           out=child[f][:m - n])
+    torch.index_select(store.type[n:m].cuda(non_blocking=True), 0, order, out=child["type"][:m - n])
+    fields = [getattr(store, f)[n:m] for f in qed.FLOAT_FIELDS]
+    torch.index_select(torch.stack([f.cuda(non_blocking=True) for f in fields]), 1, order,
+                       out=child["fields"][:, :m - n])
     out["child"] = child
     out["stats"] = [int(stats[k]) for k in STATS]
     return out
@@ -332,7 +334,7 @@ def run(s):
         ctx.graph_launch()
         stats = ctx.graph_read_stats()[0]
         for t in s["child"].values():   # each launch is another step, with other counts
-            t[stats["count"] - n:].zero_()
+            t[..., stats["count"] - n:].zero_()
         out = _out(s, stats)
         out["spectrum"] = ctx.read_spectrum(reset=True)
         return out
