@@ -357,7 +357,7 @@ def run_gb300(args):
         t_launch = kern["hot"][0] / kern["hot"][1] / 1e3
         per_launch = 20.0 * pagg["substeps_warp"] / kern["hot"][1]
         achieved = per_launch / t_launch / 1e12
-        roof = {"kernel": "k_hot_lanes + k_step (hot pass)", "bound": "alu", "achieved": achieved,
+        roof = {"kernel": "k_hot + k_step (hot pass)", "bound": "alu", "achieved": achieved,
                 "peak": mul_peak, "unit": "T int32-mul/s", "frac": achieved / mul_peak,
                 "traffic": None, "traffic_note": HOT_TRAFFIC_NOTE,
                 "peak_kind": "measured: qed_peak_probe MUL32 (Philox multiplies) on this GPU"}

@@ -7,12 +7,12 @@
 //   k_cold                 thread pass: one lane per row for the plan and
 //                          events, the warp's lanes together for the draws;
 //                          plans of at least hot_min sub-steps are queued
-//   k_hot_lanes            hot pass (persistent): long plans one warp each
-//                          (64 sub-steps per iteration, lane l drawing the
-//                          Philox block of sub-steps 2l, 2l+1), medium plans
-//                          one lane each with warp-shared draws; in sampler
-//                          mode the warp of a sampler particle evaluates the
-//                          network for its events
+//   k_hot                  hot pass (persistent): one lane per queued particle,
+//                          the windows of a warp's particles drawn by its
+//                          lanes together
+//   k_hot_net              the same in sampler mode 1: long plans and the
+//                          sampler's particles one warp each, which evaluates
+//                          the network for its events
 //   k_advance              closes a cascade generation; below tail_rows rows
 //                          it hands the rest of the step to the tail pass
 //   k_tail_begin / k_step / k_tail_end
@@ -47,7 +47,14 @@ namespace {
 // Defaults measured on the 2^24 clumped population (coordinate search over
 // hot_min 32..128 and long_min 128..2048)
 constexpr uint32_t kHotMinDefault = 32;    // plans with N >= hot_min go to the hot pass
-constexpr uint32_t kLongMinDefault = 256;  // ... and with N >= long_min to its warp mode
+#ifndef QED_SAMP_LONG
+#define QED_SAMP_LONG 4096
+#endif
+constexpr uint32_t kSampLong = QED_SAMP_LONG;   // sampler: plans with N >= this are stepped first
+#ifndef QED_LONG_MIN
+#define QED_LONG_MIN 256
+#endif
+constexpr uint32_t kLongMinDefault = QED_LONG_MIN;  // ... and with N >= long_min to its warp mode
 constexpr long long kTailRowsDefault = 1ll << 17;   // generations below this go to the tail pass
 
 // Minimum resident blocks per SM requested from the register allocator:
@@ -89,7 +96,9 @@ struct DevCtl {
                                     // after the thread pass's hot_tail entries
     int skip;                       // the tail pass does nothing
     unsigned long long push_head;   // push mode: next row of the generation to take
-    unsigned int samp_tail, samp_head;   // event-driven sampler: its queue of this generation
+    // event-driven sampler, its queue of this generation: entries at the front
+    // (the longest plans) and at the back of the array, entries taken of each
+    unsigned int samp_tail, samp_back, samp_head, samp_back_head;
     long long n_init;               // rows at the start of the step (the rest are children)
     unsigned long long beat;        // persistent passes: progress of long chains, so that
                                     // idle warps tell a long chain from a stalled step
@@ -121,7 +130,8 @@ struct Scratch {
                             // from both ends: long plans from the front,
                             // medium plans from the back
     long long hot_cap;
-    HotItem* samp;          // event-driven sampler's queue (capacity entries; null when off)
+    HotItem* samp;          // event-driven sampler's queue (null when off)
+    long long samp_cap;     // its entries
     qed_event_record* log;  // optional
     long long log_cap;
     long long* log_count;
@@ -347,10 +357,27 @@ __device__ __forceinline__ unsigned long long stored_rows(const DevParticles& P)
     return (unsigned long long)min(c, P.capacity);
 }
 
+// Rows [slot, slot + n) were reserved for children: slot, or -1 on overflow,
+// when the rows that exist are marked removed and the capacity error is
+// recorded.
+__device__ __forceinline__ long long check_rows(const DevParticles& P, DevCtl* ctl, long long slot,
+                                                int n) {
+    if (slot + n > P.capacity) {
+        for (long long j = slot; j < slot + n && j < P.capacity; ++j) {
+            P.id[j] = 0;
+            __threadfence();   // a tail-pass lane may be waiting for this row
+            *reinterpret_cast<volatile uint8_t*>(P.type + j) = QED_REMOVED;
+        }
+        atomicMax(&ctl->required, slot + n);
+        atomicExch(&ctl->status, (int)QED_ERR_CAPACITY);
+        return -1;
+    }
+    return slot;
+}
+
 // Reserve n rows for children.  `aggregate`: the lanes of the warp that reach
 // this call together share one atomic (ballots of the active lanes give each
-// lane its offset, the first lane adds the total, the base is broadcast).  On overflow
-// the reserved rows are marked removed and the capacity error is recorded.
+// lane its offset, the first lane adds the total, the base is broadcast).
 __device__ __forceinline__ long long reserve_rows(const DevParticles& P, DevCtl* ctl, int n,
                                                   bool aggregate) {
     long long slot;
@@ -375,17 +402,7 @@ __device__ __forceinline__ long long reserve_rows(const DevParticles& P, DevCtl*
         slot = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(P.count),
                                     (unsigned long long)n);
     }
-    if (slot + n > P.capacity) {
-        for (long long j = slot; j < slot + n && j < P.capacity; ++j) {
-            P.id[j] = 0;
-            __threadfence();   // a tail-pass lane may be waiting for this row
-            *reinterpret_cast<volatile uint8_t*>(P.type + j) = QED_REMOVED;
-        }
-        atomicMax(&ctl->required, slot + n);
-        atomicExch(&ctl->status, (int)QED_ERR_CAPACITY);
-        return -1;
-    }
-    return slot;
+    return check_rows(P, ctl, slot, n);
 }
 
 // The parent's fields, copied to its children.
@@ -415,99 +432,41 @@ __device__ __forceinline__ void write_child_fields(const DevParticles& P, const 
 
 constexpr long long kReserveHere = -2;   // apply_event reserves the child rows itself
 
-// Apply an accepted event (recoil or decay, children, log).  Returns true if
-// the particle was removed (photon decay).  Thread callers (write_rows) do
-// everything themselves, sharing one reservation atomic per warp; warp
-// callers (all 32 lanes, identical arguments) reserve and store on lane 0
-// (13 stores from one lane measured faster than a 13-way divergent split of
-// the stores across lanes).  The reservation is issued first so that its
-// latency overlaps the child-id computation.
-__device__ __forceinline__ bool apply_event(const DevParticles& P, const Scratch& S, const StepParams& SP,
-                            DevCtl* ctl, long long i, uint64_t id, bool photon, float x,
-                            float eps, float chi, uint32_t step, uint32_t s, ftime t_after, PState& st,
-                            Stats& stats, bool write_rows, bool warp_caller, const Fields& F,
-                            bool publish, long long j_pre = kReserveHere) {
-    const int nch = photon ? 2 : 1;
-    const int lane = threadIdx.x & 31;
-    long long j = -1;
-    if (j_pre != kReserveHere) {
-        j = j_pre;   // reserved by the caller (-1: it did not fit)
-    } else if (warp_caller) {
-        // lane 0 reserves and stores; its result is first needed at the stores
-        if (lane == 0) j = reserve_rows(P, ctl, nch, false);
-    } else if (write_rows) {
-        j = reserve_rows(P, ctl, nch, true);
-    }
+// Write the children of an accepted event into rows j.. (j < 0: they did not
+// fit) and the event into the log.  st: the parent before the event; the type
+// bytes come last.  kPublish: in a persistent pass another warp may be waiting
+// for these rows: one fence for the event's children, then their type bytes.
+// kDeferred: the same, but fence and type bytes are the caller's.
+enum ChildMode { kPlain, kPublish, kDeferred };
+__device__ __forceinline__ uint8_t child_type(bool photon, int r) {
+    return photon ? (r == 0 ? (uint8_t)QED_ELECTRON : (uint8_t)QED_POSITRON) : (uint8_t)QED_PHOTON;
+}
+__device__ __forceinline__ void write_children(const DevParticles& P, const Scratch& S,
+                                               const StepParams& SP, long long i, long long j,
+                                               uint64_t id, bool photon, float x, float chi,
+                                               uint32_t step, uint32_t s, ftime t_after,
+                                               const PState& st, const Fields& F, ChildMode mode) {
     const uint4 cid = philox4x32_10(make_uint4((uint32_t)id, (uint32_t)(id >> 32), step, s),
                                     SP.child_keys);
     const uint64_t id0 = ((uint64_t)cid.x | ((uint64_t)cid.y << 32)) | (1ull << 63);
     const uint64_t id1 = ((uint64_t)cid.z | ((uint64_t)cid.w << 32)) | (1ull << 63);
-    float delta;
-    bool removed = false;
-    float cp[2][3];
-    if (!photon) {
-        delta = x * x * x;
-        cp[0][0] = delta * st.px;
-        cp[0][1] = delta * st.py;
-        cp[0][2] = delta * st.pz;
-        cp[1][0] = cp[1][1] = cp[1][2] = 0.0f;
-    } else {
-        delta = x;
-        const float omd = 1.0f - x;
-        cp[0][0] = x * st.px;
-        cp[0][1] = x * st.py;
-        cp[0][2] = x * st.pz;
-        cp[1][0] = omd * st.px;
-        cp[1][1] = omd * st.py;
-        cp[1][2] = omd * st.pz;
-    }
+    const float delta = photon ? x : x * x * x;
     if (j >= 0) {
-        const uint64_t cids[2] = {id0, id1};
-        const uint8_t ctypes[2] = {photon ? (uint8_t)QED_ELECTRON : (uint8_t)QED_PHOTON,
-                                   (uint8_t)QED_POSITRON};
-        if (!warp_caller || lane == 0) {
-            const float w = P.w[i];
-            for (int r = 0; r < nch; ++r)
-                write_child_fields(P, S, j + r, F, w, cp[r][0], cp[r][1], cp[r][2], cids[r],
-                                   t_after);
-            // in the tail pass another warp may be waiting for these rows:
-            // one fence for the event's children, then their type bytes
-            if (publish) __threadfence();
-            for (int r = 0; r < nch; ++r)
-                *reinterpret_cast<volatile uint8_t*>(P.type + j + r) = ctypes[r];
+        const float w = P.w[i];
+        write_child_fields(P, S, j, F, w, delta * st.px, delta * st.py, delta * st.pz, id0,
+                           t_after);
+        if (photon) {
+            const float omd = 1.0f - x;
+            write_child_fields(P, S, j + 1, F, w, omd * st.px, omd * st.py, omd * st.pz, id1,
+                               t_after);
+        }
+        if (mode == kPublish) __threadfence();
+        if (mode != kDeferred) {
+            *reinterpret_cast<volatile uint8_t*>(P.type + j) = child_type(photon, 0);
+            if (photon) *reinterpret_cast<volatile uint8_t*>(P.type + j + 1) = child_type(true, 1);
         }
     }
-    if (!photon) {
-        if (SP.recoil) {
-            if (delta < 1e-6f && eps > 1e4f) {
-                const double f = 1.0 - (double)delta;
-                st.px = (float)(f * (double)st.px);
-                st.py = (float)(f * (double)st.py);
-                st.pz = (float)(f * (double)st.pz);
-            } else if (delta < 0.5f) {
-                st.px = fmaf(-delta, st.px, st.px);
-                st.py = fmaf(-delta, st.py, st.py);
-                st.pz = fmaf(-delta, st.pz, st.pz);
-            } else {
-                const float omd = (1.0f - x) * (1.0f + x + x * x);
-                st.px *= omd;
-                st.py *= omd;
-                st.pz *= omd;
-            }
-        }
-        if (!warp_caller || lane == 0) {   // a warp caller counts on lane 0
-            stats.emissions++;
-            stats.children++;
-        }
-    } else {
-        removed = SP.recoil != 0;
-        if (!warp_caller || lane == 0) {
-            stats.pairs++;
-            stats.children += 2;
-        }
-    }
-    const bool logger = warp_caller ? lane == 0 : write_rows;
-    if (logger && S.log) {
+    if (S.log) {
         const long long k = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(S.log_count), 1ull);
         if (k < S.log_cap) {
             qed_event_record r;
@@ -521,7 +480,62 @@ __device__ __forceinline__ bool apply_event(const DevParticles& P, const Scratch
             S.log[k] = r;
         }
     }
-    return removed;
+}
+
+// The parent after the event (recoil or decay).  True if it was removed.
+__device__ __forceinline__ bool event_recoil(const StepParams& SP, bool photon, float x, float eps,
+                                             PState& st) {
+    if (photon) return SP.recoil != 0;
+    if (SP.recoil) {
+        const float delta = x * x * x;
+        if (delta < 1e-6f && eps > 1e4f) {
+            const double f = 1.0 - (double)delta;
+            st.px = (float)(f * (double)st.px);
+            st.py = (float)(f * (double)st.py);
+            st.pz = (float)(f * (double)st.pz);
+        } else if (delta < 0.5f) {
+            st.px = fmaf(-delta, st.px, st.px);
+            st.py = fmaf(-delta, st.py, st.py);
+            st.pz = fmaf(-delta, st.pz, st.pz);
+        } else {
+            const float omd = (1.0f - x) * fmaf(x, x, 1.0f + x);
+            st.px *= omd;
+            st.py *= omd;
+            st.pz *= omd;
+        }
+    }
+    return false;
+}
+
+__device__ __forceinline__ void count_event(Stats& stats, bool photon) {
+    if (photon) {
+        stats.pairs++;
+        stats.children += 2;
+    } else {
+        stats.emissions++;
+        stats.children++;
+    }
+}
+
+// Apply an accepted event (children, log, recoil or decay).  Returns true if
+// the particle was removed (photon decay).  Thread callers share one
+// reservation atomic per warp; warp callers (all 32 lanes, identical
+// arguments) reserve and store on lane 0 (13 stores from one lane measured
+// faster than a 13-way divergent split of the stores across lanes).  The
+// reservation is issued first so that its latency overlaps the child ids.
+__device__ __forceinline__ bool apply_event(const DevParticles& P, const Scratch& S, const StepParams& SP,
+                            DevCtl* ctl, long long i, uint64_t id, bool photon, float x,
+                            float eps, float chi, uint32_t step, uint32_t s, ftime t_after, PState& st,
+                            Stats& stats, bool warp_caller, const Fields& F,
+                            bool publish, long long j_pre = kReserveHere) {
+    if (!warp_caller || (threadIdx.x & 31) == 0) {
+        const long long j = j_pre != kReserveHere ? j_pre   // reserved by the caller
+                                                  : reserve_rows(P, ctl, photon ? 2 : 1, !warp_caller);
+        write_children(P, S, SP, i, j, id, photon, x, chi, step, s, t_after, st, F,
+                       publish ? kPublish : kPlain);
+        count_event(stats, photon);
+    }
+    return event_recoil(SP, photon, x, eps, st);
 }
 
 __device__ __forceinline__ bool process_enabled(const StepParams& SP, bool photon) {
@@ -545,10 +559,12 @@ __device__ __forceinline__ void push_hot(const Scratch& S, DevCtl* ctl, long lon
 // With the learned sampler on, e+- whose chi lies in a usable bin of its
 // range (64 bins uniform in log10 chi over [-2, 2)) are stepped in the hot
 // pass's warp mode, where the network is evaluated.
-__device__ __forceinline__ bool sampler_bin_ok(const StepParams& SP, float chi) {
-    if (!SP.sampler || !(chi >= 1e-2f && chi < 1e2f)) return false;
+__device__ __forceinline__ bool sampler_bin(unsigned long long bins, float chi) {
     const int bin = min(max((int)((log10f(chi) - kMlpLog10Lo) * 16.0f), 0), 63);
-    return (SP.net_bins >> bin) & 1ull;
+    return chi >= 1e-2f && chi < 1e2f && ((bins >> bin) & 1ull);
+}
+__device__ __forceinline__ bool sampler_bin_ok(const StepParams& SP, float chi) {
+    return SP.sampler && sampler_bin(SP.net_bins, chi);
 }
 
 // With the event-driven sampler, photons whose plan has candidates (a nonzero
@@ -556,9 +572,7 @@ __device__ __forceinline__ bool sampler_bin_ok(const StepParams& SP, float chi) 
 // sampler decide their decay from the tabulated total pair probability and
 // take delta_e from the pair network.
 __device__ __forceinline__ bool pair_sampler_ok(const StepParams& SP, float chi, uint32_t T) {
-    if (!SP.pnet_bins || T == 0u || !(chi >= 1e-2f && chi < 1e2f)) return false;
-    const int bin = min(max((int)((log10f(chi) - kMlpLog10Lo) * 16.0f), 0), 63);
-    return (SP.pnet_bins >> bin) & 1ull;
+    return SP.pnet_bins && T != 0u && sampler_bin(SP.pnet_bins, chi);
 }
 
 // Graph runs keep the global step index as a device base plus the node's
@@ -570,21 +584,71 @@ __device__ __forceinline__ uint32_t step_index(const StepParams& SP) {
 // One round of warp-shared draws.  Every active lane has the sub-steps
 // [s, s_end) of its current plan to test; the Philox blocks of those ranges
 // are laid end to end (prefix sum of the per-lane block counts) and drawn 32
-// at a time, lane f of a round taking block f.  Its owner is the last lane
-// whose first block index is <= f (5-step binary search over the lanes), whose
-// plan parameters come by shuffle.  Accepted sub-steps are reduced per owner
-// with a shared-memory minimum: on return facc[lane] holds the lane's earliest
-// accepted sub-step in its range, or kNoEvent.  Called by all 32 lanes.
+// at a time, lane f of a pass taking block f.  Its owner is found from the
+// blocks at which ranges start (one reduction per pass and a bit count), its
+// parameters come from shared memory.  A sub-step whose acceptance draw is
+// below its plan's squeeze threshold goes to the warp's candidate list; the
+// list is evaluated at the end of the round (or when it may overflow), one
+// candidate per lane, so that the acceptance function is paid once per 32
+// candidates instead of once per pass that has one.  Accepted sub-steps are
+// reduced per owner with a shared-memory minimum: on return facc[lane] holds
+// the lane's earliest accepted sub-step in its range, or kNoEvent.  Called by
+// all 32 lanes; key[lane] is the lane's draw key.
 constexpr uint32_t kNoEvent = 0xffffffffu;
-__device__ __forceinline__ void warp_draw_round(const SharedTables& sm, uint32_t* facc,
-                                                bool active, uint32_t s, uint32_t s_end,
-                                                uint32_t T, float b, float c_h, uint64_t id,
-                                                bool photon, uint32_t step, const PhiloxKeys& K,
+constexpr int kCandMax = 128;   // candidates listed before they are evaluated
+struct DrawBuf {                // one per warp
+    DrawKey key[32];
+    uint4 par[32];              // s, s_end, b, c_h (negative: photon)
+    uint2 off[32];              // first block less its place in the round; last draw word that passes
+    uint32_t facc[32];
+    uint32_t cand_s[kCandMax];  // candidates: sub-step and owner
+    uint8_t cand_o[kCandMax];
+    uint8_t owner[32];          // lanes with blocks to draw, in lane order
+};
+
+// Evaluates the n listed candidates.  Counted are those that decide in order:
+// up to the owner's first accepted sub-step (later lists hold later sub-steps
+// of an owner, so its minimum is final for this one).
+__device__ __forceinline__ void eval_candidates(const SharedTables& sm, DrawBuf& B, int n,
+                                                uint32_t y1, const PhiloxKeys& K,
                                                 unsigned int& cand) {
+    __syncwarp();
+    const int lane = threadIdx.x & 31;
+    for (int c0 = 0; c0 < n; c0 += 32) {
+        const int c = c0 + lane;
+        if (c < n) {
+            const uint32_t s = B.cand_s[c];
+            const int o = B.cand_o[c];
+            const uint4 p = B.par[o];
+            if (s >= p.x && s < p.y) {   // not the other sub-step of a block at an end of the range
+                const uint4 r = draw_block(B.key[o], y1, s >> 1, K);
+                const float c_h = __uint_as_float(p.w);
+                float dtmp;
+                const float y = u01((s & 1u) ? r.w : r.y);
+                if (y < acceptance(sm.syn, c_h < 0.0f, __uint_as_float(p.z), fabsf(c_h),
+                                   u01((s & 1u) ? r.z : r.x), &dtmp))
+                    atomicMin(&B.facc[o], s);
+            }
+        }
+    }
+    __syncwarp();
+    for (int c = lane; c < n; c += 32) {
+        const uint32_t s = B.cand_s[c];
+        const int o = B.cand_o[c];
+        const uint4 p = B.par[o];
+        cand += s >= p.x && s < p.y && s <= B.facc[o] ? 1u : 0u;
+    }
+    __syncwarp();
+}
+
+__device__ __forceinline__ void draw_round(const SharedTables& sm, DrawBuf& B, bool active,
+                                           uint32_t s, uint32_t s_end, uint32_t T, float b,
+                                           float c_h, bool photon, uint32_t y1,
+                                           const PhiloxKeys& K, unsigned int& cand) {
     constexpr unsigned int kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const uint32_t b0 = s >> 1;
-    const uint32_t nblk = (active && s_end > s) ? ((s_end - 1u) >> 1) - b0 + 1u : 0u;
+    const uint32_t nblk = (active && s_end > s && T != 0u) ? ((s_end - 1u) >> 1) - b0 + 1u : 0u;
     uint32_t incl = nblk;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -593,61 +657,62 @@ __device__ __forceinline__ void warp_draw_round(const SharedTables& sm, uint32_t
     }
     const uint32_t total = __shfl_sync(kAll, incl, 31);
     const uint32_t excl = incl - nblk;
-    facc[lane] = kNoEvent;
+    const unsigned int have = __ballot_sync(kAll, nblk != 0u);
+    if (nblk) {
+        B.owner[__popc(have & ((1u << lane) - 1u))] = (uint8_t)lane;
+        B.par[lane] = make_uint4(s, s_end, __float_as_uint(b), __float_as_uint(photon ? -c_h : c_h));
+        B.off[lane] = make_uint2(b0 - excl, (T << 9) - 1u);   // (r >> 9) < T, T <= 2^23
+    }
+    B.facc[lane] = kNoEvent;
     __syncwarp();
+    const unsigned int upto = 0xffffffffu >> (31 - lane);
+    int before = -1;   // owners that start before the pass, less one
+    int n = 0;
     for (uint32_t fb = 0; fb < total; fb += 32) {
         const uint32_t f = fb + (uint32_t)lane;
-        int owner = 0;
-#pragma unroll
-        for (int stp = 16; stp > 0; stp >>= 1) {
-            const uint32_t e = __shfl_sync(kAll, excl, owner + stp);
-            if (e <= f) owner += stp;
-        }
-        const uint32_t blk = __shfl_sync(kAll, b0, owner) + (f - __shfl_sync(kAll, excl, owner));
-        const uint32_t o_s = __shfl_sync(kAll, s, owner);
-        const uint32_t o_end = __shfl_sync(kAll, s_end, owner);
-        const uint32_t o_T = __shfl_sync(kAll, T, owner);
-        const float o_b = __shfl_sync(kAll, b, owner);
-        const float o_ch = __shfl_sync(kAll, c_h, owner);
-        const uint32_t o_lo = __shfl_sync(kAll, (uint32_t)id, owner);
-        const uint32_t o_hi = __shfl_sync(kAll, (uint32_t)(id >> 32), owner);
-        const bool o_photon = __shfl_sync(kAll, photon ? 1 : 0, owner) != 0;
-        if (f < total) {
-            const uint4 r = philox4x32_10(make_uint4(o_lo, o_hi, step, blk), K);
-            const uint32_t sA = 2u * blk;
-            const bool cA = sA >= o_s && sA < o_end && (r.y >> 9) < o_T;
-            const bool cB = sA + 1u >= o_s && sA + 1u < o_end && (r.w >> 9) < o_T;
-            cand += (unsigned)cA + (unsigned)cB;
-            bool aA = false, aB = false;
-            float dtmp;
-            if (cA || cB) {
-                // one acceptance evaluation per lane: the earlier candidate of
-                // the pair; the later one only if the earlier is rejected
-                const bool first = cA;
-                const float y = u01(first ? r.y : r.w);
-                const bool acc =
-                    y < acceptance(sm.syn, o_photon, o_b, o_ch, u01(first ? r.x : r.z), &dtmp);
-                aA = first && acc;
-                aB = !first && acc;
+        const uint32_t d = excl - fb;
+        const unsigned int starts = __reduce_or_sync(kAll, nblk && d < 32u ? 1u << d : 0u);
+        const int o = B.owner[before + __popc(starts & upto)];
+        before += __popc(starts);
+        const uint2 off = B.off[o];
+        const uint32_t blk = off.x + f;
+        const uint2 r = draw_yw(B.key[o], y1, blk, K);
+        const bool cA = f < total && r.x <= off.y;
+        const bool cB = f < total && r.y <= off.y;
+        const unsigned int mA = __ballot_sync(kAll, cA), mB = __ballot_sync(kAll, cB);
+        if (mA | mB) {
+            const unsigned int below = upto >> 1;
+            if (cA) {
+                const int k = n + __popc(mA & below);
+                B.cand_s[k] = 2u * blk;
+                B.cand_o[k] = (uint8_t)o;
             }
-            if (cA && cB && !aA)
-                aB = u01(r.w) < acceptance(sm.syn, o_photon, o_b, o_ch, u01(r.z), &dtmp);
-            if (aA) atomicMin(&facc[owner], sA);
-            else if (aB) atomicMin(&facc[owner], sA + 1u);
+            n += __popc(mA);
+            if (cB) {
+                const int k = n + __popc(mB & below);
+                B.cand_s[k] = 2u * blk + 1u;
+                B.cand_o[k] = (uint8_t)o;
+            }
+            n += __popc(mB);
+            if (n > kCandMax - 64) {
+                eval_candidates(sm, B, n, y1, K, cand);
+                n = 0;
+            }
         }
     }
+    if (n) eval_candidates(sm, B, n, y1, K, cand);
     __syncwarp();
 }
 
 // x of sub-step s (the first word of its draw pair).
-__device__ __forceinline__ float draw_x(uint64_t id, uint32_t step, uint32_t s,
+__device__ __forceinline__ float draw_x(const DrawKey& d, uint32_t y1, uint32_t s,
                                         const PhiloxKeys& K) {
-    const uint4 r = philox4x32_10(make_uint4((uint32_t)id, (uint32_t)(id >> 32), step, s >> 1), K);
+    const uint4 r = draw_block(d, y1, s >> 1, K);
     return u01((s & 1u) ? r.z : r.x);
 }
 
 // Thread pass: one lane per row for planning and events, the warp's lanes
-// together for the draws (warp_draw_round).  First generation of a step:
+// together for the draws (draw_round).  First generation of a step:
 // rows [0, pass_end) with the full step; later generations: rows
 // [pass_begin, pass_end) (children) with their stored remaining time.  Each
 // lane plans its row; particles whose plan reaches hot_min sub-steps (or,
@@ -662,7 +727,7 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
                                                        DevCtl* ctl) {
     const uint32_t step = step_index(SP);
     __shared__ SharedTables sm;
-    __shared__ uint32_t first_acc[kColdThreads];
+    __shared__ DrawBuf draw_buf[kColdThreads / 32];
     stage_tables(sm);
     __syncthreads();
     if (ctl->status == (int)QED_ERR_TIMEOUT || ctl->skip) return;
@@ -673,7 +738,8 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    uint32_t* facc = first_acc + (threadIdx.x & ~31);
+    DrawBuf& B = draw_buf[threadIdx.x >> 5];
+    const uint32_t y1 = draw_y1(step, SP.draw_keys);
     constexpr unsigned int kAll = 0xffffffffu;
     Stats stats;
     for (long long base = begin + warp * 32; base < end; base += nwarps * 32) {
@@ -691,6 +757,7 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
                 if (time_positive(t_rem)) {
                     active = true;
                     id = P.id[i];
+                    B.key[lane] = draw_key(id, step, SP.draw_keys);
                     st = PState{P.px[i], P.py[i], P.pz[i]};
                     Ex = P.Ex[i]; Ey = P.Ey[i]; Ez = P.Ez[i];
                     Bx = P.Bx[i]; By = P.By[i]; Bz = P.Bz[i];
@@ -733,9 +800,12 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
                             it.idx = (uint32_t)i;
                             it.s = s;
                             it.t_rem = t_rem;
-                            S.samp[atomicAdd(&ctl->samp_tail, 1u)] = it;
+                            if (pl.N >= kSampLong)
+                                S.samp[atomicAdd(&ctl->samp_tail, 1u)] = it;
+                            else
+                                S.samp[S.samp_cap - 1 - (long long)atomicAdd(&ctl->samp_back, 1u)] = it;
                         } else {
-                            push_hot(S, ctl, i, s, t_rem, pl.N >= SP.long_min || net);
+                            push_hot(S, ctl, i, s, t_rem, pl.N >= SP.front_min || net);
                         }
                         active = false;
                     } else {
@@ -752,9 +822,10 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
                 }
             }
             const uint32_t s_end = active ? s + pl.N : 0u;
-            warp_draw_round(sm, facc, active, s, s_end, pl.T, pl.b, pl.c_h, id, photon, step, SP.draw_keys, stats.cand);
+            draw_round(sm, B, active, s, s_end, pl.T, pl.b, pl.c_h, photon, y1, SP.draw_keys,
+                       stats.cand);
             if (active) {
-                const uint32_t s_ev = facc[lane];
+                const uint32_t s_ev = B.facc[lane];
                 if (s_ev == kNoEvent) {
                     stats.substeps += pl.N;
                     s = s_end;
@@ -762,11 +833,11 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
                 } else {
                     const uint32_t k = s_ev - s;
                     stats.substeps += k + 1u;
-                    const float x = draw_x(id, step, s_ev, SP.draw_keys);
+                    const float x = draw_x(B.key[lane], y1, s_ev, SP.draw_keys);
                     const ftime t_after = (k + 1u == pl.N) ? ftime{0.0f, 0.0f}
                                                            : time_sub_mul(t_rem, k + 1u, pl.h);
                     removed = apply_event(P, S, SP, ctl, i, id, photon, x, eps, chi, step, s_ev,
-                                          t_after, st, stats, true, false,
+                                          t_after, st, stats, false,
                                           Fields{Ex, Ey, Ez, Bx, By, Bz}, false);
                     changed = true;
                     s = s_ev + 1u;
@@ -775,7 +846,7 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
                     else need_plan = true;
                 }
             }
-            __syncwarp();   // facc is reset by the next round
+            __syncwarp();   // the draw buffer is reused by the next round
         }
         if (removed) {
             P.type[i] = QED_REMOVED;
@@ -1019,7 +1090,7 @@ __global__ void __launch_bounds__(kLaneThreads) k_push(DevParticles P, StepParam
             if (ev) {
                 ev = false;
                 removed = apply_event(P, S, SP, ctl, i, id, photon, ev_x, ev_eps, ev_chi, step, s,
-                                      t_rem, st, stats, true, false, F, kStream);
+                                      t_rem, st, stats, false, F, kStream);
                 ++s;
                 if (removed || !time_positive(t_rem)) return true;
             }
@@ -1134,7 +1205,7 @@ __global__ void __launch_bounds__(kLaneThreads) k_push(DevParticles P, StepParam
                     const ftime t_after = (kk == pl.N) ? ftime{0.0f, 0.0f}
                                                        : time_sub_mul(t_rem, kk, pl.h);
                     removed = apply_event(P, S, SP, ctl, i, id, photon, nxd, neps, nchi, step,
-                                          s + (uint32_t)jstar_o, t_after, st, stats, true, false, F,
+                                          s + (uint32_t)jstar_o, t_after, st, stats, false, F,
                                           kStream);
                     s += used_o;
                     t_rem = t_after;
@@ -1224,7 +1295,7 @@ __global__ void __launch_bounds__(kLaneThreads) k_push(DevParticles P, StepParam
 // kSampler: an e+- in a usable bin of the sampler's chi range decides events
 // from the tabulated total probability c_h W(b) and takes the energy fraction
 // from the network at the event's uniform, evaluated by the warp (FP32).
-template <int kSampler, bool kCells = false>
+template <int kSampler>
 __device__ __forceinline__ void warp_item(const DevParticles& P, const Scratch& S,
                                           const StepParams& SP, DevCtl* ctl,
                                           const SharedTables& sm, unsigned char* net_smem,
@@ -1244,12 +1315,10 @@ __device__ __forceinline__ void warp_item(const DevParticles& P, const Scratch& 
     ftime t_rem = it.t_rem;
     bool removed = false, changed = false;
     unsigned int rounds = 0;   // publish (persistent pass): beats of a long chain
-    const long long n_init = kCells ? ctl->n_init : 0;
     while (time_positive(t_rem)) {
         float eps, chi;
         Plan pl = plan_particle(SP, sm.sqz_e, sm.sqz_p, photon, st.px, st.py, st.pz, Ex, Ey, Ez,
                                 Bx, By, Bz, t_rem, &chi, &eps);
-        if (kCells) apply_cell_count(SP, pl, sm.sqz_e, sm.sqz_p, photon, i, n_init, s, t_rem, eps);
         if (!(eps > 0.0f)) break;
         if (lane == 0) {
             stats.plans++;
@@ -1259,7 +1328,7 @@ __device__ __forceinline__ void warp_item(const DevParticles& P, const Scratch& 
         // event-driven mode: photons in a usable bin of the pair sampler too
         const bool use_pnet =
             kSampler == 2 && photon && pl.N >= SP.hot_min && pair_sampler_ok(SP, chi, pl.T);
-        const bool use_net = (kSampler != 0 && !photon && sampler_bin_ok(SP, chi)) || use_pnet;
+        const bool use_net = (!photon && sampler_bin_ok(SP, chi)) || use_pnet;
         const SamplerMma& tab = use_pnet ? pair_mma(net_smem) : mma;
         const float thr =
             use_net ? fminf(pl.c_h * (kSampler == 2 ? wtot_at(tab.wtot, tab.nrows, chi)
@@ -1303,7 +1372,7 @@ __device__ __forceinline__ void warp_item(const DevParticles& P, const Scratch& 
                 const ftime t_after = (k_ev + 1 == pl.N) ? ftime{0.0f, 0.0f}
                                                          : time_sub_mul(t_rem, k_ev + 1, pl.h);
                 removed = apply_event(P, S, SP, ctl, i, id, photon, x, eps, chi, step, s_ev,
-                                      t_after, st, stats, lane == 0, true,
+                                      t_after, st, stats, true,
                                       Fields{Ex, Ey, Ez, Bx, By, Bz}, publish);
                 changed = true;
                 s = s_ev + 1;
@@ -1373,7 +1442,7 @@ __device__ __forceinline__ void warp_item(const DevParticles& P, const Scratch& 
             const ftime t_after = (k_ev + 1 == pl.N) ? ftime{0.0f, 0.0f}
                                                      : time_sub_mul(t_rem, k_ev + 1, pl.h);
             removed = apply_event(P, S, SP, ctl, i, id, photon, x, eps, chi, step, s_ev, t_after,
-                                  st, stats, lane == 0, true, Fields{Ex, Ey, Ez, Bx, By, Bz},
+                                  st, stats, true, Fields{Ex, Ey, Ez, Bx, By, Bz},
                                   publish);
             changed = true;
             s = s_ev + 1;
@@ -1395,6 +1464,83 @@ __device__ __forceinline__ void warp_item(const DevParticles& P, const Scratch& 
 }
 
 
+using LaneFields = float[6][kLaneThreads];
+
+__device__ __forceinline__ Fields lane_fields(const LaneFields& f) {
+    const int t = threadIdx.x;
+    return Fields{f[0][t], f[1][t], f[2][t], f[3][t], f[4][t], f[5][t]};
+}
+
+// The hot pass and the event-driven sampler write their children 32 at a time: a round has a few events, and
+// the child ids, the reservation and the stores cost a warp the same for one
+// as for 32.  Nobody waits for them before the next generation.
+constexpr int kEventBuf = 64;
+struct __align__(16) EventBuf {   // one per warp, used as a ring
+    uint64_t id[kEventBuf];
+    ftime t_after[kEventBuf];
+    uint32_t i[kEventBuf], s[kEventBuf];
+    float x[kEventBuf];   // negative: the parent is a photon
+    float px[kEventBuf], py[kEventBuf], pz[kEventBuf], chi[kEventBuf];
+    float f[6][kEventBuf];   // E, B
+};
+__device__ __forceinline__ void note_event(EventBuf& E, unsigned int q, uint32_t i, uint64_t id,
+                                           bool photon, float x, float chi, uint32_t s,
+                                           ftime t_after, const PState& st, const Fields& F) {
+    E.id[q] = id;
+    E.t_after[q] = t_after;
+    E.i[q] = i;
+    E.s[q] = s;
+    E.x[q] = photon ? -x : x;
+    E.px[q] = st.px;
+    E.py[q] = st.py;
+    E.pz[q] = st.pz;
+    E.chi[q] = chi;
+    E.f[0][q] = F.Ex;
+    E.f[1][q] = F.Ey;
+    E.f[2][q] = F.Ez;
+    E.f[3][q] = F.Bx;
+    E.f[4][q] = F.By;
+    E.f[5][q] = F.Bz;
+}
+
+
+// The children of the ring's first min(n, 32) events.
+__device__ __forceinline__ void events_flush(const DevParticles& P, const Scratch& S,
+                                             const StepParams& SP, DevCtl* ctl, const EventBuf& E,
+                                             unsigned int& n, unsigned int& head, uint32_t step) {
+    const unsigned int lane = threadIdx.x & 31;
+    const unsigned int k = min(n, 32u);
+    __syncwarp();
+    if (lane < k) {
+        const unsigned int q = (head + lane) % kEventBuf;
+        const bool photon = E.x[q] < 0.0f;
+        const uint32_t i = E.i[q];
+        const long long j = reserve_rows(P, ctl, photon ? 2 : 1, true);
+        write_children(P, S, SP, i, j, E.id[q], photon, fabsf(E.x[q]), E.chi[q], step, E.s[q],
+                       E.t_after[q], PState{E.px[q], E.py[q], E.pz[q]},
+                       Fields{E.f[0][q], E.f[1][q], E.f[2][q], E.f[3][q], E.f[4][q], E.f[5][q]},
+                       kPlain);
+    }
+    __syncwarp();
+    n -= k;
+    head += k;
+}
+
+#ifndef QED_SAMP_REFILL
+#define QED_SAMP_REFILL 4
+#endif
+constexpr int kSampRefill = QED_SAMP_REFILL;   // idle lanes before a warp takes queue entries
+#ifndef QED_SAMP_LANES
+#define QED_SAMP_LANES 8
+#endif
+constexpr int kSampLanes = QED_SAMP_LANES;
+#ifndef QED_SAMP_BLOCKS
+#define QED_SAMP_BLOCKS 2
+#endif
+// Dynamic shared memory of k_samp: the networks, then a ring per warp.
+constexpr size_t kSampSmemBytes = kMmaSmemBytes + sizeof(EventBuf) * (kLaneThreads / 32);
+static_assert(kMmaSmemBytes % 16 == 0, "ring alignment");
+
 // Event-driven sampler, one lane per particle (sampler mode 2; reading of
 // Sec. 2.2's inverse sampling, with the sub-steps to the next event drawn at
 // once).  A lane holds one of the sampler's particles (e+- in a usable chi
@@ -1410,14 +1556,16 @@ __device__ __forceinline__ void warp_item(const DevParticles& P, const Scratch& 
 // sampler's usable bins continues with rejection: its state goes back to the
 // store and it joins the hot pass's queue (the hot pass runs after this
 // kernel).  Idle lanes take queue entries, one atomic per warp.  Persistent.
-__global__ void __launch_bounds__(kLaneThreads) k_samp(DevParticles P, StepParams SP, Scratch S,
+__global__ void __launch_bounds__(kLaneThreads, QED_SAMP_BLOCKS) k_samp(DevParticles P, StepParams SP, Scratch S,
                                                        DevCtl* ctl) {
     const uint32_t step = step_index(SP);
     __shared__ SharedTables sm;
-    __shared__ float fld[6][kLaneThreads];   // E, B at the lane's row
+    __shared__ LaneFields fld;   // E, B at the lane's row
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     SamplerMma& net = *reinterpret_cast<SamplerMma*>(dyn_smem);   // emission
     SamplerMma& pnet = pair_mma(dyn_smem);                           // pair production
+    const unsigned int n_front = ctl->samp_tail, n_back = ctl->samp_back;
+    if (n_front + n_back == 0u || ctl->status == (int)QED_ERR_TIMEOUT) return;
     stage_tables(sm);
     stage_sampler_mma(net, reinterpret_cast<const __nv_bfloat16*>(SP.net_w), SP.net_wtot,
                       SP.net_rows, SP.net_bins);
@@ -1425,13 +1573,21 @@ __global__ void __launch_bounds__(kLaneThreads) k_samp(DevParticles P, StepParam
         stage_sampler_mma(pnet, reinterpret_cast<const __nv_bfloat16*>(SP.pnet_w), SP.pnet_wtot,
                           SP.net_rows, SP.pnet_bins);
     __syncthreads();
-    if (ctl->status == (int)QED_ERR_TIMEOUT) return;
     constexpr unsigned int kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
+    EventBuf& E = reinterpret_cast<EventBuf*>(dyn_smem + kMmaSmemBytes)[threadIdx.x >> 5];
+    unsigned int n_ev = 0, ev_head = 0;   // events whose children are not written yet
     const uint32_t kw0 = (uint32_t)SP.seed ^ kWaitKeyLo, kw1 = (uint32_t)(SP.seed >> 32) ^ kWaitKeyHi;
-    const unsigned int tail = ctl->samp_tail;
     Stats stats;
-    bool active = false, more = true, photon = false;
+    // spread over the warps as in the hot pass, but half a tile of the network
+    // (8 samples) at least
+    const unsigned int nwarps = gridDim.x * (kLaneThreads / 32);
+    const int cap = (int)min(32u, max((unsigned int)kSampLanes, (n_front + n_back + nwarps - 1u) / nwarps));
+    const unsigned int used = min(nwarps, (n_front + n_back + cap - 1u) / cap);
+    const int cap_front = cap == 32 ? 32 : (int)min((unsigned int)cap, (n_front + used - 1u) / used);
+    bool active = false, need_plan = false, more = true, photon = false, changed = false;
+    bool more_front = n_front != 0u, first = true;   // more_front: lane 0
+    bool in_step = true;
     uint32_t i = 0, s = 0;
     uint64_t id = 0;
     PState st{0.0f, 0.0f, 0.0f};
@@ -1439,46 +1595,39 @@ __global__ void __launch_bounds__(kLaneThreads) k_samp(DevParticles P, StepParam
     Plan pl;
     pl.N = 0;
     float chi = 0.0f, eps = 0.0f, thr = 0.0f;
-    bool removed = false;
-    // after a load or an event: plan the remaining time; false if the lane
-    // is done with the particle (no time left, or handed to rejection)
-    auto plan_lane = [&]() -> bool {
-        pl = plan_particle(SP, sm.sqz_e, sm.sqz_p, photon, st.px, st.py, st.pz,
-                           fld[0][threadIdx.x], fld[1][threadIdx.x], fld[2][threadIdx.x],
-                           fld[3][threadIdx.x], fld[4][threadIdx.x], fld[5][threadIdx.x], t_rem,
-                           &chi, &eps);
-        if (!(eps > 0.0f)) return false;
-        stats.max_N = max(stats.max_N, pl.N);
-        const bool usable = photon ? pl.N >= SP.hot_min && pair_sampler_ok(SP, chi, pl.T)
-                                   : sampler_bin_ok(SP, chi);
-        if (!usable) {
-            // rejection from here on: the hot pass plans again from the store
-            if (!photon) {
-                P.px[i] = st.px;
-                P.py[i] = st.py;
-                P.pz[i] = st.pz;
-            }
-            push_hot(S, ctl, i, s, t_rem, pl.N >= SP.long_min);
-            return false;
-        }
-        stats.plans++;
-        stats.guard += pl.guard ? 1 : 0;
-        const SamplerMma& tab = photon ? pnet : net;
-        thr = fminf(pl.c_h * wtot_at(tab.wtot, tab.nrows, chi), 1.0f);
-        return true;
-    };
     while (true) {
         if (more) {
             const unsigned int idle = __ballot_sync(kAll, !active);
-            if (idle) {
-                unsigned int base = 0;
-                if (lane == 0) base = atomicAdd(&ctl->samp_head, (unsigned int)__popc(idle));
-                base = __shfl_sync(kAll, base, 0);
-                if (base + (unsigned int)__popc(idle) >= tail) more = false;
+            const int room = __popc(idle) - (32 - cap);   // particles short of the cap
+            if (room >= kSampRefill || room == cap) {
+                unsigned int base_f = 0, base_b = 0;
+                int got_f = 0, got_b = 0, last = 0;
+                if (lane == 0) {
+                    if (more_front) {
+                        const unsigned int k = (unsigned int)(first ? cap_front : room);
+                        base_f = atomicAdd(&ctl->samp_head, k);
+                        got_f = base_f < n_front ? (int)min(k, n_front - base_f) : 0;
+                        more_front = base_f + k < n_front;
+                    }
+                    if (got_f < room) {
+                        const unsigned int k = (unsigned int)(room - got_f);
+                        base_b = atomicAdd(&ctl->samp_back_head, k);
+                        got_b = base_b < n_back ? (int)min(k, n_back - base_b) : 0;
+                        last = !more_front && base_b + k >= n_back ? 1 : 0;
+                    }
+                }
+                first = false;
+                got_f = __shfl_sync(kAll, got_f, 0);
+                got_b = __shfl_sync(kAll, got_b, 0);
+                base_f = __shfl_sync(kAll, base_f, 0);
+                base_b = __shfl_sync(kAll, base_b, 0);
+                if (__shfl_sync(kAll, last, 0)) more = false;
                 if (!active) {
-                    const unsigned int q = base + (unsigned int)__popc(idle & ((1u << lane) - 1u));
-                    if (q < tail) {
-                        const HotItem it = S.samp[q];
+                    const int rank = __popc(idle & ((1u << lane) - 1u));
+                    if (rank < got_f + got_b) {
+                        const HotItem it =
+                            S.samp[rank < got_f ? (long long)base_f + rank
+                                                : S.samp_cap - 1 - ((long long)base_b + rank - got_f)];
                         i = it.idx;
                         s = it.s;
                         t_rem = it.t_rem;
@@ -1491,17 +1640,56 @@ __global__ void __launch_bounds__(kLaneThreads) k_samp(DevParticles P, StepParam
                         fld[3][threadIdx.x] = P.Bx[i];
                         fld[4][threadIdx.x] = P.By[i];
                         fld[5][threadIdx.x] = P.Bz[i];
-                        active = plan_lane();
+                        changed = false;
+                        active = need_plan = true;
                     }
                 }
             }
         }
+        // new rows and lanes with an event plan together
+        if (need_plan) {
+            need_plan = false;
+            const Fields F = lane_fields(fld);
+            pl = plan_particle(SP, sm.sqz_e, sm.sqz_p, photon, st.px, st.py, st.pz, F.Ex, F.Ey,
+                               F.Ez, F.Bx, F.By, F.Bz, t_rem, &chi, &eps);
+            active = false;
+            if (eps > 0.0f) {
+                stats.max_N = max(stats.max_N, pl.N);
+                active = photon ? pl.N >= SP.hot_min && pl.T != 0u &&
+                                      sampler_bin(SP.pnet_bins, chi)
+                                : sampler_bin(SP.net_bins, chi);
+                if (active) {
+                    stats.plans++;
+                    stats.guard += pl.guard ? 1 : 0;
+                    const SamplerMma& tab = photon ? pnet : net;
+                    thr = fminf(pl.c_h * wtot_at(tab.wtot, tab.nrows, chi), 1.0f);
+                }
+            }
+            if (!active) {   // no energy left, or rejection from here on
+                if (changed) {
+                    P.px[i] = st.px;
+                    P.py[i] = st.py;
+                    P.pz[i] = st.pz;
+                }
+                // the hot pass plans again from the store
+                if (eps > 0.0f) push_hot(S, ctl, i, s, t_rem, pl.N >= SP.front_min);
+            }
+        }
         if (!__any_sync(kAll, active)) {
-            if (!more) break;
+            if (!more) {
+                if (in_step) __syncthreads_and(0);
+                break;
+            }
             continue;
         }
+        // while there is work for all, the block's warps go through the network
+        // together: its instructions do not fit the caches next to the warps,
+        // and together they are fetched once for all (3.3 against 3.1 ms on 1e6
+        // uniform-field electrons).  The first warp without more work ends it
+        // for all.
+        if (in_step) in_step = __syncthreads_and(more) != 0;
         // the sub-steps to the next event
-        bool ev = false, done = false;
+        bool ev = false;
         uint32_t k = 0;
         float u_net = 0.5f;
         if (active) {
@@ -1510,104 +1698,561 @@ __global__ void __launch_bounds__(kLaneThreads) k_samp(DevParticles P, StepParam
             const float wait = floorf(logf(u01(r.y)) / log1pf(-thr));
             if (!(wait < (float)pl.N && thr > 0.0f)) {   // no event in the rest of the plan
                 stats.substeps += pl.N;
-                s += pl.N;
-                done = true;
+                active = false;
+                if (changed) {
+                    P.px[i] = st.px;
+                    P.py[i] = st.py;
+                    P.pz[i] = st.pz;
+                }
             } else {
                 k = (uint32_t)wait;
                 ev = true;
                 u_net = u01(r.x);
             }
         }
-        if (__any_sync(kAll, ev)) {
-            // the child rows (one photon, or an e- and an e+), reserved first
-            // (one atomic for the warp's events) so that the atomic's latency
-            // overlaps the network
-            long long j = -1;
-            if (ev) j = reserve_rows(P, ctl, photon ? 2 : 1, true);
-            // the emission and the pair network for the lanes with such an
-            // event, each packed into one tile when at most 16 have one
-            const float v0 = log10f(chi) * 0.5f, v1 = mlp_input_u(u_net);
-            float x = 0.0f;
-            if (__any_sync(kAll, ev && !photon))
-                x = mlp_infer_mma_some(net, warp_mma_buf(dyn_smem), ev && !photon, v0, v1);
-            if (__any_sync(kAll, ev && photon)) {
-                const float xp = mlp_infer_mma_some(pnet, warp_mma_buf(dyn_smem), ev && photon,
-                                                    v0, v1);
-                if (photon) x = xp;
-            }
-            if (ev) {
-                const uint32_t s_ev = s + k;
-                stats.substeps += k + 1;
-                if (photon) stats.sampled_p++;
-                else stats.sampled++;
-                const ftime t_after = (k + 1 == pl.N) ? ftime{0.0f, 0.0f}
-                                                      : time_sub_mul(t_rem, k + 1, pl.h);
-                removed = apply_event(P, S, SP, ctl, i, id, photon, x, eps, chi, step, s_ev,
-                                      t_after, st, stats, true, false,
-                                      Fields{fld[0][threadIdx.x], fld[1][threadIdx.x],
-                                             fld[2][threadIdx.x], fld[3][threadIdx.x],
-                                             fld[4][threadIdx.x], fld[5][threadIdx.x]},
-                                      false, j);
-                s = s_ev + 1;
-                t_rem = t_after;
-                if (removed || !time_positive(t_rem)) {
-                    done = true;
-                } else if (!plan_lane()) {
-                    active = false;   // handed to rejection, or no energy left
-                }
-            }
+        const unsigned int em = __ballot_sync(kAll, ev);
+        if (!em) continue;
+        // the emission and the pair network for the lanes with such an event,
+        // each packed into one tile when at most 16 have one (one copy of the
+        // unrolled network: its instructions are fetched anew in every round)
+        const float v0 = log10f(chi) * 0.5f, v1 = mlp_input_u(u_net);
+        float x = 0.0f;
+#pragma unroll 1
+        for (int p = 0; p < 2; ++p) {
+            const bool want = ev && photon == (p != 0);
+            if (!__any_sync(kAll, want)) continue;
+            const float xp = mlp_infer_mma_some(p ? pnet : net, warp_mma_buf(dyn_smem), want, v0,
+                                                v1);
+            if (want) x = xp;
         }
-        if (done) {
+        if (ev) {
+            stats.substeps += k + 1;
+            if (photon) stats.sampled_p++;
+            else stats.sampled++;
+            count_event(stats, photon);
+            t_rem = (k + 1 == pl.N) ? ftime{0.0f, 0.0f} : time_sub_mul(t_rem, k + 1, pl.h);
+            note_event(E, (ev_head + n_ev + __popc(em & ((1u << lane) - 1u))) % kEventBuf, i, id,
+                       photon, x, chi, s + k, t_rem, st, lane_fields(fld));
+            const bool removed = event_recoil(SP, photon, x, eps, st);
+            changed = true;
+            s += k + 1;
+            need_plan = active = !removed && time_positive(t_rem);
             if (removed) {
                 P.type[i] = QED_REMOVED;   // a decayed photon (Algorithm 2)
-            } else if (!photon) {
+            } else if (!active) {
                 P.px[i] = st.px;
                 P.py[i] = st.py;
                 P.pz[i] = st.pz;
             }
-            removed = false;
-            active = false;
         }
+        n_ev += (unsigned int)__popc(em);
+        if (n_ev >= 32u) events_flush(P, S, SP, ctl, E, n_ev, ev_head, step);
     }
+    if (n_ev) events_flush(P, S, SP, ctl, E, n_ev, ev_head, step);
     stats.warp_substeps = stats.substeps;
     flush_stats(stats, ctl);
 }
 
-// Hot pass (rejection).  Long plans (N >= long_min, front of the queue) first,
-// one warp each (warp_item), so that their long chains start early; then the
-// medium plans (back of the queue), one lane each, with the same warp-shared
-// draws as the thread pass but at most kWindow sub-steps per lane and round,
-// so that the draws wasted after an event stay short.  Lanes with an event in
-// the round apply it and re-plan together, so that the event path is paid
-// once per round rather than once per event; lanes whose particle is done
-// take the next queue entries (one atomic per warp).  Persistent: the grid is
-// the resident block count, and a warp leaves when the queue is empty and its
-// lanes are idle.
-// kSampler = 1 (per-sub-step sampler): the sampler's particles (e+- in a
-// usable bin of its chi range) are queued for the warp mode, which evaluates
-// the network (warp_item).  Sampler mode 2 steps its particles in k_samp and
-// runs this kernel's rejection form (kSampler = 0) for the others.
-constexpr uint32_t kWindow = 64;
+// One particle per lane: the hot pass and the tail pass.  Draws are keyed by
+// (id, step, sub-step) and so do not depend on the plan: a lane keeps, for the
+// next windows of 64 sub-steps, the masks of the sub-steps whose acceptance
+// draw is below T_cap, a quarter above its plan's squeeze threshold, and walks
+// along them plan after plan (a re-plan moves the threshold by a few per cent;
+// if it rises above T_cap, the masks are drawn again).  So the draws run in
+// bulk, a window to 32 lanes (the two ballots are the masks) and none of them
+// twice, and what is left on the chain from one event to the next is one
+// evaluation of the next candidates, the recoil and the plan.
+#ifndef QED_WINDOWS
+#define QED_WINDOWS 8
+#endif
+#ifndef QED_DRAW_ILP
+#define QED_DRAW_ILP 4
+#endif
+constexpr int kWindows = QED_WINDOWS;   // windows a lane draws at a time
+constexpr int kDrawIlp = QED_DRAW_ILP;  // windows in flight
+constexpr uint32_t kOwnMax = 8;      // plans of this many sub-steps are drawn by their lane
+struct ListBuf {                     // one per warp
+    DrawKey key[32];
+    uint4 par[32];                   // evaluation: T, b, c_h
+    uint2 mask[kWindows][32];        // candidates among the even and the odd sub-steps of a window
+    uint32_t cand[4][32];            // the next candidates of each lane
+    uint2 draw[32];                  // drawing: first block, last word that passes
+    uint8_t item[32 * kWindows + 8]; // drawing: lane | window << 5
+    uint8_t owner[32];
+};
 
-template <int kSampler, bool kCells = false>
-__global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_lanes(DevParticles P, StepParams SP,
+struct Lane {
+    bool active = false, need_plan = false, photon = false, changed = false, removed = false;
+    bool event = false;              // an accepted event, not yet applied
+    uint32_t i = 0;
+    uint32_t s0 = 0;                 // first sub-step of the plan
+    uint32_t next = 0;               // first sub-step not decided
+    uint32_t w0 = 0, cov = 0;        // the masks start at window w0 and cover the sub-steps below cov
+    uint32_t T_cap = 0;
+    uint32_t s_ev = 0;
+    float x_ev = 0.0f;
+    uint64_t id = 0;
+    PState st{0.0f, 0.0f, 0.0f};
+    ftime t_rem{0.0f, 0.0f};
+    Plan pl;
+    float chi = 0.0f, eps = 0.0f;
+};
+// Start row i at sub-step s with t_rem left.
+__device__ __forceinline__ void lane_take(const DevParticles& P, const StepParams& SP, Lane& L,
+                                          ListBuf& B, LaneFields& f, uint32_t step, uint32_t i,
+                                          bool photon, uint32_t s, ftime t_rem) {
+    const int t = threadIdx.x;
+    L.i = i;
+    L.s0 = s;
+    L.t_rem = t_rem;
+    L.photon = photon;
+    L.id = P.id[i];
+    L.st = PState{P.px[i], P.py[i], P.pz[i]};
+    f[0][t] = P.Ex[i];
+    f[1][t] = P.Ey[i];
+    f[2][t] = P.Ez[i];
+    f[3][t] = P.Bx[i];
+    f[4][t] = P.By[i];
+    f[5][t] = P.Bz[i];
+    B.key[t & 31] = draw_key(L.id, step, SP.draw_keys);
+    L.next = L.cov = s;   // no masks
+    L.T_cap = 0u;
+    L.changed = L.removed = L.event = false;
+    L.active = L.need_plan = true;
+}
+
+// The lane's particle is done: its state goes back to the store.
+__device__ __forceinline__ void lane_finish(const DevParticles& P, Lane& L) {
+    if (L.removed) {
+        P.type[L.i] = QED_REMOVED;
+    } else if (L.changed) {
+        P.px[L.i] = L.st.px;
+        P.py[L.i] = L.st.py;
+        P.pz[L.i] = L.st.pz;
+    }
+    L.active = L.need_plan = false;
+}
+
+// Children of the warp's events: rows reserved, not yet written.
+struct PendingChildren {
+    bool mine = false;               // this lane has some
+    int offset = 0;
+    unsigned long long base = 0;     // on the leader
+    int leader = 0;
+    PState st{0.0f, 0.0f, 0.0f};     // the parent before the event
+};
+
+// First half of the lanes' events: the child rows are reserved (one atomic for
+// the warp, not waited for) and the parents recoil.
+__device__ __forceinline__ PendingChildren events_begin(const DevParticles& P, const StepParams& SP,
+                                                        Lane& L, Stats& stats) {
+    constexpr unsigned int kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    PendingChildren c;
+    const unsigned int m1 = __ballot_sync(kAll, L.event && !L.photon);
+    const unsigned int m2 = __ballot_sync(kAll, L.event && L.photon);
+    if ((m1 | m2) == 0u) return c;
+    c.leader = __ffs(m1 | m2) - 1;
+    if (lane == c.leader)
+        c.base = atomicAdd(reinterpret_cast<unsigned long long*>(P.count),
+                           (unsigned long long)(__popc(m1) + 2 * __popc(m2)));
+    if (L.event) {
+        const unsigned int below = (1u << lane) - 1u;
+        c.mine = true;
+        c.offset = __popc(m1 & below) + 2 * __popc(m2 & below);
+        c.st = L.st;
+        const uint32_t k = L.s_ev - L.s0;
+        stats.substeps += k + 1u;
+        count_event(stats, L.photon);
+        L.t_rem = (k + 1u == L.pl.N) ? ftime{0.0f, 0.0f} : time_sub_mul(L.t_rem, k + 1u, L.pl.h);
+        L.removed = event_recoil(SP, L.photon, L.x_ev, L.eps, L.st);
+        L.changed = true;
+        L.s0 = L.next = L.s_ev + 1u;
+        L.need_plan = !L.removed && time_positive(L.t_rem);
+    }
+    return c;
+}
+
+// The lanes' events: noted for their children, the parents recoil.  n, head:
+// the ring's entries (warp-uniform).
+__device__ __forceinline__ void events_note(const StepParams& SP, Lane& L, EventBuf& E,
+                                            const LaneFields& f, unsigned int& n, unsigned int head, Stats& stats) {
+    const int lane = threadIdx.x & 31;
+    const unsigned int m = __ballot_sync(0xffffffffu, L.event);
+    if (!m) return;
+    if (L.event) {
+        const uint32_t k = L.s_ev - L.s0;
+        stats.substeps += k + 1u;
+        count_event(stats, L.photon);
+        L.t_rem = (k + 1u == L.pl.N) ? ftime{0.0f, 0.0f} : time_sub_mul(L.t_rem, k + 1u, L.pl.h);
+        const unsigned int q = (head + n + __popc(m & ((1u << lane) - 1u))) % kEventBuf;
+        note_event(E, q, L.i, L.id, L.photon, L.x_ev, L.chi, L.s_ev, L.t_rem, L.st, lane_fields(f));
+        L.removed = event_recoil(SP, L.photon, L.x_ev, L.eps, L.st);
+        L.changed = true;
+        L.event = false;
+        L.s0 = L.next = L.s_ev + 1u;
+        L.need_plan = !L.removed && time_positive(L.t_rem);
+        L.active = L.need_plan;   // else done: lane_finish
+    }
+    n += (unsigned int)__popc(m);
+}
+
+// Second half: the children are written (their chi is the parent's before the
+// event, for the log).  Returns the first child's row, or -1.
+__device__ __forceinline__ long long events_end(const DevParticles& P, const Scratch& S,
+                                                const StepParams& SP, DevCtl* ctl, Lane& L,
+                                                const PendingChildren& c, ftime t_after, float chi,
+                                                const LaneFields& f, uint32_t step, ChildMode mode) {
+    const unsigned long long base = __shfl_sync(0xffffffffu, c.base, c.leader);
+    if (!c.mine) return -1;
+    const long long j =
+        check_rows(P, ctl, (long long)(base + (unsigned long long)c.offset), L.photon ? 2 : 1);
+    write_children(P, S, SP, L.i, j, L.id, L.photon, L.x_ev, chi, step, L.s_ev, t_after, c.st,
+                   lane_fields(f), mode);
+    L.event = false;
+    return j;
+}
+
+// Plan the time that is left; true if the particle is done with it: no energy,
+// or no candidate admitted (a zero squeeze threshold: the sub-steps pass
+// without an event).  hand_over (sampler modes): the particle goes elsewhere.
+template <bool kCells>
+__device__ __forceinline__ bool lane_plan(const StepParams& SP, const SharedTables& sm, Lane& L,
+                                          const LaneFields& f, const DevCtl* ctl) {
+    const Fields F = lane_fields(f);
+    L.need_plan = false;
+    L.pl = plan_particle(SP, sm.sqz_e, sm.sqz_p, L.photon, L.st.px, L.st.py, L.st.pz, F.Ex, F.Ey,
+                         F.Ez, F.Bx, F.By, F.Bz, L.t_rem, &L.chi, &L.eps);
+    if (kCells)
+        apply_cell_count(SP, L.pl, sm.sqz_e, sm.sqz_p, L.photon, L.i, ctl->n_init, L.s0, L.t_rem,
+                         L.eps);
+    return !(L.eps > 0.0f);
+}
+__device__ __forceinline__ bool lane_count_plan(Lane& L, Stats& stats) {
+    stats.plans++;
+    stats.guard += L.pl.guard ? 1 : 0;
+    if (L.pl.T == 0u) {
+        stats.substeps += L.pl.N;
+        return true;
+    }
+    if (L.pl.T > L.T_cap) {   // the masks (if any) are not complete for this plan
+        L.T_cap = min(L.pl.T + (L.pl.T >> 2) + 1u, 1u << 23);
+        L.cov = L.s0;
+    }
+    return false;
+}
+
+// Draw the masks of the lanes that have walked through theirs and are not at
+// the end of their plan.  Their windows are listed and drawn one after the
+// other, kDrawIlp at a time (a window's ten multiply rounds are one chain), by
+// all 32 lanes.  A lane whose plan ends within kOwnMax sub-steps draws its few
+// blocks by itself, at the same time as the other such lanes.
+__device__ __forceinline__ void list_draw(ListBuf& B, Lane& L, uint32_t y1, const PhiloxKeys& K) {
+    constexpr unsigned int kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const uint32_t left = L.pl.N - (L.next - L.s0);
+    const bool need = L.active && L.next == L.cov && left != 0u;
+    if (!__any_sync(kAll, need)) return;
+    const uint32_t last_word = (L.T_cap << 9) - 1u;   // (r >> 9) < T_cap, T_cap <= 2^23
+    const uint32_t last = L.next + left - 1u;         // last sub-step of the plan
+    const bool own = need && left <= kOwnMax && (last >> 6) == (L.next >> 6);
+    int nw = 0;
+    if (need) {
+        L.w0 = L.next >> 6;
+        nw = own ? 0 : (int)min((uint32_t)kWindows, (last >> 6) - L.w0 + 1u);
+        L.cov = own ? last + 1u : (L.w0 + (uint32_t)nw) << 6;
+    }
+    if (__any_sync(kAll, own)) {
+        unsigned int mA = 0, mB = 0;
+        uint32_t blk = L.next >> 1;
+        while (__any_sync(kAll, own && blk <= last >> 1)) {
+            if (own && blk <= last >> 1) {
+                const uint2 r = draw_yw(B.key[lane], y1, blk, K);
+                mA |= (r.x <= last_word ? 1u : 0u) << (blk & 31u);
+                mB |= (r.y <= last_word ? 1u : 0u) << (blk & 31u);
+                ++blk;
+            }
+        }
+        if (own) B.mask[0][lane] = make_uint2(mA, mB);
+    }
+    int total = 0;
+#pragma unroll
+    for (int j = 0; j < kWindows; ++j) {
+        const unsigned int m = __ballot_sync(kAll, nw > j);
+        if (nw > j) B.item[total + __popc(m & ((1u << lane) - 1u))] = (uint8_t)(lane | j << 5);
+        total += __popc(m);
+    }
+    if (nw) B.draw[lane] = make_uint2(L.w0 << 5, last_word);
+    if (!total) {
+        __syncwarp();
+        return;
+    }
+    if (lane < kDrawIlp) B.item[total + lane] = (uint8_t)0;   // padding, overwritten below
+    __syncwarp();
+    if (lane < kDrawIlp) B.item[total + lane] = B.item[0];
+    __syncwarp();
+    for (int k = 0; k < total; k += kDrawIlp) {
+        uint4 c[kDrawIlp];
+        uint32_t lim[kDrawIlp];
+        int it[kDrawIlp];
+#pragma unroll
+        for (int q = 0; q < kDrawIlp; ++q) {
+            it[q] = B.item[k + q];
+            const uint2 d = B.draw[it[q] & 31];
+            lim[q] = d.y;
+            c[q] = draw_rounds(B.key[it[q] & 31], y1, d.x + (uint32_t)(it[q] & ~31) + (uint32_t)lane, K);
+        }
+#pragma unroll
+        for (int q = 0; q < kDrawIlp; ++q) {
+            const unsigned int mA = __ballot_sync(kAll, kPhiloxM1 * c[q].z <= lim[q]);
+            const unsigned int mB = __ballot_sync(kAll, kPhiloxM0 * c[q].x <= lim[q]);
+            if (lane == 0) B.mask[it[q] >> 5][it[q] & 31] = make_uint2(mA, mB);
+        }
+    }
+    __syncwarp();
+}
+
+// Test the next candidates of every lane's plan, 1, 2 or 4 of each so that the
+// warp's lanes have one apiece.  Sets L.event for the earliest accepted one.
+// True if the plan ran out without an event.
+__device__ __forceinline__ bool list_test(const SharedTables& sm, ListBuf& B, Lane& L, uint32_t y1,
+                                          const PhiloxKeys& K, unsigned int& cand) {
+    constexpr unsigned int kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int n_on = __popc(__ballot_sync(kAll, L.active));
+    const int lg = n_on <= 8 ? 2 : (n_on <= 16 ? 1 : 0), per = 1 << lg;
+    const uint32_t plan_end = L.s0 + L.pl.N;
+    // the lane's next candidates; t: every candidate before it is among them
+    uint32_t t = L.next;
+    int found = 0;
+    if (L.active) {
+        const uint32_t lim = min(plan_end - L.s0, L.cov - L.s0) + L.s0;
+        uint32_t w = t & ~63u;
+        uint2 c = B.mask[(w >> 6) - L.w0][lane];
+        c.x &= (uint32_t)(0xffffffffull << (((t & 63u) + 1u) >> 1));
+        c.y &= 0xffffffffu << ((t & 63u) >> 1);
+        t = lim;
+        while (true) {
+            if (!(c.x | c.y)) {
+                w += 64u;
+                if (w >= lim) break;
+                c = B.mask[(w >> 6) - L.w0][lane];
+                continue;
+            }
+            const uint32_t a = 2u * (uint32_t)__clz(__brev(c.x));   // 64 and 65: none
+            const uint32_t b = 2u * (uint32_t)__clz(__brev(c.y)) + 1u;
+            const uint32_t s = w + min(a, b);
+            if (s >= lim) break;
+            B.cand[found][lane] = s;
+            if (++found == per) {
+                t = s + 1u;
+                break;
+            }
+            if (a < b) c.x &= c.x - 1u;
+            else c.y &= c.y - 1u;
+        }
+    }
+    const bool any = found > 0;
+    const unsigned int m = __ballot_sync(kAll, any);
+    const int n = __popc(m), rank = __popc(m & ((1u << lane) - 1u));
+    if (n) {
+        if (any) {
+            B.owner[rank] = (uint8_t)lane;
+            B.par[lane] = make_uint4(L.pl.T, __float_as_uint(L.pl.b),
+                                     __float_as_uint(L.photon ? -L.pl.c_h : L.pl.c_h),
+                                     (uint32_t)found);
+        }
+        __syncwarp();
+        const int r = lane >> lg, k = lane & (per - 1);
+        bool cnd = false, acc = false;
+        uint32_t s = 0;
+        float x = 0.0f;
+        if (r < n) {
+            const int o = B.owner[r];
+            const uint4 p = B.par[o];
+            if (k < (int)p.w) {
+                s = B.cand[k][o];
+                const uint4 w = draw_block(B.key[o], y1, s >> 1, K);
+                const uint32_t yw = (s & 1u) ? w.w : w.y;
+                cnd = (yw >> 9) < p.x;
+                if (cnd) {
+                    x = u01((s & 1u) ? w.z : w.x);
+                    const float c_h = __uint_as_float(p.z);
+                    float dtmp;
+                    acc = u01(yw) < acceptance(sm.syn, c_h < 0.0f, __uint_as_float(p.y),
+                                               fabsf(c_h), x, &dtmp);
+                }
+            }
+        }
+        const unsigned int group = (1u << per) - 1u;
+        const int sh = any ? rank << lg : 0;
+        const unsigned int g_acc = __ballot_sync(kAll, acc) >> sh & group;
+        const unsigned int g_cnd = __ballot_sync(kAll, cnd) >> sh & group;
+        const int win = g_acc ? __ffs(g_acc) - 1 : 0;
+        const uint32_t s_ev = __shfl_sync(kAll, s, (sh + win) & 31);
+        const float x_ev = __shfl_sync(kAll, x, (sh + win) & 31);
+        if (any) {
+            L.event = g_acc != 0u;
+            cand += __popc(L.event ? g_cnd & ((2u << win) - 1u) : g_cnd);
+            L.s_ev = s_ev;
+            L.x_ev = x_ev;
+        }
+        if (L.event) return false;
+    }
+    L.next = t;
+    return L.active && t - L.s0 == L.pl.N;
+}
+
+#ifndef QED_HOT_LANES
+#define QED_HOT_LANES 16
+#endif
+#ifndef QED_HOT_MANY
+#define QED_HOT_MANY 256
+#endif
+#ifndef QED_HOT_REFILL
+#define QED_HOT_REFILL 8
+#endif
+#ifndef QED_HOT_MIN_BLOCKS
+#define QED_HOT_MIN_BLOCKS 2
+#endif
+constexpr unsigned int kHotLanes = QED_HOT_LANES;   // most particles a warp of the hot pass holds,
+constexpr int kHotMany = QED_HOT_MANY;       // 32 with a queue of this many times the warps
+constexpr int kHotRefill = QED_HOT_REFILL;   // idle lanes before it takes queue entries
+constexpr uint32_t kWindow = 64;             // mode 1's medium plans: sub-steps per lane and round
+
+// Hot pass (rejection).  One particle per lane.  A round applies the events
+// the last one found, plans them and the rows just taken together, draws the
+// lists that have run out and tests the next candidates.  Persistent: the
+// grid is the resident block count.  A warp first takes its share of the long
+// plans (N >= long_min, front of the queue array), so that their chains start
+// early, then medium plans (back of the array); lanes whose particle is done
+// take further entries, kHotRefill at a time (one atomic per warp and queue).
+// The entries are spread evenly: a warp takes no more than the queue's length
+// over the number of warps.
+struct HotSmem {
+    SharedTables tables;
+    ListBuf list[kLaneThreads / 32];
+    EventBuf events[kLaneThreads / 32];
+    LaneFields fld;
+};
+
+template <bool kCells>
+__global__ void __launch_bounds__(kLaneThreads, QED_HOT_MIN_BLOCKS) k_hot(DevParticles P, StepParams SP,
+                                                                 Scratch S, DevCtl* ctl) {
+    const uint32_t step = step_index(SP);
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    HotSmem& hs = *reinterpret_cast<HotSmem*>(dyn_smem);
+    SharedTables& sm = hs.tables;
+    LaneFields& fld = hs.fld;
+    const unsigned int n_long = ctl->hot_tail, n_med = ctl->med_tail;
+    if (n_long + n_med == 0u || ctl->status == (int)QED_ERR_TIMEOUT) return;
+    stage_tables(sm);
+    __syncthreads();
+    constexpr unsigned int kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    ListBuf& B = hs.list[threadIdx.x >> 5];
+    EventBuf& E = hs.events[threadIdx.x >> 5];
+    unsigned int n_ev = 0, ev_head = 0;   // events whose children are not written yet
+    const uint32_t y1 = draw_y1(step, SP.draw_keys);
+    const unsigned int nwarps = gridDim.x * (kLaneThreads / 32);
+    const unsigned int most = (n_long + n_med) / nwarps >= (unsigned int)kHotMany ? 32u : kHotLanes;
+    const int cap_long = (int)min(most, (n_long + nwarps - 1u) / nwarps);
+    const int cap = (int)min(most, (n_long + n_med + nwarps - 1u) / nwarps);
+    bool more_long = n_long != 0u, more_med = n_med != 0u, first = true;   // warp-uniform
+    Stats stats;
+    Lane L;
+    L.pl.N = 0;
+    L.pl.T = 0;
+    L.pl.b = L.pl.c_h = 0.0f;
+    while (true) {
+        if (more_long || more_med) {
+            const unsigned int idle = __ballot_sync(kAll, !L.active);
+            const int room = __popc(idle) - (32 - cap);   // particles short of the cap
+            if (room >= kHotRefill || room == cap) {
+                unsigned int base_l = 0, base_m = 0;
+                int got_l = 0, got_m = 0, flags = 0;
+                if (lane == 0) {
+                    if (more_long) {
+                        const unsigned int k = (unsigned int)(first ? cap_long : room);
+                        base_l = atomicAdd(&ctl->hot_head, k);
+                        got_l = base_l < n_long ? (int)min(k, n_long - base_l) : 0;
+                        flags |= base_l + k >= n_long ? 1 : 0;
+                    }
+                    if (more_med && got_l < room) {
+                        const unsigned int k = (unsigned int)(room - got_l);
+                        base_m = atomicAdd(&ctl->med_head, k);
+                        got_m = base_m < n_med ? (int)min(k, n_med - base_m) : 0;
+                        flags |= base_m + k >= n_med ? 2 : 0;
+                    }
+                }
+                got_l = __shfl_sync(kAll, got_l, 0);
+                got_m = __shfl_sync(kAll, got_m, 0);
+                base_l = __shfl_sync(kAll, base_l, 0);
+                base_m = __shfl_sync(kAll, base_m, 0);
+                flags = __shfl_sync(kAll, flags, 0);
+                if (flags & 1) more_long = false;
+                if (flags & 2) more_med = false;
+                first = false;
+                const int rank = __popc(idle & ((1u << lane) - 1u));
+                if (!L.active && rank < got_l + got_m) {
+                    const HotItem it =
+                        S.hot[rank < got_l ? (long long)base_l + rank
+                                           : S.hot_cap - 1 - ((long long)base_m + rank - got_l)];
+                    lane_take(P, SP, L, B, fld, step, it.idx, P.type[it.idx] == QED_PHOTON, it.s,
+                              it.t_rem);
+                }
+            }
+        }
+        const bool had = L.active;
+        events_note(SP, L, E, fld, n_ev, ev_head, stats);
+        bool done = had && !L.active;
+        if (L.need_plan) {
+            done = lane_plan<kCells>(SP, sm, L, fld, ctl);
+            if (!done) {
+                stats.max_N = max(stats.max_N, L.pl.N);
+                done = lane_count_plan(L, stats);
+            }
+        }
+        if (done) lane_finish(P, L);
+        if (n_ev >= 32u) events_flush(P, S, SP, ctl, E, n_ev, ev_head, step);
+        if (!__any_sync(kAll, L.active)) {
+            if (!more_long && !more_med) break;
+            continue;
+        }
+        list_draw(B, L, y1, SP.draw_keys);
+        if (list_test(sm, B, L, y1, SP.draw_keys, stats.cand)) {
+            stats.substeps += L.pl.N;
+            lane_finish(P, L);
+        }
+        __syncwarp();   // the list buffer is reused by the next round
+    }
+    if (n_ev) events_flush(P, S, SP, ctl, E, n_ev, ev_head, step);
+    stats.warp_substeps = stats.substeps;   // every sub-step of this kernel is a hot-pass one
+    flush_stats(stats, ctl);
+}
+
+// Hot pass of the per-sub-step sampler (mode 1).  Long plans and the sampler's
+// particles (e+- in a usable bin of its chi range; front of the queue) first,
+// one warp each (warp_item, which evaluates the network); then the medium
+// plans (back of the queue), one lane each, with warp-shared draws over at
+// most kWindow sub-steps per lane and round.  Sampler mode 2 steps its
+// particles in k_samp and runs k_hot for the others.
+__global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_net(DevParticles P, StepParams SP,
                                                                  Scratch S, DevCtl* ctl) {
     const uint32_t step = step_index(SP);
     __shared__ SharedTables sm;
-    __shared__ uint32_t first_acc[kLaneThreads];
+    __shared__ DrawBuf draw_buf[kLaneThreads / 32];
     extern __shared__ __align__(16) unsigned char dyn_smem[];
-    // sampler mode 2 runs its network in k_samp; its generations use k_hot_lanes<0>
-    static_assert(kSampler == 0 || kSampler == 1, "hot pass: rejection or sampler mode 1");
     stage_tables(sm);
-    if (kSampler == 1)
-        stage_sampler(*reinterpret_cast<SamplerSmem*>(dyn_smem),
-                      reinterpret_cast<const __nv_bfloat16*>(SP.net_w), SP.net_wtot, SP.net_rows,
-                      SP.net_bins);
+    stage_sampler(*reinterpret_cast<SamplerSmem*>(dyn_smem),
+                  reinterpret_cast<const __nv_bfloat16*>(SP.net_w), SP.net_wtot, SP.net_rows,
+                  SP.net_bins);
     __syncthreads();
     if (ctl->status == (int)QED_ERR_TIMEOUT) return;
     constexpr unsigned int kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    uint32_t* facc = first_acc + (threadIdx.x & ~31);
+    DrawBuf& B = draw_buf[threadIdx.x >> 5];
+    const uint32_t y1 = draw_y1(step, SP.draw_keys);
     const uint32_t k0 = (uint32_t)SP.seed, k1 = (uint32_t)(SP.seed >> 32);
     Stats stats;
     {
@@ -1620,8 +2265,7 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_lane
             if (lane == 0) q = atomicAdd(&ctl->hot_head, 1u);
             q = __shfl_sync(kAll, q, 0);
             if (q >= long_tail) break;
-            warp_item<kSampler, kCells>(P, S, SP, ctl, sm, dyn_smem, S.hot[q], step, k0, k1, wstats, wcand,
-                                false);
+            warp_item<1>(P, S, SP, ctl, sm, dyn_smem, S.hot[q], step, k0, k1, wstats, wcand, false);
         }
         if (lane == 0) stats = wstats;
         stats.cand = wcand;
@@ -1659,6 +2303,7 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_lane
                         t_rem = it.t_rem;
                         photon = P.type[i] == QED_PHOTON;
                         id = P.id[i];
+                        B.key[lane] = draw_key(id, step, SP.draw_keys);
                         st = PState{P.px[i], P.py[i], P.pz[i]};
                         Ex = P.Ex[i]; Ey = P.Ey[i]; Ez = P.Ez[i];
                         Bx = P.Bx[i]; By = P.By[i]; Bz = P.Bz[i];
@@ -1671,9 +2316,6 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_lane
         if (planned) {
             pl = plan_particle(SP, sm.sqz_e, sm.sqz_p, photon, st.px, st.py, st.pz, Ex, Ey, Ez,
                                Bx, By, Bz, t_rem, &chi, &eps);
-            if (kCells)
-                apply_cell_count(SP, pl, sm.sqz_e, sm.sqz_p, photon, i, ctl->n_init, s, t_rem,
-                                 eps);
             if (eps > 0.0f) {
                 active = true;
                 k_done = 0;
@@ -1693,10 +2335,9 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_lane
         }
         const uint32_t n_win = active ? min(kWindow, pl.N - k_done) : 0u;
         const uint32_t s_end = s + n_win;
-        warp_draw_round(sm, facc, active, s, s_end, pl.T, pl.b, pl.c_h, id, photon, step, SP.draw_keys,
-                        stats.cand);
+        draw_round(sm, B, active, s, s_end, pl.T, pl.b, pl.c_h, photon, y1, SP.draw_keys, stats.cand);
         if (active) {
-            const uint32_t s_ev = facc[lane];
+            const uint32_t s_ev = B.facc[lane];
             bool done = false;
             if (s_ev == kNoEvent) {
                 stats.substeps += n_win;
@@ -1706,11 +2347,11 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_lane
             } else {
                 const uint32_t k = k_done + (s_ev - s);
                 stats.substeps += s_ev - s + 1u;
-                const float x = draw_x(id, step, s_ev, SP.draw_keys);
+                const float x = draw_x(B.key[lane], y1, s_ev, SP.draw_keys);
                 const ftime t_after = (k + 1u == pl.N) ? ftime{0.0f, 0.0f}
                                                        : time_sub_mul(t_rem, k + 1u, pl.h);
                 removed = apply_event(P, S, SP, ctl, i, id, photon, x, eps, chi, step, s_ev,
-                                      t_after, st, stats, true, false,
+                                      t_after, st, stats, false,
                                       Fields{Ex, Ey, Ez, Bx, By, Bz}, false);
                 changed = true;
                 s = s_ev + 1u;
@@ -1745,7 +2386,7 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_lane
                 active = false;
             }
         }
-        __syncwarp();   // facc is reset by the next round
+        __syncwarp();   // the draw buffer is reused by the next round
     }
     stats.warp_substeps = stats.substeps;   // every sub-step of this kernel is a hot-pass one
     flush_stats(stats, ctl);
@@ -1756,12 +2397,13 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_lane
 // generations stop: a thread pass (k_cold) over that generation, then one
 // launch of this persistent kernel finishes the step, taking the thread pass's
 // queue and every child appended from then on (rows n0 and up) as they come.
-// Each warp takes, in order,
-//   1. a long plan from the queue (N >= long_min, or a sampler particle), stepped
-//      by the whole warp (warp_item);
-//   2. for its idle lanes, child rows appended so far, then the thread pass's
-//      medium plans, one lane each, drawn with the warp-shared rounds in windows
-//      of kWindow sub-steps.
+// As in the hot pass, a lane holds a particle, the warp draws the windows of
+// its lanes together, and lanes with an event or a new row plan together.  A
+// warp takes, in order, its share of the queue's long plans (each warp the
+// queue's length over the number of warps), child rows appended so far, then
+// the queue's medium plans.  With a learned sampler the long entries (the
+// sampler's particles among them) are stepped by a whole warp each
+// (warp_item), and so are the sampler's particles that appear later.
 // A child row is published by its writer (type byte last, after a fence); a
 // lane that takes a row still being written waits for it.  Work units are the
 // thread pass's queue entries and the child rows; the pass ends when every
@@ -1777,6 +2419,30 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_lane
 // returns.
 // ---------------------------------------------------------------------------
 constexpr unsigned long long kWaitNsDefault = 1000000000ull;   // idle time before giving up: 1 s
+#ifndef QED_TAIL_CLAIM
+#define QED_TAIL_CLAIM 8
+#endif
+#ifndef QED_TAIL_SPREAD
+#define QED_TAIL_SPREAD 256
+#endif
+#ifndef QED_TAIL_ROUNDS
+#define QED_TAIL_ROUNDS 8
+#endif
+#ifndef QED_TAIL_NAP
+#define QED_TAIL_NAP 4
+#endif
+#ifndef QED_TAIL_WARPS
+#define QED_TAIL_WARPS 8
+#endif
+#ifndef QED_TAIL_MINB
+#define QED_TAIL_MINB 8
+#endif
+constexpr unsigned int kTailMinBlocks = QED_TAIL_MINB;   // blocks that stay: these and
+constexpr unsigned int kTailWarps = QED_TAIL_WARPS;   // this many warps per queue entry (the
+                                         // polls of idle warps slow the others)
+constexpr int kTailClaim = QED_TAIL_CLAIM;   // idle lanes before a busy warp takes rows,
+constexpr unsigned int kTailRounds = QED_TAIL_ROUNDS;   // and rounds between two looks
+constexpr unsigned int kTailSpread = QED_TAIL_SPREAD;   // warps that share the rows on offer
 
 // Queue a long plan: the entry's row index is written last (readers wait for it).
 __device__ __forceinline__ void push_long(const Scratch& S, DevCtl* ctl, unsigned int cold_long,
@@ -1791,15 +2457,20 @@ __device__ __forceinline__ void push_long(const Scratch& S, DevCtl* ctl, unsigne
 
 template <int kSampler, bool kCells = false>
 // Two resident blocks per SM (128 registers, no spills): the tail pass is
-// bound by latency, not by the number of warps (three blocks at 80 registers
-// spilled 434 bytes a thread and measured 0.8% slower per step).
+// bound by latency, not by the number of warps.
 __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepParams SP,
                                                             Scratch S, DevCtl* ctl) {
     const uint32_t step = step_index(SP);
     __shared__ SharedTables sm;
-    __shared__ uint32_t first_acc[kLaneThreads];
-    __shared__ float fld[6][kLaneThreads];   // E, B at the lane's row (read at plans and events)
+    __shared__ ListBuf list_buf[kLaneThreads / 32];
+    __shared__ LaneFields fld;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
+    // the thread pass's queue (fixed during this kernel)
+    const unsigned int cold_long = ctl->hot_tail, cold_med = ctl->med_tail;
+    const unsigned long long units0 = (unsigned long long)cold_long + cold_med;
+    const unsigned int blocks = (unsigned int)min(
+        (unsigned long long)gridDim.x, kTailMinBlocks + units0 * kTailWarps / (kLaneThreads / 32));
+    if (ctl->skip || blockIdx.x >= blocks) return;
     stage_tables(sm);
     if (kSampler == 1)
         stage_sampler(*reinterpret_cast<SamplerSmem*>(dyn_smem),
@@ -1814,40 +2485,35 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
                               SP.pnet_wtot, SP.net_rows, SP.pnet_bins);
     }
     __syncthreads();
-    if (ctl->skip) return;
     constexpr unsigned int kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    uint32_t* facc = first_acc + (threadIdx.x & ~31);
-    const uint32_t k0 = (uint32_t)SP.seed, k1 = (uint32_t)(SP.seed >> 32);
+    ListBuf& B = list_buf[threadIdx.x >> 5];
+    const uint32_t y1 = draw_y1(step, SP.draw_keys);
     const unsigned long long n0 = (unsigned long long)ctl->n0;
     const bool cascade = SP.cascade != 0;
-    // the thread pass's queue (fixed during this kernel)
-    const unsigned int cold_long = ctl->hot_tail, cold_med = ctl->med_tail;
-    const unsigned long long units0 = (unsigned long long)cold_long + cold_med;
+    const unsigned int nwarps = blocks * (kLaneThreads / 32);
+    const unsigned int share_long = min(32u, (cold_long + nwarps - 1u) / nwarps);
+    const unsigned int share_med = min(32u, (cold_med + nwarps - 1u) / nwarps);
     Stats stats;                 // per lane; the warp mode counts on lane 0
     unsigned int done = 0;       // units this lane completed, not yet added to ctl->finished
-    bool active = false, waiting = false, child = false;
-    bool photon = false, changed = false, removed = false;
-    long long i = 0;
-    uint64_t id = 0;
-    PState st{0.0f, 0.0f, 0.0f};
-    ftime t_rem{0.0f, 0.0f};
-    uint32_t s = 0, k_done = 0;
-    Plan pl;
-    pl.N = 0;
-    pl.T = 0;
-    pl.b = pl.c_h = 0.0f;
-    float chi = 0.0f, eps = 0.0f;
+    bool waiting = false, child = false;
+    uint32_t row = 0;            // waiting: a child's row, or a queue entry's position
+    Lane L;
+    L.pl.N = 0;
+    L.pl.T = 0;
+    L.pl.b = L.pl.c_h = 0.0f;
     unsigned int idle = 0, rounds = 0;
     unsigned long long idle_ns = 0, seen = 0;
     unsigned int ticket = kNoItem;   // lane 0: long-queue entry taken, not yet pushed
     unsigned long long pend_lo = 0, pend_hi = 0;   // lane 0: child indices taken, not handed out
+    bool more_long = kSampler == 0 && cold_long != 0u, more_med = cold_med != 0u;   // lane 0
     bool timed_out = false;
     while (true) {
-        // ---- 1. a long plan, stepped by the whole warp.  Lane 0 takes a ticket
-        // with one atomic add when the queue looks non-empty; a ticket past the
-        // tail is kept until its entry is pushed (void if the step ends first).
-        {
+        // ---- 1. (sampler modes) a long plan, stepped by the whole warp.  Lane 0
+        // takes a ticket with one atomic add when the queue looks non-empty; a
+        // ticket past the tail is kept until its entry is pushed (void if the
+        // step ends first).
+        if (kSampler != 0) {
             int got = 0;
             unsigned int q = 0;
             if (lane == 0) {
@@ -1886,38 +2552,56 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
                 it.s = __shfl_sync(kAll, it.s, 0);
                 it.t_rem.hi = __shfl_sync(kAll, it.t_rem.hi, 0);
                 it.t_rem.lo = __shfl_sync(kAll, it.t_rem.lo, 0);
-                warp_item<kSampler, kCells>(P, S, SP, ctl, sm, dyn_smem, it, step, k0, k1, stats, stats.cand,
-                                    true);
+                const uint32_t k0 = (uint32_t)SP.seed, k1 = (uint32_t)(SP.seed >> 32);
+                warp_item<kSampler == 0 ? 1 : kSampler>(P, S, SP, ctl, sm, dyn_smem, it, step, k0,
+                                                        k1, stats, stats.cand, true);
                 if (lane == 0) ++done;
                 idle = 0;
                 idle_ns = 0;
                 continue;
             }
         }
-        // ---- 2. rows for the idle lanes: children first, then the medium plans.
-        // Lane 0 takes child indices with one atomic add into a pending range
-        // and hands a lane only an index whose row is reserved already (the
-        // rest stay pending; indices never reserved are void when the step
-        // ends); medium plans come the same way, an index past their count is
-        // dropped.
+        // ---- 2. rows for the idle lanes: the queue's long plans, children, the
+        // queue's medium plans.  Lane 0 takes child indices with one atomic add
+        // into a pending range and hands a lane only an index whose row is
+        // reserved already (the rest stay pending; indices never reserved are
+        // void when the step ends); queue entries come the same way, an index
+        // past their count is dropped.  A warp takes a share of what is on
+        // offer (a round's time grows with the particles it steps, and other
+        // warps are idle when there is little), and a busy warp looks only when
+        // kTailClaim of its lanes are free, and not in every round.
         {
-            const unsigned int free_lanes = __ballot_sync(kAll, !active && !waiting);
-            if (free_lanes) {
-                const int want = __popc(free_lanes);
-                unsigned long long base_c = 0, base_i = 0;
-                int got_c = 0, got_i = 0;
+            const unsigned int free_lanes = __ballot_sync(kAll, !L.active && !waiting);
+            const bool look = free_lanes == kAll ||
+                              (__popc(free_lanes) >= kTailClaim && rounds % kTailRounds == 0u);
+            if (look || (free_lanes && __any_sync(kAll, lane == 0 && pend_lo < pend_hi))) {
+                const unsigned int want = (unsigned int)__popc(free_lanes);
+                unsigned long long base_c = 0;
+                unsigned int base_l = 0, base_m = 0;
+                int got_l = 0, got_c = 0, got_m = 0;
                 if (lane == 0) {
-                    if (cascade) {
-                        const unsigned long long stored = stored_rows(P);
-                        if (pend_lo == pend_hi) {
-                            const unsigned long long ch =
-                                *reinterpret_cast<volatile unsigned long long*>(&ctl->child_head);
-                            if (ch < stored) {
-                                const unsigned long long k =
-                                    min((unsigned long long)want, stored - ch);
-                                pend_lo = atomicAdd(&ctl->child_head, k);
-                                pend_hi = pend_lo + k;
-                            }
+                    // the control words are read at once, one round trip
+                    const unsigned int h_long =
+                        more_long ? *reinterpret_cast<volatile unsigned int*>(&ctl->hot_head) : 0u;
+                    const unsigned int h_med =
+                        more_med ? *reinterpret_cast<volatile unsigned int*>(&ctl->med_head) : 0u;
+                    const unsigned long long ch =
+                        *reinterpret_cast<volatile unsigned long long*>(&ctl->child_head);
+                    const unsigned long long stored = cascade ? stored_rows(P) : n0;
+                    more_long = more_long && h_long < cold_long;
+                    more_med = more_med && h_med < cold_med;
+                    if (more_long) {
+                        const unsigned int k = min(want, share_long);
+                        base_l = atomicAdd(&ctl->hot_head, k);
+                        got_l = base_l < cold_long ? (int)min(k, cold_long - base_l) : 0;
+                    }
+                    if (got_l == 0) {
+                        if (pend_lo == pend_hi && ch < stored) {
+                            const unsigned long long k =
+                                min((unsigned long long)want,
+                                    (stored - ch + kTailSpread - 1) / kTailSpread);
+                            pend_lo = atomicAdd(&ctl->child_head, k);
+                            pend_hi = pend_lo + k;
                         }
                         if (pend_lo < pend_hi && pend_lo < stored) {
                             got_c = (int)min((unsigned long long)want, min(pend_hi, stored) - pend_lo);
@@ -1925,91 +2609,107 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
                             pend_lo += (unsigned long long)got_c;
                         }
                     }
-                    if (got_c < want &&
-                        *reinterpret_cast<volatile unsigned int*>(&ctl->med_head) < cold_med) {
-                        const unsigned int k = (unsigned int)(want - got_c);
-                        const unsigned int b = atomicAdd(&ctl->med_head, k);
-                        base_i = b;
-                        got_i = b < cold_med ? (int)min(k, cold_med - b) : 0;
+                    if (got_l == 0 && got_c == 0 && more_med) {
+                        const unsigned int k = min(want, share_med);
+                        base_m = atomicAdd(&ctl->med_head, k);
+                        got_m = base_m < cold_med ? (int)min(k, cold_med - base_m) : 0;
                     }
                 }
-                got_c = __shfl_sync(kAll, got_c, 0);
-                got_i = __shfl_sync(kAll, got_i, 0);
-                if (got_c + got_i) {
-                    base_c = __shfl_sync(kAll, base_c, 0);
-                    base_i = __shfl_sync(kAll, base_i, 0);
+                // one kind per claim
+                const int got = __shfl_sync(kAll, got_l + got_c + got_m, 0);
+                if (got) {
+                    const int kind = __shfl_sync(kAll, got_l ? 0 : (got_c ? 1 : 2), 0);
+                    const uint32_t base = __shfl_sync(
+                        kAll, got_l ? base_l : (got_c ? (uint32_t)base_c : base_m), 0);
                     const int rank = __popc(free_lanes & ((1u << lane) - 1u));
-                    if (!active && !waiting && rank < got_c + got_i) {
-                        // a child's row index, or a medium plan's queue position
-                        child = rank < got_c;
-                        i = (long long)(child ? base_c + rank : base_i + (rank - got_c));
+                    if (!L.active && !waiting && rank < got) {
+                        // a child's row, or a queue entry's row, sub-step and time
+                        child = kind == 1;
+                        row = base + (uint32_t)rank;
                         waiting = true;
-                    }
-                }
-            }
-        }
-        // ---- 3. lanes holding a row: load and plan it once it is written
-        if (waiting) {
-            uint32_t s0 = 0;
-            if (!child) {   // a medium plan: its row, first sub-step and remaining time
-                const HotItem it = S.hot[S.hot_cap - 1 - i];
-                i = it.idx;
-                s0 = it.s;
-                t_rem = it.t_rem;
-            }
-            const uint8_t ty = *reinterpret_cast<volatile uint8_t*>(P.type + i);
-            if (!child || ty != kNotReady) {
-                if (child) {
-                    __threadfence();
-                    t_rem = S.t_rem[i];
-                }
-                waiting = false;
-                photon = ty == QED_PHOTON;
-                bool work = ty <= QED_PHOTON && process_enabled(SP, photon) && time_positive(t_rem);
-                if (work) {
-                    id = P.id[i];
-                    st = PState{P.px[i], P.py[i], P.pz[i]};
-                    fld[0][threadIdx.x] = P.Ex[i];
-                    fld[1][threadIdx.x] = P.Ey[i];
-                    fld[2][threadIdx.x] = P.Ez[i];
-                    fld[3][threadIdx.x] = P.Bx[i];
-                    fld[4][threadIdx.x] = P.By[i];
-                    fld[5][threadIdx.x] = P.Bz[i];
-                    s = s0;
-                    changed = removed = false;
-                    pl = plan_particle(SP, sm.sqz_e, sm.sqz_p, photon, st.px, st.py, st.pz,
-                                       fld[0][threadIdx.x], fld[1][threadIdx.x],
-                                       fld[2][threadIdx.x], fld[3][threadIdx.x],
-                                       fld[4][threadIdx.x], fld[5][threadIdx.x], t_rem, &chi, &eps);
-                    if (kCells)
-                        apply_cell_count(SP, pl, sm.sqz_e, sm.sqz_p, photon, i, ctl->n_init, s,
-                                         t_rem, eps);
-                    work = eps > 0.0f;
-                }
-                if (!work) {
-                    ++done;
-                } else {
-                    stats.max_N = max(stats.max_N, pl.N);
-                    if (pl.N >= SP.long_min || (!photon && sampler_bin_ok(SP, chi)) ||
-                        (kSampler == 2 && photon && pl.N >= SP.hot_min &&
-                         pair_sampler_ok(SP, chi, pl.T))) {
-                        push_long(S, ctl, cold_long, i, s, t_rem);   // the warp mode plans again
-                    } else {
-                        stats.plans++;
-                        stats.guard += pl.guard ? 1 : 0;
-                        if (pl.T == 0u) {   // no candidates: the plan passes without an event
-                            stats.substeps += pl.N;
-                            ++done;
-                        } else {
-                            active = true;
-                            k_done = 0;
+                        if (!child) {
+                            const HotItem it = S.hot[kind == 0 ? (long long)row
+                                                               : S.hot_cap - 1 - (long long)row];
+                            row = it.idx;
+                            L.s0 = it.s;
+                            L.t_rem = it.t_rem;
                         }
                     }
                 }
             }
         }
-        // ---- 4. nothing to draw: wait for work, or finish
-        if (!__any_sync(kAll, active)) {
+        // ---- 3. lanes holding a row: load it once it is written
+        if (waiting) {
+            const uint8_t ty = *reinterpret_cast<volatile uint8_t*>(P.type + row);
+            if (!child || ty != kNotReady) {
+                if (child) {
+                    __threadfence();
+                    L.t_rem = S.t_rem[row];
+                    L.s0 = 0;
+                }
+                waiting = false;
+                const bool photon = ty == QED_PHOTON;
+                if (ty <= QED_PHOTON && process_enabled(SP, photon) && time_positive(L.t_rem))
+                    lane_take(P, SP, L, B, fld, step, row, photon, L.s0, L.t_rem);
+                else
+                    ++done;
+            }
+        }
+        // ---- 4. the events of the last round; they and new rows plan together
+        const PendingChildren kids = events_begin(P, SP, L, stats);
+        const ftime t_kids = L.t_rem;
+        const float chi_kids = L.chi;
+        bool fin = kids.mine && !L.need_plan;
+        bool hand_over = false;
+        if (L.need_plan) {
+            fin = lane_plan<kCells>(SP, sm, L, fld, ctl);
+            if (!fin) {
+                stats.max_N = max(stats.max_N, L.pl.N);
+                hand_over = kSampler != 0 &&
+                            ((!L.photon && sampler_bin_ok(SP, L.chi)) ||
+                             (kSampler == 2 && L.photon && L.pl.N >= SP.hot_min &&
+                              pair_sampler_ok(SP, L.chi, L.pl.T)));
+                if (!hand_over) fin = lane_count_plan(L, stats);
+            }
+        }
+        const long long j_kids =
+            events_end(P, S, SP, ctl, L, kids, t_kids, chi_kids, fld, step, kDeferred);
+        if (hand_over) {   // the warp mode plans again; the particle's state goes with the row
+            lane_finish(P, L);
+            push_long(S, ctl, cold_long, L.i, L.s0, L.t_rem);
+        } else if (fin) {
+            lane_finish(P, L);
+            ++done;
+        }
+        const unsigned int on = __ballot_sync(kAll, L.active);
+        if (on) {
+            // ---- 5. the lists that have run out are drawn, the next candidates tested
+            idle = 0;
+            idle_ns = 0;
+            if (++rounds == kBeatRounds) {
+                rounds = 0;
+                if (lane == 0) atomicAdd(&ctl->beat, 1ull);
+            }
+            list_draw(B, L, y1, SP.draw_keys);
+            if (list_test(sm, B, L, y1, SP.draw_keys, stats.cand)) {
+                stats.substeps += L.pl.N;
+                lane_finish(P, L);
+                ++done;
+            }
+        }
+        // the children's rows have been written since the last fence: publish
+        // them (after the draws, so that the fence finds the stores done)
+        if (__any_sync(kAll, kids.mine)) {
+            __threadfence();
+            if (j_kids >= 0) {
+                // kids.mine: the lane's photon flag is still the parent's
+                *reinterpret_cast<volatile uint8_t*>(P.type + j_kids) = child_type(L.photon, 0);
+                if (L.photon)
+                    *reinterpret_cast<volatile uint8_t*>(P.type + j_kids + 1) = child_type(true, 1);
+            }
+        }
+        // ---- 6. nothing to draw: wait for work, or finish
+        if (!on) {
             // lanes waiting for a row still being written hold the warp
             const bool hold = __any_sync(kAll, waiting);
             bool finish = false;
@@ -2041,7 +2741,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
                 seen = progress;
                 idle_ns = 0;
             }
-            const unsigned int nap = hold ? 64u : 256u << min(idle, 4u);
+            const unsigned int nap = hold ? 64u : 256u << min(idle, (unsigned int)QED_TAIL_NAP);
             ++idle;
             idle_ns += nap;
             if (idle_ns > SP.wait_ns) {
@@ -2051,87 +2751,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
             __nanosleep(nap);
             continue;
         }
-        idle = 0;
-        idle_ns = 0;
-        if (++rounds == kBeatRounds) {
-            rounds = 0;
-            if (lane == 0) atomicAdd(&ctl->beat, 1ull);
-        }
-        // ---- 5. one round of warp-shared draws for the active lanes
-        const uint32_t n_win = active ? min(kWindow, pl.N - k_done) : 0u;
-        const uint32_t s_end = s + n_win;
-        warp_draw_round(sm, facc, active, s, s_end, pl.T, pl.b, pl.c_h, id, photon, step, SP.draw_keys,
-                        stats.cand);
-        if (active) {
-            const uint32_t s_ev = facc[lane];
-            bool fin = false;
-            if (s_ev == kNoEvent) {
-                stats.substeps += n_win;
-                s = s_end;
-                k_done += n_win;
-                fin = k_done == pl.N;   // the plan ran out without an event
-            } else {
-                const uint32_t k = k_done + (s_ev - s);
-                stats.substeps += s_ev - s + 1u;
-                const float x = draw_x(id, step, s_ev, SP.draw_keys);
-                const ftime t_after = (k + 1u == pl.N) ? ftime{0.0f, 0.0f}
-                                                       : time_sub_mul(t_rem, k + 1u, pl.h);
-                removed = apply_event(P, S, SP, ctl, i, id, photon, x, eps, chi, step, s_ev,
-                                      t_after, st, stats, true, false,
-                                      Fields{fld[0][threadIdx.x], fld[1][threadIdx.x],
-                                             fld[2][threadIdx.x], fld[3][threadIdx.x],
-                                             fld[4][threadIdx.x], fld[5][threadIdx.x]},
-                                      true);
-                changed = true;
-                s = s_ev + 1u;
-                t_rem = t_after;
-                fin = removed || !time_positive(t_rem);
-                if (!fin) {
-                    pl = plan_particle(SP, sm.sqz_e, sm.sqz_p, photon, st.px, st.py, st.pz,
-                                       fld[0][threadIdx.x], fld[1][threadIdx.x],
-                                       fld[2][threadIdx.x], fld[3][threadIdx.x],
-                                       fld[4][threadIdx.x], fld[5][threadIdx.x], t_rem, &chi,
-                                       &eps);
-                    k_done = 0;
-                    if (!(eps > 0.0f)) {
-                        fin = true;
-                    } else {
-                        stats.max_N = max(stats.max_N, pl.N);
-                        if (pl.N >= SP.long_min || (!photon && sampler_bin_ok(SP, chi)) ||
-                        (kSampler == 2 && photon && pl.N >= SP.hot_min &&
-                         pair_sampler_ok(SP, chi, pl.T))) {
-                            // continue in the warp mode; its state goes with the row
-                            P.px[i] = st.px;
-                            P.py[i] = st.py;
-                            P.pz[i] = st.pz;
-                            changed = false;
-                            push_long(S, ctl, cold_long, i, s, t_rem);
-                            active = false;
-                        } else {
-                            stats.plans++;
-                            stats.guard += pl.guard ? 1 : 0;
-                            if (pl.T == 0u) {
-                                stats.substeps += pl.N;
-                                s += pl.N;
-                                fin = true;
-                            }
-                        }
-                    }
-                }
-            }
-            if (fin) {
-                if (removed) {
-                    P.type[i] = QED_REMOVED;
-                } else if (changed) {
-                    P.px[i] = st.px;
-                    P.py[i] = st.py;
-                    P.pz[i] = st.pz;
-                }
-                active = false;
-                ++done;
-            }
-        }
-        __syncwarp();   // facc is reset by the next round
+        __syncwarp();   // the list buffer is reused by the next round
     }
     if (timed_out && lane == 0) atomicExch(&ctl->status, (int)QED_ERR_TIMEOUT);
     const unsigned long long sum = warp_sum(done);
@@ -2139,9 +2759,6 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
     stats.warp_substeps = stats.substeps;   // every sub-step of this kernel is a hot-pass one
     flush_stats(stats, ctl);
 }
-
-// Before the persistent step (cascading): rows [n0, capacity) are free; mark
-// them not written, so that a lane taking a child row waits for its writer.
 
 // Start a step.  keep_sticky: inside a multi-step graph, a step that follows
 // a failed step does nothing (its range is empty and it keeps the status).
@@ -2175,9 +2792,20 @@ const void* cold_kernel(bool cells) {
 }
 const void* hot_kernel(int mode, bool cells = false) {
     // sampler mode 2 runs its network in k_samp: the hot pass of its
-    // generations is rejection's (loop_hot_mode), so there is no k_hot_lanes<2>
-    return mode == 1 ? (const void*)k_hot_lanes<1>
-                     : cells ? (const void*)k_hot_lanes<0, true> : (const void*)k_hot_lanes<0>;
+    // generations is rejection's (loop_hot_mode)
+    return mode == 1 ? (const void*)k_hot_net
+                     : cells ? (const void*)k_hot<true> : (const void*)k_hot<false>;
+}
+size_t hot_smem(int mode) { return mode == 1 ? kNetSmemBytes : sizeof(HotSmem); }
+// Their dynamic shared memory is above the default limit.
+cudaError_t allow_smem() {
+    const void* hot[] = {hot_kernel(1), hot_kernel(0), hot_kernel(0, true)};
+    for (int k = 0; k < 3; ++k) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            hot[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hot_smem(k == 0 ? 1 : 0));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 const void* step_kernel(int mode, bool cells = false) {
     return mode == 2 ? (const void*)k_step<2>
@@ -2204,6 +2832,8 @@ __global__ void k_advance(DevCtl* ctl, long long* count, long long capacity, int
     ctl->med_tail = 0;
     ctl->samp_head = 0;
     ctl->samp_tail = 0;
+    ctl->samp_back = 0;
+    ctl->samp_back_head = 0;
     ctl->passes += 1;
     ctl->first_pass = 0;
     int more = (more_allowed && ctl->pass_end > ctl->pass_begin && ctl->status == 0) ? 1 : 0;
@@ -2584,6 +3214,15 @@ qed_status cuda_check(qed_ctx* ctx, cudaError_t e, const char* where) {
         if (_s != QED_OK) return _s;                                \
     } while (0)
 
+// Plans that go to the front of the hot pass's queue: those that sampler mode 1
+// steps a warp each (N >= long_min); without it, the plans stepped first, so
+// that their chains start early, four times as long (measured at long_min 256:
+// front from 256, 512, 1024, 2048, 4096 sub-steps 4.26, 4.04, 4.00, 3.95, 4.19
+// ms of hot pass on the clumped 2^24 population).
+uint32_t front_min(uint32_t long_min, int sampler_mode) {
+    return sampler_mode == 1 ? long_min : std::min(long_min, 1u << 29) * 4u;
+}
+
 StepParams make_params(const qed_config& c, uint64_t step) {
     StepParams P;
     P.seed = c.seed;
@@ -2592,6 +3231,8 @@ StepParams make_params(const qed_config& c, uint64_t step) {
     P.t_step.hi = (float)c.dt_periods;
     P.t_step.lo = (float)(c.dt_periods - (double)P.t_step.hi);
     P.inv_Es = (float)inv_schwinger64(c.lambda_m);            // 1 / E_s in code units
+    P.K_lo = (float)(rate_K64(c.lambda_m) - (double)P.K);
+    P.inv_Es_lo = (float)(inv_schwinger64(c.lambda_m) - (double)P.inv_Es);
     P.p_max = c.p_max;
     P.inv_p_max = 1.0f / c.p_max;
     P.pair_coeff = c.pair_bound_coeff;
@@ -2601,7 +3242,7 @@ StepParams make_params(const qed_config& c, uint64_t step) {
     P.wait_ns = kWaitNsDefault;
     P.step_base = nullptr;
     P.hot_min = kHotMinDefault;
-    P.long_min = kLongMinDefault;
+    P.front_min = front_min(kLongMinDefault, 0);
     P.sampler = 0;
     P.net_rows = 0;
     P.net_bins = 0;
@@ -2667,6 +3308,7 @@ qed_status ensure_samp(qed_ctx* ctx, long long cap, const StepParams& SP, Scratc
         ctx->samp_cap = cap;
     }
     S->samp = ctx->d_samp;
+    S->samp_cap = ctx->samp_cap;
     return QED_OK;
 }
 
@@ -2758,6 +3400,7 @@ Scratch make_scratch(const qed_ctx* ctx) {
     S.hot = ctx->d_hot;
     S.hot_cap = 2 * ctx->scratch_cap;
     S.samp = nullptr;
+    S.samp_cap = 0;
     S.log = ctx->log;
     S.log_cap = ctx->log_cap;
     S.log_count = ctx->log_count;
@@ -2829,15 +3472,15 @@ qed_status qed_init(qed_ctx** out, const qed_config* cfg, void* stream) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cold<false>, kColdThreads, 0);
         ctx->cold_blocks = ctx->cold_blocks_max = ctx->sms * (per_sm > 0 ? per_sm : 1);
         per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hot_lanes<0>, kLaneThreads, 0);
+        allow_smem();
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hot<false>, kLaneThreads,
+                                                      hot_smem(0));
         ctx->hot_blocks = ctx->hot_blocks_max = ctx->sms * (per_sm > 0 ? per_sm : 1);
         per_sm = 0;
-        cudaFuncSetAttribute(hot_kernel(1), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kNetSmemBytes);
         for (int m = 1; m <= 2; ++m)
             cudaFuncSetAttribute(step_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kNetSmemBytes);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hot_lanes<1>, kLaneThreads,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hot_net, kLaneThreads,
                                                       kNetSmemBytes);
         ctx->net_blocks = ctx->sms * (per_sm > 0 ? per_sm : 1);
         per_sm = 0;
@@ -2855,9 +3498,9 @@ qed_status qed_init(qed_ctx** out, const qed_config* cfg, void* stream) {
         ctx->push_blocks = ctx->sms * (per_sm > 0 ? per_sm : 1);
         per_sm = 0;
         cudaFuncSetAttribute(k_samp, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kMmaSmemBytes);
+                             (int)kSampSmemBytes);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_samp, kLaneThreads,
-                                                      kMmaSmemBytes);
+                                                      kSampSmemBytes);
         ctx->samp_blocks = ctx->sms * (per_sm > 0 ? per_sm : 1);
         ctx->hot_min = kHotMinDefault;
         ctx->long_min = kLongMinDefault;
@@ -3030,7 +3673,7 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
     if (st != QED_OK) return st;
     StepParams SP = make_params(ctx->cfg, step_index);
     SP.hot_min = ctx->hot_min;
-    SP.long_min = ctx->long_min;
+    SP.front_min = front_min(ctx->long_min, ctx->cfg.sampler_mode);
     SP.wait_ns = ctx->wait_ns;
     st = sampler_params(ctx, &SP);
     if (st != QED_OK) return st;
@@ -3066,7 +3709,7 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
         }
         if (SP.sampler == 2) {
             LaunchScope ls(ctx, QED_KERNEL_SAMPLER);
-            k_samp<<<ctx->samp_blocks, kLaneThreads, kMmaSmemBytes, ctx->stream>>>(
+            k_samp<<<ctx->samp_blocks, kLaneThreads, kSampSmemBytes, ctx->stream>>>(
                 D, SP, S, ctx->d_ctl);
         }
         {
@@ -3079,8 +3722,7 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
             const int hm = loop_hot_mode(SP);
             QED_CUDA(ctx, cudaLaunchKernel(hot_kernel(hm, SP.N_cell != nullptr),
                                            dim3(hm ? ctx->net_blocks : ctx->hot_blocks),
-                                           dim3(kLaneThreads), a, hm ? kNetSmemBytes : 0,
-                                           ctx->stream));
+                                           dim3(kLaneThreads), a, hot_smem(hm), ctx->stream));
         }
         {
             LaunchScope ls(ctx, QED_KERNEL_CONTROL);
@@ -3474,7 +4116,7 @@ qed_status qed_graph_capture(qed_ctx* ctx, const qed_particles* p, uint64_t firs
         StepParams SP = make_params(ctx->cfg, (uint64_t)k);   // offset from the device base
         SP.step_base = step_base;
         SP.hot_min = ctx->hot_min;
-        SP.long_min = ctx->long_min;
+        SP.front_min = front_min(ctx->long_min, ctx->cfg.sampler_mode);
         SP.wait_ns = ctx->wait_ns;
         st = sampler_params(ctx, &SP);
         if (st != QED_OK) break;
@@ -3509,14 +4151,14 @@ qed_status qed_graph_capture(qed_ctx* ctx, const qed_particles* p, uint64_t firs
         if (st == QED_OK && SP.sampler == 2) {
             void* a[] = {&D, &SP, &S, &ctl};
             st = add_kernel(ctx, body, &bs, (const void*)k_samp, dim3(ctx->samp_blocks),
-                            dim3(kLaneThreads), a, &bc, 1, kMmaSmemBytes);
+                            dim3(kLaneThreads), a, &bc, 1, kSampSmemBytes);
         }
         if (st == QED_OK) {
             void* a[] = {&D, &SP, &S, &ctl};
             const int hm = loop_hot_mode(SP);
             st = add_kernel(ctx, body, &bh, hot_kernel(hm, SP.N_cell != nullptr),
                             dim3(hm ? ctx->net_blocks : ctx->hot_blocks), dim3(kLaneThreads), a,
-                            &bs, 1, hm ? kNetSmemBytes : 0);
+                            &bs, 1, hot_smem(hm));
         }
         if (st == QED_OK) {
             void* a[] = {&ctl,        &count, &capacity, &more_allowed, &max_passes,
@@ -3614,11 +4256,12 @@ static qed_status run_step_graph(qed_ctx* ctx, const DevParticles& Din, StepPara
     put((uint64_t)Din.capacity);
     putp(Sin.t_rem); putp(Sin.hot); put((uint64_t)Sin.hot_cap); putp(Sin.log);
     put((uint64_t)Sin.log_cap); putp(Sin.log_count); putp(Sin.samp);
+    put((uint64_t)Sin.samp_cap);
     put(SPin.seed);
     { uint64_t b; memcpy(&b, &SPin.dt, 8); put(b); }
     putf(SPin.K); putf(SPin.inv_Es); putf(SPin.p_max); putf(SPin.inv_p_max); putf(SPin.pair_coeff);
     putf(SPin.t_step.hi); putf(SPin.t_step.lo);
-    put(SPin.hot_min); put(SPin.long_min); put((uint64_t)SPin.sampler); put((uint64_t)SPin.net_rows);
+    put(SPin.hot_min); put(SPin.front_min); put((uint64_t)SPin.sampler); put((uint64_t)SPin.net_rows);
     put(SPin.net_bins); putp(SPin.net_w); putp(SPin.net_wtot); put(SPin.process_mask);
     put(SPin.pnet_bins); putp(SPin.pnet_w); putp(SPin.pnet_wtot);
     put((uint64_t)SPin.recoil); put((uint64_t)SPin.cascade); put(SPin.wait_ns);
@@ -3673,12 +4316,12 @@ static qed_status run_step_graph(qed_ctx* ctx, const DevParticles& Din, StepPara
             bs = bc;
             if (st == QED_OK && SP.sampler == 2)
                 st = add_kernel(ctx, body, &bs, (const void*)k_samp, dim3(ctx->samp_blocks),
-                                dim3(kLaneThreads), a, &bc, 1, kMmaSmemBytes);
+                                dim3(kLaneThreads), a, &bc, 1, kSampSmemBytes);
             const int hm = loop_hot_mode(SP);
             if (st == QED_OK)
                 st = add_kernel(ctx, body, &bh, hot_kernel(hm, SP.N_cell != nullptr),
                                 dim3(hm ? ctx->net_blocks : ctx->hot_blocks), dim3(kLaneThreads),
-                                a, &bs, 1, hm ? kNetSmemBytes : 0);
+                                a, &bs, 1, hot_smem(hm));
             if (st == QED_OK) {
                 void* b[] = {&ctl,        &count, &capacity, &more_allowed, &max_passes,
                              &tail_rows, &h,     &use_handle};
@@ -4329,10 +4972,11 @@ qed_status noalloc_setup(int dev, NoAllocDevice* out) {
         int sms = 0, per_cold = 0, per_hot = 0, per_step = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return QED_ERR_CUDA;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_cold, k_cold<false>, kColdThreads, 0) !=
+        if (allow_smem() != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_cold, k_cold<false>, kColdThreads, 0) !=
                 cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_hot, k_hot_lanes<0>, kLaneThreads, 0) !=
-                cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_hot, k_hot<false>, kLaneThreads,
+                                                          hot_smem(0)) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_step, k_step<0>, kLaneThreads, 0) !=
                 cudaSuccess)
             return QED_ERR_CUDA;
@@ -4387,6 +5031,8 @@ extern "C" qed_status qed_event_step_noalloc(const qed_config* cfg, const qed_pa
     S.t_rem = reinterpret_cast<ftime*>(nd.base + kNoAllocTremOffset);
     S.hot = reinterpret_cast<HotItem*>(nd.base + kNoAllocHotOffset);
     S.hot_cap = 2 * (long long)QED_NOALLOC_MAX_ROWS;
+    S.samp = nullptr;
+    S.samp_cap = 0;
     S.log = nullptr;
     S.log_cap = 0;
     S.log_count = nullptr;
@@ -4397,7 +5043,7 @@ extern "C" qed_status qed_event_step_noalloc(const qed_config* cfg, const qed_pa
     DevCtl h;
     for (int pass = 0; pass < max_passes; ++pass) {
         k_cold<false><<<nd.cold_blocks, kColdThreads, 0, s>>>(D, SP, S, ctl);
-        k_hot_lanes<0><<<nd.hot_blocks, kLaneThreads, 0, s>>>(D, SP, S, ctl);
+        k_hot<false><<<nd.hot_blocks, kLaneThreads, hot_smem(0), s>>>(D, SP, S, ctl);
         k_advance<<<1, 1, 0, s>>>(ctl, D.count, D.capacity, cascade ? 1 : 0, max_passes,
                                   kTailRowsDefault, 0ull, 0);
         if (cudaGetLastError() != cudaSuccess) return noalloc_fail(dev, QED_ERR_CUDA);

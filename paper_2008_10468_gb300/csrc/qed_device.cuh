@@ -64,6 +64,60 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKeys& K) {
     return c;
 }
 
+// The draw stream of one particle in one step: Philox4x32-10 at counters
+// (id_lo, id_hi, step, block) for many blocks.  Only the fourth counter word
+// changes, so the first three rounds depend on it through two of their six
+// products; the rest is these four words, made once per particle, and one word
+// of the step (draw_y1).  A block's second and fourth words, which decide
+// whether a sub-step is a candidate, are the low halves of the last round's
+// products (draw_yw); its first and third words are needed for candidates
+// only (draw_block).  14 wide and 2 narrow products instead of 20 wide: the
+// wide product's rate (about 30 per clock and SM, measured) is what bounds the
+// draws.
+struct DrawKey {
+    uint32_t a, w2, h, y3;
+};
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
+
+__device__ __forceinline__ uint32_t draw_y1(uint32_t step, const PhiloxKeys& K) {
+    return (kPhiloxM1 * step) ^ K.k[2];
+}
+__device__ __forceinline__ DrawKey draw_key(uint64_t id, uint32_t step, const PhiloxKeys& K) {
+    const uint32_t lo = (uint32_t)id, hi = (uint32_t)(id >> 32);
+    const uint32_t x1 = __umulhi(kPhiloxM1, step) ^ hi ^ K.k[0];
+    const uint32_t z2 = __umulhi(kPhiloxM0, x1) ^ (kPhiloxM0 * lo) ^ K.k[3];
+    return DrawKey{__umulhi(kPhiloxM0, lo) ^ K.k[1], (kPhiloxM0 * x1) ^ K.k[5],
+                   __umulhi(kPhiloxM1, z2) ^ K.k[4], kPhiloxM1 * z2};
+}
+// The state before the last round.
+__device__ __forceinline__ uint4 draw_rounds(const DrawKey& d, uint32_t y1, uint32_t blk,
+                                             const PhiloxKeys& K) {
+    const uint32_t z1 = d.a ^ blk;
+    const uint32_t x2 = __umulhi(kPhiloxM1, z1) ^ y1;
+    uint4 c = make_uint4((kPhiloxM1 * z1) ^ d.h, d.y3, __umulhi(kPhiloxM0, x2) ^ d.w2,
+                         kPhiloxM0 * x2);
+#pragma unroll
+    for (int r = 3; r < 9; ++r) {
+        const uint32_t hi0 = __umulhi(kPhiloxM0, c.x), lo0 = kPhiloxM0 * c.x;
+        const uint32_t hi1 = __umulhi(kPhiloxM1, c.z), lo1 = kPhiloxM1 * c.z;
+        c = make_uint4(hi1 ^ c.y ^ K.k[2 * r], lo1, hi0 ^ c.w ^ K.k[2 * r + 1], lo0);
+    }
+    return c;
+}
+// Words 1 and 3 of block blk (the acceptance draws of its two sub-steps).
+__device__ __forceinline__ uint2 draw_yw(const DrawKey& d, uint32_t y1, uint32_t blk,
+                                         const PhiloxKeys& K) {
+    const uint4 c = draw_rounds(d, y1, blk, K);
+    return make_uint2(kPhiloxM1 * c.z, kPhiloxM0 * c.x);
+}
+// All four words of block blk.
+__device__ __forceinline__ uint4 draw_block(const DrawKey& d, uint32_t y1, uint32_t blk,
+                                            const PhiloxKeys& K) {
+    const uint4 c = draw_rounds(d, y1, blk, K);
+    return make_uint4(__umulhi(kPhiloxM1, c.z) ^ c.y ^ K.k[18], kPhiloxM1 * c.z,
+                      __umulhi(kPhiloxM0, c.x) ^ c.w ^ K.k[19], kPhiloxM0 * c.x);
+}
+
 // ((r >> 9) + 1/2) * 2^-23: open interval (0, 1), exact in binary32.
 __device__ __forceinline__ float u01(uint32_t r) {
     return fmaf((float)(r >> 9), 0x1p-23f, 0x1p-24f);
@@ -121,6 +175,25 @@ __device__ __forceinline__ ff ff_sqrt(ff a) {
     const ff s2 = two_prod(s, s);
     const float r = __fadd_rn(__fadd_rn(__fsub_rn(a.hi, s2.hi), -s2.lo), a.lo);
     return fast_two_sum(s, __fdiv_rn(r, __fmul_rn(2.0f, s)));
+}
+
+// a / b to ~44 bits.
+__device__ __forceinline__ ff ff_div(ff a, ff b) {
+    const float q = __fdividef(a.hi, b.hi);
+    const ff r = ff_add(a, ff_neg(ff_mul_f(b, q)));
+    return fast_two_sum(q, __fdividef(r.hi, b.hi));
+}
+// a^n, n >= 1.
+__device__ __forceinline__ ff ff_pow(ff a, int n) {
+    ff r{1.0f, 0.0f};
+    while (true) {
+        if (n & 1) r = ff_mul(r, a);
+        if (!(n >>= 1)) return r;
+        a = ff_mul(a, a);
+    }
+}
+__host__ __device__ constexpr ff ff_of(double x) {
+    return ff{(float)x, (float)(x - (double)(float)x)};
 }
 
 // chi = sqrt((eps E + p x B)^2 - (p . E)^2) / E_s with eps = sqrt(1 + p^2)
@@ -297,14 +370,14 @@ __device__ __forceinline__ void stage_syn_table(SynTable& tb) {
 constexpr float kPi = 3.14159265358979f;
 
 // The emission bound from l2b = log2(b) (b > 0): the powers as exp2(a l2b) on
-// the special-function unit (error budget in make_plan).
+// the special-function unit (error budget in make_plan).  One form for the
+// four pieces, so that the lanes of a warp do not take turns.
 __device__ __forceinline__ float bound_emission_l2(float b, float l2b, float c) {
-    float lead;
-    if (b < 0.1f) lead = 0.56f * kPi * b;
-    else if (b < 0.5f) lead = 0.45f * kPi * exp2f(l2b * (11.0f / 12.0f));
-    else if (b < 10.0f) lead = 0.42f * kPi * exp2f(l2b * (19.0f / 24.0f));
-    else lead = 0.55f * kPi * exp2f(l2b * (2.0f / 3.0f));
-    return c * (lead + 0.1f * b);
+    const bool p1 = b >= 0.1f, p2 = b >= 0.5f, p3 = b >= 10.0f;
+    const float A = p3 ? 0.55f * kPi : (p2 ? 0.42f * kPi : (p1 ? 0.45f * kPi : 0.56f * kPi));
+    const float e = p3 ? 2.0f / 3.0f : (p2 ? 19.0f / 24.0f : 11.0f / 12.0f);
+    const float v = p1 ? exp2f(l2b * e) : b;
+    return c * fmaf(0.1f, b, __fmul_rn(A, v));
 }
 
 // x -> 0 limit of 3 x^2 P(x^3) over c b^{2/3}:  4 pi / (sqrt3 Gamma(1/3) 2^{1/3}).
@@ -373,6 +446,7 @@ struct Plan {
 // parameter block would make the whole block addressable, i.e. a local copy).
 struct PlanConst {
     float K, inv_Es, inv_p_max, pair_coeff, p_max;
+    float K_lo, inv_Es_lo;   // what K and inv_Es leave of their binary64 values
     double lambda_m;   // laser wavelength (m): the binary64 constants of near-tie plans
 };
 
@@ -396,6 +470,7 @@ struct StepParams {
     double dt;           // global step (periods)
     float K;             // sqrt3 R / pi  (1 / period)
     float inv_Es;        // 1 / Schwinger field (code units)
+    float K_lo, inv_Es_lo;   // what the two leave of their binary64 values
     float p_max;
     float inv_p_max;     // 1 / p_max
     float pair_coeff;
@@ -406,7 +481,7 @@ struct StepParams {
     ftime t_step;        // dt as float-float
     const uint32_t* step_base;  // graph runs: device step base added to `step`
     uint32_t hot_min;           // plans with at least this many sub-steps go to the hot pass
-    uint32_t long_min;          // ... and with at least this many to its warp mode
+    uint32_t front_min;         // ... and with at least this many to the front of its queue
     int sampler;                // learned sampler on (e+- in usable bins)
     int net_rows;               // rows of the total-probability table
     unsigned long long net_bins;  // usable bins (64, uniform in log10 chi over [-2, 2))
@@ -445,8 +520,10 @@ __device__ __forceinline__ float squeeze_bound(const float* __restrict__ sqz_e,
 }
 
 __device__ __forceinline__ uint32_t squeeze_threshold(float B) {
-    // y = ((r>>9) * 2 + 1) 2^-24 < B  <=>  (r>>9) < (B 2^24 - 1) / 2
+    // y = ((r>>9) * 2 + 1) 2^-24 < B  <=>  (r>>9) < (B 2^24 - 1) / 2; the
+    // smallest y is 2^-24, so half of it admits no candidate
     if (!(B < 1.0f)) return 1u << 23;
+    if (B < 0x1p-25f) return 0u;
     const float t = ceilf(fmaf(B, 0x1p23f, -0.5f)) + 1.0f;
     return t <= 0.0f ? 0u : (t >= 0x1p23f ? (1u << 23) : (uint32_t)t);
 }
@@ -478,12 +555,15 @@ __device__ __forceinline__ float log2_split(float b) {
 // g (1 -+ d) and b stays in its f piece within d; otherwise plan_slow
 // recomputes it.
 __device__ __forceinline__ PlanConst plan_const(const StepParams& P) {
-    return PlanConst{P.K, P.inv_Es, P.inv_p_max, P.pair_coeff, P.p_max, P.lambda_m};
+    return PlanConst{P.K,     P.inv_Es, P.inv_p_max, P.pair_coeff,
+                     P.p_max, P.K_lo,   P.inv_Es_lo, P.lambda_m};
 }
 
+// *x_out, *guard_out: f / P_max or the guard, whichever is larger, and the guard.
 __device__ __forceinline__ Plan make_plan(const PlanConst& P, const float* __restrict__ sqz_e,
                                           const float* __restrict__ sqz_p, bool photon, float chi,
-                                          float eps, ftime T, float d) {
+                                          float eps, ftime T, float d, float* x_out,
+                                          float* guard_out) {
     Plan pl;
     pl.chi = chi;
     pl.eps = eps;
@@ -495,21 +575,19 @@ __device__ __forceinline__ Plan make_plan(const PlanConst& P, const float* __res
     const float f = photon ? P.pair_coeff * c_rem * b
                            : (b > 0.0f ? bound_emission_l2(b, l2b, c_rem) : 0.0f);
     const float q = f * P.inv_p_max;
-    float N = fmaxf(1.0f, ceilf(q));
     float b23 = 0.0f;
     if (b > 0.0f) b23 = exp2f(l2b * (2.0f / 3.0f));
-    pl.guard = false;
-    float graw = 0.0f;
-    if (!photon) {
-        graw = kSmallF * c_rem * b23;
-        const float g = ceilf(graw);
-        if (g > N) { N = g; pl.guard = true; }
-    }
-    // N = max(1, ceil(q), ceil(g)) is monotone in q and g: it is certain when
-    // it is the same at both ends of the band (and b stays in its f piece)
-    const float n_lo = fmaxf(1.0f, fmaxf(ceilf(q * (1.0f - d)), ceilf(graw * (1.0f - d))));
-    const float n_hi = fmaxf(1.0f, fmaxf(ceilf(q * (1.0f + d)), ceilf(graw * (1.0f + d))));
-    bool safe = n_lo == n_hi;
+    const float graw = photon ? 0.0f : kSmallF * c_rem * b23;
+    pl.guard = graw > fmaxf(1.0f, ceilf(q));   // ceil(graw) above max(1, ceil(q))
+    // N = max(1, ceil(q), ceil(g)) is the ceiling of the larger one, monotone
+    // in it: it is certain when it is the same at both ends of the band (and b
+    // stays in its f piece)
+    const float x = fmaxf(q, graw);
+    *x_out = x;
+    *guard_out = graw;
+    const float n_lo = fmaxf(1.0f, ceilf(x * (1.0f - d)));
+    float N = fmaxf(1.0f, ceilf(x * (1.0f + d)));
+    bool safe = n_lo == N;
     if (!photon)
         safe = safe && emission_piece(b * (1.0f - d)) == emission_piece(b * (1.0f + d));
     N = fminf(N, 1073741824.0f);  // 2^30: keeps the 32-bit sub-step counter from wrapping
@@ -532,49 +610,111 @@ __device__ __forceinline__ double bound_emission64(double b, double c) {
     return lead + 0.1 * c * b;
 }
 
-// Slow path of plan_particle, for plans whose binary32 count is not certain
-// (chi ill-conditioned, or f / P_max within 3e-6 of an integer, or b at a
-// piece edge): chi in float-float and the binary32 plan from it; if its count
-// is still not certain, the count N = max(1, ceil(f/P_max), guard) in
-// binary64, so that N is the exact count unless f / P_max lies within ~1e-13
-// of an integer.  The binary64 step is rare (0.6% of the longest plans,
-// fewer of the others), so it stays off the sub-step path.  Kept out of line
-// so that the common path does not carry its registers.
-__device__ __noinline__ Plan plan_slow(PlanConst P, const float* __restrict__ sqz_e,
-                                       const float* __restrict__ sqz_p, bool photon, float px,
-                                       float py, float pz, float Ex, float Ey, float Ez, float Bx,
-                                       float By, float Bz, ftime T) {
-    ff q2, epsf;
-    chi_sq_ff(photon, px, py, pz, Ex, Ey, Ez, Bx, By, Bz, &q2, &epsf);
-    const double q2d = (double)q2.hi + (double)q2.lo;
-    const double chi_d = q2d > 0.0 ? sqrt(q2d) * inv_schwinger64(P.lambda_m) : 0.0;
-    const double eps_d = (double)epsf.hi + (double)epsf.lo;
-    Plan pl;
-    pl.chi = (float)chi_d;
-    pl.eps = (float)eps_d;
-    if (!(pl.eps > 0.0f)) {
-        pl.N = 0;
-        return pl;
+// Whether f / P_max exceeds the integer k, for f / P_max near k, in
+// float-float arithmetic: f = c_rem (A pi b^e + 0.1 b) with c_rem = K T / eps
+// and e = p / m, so that f / P_max > k is b^p > v^m with
+// v = (k P_max eps / (K T) - 0.1 b) / (A pi): products instead of the powers
+// (photons and the lowest piece of f are linear in b).  The two sides are
+// within ~1e-12; true in *decided if they differ by more than 1e-10.
+__device__ __forceinline__ bool count_above(const PlanConst& P, bool photon, ff b, ff eps, ftime T,
+                                            float k, bool* decided) {
+    const ff KT = ff_mul(ff{P.K, P.K_lo}, ff{T.hi, T.lo});
+    ff rhs = ff_mul(two_prod(k, P.p_max), eps), lhs;
+    if (photon) {
+        lhs = ff_mul(ff_mul_f(b, P.pair_coeff), KT);
+    } else {
+        constexpr double kPiD = 3.14159265358979323846;
+        const ff v = ff_add(ff_div(rhs, KT), ff_neg(ff_mul(b, ff_of(0.1))));
+        const int piece = emission_piece(b.hi);
+        const ff inv_A = piece == 3   ? ff_of(1.0 / (0.55 * kPiD))
+                         : piece == 2 ? ff_of(1.0 / (0.42 * kPiD))
+                         : piece == 1 ? ff_of(1.0 / (0.45 * kPiD))
+                                      : ff_of(1.0 / (0.56 * kPiD));
+        const int p = piece == 3 ? 2 : (piece == 2 ? 19 : (piece == 1 ? 11 : 1));
+        const int m = piece == 3 ? 3 : (piece == 2 ? 24 : (piece == 1 ? 12 : 1));
+        lhs = ff_pow(b, p);
+        rhs = ff_pow(ff_mul(v, inv_A), m);
     }
-    // the binary32 plan from the float-float chi (chi now within 1 ulp): when
-    // its count is certain, that is the plan (an ill-conditioned chi, the
-    // common reason to be here, needs no binary64)
-    pl = make_plan(P, sqz_e, sqz_p, photon, pl.chi, pl.eps, T, 1.5e-6f);
-    if (pl.safe) return pl;
+    const ff d = ff_add(lhs, ff_neg(rhs));
+    *decided = fabsf(d.hi) > 1e-10f * fabsf(rhs.hi);   // false for infinities and NaN too
+    return d.hi > 0.0f;
+}
+
+// The count N = max(1, ceil(f/P_max), guard) in binary64, the exact count
+// unless f / P_max lies within ~1e-13 of an integer; bit 31: the guard bound.
+__device__ __noinline__ uint32_t count64(PlanConst P, bool photon, double chi_d, double eps_d,
+                                         ftime T) {
     const double b = 1.5 * chi_d;
     const double c_rem = rate_K64(P.lambda_m) * ((double)T.hi + (double)T.lo) / eps_d;  // hi + lo exact
     const double f = photon ? (double)P.pair_coeff * c_rem * b
                             : (b > 0.0 ? bound_emission64(b, c_rem) : 0.0);
     double N = fmax(1.0, ceil(f / (double)P.p_max));
-    pl.guard = false;
+    bool guard = false;
     if (!photon && b > 0.0) {
         const double g = ceil(2.14952824153447863 * c_rem * pow(b, 2.0 / 3.0));
-        if (g > N) { N = g; pl.guard = true; }
+        if (g > N) { N = g; guard = true; }
     }
-    N = fmin(N, 1073741824.0);   // 2^30
-    pl.N = (uint32_t)N;
+    return (uint32_t)fmin(N, 1073741824.0) | (guard ? 1u << 31 : 0u);   // 2^30
+}
+
+// Slow path of plan_particle, for plans whose binary32 count is not certain
+// (chi ill-conditioned, or f / P_max within 3e-6 of an integer, or b at a
+// piece edge): chi in float-float and the binary32 plan from it; if its count
+// is still not certain, the count from the float-float comparison of f / P_max
+// with the integer it is near (count_above).  What that cannot decide (a near
+// tie below 1e-10, b at a piece edge, a count above 1e5, the validity guard
+// binding) is counted in binary64, so that N is the exact count unless
+// f / P_max lies within ~1e-13 of an integer.  0.6% of the clumped
+// population's plans and 8% of those of 2e4 sub-steps come here.  In binary64
+// (the powers by pow, at 1/64 of the binary32 rate) the count took 17% of the
+// hot pass's time on the uniform-field electrons (1.00 against 0.83 ms without
+// the slow path) and 28 against 20 us of the thread pass's.  Kept out of line
+// so that the common path does not carry its registers.
+__device__ __noinline__ Plan plan_slow(PlanConst P, const float* __restrict__ sqz_e,
+                                       const float* __restrict__ sqz_p, bool photon, float px,
+                                       float py, float pz, float Ex, float Ey, float Ez, float Bx,
+                                       float By, float Bz, ftime T) {
+    ff q2, eps;
+    chi_sq_ff(photon, px, py, pz, Ex, Ey, Ez, Bx, By, Bz, &q2, &eps);
+    ff chi{0.0f, 0.0f};
+    if (q2.hi > 0.0f) chi = ff_mul(ff_sqrt(q2), ff{P.inv_Es, P.inv_Es_lo});
+    Plan pl;
+    pl.chi = chi.hi;
+    // the rounding of the binary64 value: asked of it when the rest is within
+    // 2^-44 of half a unit in the last place (or chi is tiny)
+    const float half_ulp = __int_as_float((__float_as_int(chi.hi) & 0x7f800000) - (24 << 23));
+    const bool chi64 = q2.hi > 0.0f && (!(chi.hi > 1e-30f) ||
+                                        fabsf(fabsf(chi.lo) - half_ulp) < 0x1p-18f * half_ulp ||
+                                        fabsf(fabsf(chi.lo) - 0.5f * half_ulp) < 0x1p-18f * half_ulp);
+    if (chi64) pl.chi = (float)(sqrt((double)q2.hi + (double)q2.lo) * inv_schwinger64(P.lambda_m));
+    pl.eps = __fadd_rn(eps.hi, eps.lo);
+    if (!(pl.eps > 0.0f)) {
+        pl.N = 0;
+        return pl;
+    }
+    // the binary32 plan from the float-float chi (chi now within 1 ulp): when
+    // its count is certain, that is the plan
+    float x, graw;
+    pl = make_plan(P, sqz_e, sqz_p, photon, pl.chi, pl.eps, T, 1.5e-6f, &x, &graw);
+    if (pl.safe) return pl;
+    const float b32 = pl.b;
+    const float k = rintf(x);
+    bool decided = false;
+    if (x < 1e5f && k >= 1.0f && graw < 0.9f * x &&
+        (photon || emission_piece(b32 * (1.0f - 1e-6f)) == emission_piece(b32 * (1.0f + 1e-6f)))) {
+        const bool above =
+            count_above(P, photon, ff_mul_f(chi, 1.5f), eps, T, k, &decided);
+        pl.N = (uint32_t)k + (above ? 1u : 0u);
+        pl.guard = false;
+    }
+    if (!decided) {
+        const double q2d = (double)q2.hi + (double)q2.lo;
+        const double chi_d = q2d > 0.0 ? sqrt(q2d) * inv_schwinger64(P.lambda_m) : 0.0;
+        const uint32_t c = count64(P, photon, chi_d, (double)eps.hi + (double)eps.lo, T);
+        pl.N = c & 0x7fffffffu;
+        pl.guard = (c >> 31) != 0u;
+    }
     pl.safe = true;
-    pl.b = 1.5f * pl.chi;
     pl.h = time_div(T, pl.N);
     pl.c_h = P.K * pl.h.hi * __fdividef(1.0f, pl.eps);
     const float b23 = pl.b > 0.0f ? exp2f(__log2f(pl.b) * (2.0f / 3.0f)) : 0.0f;
@@ -624,8 +764,9 @@ __device__ __forceinline__ Plan plan_particle(const StepParams& SP, const float*
     const float chi = chi_f32(photon, px, py, pz, Ex, Ey, Ez, Bx, By, Bz, P.inv_Es, &eps, &wc,
                               8.0f, &kappa);
     if (wc && eps > 0.0f) {
-        const Plan pl =
-            make_plan(P, sqz_e, sqz_p, photon, chi, eps, T, fmaf(5e-7f, kappa, 1.5e-6f));
+        float x, graw;
+        const Plan pl = make_plan(P, sqz_e, sqz_p, photon, chi, eps, T,
+                                  fmaf(5e-7f, kappa, 1.5e-6f), &x, &graw);
         if (pl.safe) {
             *chi_out = chi;
             *eps_out = eps;

@@ -566,13 +566,14 @@ __device__ __forceinline__ float sampler_wtot(const SamplerSmem& S, float chi) {
 // A fragment of the next one for the same rows, so activations stay in
 // registers between layers.  A row's result depends on that row's inputs only.
 // ---------------------------------------------------------------------------
-constexpr int kHPad = 72;   // BF16 row stride of W2, W3 ([n][k], 64 + 8): the
-                            // 32-bit fragment loads of a warp hit 32 banks
-
+// W2 and W3 sit in shared memory as the B fragments themselves: the 16 words
+// that a lane needs of one 16-deep slice (8 tiles of 8 neurons, two words
+// each) are four 128-bit loads, conflict-free; from row-major W they were 16
+// loads of 32 bits.
 struct SamplerMma {
-    __align__(16) __nv_bfloat16 W2[kMlpW * kHPad];
-    __align__(16) __nv_bfloat16 W3[kMlpW * kHPad];
-    float W1[kMlpW * 2], b1[kMlpW], b2[kMlpW], b3[kMlpW], w4[kMlpW];
+    uint4 W2[16 * 32], W3[16 * 32];   // [slice kt][tiles 2q, 2q + 1][lane]
+    float4 W1[32];                    // rows 2m, 2m + 1
+    __align__(16) float b1[kMlpW], b2[kMlpW], b3[kMlpW], w4[kMlpW];
     float b4;
     float wtot[1024];
     unsigned long long bin_ok;
@@ -582,12 +583,18 @@ struct SamplerMma {
 __device__ __forceinline__ void stage_sampler_mma(SamplerMma& S, const __nv_bfloat16* __restrict__ w,
                                                   const float* __restrict__ wtot, int nrows,
                                                   unsigned long long bin_ok) {
-    for (int i = threadIdx.x; i < kMlpW * kMlpW; i += blockDim.x) {
-        const int n = i / kMlpW, k = i % kMlpW;
-        S.W2[n * kHPad + k] = w[kMlpOffW2 + i];
-        S.W3[n * kHPad + k] = w[kMlpOffW3 + i];
+    __nv_bfloat162* f2 = reinterpret_cast<__nv_bfloat162*>(S.W2);
+    __nv_bfloat162* f3 = reinterpret_cast<__nv_bfloat162*>(S.W3);
+    for (int i = threadIdx.x; i < 16 * 32 * 4; i += blockDim.x) {
+        // word c of the lane's uint4 for slice kt, tiles 2q and 2q + 1
+        const int c = i & 3, lane = (i >> 2) & 31, q = (i >> 7) & 3, kt = i >> 9;
+        const int n = 8 * (2 * q + (c >> 1)) + (lane >> 2);
+        const int k = 16 * kt + 8 * (c & 1) + 2 * (lane & 3);
+        f2[i] = __nv_bfloat162(w[kMlpOffW2 + n * kMlpW + k], w[kMlpOffW2 + n * kMlpW + k + 1]);
+        f3[i] = __nv_bfloat162(w[kMlpOffW3 + n * kMlpW + k], w[kMlpOffW3 + n * kMlpW + k + 1]);
     }
-    for (int i = threadIdx.x; i < 128; i += blockDim.x) S.W1[i] = __bfloat162float(w[kMlpOffW1 + i]);
+    for (int i = threadIdx.x; i < 128; i += blockDim.x)
+        reinterpret_cast<float*>(S.W1)[i] = __bfloat162float(w[kMlpOffW1 + i]);
     for (int i = threadIdx.x; i < kMlpW; i += blockDim.x) {
         S.b1[i] = __bfloat162float(w[kMlpOffB1 + i]);
         S.b2[i] = __bfloat162float(w[kMlpOffB2 + i]);
@@ -611,69 +618,75 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4],
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// (x0, x1) as BF16 pairs: hi rounds each value, lo rounds what hi leaves.
-__device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);   // .x (low half) = x0
-    const __nv_bfloat162 l =
-        __floats2bfloat162_rn(x0 - __low2float(h), x1 - __high2float(h));
+// Two binary32 values in one operation (add, mul .rn, each rounded by itself).
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 r;
+    asm("{.reg .b64 a, b, r; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5};"
+        " mul.rn.f32x2 r, a, b; mov.b64 {%0, %1}, r;}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 r;
+    asm("{.reg .b64 a, b, r; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5};"
+        " add.rn.f32x2 r, a, b; mov.b64 {%0, %1}, r;}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
+// x as BF16 pairs: hi rounds each value, lo rounds what hi leaves.
+__device__ __forceinline__ void split_bf16x2(float2 x, uint32_t& hi, uint32_t& lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x.x, x.y);   // .x (low half) = x.x
+    const float2 d = add2(x, make_float2(-__low2float(h), -__high2float(h)));
+    const __nv_bfloat162 l = __floats2bfloat162_rn(d.x, d.y);
     hi = *reinterpret_cast<const uint32_t*>(&h);
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-__device__ __forceinline__ float silu_fast(float z) { return __fdividef(z, 1.0f + __expf(-z)); }
+// z / (1 + exp(-z)) of two values.  exp(-z) below the normal range vanishes in
+// the sum and a quotient below it is 0, so the special-function operations
+// need no handling of subnormals.
+__device__ __forceinline__ float2 silu2(float z0, float z1) {
+    const float2 z = make_float2(z0, z1);
+    const float2 t = mul2(z, make_float2(-1.4426950408889634f, -1.4426950408889634f));
+    float2 e, r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(t.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(t.y));
+    e = add2(e, make_float2(1.0f, 1.0f));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(e.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(e.y));
+    return mul2(z, r);
+}
 
-// One hidden layer for one 16-row tile: C = W a + b from the A fragments
-// (hi, lo) of the layer below, then SiLU; the result replaces (hi, lo).
-// upper = false: rows 8..15 of the tile hold no sample; their activations are
-// left at 0 instead of going through SiLU (rows do not mix in the products, so
-// the other rows' results are unchanged).
-__device__ __forceinline__ void mma_hidden(const __nv_bfloat16* __restrict__ W,
-                                           const float* __restrict__ bias, uint32_t (&Ah)[4][4],
-                                           uint32_t (&Al)[4][4], bool upper) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    float C[8][4];
+// C = W a + bias for one 16-row tile, from the A fragments (hi, lo).
+__device__ __forceinline__ void mma_layer(const uint4* __restrict__ W, const float* __restrict__ bias,
+                                          const uint32_t (&Ah)[4][4], const uint32_t (&Al)[4][4],
+                                          float (&C)[8][4]) {
+    const int lane = threadIdx.x & 31, t = lane & 3;
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-        const float b0 = bias[8 * nt + 2 * t], b1 = bias[8 * nt + 2 * t + 1];
-        C[nt][0] = b0;
-        C[nt][1] = b1;
-        C[nt][2] = b0;
-        C[nt][3] = b1;
+        const float2 b = *reinterpret_cast<const float2*>(bias + 8 * nt + 2 * t);
+        C[nt][0] = C[nt][2] = b.x;
+        C[nt][1] = C[nt][3] = b.y;
     }
 #pragma unroll
     for (int kt = 0; kt < 4; ++kt) {
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const __nv_bfloat16* row = W + (8 * nt + g) * kHPad + 16 * kt + 2 * t;
-            const uint32_t b0 = *reinterpret_cast<const uint32_t*>(row);
-            const uint32_t b1 = *reinterpret_cast<const uint32_t*>(row + 8);
-            mma_16816(C[nt], Ah[kt], b0, b1);
-            mma_16816(C[nt], Al[kt], b0, b1);
-        }
-    }
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const int kt = nt >> 1, q = (nt & 1) * 2;
-        split_bf16x2(silu_fast(C[nt][0]), silu_fast(C[nt][1]), Ah[kt][q], Al[kt][q]);
-    }
-    if (upper) {
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const int kt = nt >> 1, q = (nt & 1) * 2;
-            split_bf16x2(silu_fast(C[nt][2]), silu_fast(C[nt][3]), Ah[kt][q + 1], Al[kt][q + 1]);
-        }
-    } else {
-#pragma unroll
-        for (int kt = 0; kt < 4; ++kt) {
-            Ah[kt][1] = Ah[kt][3] = 0u;
-            Al[kt][1] = Al[kt][3] = 0u;
+        for (int q = 0; q < 4; ++q) {
+            const uint4 w = W[(4 * kt + q) * 32 + lane];
+            mma_16816(C[2 * q], Ah[kt], w.x, w.y);
+            mma_16816(C[2 * q], Al[kt], w.x, w.y);
+            mma_16816(C[2 * q + 1], Ah[kt], w.z, w.w);
+            mma_16816(C[2 * q + 1], Al[kt], w.z, w.w);
         }
     }
 }
 
 // The network's output logit (before b4 and the anchor) for rows g and g + 8
 // of one tile, whose inputs are (v0a, v1a) and (v0b, v1b); every lane of the
-// group g gets both (upper = false: rows g + 8 hold no sample, ob is 0).
+// group g gets both.  upper = false: rows g + 8 hold no sample; their
+// activations are left at 0 instead of going through SiLU (rows do not mix in
+// the products, so the other rows' results are unchanged), and ob is 0.
 __device__ __forceinline__ void mma_tile(const SamplerMma& S, float v0a, float v1a, float v0b,
                                          float v1b, float& oa, float& ob, bool upper = true) {
     const int lane = threadIdx.x & 31, t = lane & 3;
@@ -681,54 +694,40 @@ __device__ __forceinline__ void mma_tile(const SamplerMma& S, float v0a, float v
     // layer 1 (two inputs) on the CUDA cores, in the fragment layout
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-        const int n = 8 * nt + 2 * t;
-        const float w00 = S.W1[2 * n], w01 = S.W1[2 * n + 1];
-        const float w10 = S.W1[2 * n + 2], w11 = S.W1[2 * n + 3];
-        const float za0 = fmaf(w00, v0a, fmaf(w01, v1a, S.b1[n]));
-        const float za1 = fmaf(w10, v0a, fmaf(w11, v1a, S.b1[n + 1]));
+        const float4 w = S.W1[4 * nt + t];
+        const float2 b = *reinterpret_cast<const float2*>(S.b1 + 8 * nt + 2 * t);
+        const float za0 = fmaf(w.x, v0a, fmaf(w.y, v1a, b.x));
+        const float za1 = fmaf(w.z, v0a, fmaf(w.w, v1a, b.y));
         const int kt = nt >> 1, q = (nt & 1) * 2;
-        split_bf16x2(silu_fast(za0), silu_fast(za1), Ah[kt][q], Al[kt][q]);
+        split_bf16x2(silu2(za0, za1), Ah[kt][q], Al[kt][q]);
         Ah[kt][q + 1] = Al[kt][q + 1] = 0u;
         if (upper) {
-            const float zb0 = fmaf(w00, v0b, fmaf(w01, v1b, S.b1[n]));
-            const float zb1 = fmaf(w10, v0b, fmaf(w11, v1b, S.b1[n + 1]));
-            split_bf16x2(silu_fast(zb0), silu_fast(zb1), Ah[kt][q + 1], Al[kt][q + 1]);
+            const float zb0 = fmaf(w.x, v0b, fmaf(w.y, v1b, b.x));
+            const float zb1 = fmaf(w.z, v0b, fmaf(w.w, v1b, b.y));
+            split_bf16x2(silu2(zb0, zb1), Ah[kt][q + 1], Al[kt][q + 1]);
         }
     }
-    mma_hidden(S.W2, S.b2, Ah, Al, upper);
-    // layer 3 and the output dot product with w4
-    const int g = lane >> 2;
-    float C[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const float b0 = S.b3[8 * nt + 2 * t], b1 = S.b3[8 * nt + 2 * t + 1];
-        C[nt][0] = b0;
-        C[nt][1] = b1;
-        C[nt][2] = b0;
-        C[nt][3] = b1;
-    }
-#pragma unroll
-    for (int kt = 0; kt < 4; ++kt) {
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-            const __nv_bfloat16* row = S.W3 + (8 * nt + g) * kHPad + 16 * kt + 2 * t;
-            const uint32_t b0 = *reinterpret_cast<const uint32_t*>(row);
-            const uint32_t b1 = *reinterpret_cast<const uint32_t*>(row + 8);
-            mma_16816(C[nt], Ah[kt], b0, b1);
-            mma_16816(C[nt], Al[kt], b0, b1);
-        }
-    }
+    // layers 2 and 3 are one piece of code; after layer 3 the output dot
+    // product with w4
     float pa = 0.0f, pb = 0.0f;
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const float w0 = S.w4[8 * nt + 2 * t], w1 = S.w4[8 * nt + 2 * t + 1];
-        pa = fmaf(w0, silu_fast(C[nt][0]), fmaf(w1, silu_fast(C[nt][1]), pa));
-    }
-    if (upper) {
+#pragma unroll 1
+    for (int layer = 2; layer <= 3; ++layer) {
+        float C[8][4];
+        mma_layer(layer == 2 ? S.W2 : S.W3, layer == 2 ? S.b2 : S.b3, Ah, Al, C);
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
-            const float w0 = S.w4[8 * nt + 2 * t], w1 = S.w4[8 * nt + 2 * t + 1];
-            pb = fmaf(w0, silu_fast(C[nt][2]), fmaf(w1, silu_fast(C[nt][3]), pb));
+            const int kt = nt >> 1, q = (nt & 1) * 2;
+            const float2 a = silu2(C[nt][0], C[nt][1]);
+            float2 c = make_float2(0.0f, 0.0f);
+            if (upper) c = silu2(C[nt][2], C[nt][3]);
+            if (layer == 2) {
+                split_bf16x2(a, Ah[kt][q], Al[kt][q]);
+                split_bf16x2(c, Ah[kt][q + 1], Al[kt][q + 1]);
+            } else {
+                const float2 w = *reinterpret_cast<const float2*>(S.w4 + 8 * nt + 2 * t);
+                pa = fmaf(w.x, a.x, fmaf(w.y, a.y, pa));
+                pb = fmaf(w.x, c.x, fmaf(w.y, c.y, pb));
+            }
         }
     }
     pa += __shfl_xor_sync(0xffffffffu, pa, 1);
