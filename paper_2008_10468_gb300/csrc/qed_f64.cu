@@ -30,7 +30,7 @@ constexpr int kThreads64 = 256;
 
 struct Syn64Table {
     longlong2 main[QED_SYN64_TAIL][QED_SYN64_NPIECE];                // power j at scale 2^(60 + j)
-    int2 tail[QED_SYN64_DEG + 1 - QED_SYN64_TAIL][QED_SYN64_NPIECE];  // power j at scale 2^(48 + j)
+    int2 tail[QED_SYN64_DEG + 1 - QED_SYN64_TAIL][QED_SYN64_NPIECE];  // power j at scale 2^(46 + j)
     unsigned long long exp2[256];                                    // 2^{-i/256} at scale 2^63
 };
 
@@ -59,12 +59,11 @@ __device__ __forceinline__ int64_t horner64(int64_t p, int32_t uh, int32_t ul, i
     return (int64_t)ph * uh + c + (mid >> 31);
 }
 
-// The binary64 number V 2^(e - 60), rounded to nearest; V > 0.
+// The binary64 number V 2^(e - 60), rounded to nearest, for V >= 2^54.
 __device__ __forceinline__ double to_double(uint64_t V, int e) {
-    const int lz = __clzll((long long)V);
-    const uint64_t W = V << lz;
-    return __longlong_as_double(((int64_t)(1025 - lz + e) << 52) + (int64_t)(W >> 11) +
-                                (int64_t)((W >> 10) & 1u));
+    const int sh = 11 - __clz((int)(V >> 32));   // to 53 bits
+    return __longlong_as_double(((int64_t)(1014 + sh + e) << 52) +
+                                (int64_t)((V + (1ull << (sh - 1))) >> sh));
 }
 
 // Small-x series (subnormals included), rare: kept out of line.
@@ -107,8 +106,8 @@ __device__ __forceinline__ void syn64(const Syn64Table& T, double x, double& F, 
         r.y = c.y + __mulhi(r.y, uh);
     }
     longlong2 c = T.main[QED_SYN64_TAIL - 1][piece];
-    int64_t pf = c.x + (((int64_t)r.x * uh) >> 20);
-    int64_t pg = c.y + (((int64_t)r.y * uh) >> 20);
+    int64_t pf = c.x + (((int64_t)r.x * uh) >> 18);
+    int64_t pg = c.y + (((int64_t)r.y * uh) >> 18);
 #pragma unroll
     for (int j = QED_SYN64_TAIL - 2; j >= 0; --j) {
         c = T.main[j][piece];
@@ -119,12 +118,10 @@ __device__ __forceinline__ void syn64(const Syn64Table& T, double x, double& F, 
     int e = (k - QED_SYN64_KMIN + (QED_SYN64_KMIN + 15)) / 3 - 5;
     uint64_t vf = (uint64_t)pf, vg = (uint64_t)pg;
     if (k >= QED_SYN64_LAMBDA_FROM) {
-        // exp(-x) = 2^-n 2^{-i/256} 2^-r, x at scale 2^54, log2 e = 1 + 0.44...
-        const uint64_t X = (frac | (1ull << 52)) << (k + 2);
-        const uint64_t hi = __umul64hi(X, QED_SYN64_LOG2E_FRAC), lo = X * QED_SYN64_LOG2E_FRAC;
-        const uint64_t y = X + hi;
-        const uint64_t f = (y << 10) | (lo >> 54);
-        e -= (int)(y >> 54);
+        // exp(-x) = 2^-n 2^{-i/256} 2^-r from y = x log2 e
+        const uint64_t y = mulhi((frac | (1ull << 52)) << 11, QED_SYN64_LOG2E);   // at scale 2^(62 - k)
+        const uint64_t f = y << (2 + k);
+        e -= (int)(y >> (62 - k));
         // z = r ln 2 < 2^-8.5 at scale 2^72; 2^-r = 1 - z (1 - z (1/2 - z (1/6 - z (1/24 - z / 120))))
         const uint64_t z = mulhi(f << 8, QED_SYN64_LN2);
         const uint32_t z32 = (uint32_t)(z >> 32);
@@ -141,6 +138,10 @@ __device__ __forceinline__ void syn64(const Syn64Table& T, double x, double& F, 
     G = to_double(vg, e);
 }
 
+// 13 KB of tables per block, a row of a power's (F, G) pairs read with one
+// 128-bit load (random pieces conflict about 2.5-fold).  2^24 points: see the
+// figures above the kernels' launch.
+template <bool W1, bool W2>
 __global__ void __launch_bounds__(kThreads64) k_sweep64(const double* __restrict__ y,
                                                         double* __restrict__ F1,
                                                         double* __restrict__ F2, long long n) {
@@ -151,8 +152,8 @@ __global__ void __launch_bounds__(kThreads64) k_sweep64(const double* __restrict
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         double a, b;
         syn64(T, __ldcs(y + i), a, b);
-        if (F1) __stcs(F1 + i, a);
-        if (F2) __stcs(F2 + i, b);
+        if (W1) __stcs(F1 + i, a);
+        if (W2) __stcs(F2 + i, b);
     }
 }
 
@@ -168,6 +169,9 @@ extern "C" qed_status qed_synchrotron_F1F2_f64(const double* y, double* F1, doub
         return QED_ERR_CUDA;
     const long long blocks = ((long long)n + kThreads64 - 1) / kThreads64;
     const int grid = (int)(blocks < (long long)sms * 8 ? blocks : (long long)sms * 8);
-    k_sweep64<<<grid, kThreads64, 0, (cudaStream_t)stream>>>(y, F1, F2, (long long)n);
+    const cudaStream_t s = (cudaStream_t)stream;
+    if (F1 && F2) k_sweep64<true, true><<<grid, kThreads64, 0, s>>>(y, F1, F2, (long long)n);
+    else if (F1) k_sweep64<true, false><<<grid, kThreads64, 0, s>>>(y, F1, F2, (long long)n);
+    else k_sweep64<false, true><<<grid, kThreads64, 0, s>>>(y, F1, F2, (long long)n);
     return cudaGetLastError() == cudaSuccess ? QED_OK : QED_ERR_CUDA;
 }

@@ -28,7 +28,7 @@ generator's extended-precision series (this module does not use the oracle).
 The kernel evaluates the same polynomials in 64-bit fixed point (binary64
 arithmetic is slow on the target GPU): the words of ``fixed_tables`` are the
 60-digit coefficients times 2^{r/3} (k = 3 q + r, so that F = 2^q exp(-lam x)
-P(u)), at scale 2^(60 + j) for power j below TAIL and 2^(48 + j) in 32 bits
+P(u)), at scale 2^(60 + j) for power j below TAIL and 2^(46 + j) in 32 bits
 from there, and exp2 is 2^{-i/256} at scale 2^63.  ``eval_fixed`` is that
 evaluation in Python integers.
 """
@@ -51,8 +51,8 @@ LAMBDA_FROM = -1           # lam_k = 1 for k >= LAMBDA_FROM (x >= 1/2)
 DEG = 12
 SMALL_DEG = 6
 NPIECE = 1 + len(PARTS) * (KMAX - KMIN + 1)
-TAIL = 8                   # powers from here on are held in 32 bits
-LOG2E_FRAC = 0x71547652B82FE177   # (log2 e - 1) 2^64, rounded
+TAIL = 7                   # powers from here on are held in 32 bits
+LOG2E = 0xB8AA3B295C17F0BC        # log2 e 2^63, rounded
 LN2 = 0xB17217F7D1CF79AC          # ln 2 2^64, rounded
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -126,7 +126,7 @@ def fixed_tables(pieces):
         for i, cf in enumerate(pieces):
             k = KMIN + i // len(PARTS)
             s = mp.power(2, mp.mpf(k % 3) / 3)
-            words = [[int(mp.nint(c * s * mp.power(2, (60 if j < TAIL else 48) + j)))
+            words = [[int(mp.nint(c * s * mp.power(2, (60 if j < TAIL else 46) + j)))
                       for j, c in enumerate(f)] for f in cf]
             for f in words:
                 # every partial sum stays within its word
@@ -165,18 +165,16 @@ def eval_fixed(tables, x):
         r = tail[piece][DEG - TAIL][f]
         for j in range(DEG - TAIL - 1, -1, -1):
             r = tail[piece][j][f] + ((r * uh) >> 32)
-        p = main[piece][TAIL - 1][f] + ((r * uh) >> 20)
+        p = main[piece][TAIL - 1][f] + ((r * uh) >> 18)
         for j in range(TAIL - 2, -1, -1):
             ph, pl = p >> 32, (p & 0xFFFFFFFF) >> 1
             p = main[piece][j][f] + ph * uh + ((ph * ul + pl * uh) >> 31)
         out.append(p)
     e = q
     if k >= LAMBDA_FROM:
-        X = ((1 << 52) | frac) << (k + 2)
-        full = X * LOG2E_FRAC
-        y = X + (full >> 64)
-        n = y >> 54
-        f64 = ((y << 10) & ((1 << 64) - 1)) | ((full & ((1 << 64) - 1)) >> 54)
+        y = _mulhi(((1 << 52) | frac) << 11, LOG2E)       # m log2 e, scale 2^62
+        n = y >> (62 - k)
+        f64 = (y << (2 + k)) & ((1 << 64) - 1)
         i = f64 >> 56
         z = _mulhi((f64 << 8) & ((1 << 64) - 1), LN2)     # scale 2^72
         z32 = z >> 32
@@ -190,9 +188,8 @@ def eval_fixed(tables, x):
         e = q - n
     res = []
     for V in out:
-        lz = 64 - V.bit_length()
-        W = V << lz
-        bits = ((1022 + 3 - lz + e) << 52) + (W >> 11) + ((W >> 10) & 1)
+        sh = V.bit_length() - 53
+        bits = ((1022 - 60 + 52 + sh + e) << 52) + ((V + (1 << (sh - 1))) >> sh)
         res.append(struct.unpack("<d", struct.pack("<q", bits))[0])
     return tuple(res)
 
@@ -257,7 +254,7 @@ def write_header(table, fixed, path=OUT):
         lines.append("    {" + ", ".join("%.17g" % v for v in small[f]) + "},")
     lines.append("};")
     lines.append("// the same coefficients times 2^{(k mod 3)/3} in fixed point: power j < %d at" % TAIL)
-    lines.append("// scale 2^(60 + j), the others at 2^(48 + j); pairs (F, G) by power, then piece")
+    lines.append("// scale 2^(60 + j), the others at 2^(46 + j); pairs (F, G) by power, then piece")
     lines.append("#define QED_SYN64_TAIL %d" % TAIL)
     lines.append("static __device__ const longlong2 qed_syn64_main[QED_SYN64_TAIL][QED_SYN64_NPIECE] = {")
     for j in range(TAIL):
@@ -272,7 +269,7 @@ def write_header(table, fixed, path=OUT):
     for i in range(0, 256, 8):
         lines.append("    " + ", ".join("0x%016xull" % w for w in exp2[i:i + 8]) + ",")
     lines.append("};")
-    lines.append("#define QED_SYN64_LOG2E_FRAC 0x%016xull" % LOG2E_FRAC)
+    lines.append("#define QED_SYN64_LOG2E 0x%016xull" % LOG2E)
     lines.append("#define QED_SYN64_LN2 0x%016xull" % LN2)
     with open(path, "w") as fh:
         fh.write("\n".join(lines) + "\n")
