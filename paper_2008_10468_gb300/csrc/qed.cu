@@ -3166,8 +3166,9 @@ struct qed_ctx {
     NetState nets[2];
     int net_sel;
     float* d_partial;          // per-block partial gradients
-    float* d_batch;            // training inputs (2 per sample), targets and weights
-    int batch_cap;
+    float* d_batch;            // training inputs (2 per sample), targets and weights,
+                               // or the two-kernel step's arrays (train_floats)
+    size_t batch_cap;          // floats
     float* d_loss;
     // multi-step graph
     cudaGraph_t graph;
@@ -4360,6 +4361,27 @@ constexpr int kEvalU = 1024;        // evaluation points in u per row
 // The network the qed_sampler_* calls address (qed_sampler_process).
 NetState& cur_net(qed_ctx* ctx) { return ctx->nets[ctx->net_sel]; }
 
+// Launch of a kernel that may start before the one
+// before it in the stream has ended: it waits for it itself (chain_wait).
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*f)(P...), int blocks, int threads, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned int)blocks);
+    c.blockDim = dim3((unsigned int)threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, f, static_cast<P>(args)...);
+}
+
+// Batches whose tiles have a block of k_mlp_grad each are trained by k_train_fwd
+// and k_train_update; larger ones fill the GPU with k_mlp_grad.
+bool two_kernel_step(const qed_ctx* ctx, int ntiles) { return ntiles <= ctx->sms * 2; }
+
 qed_status sampler_alloc(qed_ctx* ctx, int max_batch) {
     if (!cur_net(ctx).d_theta) {
         QED_CUDA(ctx, cudaMalloc(&cur_net(ctx).d_theta, sizeof(float) * kMlpParams));
@@ -4379,13 +4401,22 @@ qed_status sampler_alloc(qed_ctx* ctx, int max_batch) {
                                                       cur_net(ctx).d_wtot);
         QED_CUDA(ctx, cudaGetLastError());
     }
-    if (max_batch > 0 && ctx->d_batch && ctx->batch_cap < max_batch) {
-        cudaFree(ctx->d_batch);
-        ctx->d_batch = nullptr;
-    }
-    if (max_batch > 0 && !ctx->d_batch) {
-        QED_CUDA(ctx, cudaMalloc(&ctx->d_batch, sizeof(float) * 4 * (size_t)max_batch));
-        ctx->batch_cap = max_batch;
+    if (max_batch > 0) {
+        const int ntiles = (max_batch + kTileS - 1) / kTileS;
+        const size_t need = two_kernel_step(ctx, ntiles) ? train_floats(ntiles) : 4 * (size_t)max_batch;
+        if (ctx->d_batch && ctx->batch_cap < need) {
+            cudaFree(ctx->d_batch);
+            ctx->d_batch = nullptr;
+        }
+        if (!ctx->d_batch) {
+            QED_CUDA(ctx, cudaMalloc(&ctx->d_batch, sizeof(float) * need));
+            ctx->batch_cap = need;
+        }
+        QED_CUDA(ctx, cudaFuncSetAttribute(k_train_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)sizeof(FwdSmem)));
+        QED_CUDA(ctx, cudaFuncSetAttribute(k_train_update,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)sizeof(UpdSmem)));
     }
     return QED_OK;
 }
@@ -4607,22 +4638,35 @@ qed_status qed_sampler_train(qed_ctx* ctx, uint64_t seed, int64_t samples, int b
     // the pair network learns chi_gamma >= 0.25 only: below, the pair rate
     // is negligible and the spectrum a spike at 1/2 (rejection keeps those)
     const float l10_lo = ctx->net_sel == 1 ? kPairLog10Lo : kMlpLog10Lo;
+    NetState& net = cur_net(ctx);
     for (long long k = 0; k < steps; ++k) {
-        k_sampler_batch<<<(batch + 255) / 256, 256, 0, ctx->stream>>>(
-            (uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)k, batch, l10_lo, kMlpLog10Hi,
-            cur_net(ctx).d_cdf, kCdfRows, kCdfM, v, tgt, wgt);
         const bool last = k + 1 == steps;
         if (last) QED_CUDA(ctx, cudaMemsetAsync(ctx->d_loss, 0, sizeof(float), ctx->stream));
-        k_mlp_grad<<<grid, 256, sizeof(TrainSmem), ctx->stream>>>(
-            cur_net(ctx).d_theta, v, tgt, wgt, batch, 1, cur_net(ctx).d_cdf, kCdfRows, kCdfM, ctx->d_partial,
-            last ? ctx->d_loss : nullptr);
         p1 *= b1;
         p2 *= b2;
         // cosine decay of the step size over the run
         const float lr_k = lr * 0.5f * (1.0f + cosf(3.14159265f * (float)k / (float)steps));
-        k_mlp_adam<<<(kMlpParams + 255) / 256, 256, 0, ctx->stream>>>(
-            ctx->d_partial, grid, cur_net(ctx).d_theta, cur_net(ctx).d_m1, cur_net(ctx).d_m2, cur_net(ctx).d_wbf, lr_k, b1, b2,
-            1e-8f, (float)(1.0 - p1), (float)(1.0 - p2), 1, nullptr);
+        if (two_kernel_step(ctx, ntiles)) {
+            QED_CUDA(ctx, launch_chained(k_train_fwd, ntiles * (kTileS / kFwdS), kFwdThreads, sizeof(FwdSmem),
+                                         ctx->stream, (const float*)net.d_theta, (uint32_t)seed,
+                                         (uint32_t)(seed >> 32), (uint32_t)k, batch, l10_lo,
+                                         kMlpLog10Hi, (const float*)net.d_cdf, kCdfRows, kCdfM,
+                                         ntiles, ctx->d_batch, last ? ctx->d_loss : nullptr));
+            QED_CUDA(ctx, launch_chained(k_train_update, kUpdBlocks, 256, sizeof(UpdSmem), ctx->stream,
+                                         (const float*)ctx->d_batch, ntiles, net.d_theta, net.d_m1,
+                                         net.d_m2, net.d_wbf, lr_k, b1, b2, 1e-8f,
+                                         (float)(1.0 - p1), (float)(1.0 - p2)));
+        } else {
+            k_sampler_batch<<<(batch + 255) / 256, 256, 0, ctx->stream>>>(
+                (uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)k, batch, l10_lo, kMlpLog10Hi,
+                net.d_cdf, kCdfRows, kCdfM, v, tgt, wgt);
+            k_mlp_grad<<<grid, 256, sizeof(TrainSmem), ctx->stream>>>(
+                net.d_theta, v, tgt, wgt, batch, 1, net.d_cdf, kCdfRows, kCdfM, ctx->d_partial,
+                last ? ctx->d_loss : nullptr);
+            k_mlp_adam<<<(kMlpParams + 255) / 256, 256, 0, ctx->stream>>>(
+                ctx->d_partial, grid, net.d_theta, net.d_m1, net.d_m2, net.d_wbf, lr_k, b1, b2,
+                1e-8f, (float)(1.0 - p1), (float)(1.0 - p2), 1, nullptr);
+        }
         QED_CUDA(ctx, cudaGetLastError());
     }
     cur_net(ctx).adam_t += steps;

@@ -143,16 +143,11 @@ __device__ __forceinline__ float cdf_row_density(const float* __restrict__ row, 
 // target x from the two neighbouring CDF rows (linear in log10 chi), and the
 // weight p(x), the density of x at the target: with it the squared error
 // p^2 (x - t)^2 is, to first order, the squared error of the CDF.
-__global__ void k_sampler_batch(uint32_t k0, uint32_t k1, uint32_t batch_index, int B,
-                                float l10_lo, float l10_hi,
-                                const float* __restrict__ cdf, int nrows, int M,
-                                float* __restrict__ v, float* __restrict__ target,
-                                float* __restrict__ weight) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= B) return;
+__device__ __forceinline__ void train_sample(uint32_t k0, uint32_t k1, uint32_t batch_index, int s,
+                                             float l10_lo, float l10_hi, float& l10, float& u,
+                                             float& L) {
     const uint4 r = philox4x32_10(make_uint4((uint32_t)s, batch_index, 0x5A4D4C50u, 0u), k0, k1);
-    const float l10 = l10_lo + (l10_hi - l10_lo) * u01(r.x);
-    float u, L;
+    l10 = l10_lo + (l10_hi - l10_lo) * u01(r.x);
     if (r.z & 1u) {
         u = u01(r.y);
         L = logitf_(u);
@@ -160,6 +155,17 @@ __global__ void k_sampler_batch(uint32_t k0, uint32_t k1, uint32_t batch_index, 
         L = (2.0f * u01(r.w) - 1.0f) * 16.0f;
         u = 1.0f / (1.0f + expf(-L));
     }
+}
+
+__global__ void k_sampler_batch(uint32_t k0, uint32_t k1, uint32_t batch_index, int B,
+                                float l10_lo, float l10_hi,
+                                const float* __restrict__ cdf, int nrows, int M,
+                                float* __restrict__ v, float* __restrict__ target,
+                                float* __restrict__ weight) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= B) return;
+    float l10, u, L;
+    train_sample(k0, k1, batch_index, s, l10_lo, l10_hi, l10, u, L);
     const float pos = (l10 - kMlpLog10Lo) / (kMlpLog10Hi - kMlpLog10Lo) * (float)(nrows - 1);
     const int i = min((int)pos, nrows - 2);
     const float w = pos - (float)i;
@@ -414,6 +420,39 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ thet
     if ((t & 31) == 0 && t < kTileS && loss_out) atomicAdd(loss_out, l / (float)B);
 }
 
+// One Adam step of parameter i, and its BF16 copy.
+// p: its value and moments before.
+__device__ __forceinline__ void adam_step(int i, float g, float3 p, float* __restrict__ theta,
+                                          float* __restrict__ m1, float* __restrict__ m2,
+                                          __nv_bfloat16* __restrict__ wbf, float lr, float beta1,
+                                          float beta2, float eps, float bc1, float bc2) {
+    // the roundings written out: two callers have to agree bit for bit
+    const float a = fmaf(1.0f - beta1, g, __fmul_rn(beta1, p.y));
+    const float b = fmaf(__fmul_rn(1.0f - beta2, g), g, __fmul_rn(beta2, p.z));
+    m1[i] = a;
+    m2[i] = b;
+    const float th = p.x - lr * (a / bc1) / (sqrtf(b / bc2) + eps);
+    theta[i] = th;
+    wbf[i] = __float2bfloat16_rn(th);
+}
+
+// Kernels of a chain (launched with programmatic stream serialisation): all
+// that reads or writes memory of the kernel before comes after chain_wait; the
+// next kernel's blocks may start once every block here has called chain_next.
+// Such memory changes while the kernel runs: it is read by __ldcg, never
+// through a const __restrict__ pointer (whose loads may move up or be stale).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void copy16_async(float* smem, const float4* g) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::
+                 "r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(g) : "memory");
+}
+__device__ __forceinline__ void copies_wait() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // Sum the partial gradients; optionally apply one Adam step and refresh the
 // BF16 copy.  grad_out (nullable) receives the summed gradient.
 __global__ void k_mlp_adam(const float* __restrict__ partial, int nparts, float* __restrict__ theta,
@@ -425,14 +464,364 @@ __global__ void k_mlp_adam(const float* __restrict__ partial, int nparts, float*
     float g = 0.0f;
     for (int p = 0; p < nparts; ++p) g += partial[(size_t)p * kMlpParams + i];
     if (grad_out) grad_out[i] = g;
-    if (!apply) return;
-    const float a = beta1 * m1[i] + (1.0f - beta1) * g;
-    const float b = beta2 * m2[i] + (1.0f - beta2) * g * g;
-    m1[i] = a;
-    m2[i] = b;
-    const float th = theta[i] - lr * (a / bc1) / (sqrtf(b / bc2) + eps);
-    theta[i] = th;
-    wbf[i] = __float2bfloat16_rn(th);
+    if (apply)
+        adam_step(i, g, make_float3(theta[i], m1[i], m2[i]), theta, m1, m2, wbf, lr, beta1, beta2, eps, bc1, bc2);
+}
+
+// ---------------------------------------------------------------------------
+// One training step as two kernels, for batches of at most two tiles per SM
+// (every block of k_mlp_grad then has one tile).  The sums are those of
+// k_mlp_grad and k_mlp_adam in the same order, so the weights are the same bit
+// for bit; what changes is who forms them.  A batch of 2048 is 32 tiles, i.e.
+// 32 blocks of k_mlp_grad on 152 SMs, each with 17 shared-memory loads for 16
+// multiply-adds, and its targets (an inverse-CDF search of 24 dependent loads)
+// are not used by the CDF loss.  Here 16 samples are a block of the forward and
+// backward pass (128 blocks), which writes the activations and their gradients,
+// and an 8 x 8 piece of a weight matrix over all samples is a block of the
+// second kernel (144 blocks), which applies Adam to it.  Operands come by
+// 128-bit loads, four multiply-adds to a load; the kernels are launched
+// chained, so that their starts overlap.  Bound by latency: of 19 us a step at
+// batch 2048 (51.6 with the three kernels; 23.9 unchained) 7.5 are the forward
+// and backward pass and 3.5 the update, in chains of 64 multiply-adds (their
+// order is kept), the rest lies between the kernels.
+// ---------------------------------------------------------------------------
+constexpr int kFwdS = 16;        // samples per block of the forward and backward pass
+constexpr int kFwdPad = kMlpW + 4;
+constexpr int kFwdQ = 4;         // ... per thread
+constexpr int kFwdThreads = kMlpW * kFwdS / kFwdQ;
+// Per-sample arrays of the second kernel, [8 groups][samples][8 values] each
+// (samples padded to whole tiles), then v (2 per sample) and dout.
+enum { kTrA1, kTrA2, kTrA3, kTrD1, kTrD2, kTrD3, kTrArrays };
+__host__ __device__ inline size_t train_floats(int ntiles) {
+    return (size_t)ntiles * kTileS * (kTrArrays * kMlpW + 3);
+}
+
+struct FwdSmem {
+    float W2[kMlpW * kFwdPad], W3[kMlpW * kFwdPad];
+    float A[kFwdS * kFwdPad], D[kFwdS * kFwdPad];
+    float W1[kMlpW * 2], b1[kMlpW], b2[kMlpW], b3[kMlpW], w4[kMlpW];
+    float v[kFwdS * 2], dout[kFwdS];
+    float b4;
+};
+
+// acc[q] = b + sum_j W[n][j] in[s0 + q][j], j in order.
+__device__ __forceinline__ void fwd_layer(const float* __restrict__ W, float b,
+                                          const float* __restrict__ in, int n, int s0,
+                                          float (&acc)[kFwdQ]) {
+#pragma unroll
+    for (int q = 0; q < kFwdQ; ++q) acc[q] = b;
+#pragma unroll 4
+    for (int j = 0; j < kMlpW; j += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(W + n * kFwdPad + j);
+#pragma unroll
+        for (int q = 0; q < kFwdQ; ++q) {
+            const float4 a = *reinterpret_cast<const float4*>(in + (s0 + q) * kFwdPad + j);
+            acc[q] = fmaf(w.x, a.x, acc[q]);
+            acc[q] = fmaf(w.y, a.y, acc[q]);
+            acc[q] = fmaf(w.z, a.z, acc[q]);
+            acc[q] = fmaf(w.w, a.w, acc[q]);
+        }
+    }
+}
+
+// acc[q] = sum_m W[m][j] d[s0 + q][m], m in order.
+__device__ __forceinline__ void bwd_layer(const float* __restrict__ W, const float* __restrict__ d,
+                                          int j, int s0, float (&acc)[kFwdQ]) {
+#pragma unroll
+    for (int q = 0; q < kFwdQ; ++q) acc[q] = 0.0f;
+#pragma unroll 4
+    for (int m = 0; m < kMlpW; m += 4) {
+        float w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = W[(m + i) * kFwdPad + j];
+#pragma unroll
+        for (int q = 0; q < kFwdQ; ++q) {
+            const float4 a = *reinterpret_cast<const float4*>(d + (s0 + q) * kFwdPad + m);
+            acc[q] = fmaf(w[0], a.x, acc[q]);
+            acc[q] = fmaf(w[1], a.y, acc[q]);
+            acc[q] = fmaf(w[2], a.z, acc[q]);
+            acc[q] = fmaf(w[3], a.w, acc[q]);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kFwdThreads) k_train_fwd(const float* theta, uint32_t k0,
+                                                   uint32_t k1, uint32_t batch_index, int B,
+                                                   float l10_lo, float l10_hi,
+                                                   const float* __restrict__ cdf, int nrows, int M,
+                                                   int ntiles, float* buf,
+                                                   float* __restrict__ loss_out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    FwdSmem& S = *reinterpret_cast<FwdSmem*>(smem_raw);
+    const int t = threadIdx.x, n = t & 63, s0 = (t >> 6) * kFwdQ;
+    const int base = blockIdx.x * kFwdS, total = ntiles * kTileS;
+    // the samples come before the wait for the last step's weights
+    if (t < kFwdS) {
+        const int s = base + t;
+        float v0 = 0.0f, v1 = 0.0f;
+        if (s < B) {
+            float l10, u, L;
+            train_sample(k0, k1, batch_index, s, l10_lo, l10_hi, l10, u, L);
+            v0 = l10 * 0.5f;
+            v1 = L * kMlpLogitScale;
+        }
+        S.v[2 * t] = v0;
+        S.v[2 * t + 1] = v1;
+    }
+    chain_wait();
+    chain_next();
+    {
+        constexpr int kLoads = kMlpW * kMlpW / 4 / kFwdThreads;
+        const float4* w2 = reinterpret_cast<const float4*>(theta + kMlpOffW2);
+        const float4* w3 = reinterpret_cast<const float4*>(theta + kMlpOffW3);
+        float4 a[kLoads], b[kLoads];
+#pragma unroll
+        for (int k = 0; k < kLoads; ++k) {
+            a[k] = __ldcg(w2 + t + kFwdThreads * k);
+            b[k] = __ldcg(w3 + t + kFwdThreads * k);
+        }
+        const auto put = [&](float* W, int i, const float4& w) {   // i: float4 of the matrix
+            *reinterpret_cast<float4*>(W + (i >> 4) * kFwdPad + 4 * (i & 15)) =
+                make_float4(train_weight(w.x, 1), train_weight(w.y, 1), train_weight(w.z, 1),
+                            train_weight(w.w, 1));
+        };
+#pragma unroll
+        for (int k = 0; k < kLoads; ++k) {
+            put(S.W2, t + kFwdThreads * k, a[k]);
+            put(S.W3, t + kFwdThreads * k, b[k]);
+        }
+    }
+    if (t < 128) S.W1[t] = train_weight(__ldcg(theta + kMlpOffW1 + t), 1);
+    if (t < 64) {
+        S.b1[t] = train_weight(__ldcg(theta + kMlpOffB1 + t), 1);
+        S.b2[t] = train_weight(__ldcg(theta + kMlpOffB2 + t), 1);
+    } else if (t < 128) {
+        S.b3[t - 64] = train_weight(__ldcg(theta + kMlpOffB3 + t - 64), 1);
+        S.w4[t - 64] = train_weight(__ldcg(theta + kMlpOffW4 + t - 64), 1);
+    }
+    if (t == 0) S.b4 = train_weight(__ldcg(theta + kMlpOffB4), 1);
+    if (t < 2 * kFwdS) buf[(size_t)kTrArrays * kMlpW * total + 2 * base + t] = S.v[t];
+    __syncthreads();
+    // this thread's place in array `a` of the second kernel
+    const auto out = [&](int a, int q) -> float& {
+        return buf[((size_t)(a * 8 + (n >> 3)) * total + base + s0 + q) * 8 + (n & 7)];
+    };
+    float z1[kFwdQ], z2[kFwdQ], z3[kFwdQ];
+#pragma unroll
+    for (int q = 0; q < kFwdQ; ++q) {
+        const int s = s0 + q;
+        z1[q] = fmaf(S.W1[2 * n], S.v[2 * s], fmaf(S.W1[2 * n + 1], S.v[2 * s + 1], S.b1[n]));
+        const float a = siluf_(z1[q]);
+        S.A[s * kFwdPad + n] = a;
+        out(kTrA1, q) = a;
+    }
+    __syncthreads();
+    fwd_layer(S.W2, S.b2[n], S.A, n, s0, z2);
+#pragma unroll
+    for (int q = 0; q < kFwdQ; ++q) {
+        const float a = siluf_(z2[q]);
+        S.D[(s0 + q) * kFwdPad + n] = a;
+        out(kTrA2, q) = a;
+    }
+    __syncthreads();
+    fwd_layer(S.W3, S.b3[n], S.D, n, s0, z3);
+#pragma unroll
+    for (int q = 0; q < kFwdQ; ++q) {
+        const float a = siluf_(z3[q]);
+        S.A[(s0 + q) * kFwdPad + n] = a;
+        out(kTrA3, q) = a;
+    }
+    __syncthreads();
+    if (t < kFwdS) {
+        float o = S.b4 + anchor_of_v1(S.v[2 * t + 1]);
+#pragma unroll 4
+        for (int j = 0; j < kMlpW; j += 4) {
+            const float4 w = *reinterpret_cast<const float4*>(S.w4 + j);
+            const float4 a = *reinterpret_cast<const float4*>(S.A + t * kFwdPad + j);
+            o = fmaf(w.x, a.x, o);
+            o = fmaf(w.y, a.y, o);
+            o = fmaf(w.z, a.z, o);
+            o = fmaf(w.w, a.w, o);
+        }
+        const float x = sigmoidf_(o);
+        const bool ok = base + t < B;
+        float c, p;
+        cdf_at(cdf, nrows, M, 2.0f * S.v[2 * t], x, &c, &p);
+        const float u = 1.0f / (1.0f + expf(-anchor_of_v1(S.v[2 * t + 1])));
+        const float r = ok ? c - u : 0.0f;
+        const float d = (2.0f / (float)B) * r * p * x * (1.0f - x);
+        S.dout[t] = d;
+        buf[(size_t)(kTrArrays * kMlpW + 2) * total + base + t] = d;
+        if (loss_out) {
+            float l = r * r;
+#pragma unroll
+            for (int k = 8; k > 0; k >>= 1) l += __shfl_xor_sync(0xffffu, l, k);
+            if (t == 0) atomicAdd(loss_out, l / (float)B);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kFwdQ; ++q) {
+        const float d = S.dout[s0 + q] * S.w4[n] * dsiluf_(z3[q]);
+        S.D[(s0 + q) * kFwdPad + n] = d;
+        out(kTrD3, q) = d;
+    }
+    __syncthreads();
+    float acc[kFwdQ];
+    bwd_layer(S.W3, S.D, n, s0, acc);
+#pragma unroll
+    for (int q = 0; q < kFwdQ; ++q) {
+        const float d = acc[q] * dsiluf_(z2[q]);
+        S.A[(s0 + q) * kFwdPad + n] = d;
+        out(kTrD2, q) = d;
+    }
+    __syncthreads();
+    bwd_layer(S.W2, S.A, n, s0, acc);
+#pragma unroll
+    for (int q = 0; q < kFwdQ; ++q) out(kTrD1, q) = acc[q] * dsiluf_(z1[q]);
+}
+
+// Blocks 0..63 own 8 x 8 pieces of W3 (and those of the first column b3),
+// 64..127 of W2 (and b2), 128..135 eight weights of w4 each (and b4),
+// 136..143 eight rows of W1 (and b1).  A chunk of 32 tiles is in shared memory
+// at a time; a thread forms a 4 x 2 piece of one tile's sum.
+constexpr int kUpdTiles = 32;
+constexpr int kUpdStride = kTileS * 8 + 8;   // tiles of a warp's four slots in different banks
+struct UpdSmem {
+    float X[kUpdTiles * kUpdStride], Y[kUpdTiles * kUpdStride];
+    float part[kUpdTiles * 64];
+    float bias[kUpdTiles * 8];
+};
+constexpr int kUpdBlocks = 144;
+
+__global__ void __launch_bounds__(256) k_train_update(const float* buf, int ntiles, float* theta,
+                                                      float* m1, float* m2,
+                                                      __nv_bfloat16* wbf, float lr,
+                                                      float beta1, float beta2, float eps,
+                                                      float bc1, float bc2) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    UpdSmem& S = *reinterpret_cast<UpdSmem*>(smem_raw);
+    const int t = threadIdx.x, total = ntiles * kTileS;
+    const int role = blockIdx.x < 128 ? (int)blockIdx.x >> 6 : 2 + (((int)blockIdx.x - 128) >> 3);
+    const int gn = role < 2 ? ((int)blockIdx.x & 63) >> 3 : (int)blockIdx.x & 7;
+    const int gj = (int)blockIdx.x & 7;
+    const float* vg = buf + (size_t)kTrArrays * kMlpW * total;
+    const float* dg = vg + 2 * (size_t)total;
+    const int xa = role == 0 ? kTrD3 : (role == 1 ? kTrD2 : (role == 2 ? kTrA3 : kTrD1));
+    const float4* X4 = reinterpret_cast<const float4*>(buf + (size_t)(xa * 8 + gn) * total * 8);
+    const float4* Y4 = reinterpret_cast<const float4*>(
+        buf + (size_t)((role == 0 ? kTrA2 : kTrA1) * 8 + gj) * total * 8);
+    const bool bias = role == 3 || (role < 2 && gj == 0);
+    // this thread's parameter (threads below 72)
+    int i_par = -1;
+    if (t < 64) {
+        if (role < 2)
+            i_par = (role == 0 ? kMlpOffW3 : kMlpOffW2) + (gn * 8 + (t >> 3)) * kMlpW + gj * 8 + (t & 7);
+        else if (role == 2)
+            i_par = t < 8 ? kMlpOffW4 + gn * 8 + t : -1;
+        else
+            i_par = t < 16 ? kMlpOffW1 + 2 * gn * 8 + t : -1;
+    } else if (t < 72) {
+        if (bias)
+            i_par = (role == 0 ? kMlpOffB3 : (role == 1 ? kMlpOffB2 : kMlpOffB1)) + gn * 8 + t - 64;
+        else if (role == 2 && gn == 0 && t == 64)
+            i_par = kMlpOffB4;
+    }
+    // its state was written by the last step's update, which has ended: the
+    // blocks before this one in the chain have waited for it
+    float3 par = make_float3(0.0f, 0.0f, 0.0f);
+    if (i_par >= 0) 
+        par = make_float3(__ldcg(theta + i_par), __ldcg(m1 + i_par), __ldcg(m2 + i_par));
+    chain_wait();
+    chain_next();
+    float g = 0.0f, gb = 0.0f;   // threads below 64: this thread's weight; below 8: its bias
+    for (int c0 = 0; c0 < ntiles; c0 += kUpdTiles) {
+        const int nt = min(kUpdTiles, ntiles - c0);
+        __syncthreads();   // the last chunk has been summed
+        for (int i = t; i < nt * kTileS * 2; i += 256) {
+            const int tile = i >> 7, r = i & 127;   // 128 float4 a tile
+            copy16_async(S.X + tile * kUpdStride + 4 * r, X4 + (size_t)c0 * kTileS * 2 + i);
+            if (role < 2)
+                copy16_async(S.Y + tile * kUpdStride + 4 * r, Y4 + (size_t)c0 * kTileS * 2 + i);
+        }
+        if (role >= 2)   // dout, or v: one or two values a sample
+            for (int i = t; i < nt * kTileS; i += 256) {
+                const size_t s = (size_t)c0 * kTileS + i;
+                if (role == 2) {
+                    S.Y[i] = __ldcg(dg + s);
+                } else {
+                    S.Y[2 * i] = __ldcg(vg + 2 * s);
+                    S.Y[2 * i + 1] = __ldcg(vg + 2 * s + 1);
+                }
+            }
+        copies_wait();
+        __syncthreads();
+        const int tile = t >> 3, u = t & 7;
+        if (tile < nt) {
+            const float* X = S.X + tile * kUpdStride;
+            if (role < 2) {
+                const int n = (u & 1) * 4, j = (u >> 1) * 2;
+                const float* Y = S.Y + tile * kUpdStride;
+                float a[4][2];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a[i][0] = a[i][1] = 0.0f;
+#pragma unroll 8
+                for (int s = 0; s < kTileS; ++s) {
+                    const float4 x = *reinterpret_cast<const float4*>(X + 8 * s + n);
+                    const float2 y = *reinterpret_cast<const float2*>(Y + 8 * s + j);
+                    a[0][0] = fmaf(x.x, y.x, a[0][0]);
+                    a[0][1] = fmaf(x.x, y.y, a[0][1]);
+                    a[1][0] = fmaf(x.y, y.x, a[1][0]);
+                    a[1][1] = fmaf(x.y, y.y, a[1][1]);
+                    a[2][0] = fmaf(x.z, y.x, a[2][0]);
+                    a[2][1] = fmaf(x.z, y.y, a[2][1]);
+                    a[3][0] = fmaf(x.w, y.x, a[3][0]);
+                    a[3][1] = fmaf(x.w, y.y, a[3][1]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    S.part[tile * 64 + (n + i) * 8 + j] = a[i][0];
+                    S.part[tile * 64 + (n + i) * 8 + j + 1] = a[i][1];
+                }
+            } else if (role == 2) {
+                const float* d = S.Y + tile * kTileS;
+                float a = 0.0f, b = 0.0f;
+#pragma unroll 8
+                for (int s = 0; s < kTileS; ++s) {
+                    a = fmaf(d[s], X[8 * s + u], a);
+                    b += d[s];
+                }
+                S.part[tile * 64 + u] = a;
+                S.bias[tile * 8 + u] = b;
+            } else {
+                const float* v = S.Y + tile * kTileS * 2;
+                float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll 8
+                for (int s = 0; s < kTileS; ++s) {
+                    const float d = X[8 * s + u];
+                    a0 = fmaf(d, v[2 * s], a0);
+                    a1 = fmaf(d, v[2 * s + 1], a1);
+                }
+                S.part[tile * 64 + 2 * u] = a0;
+                S.part[tile * 64 + 2 * u + 1] = a1;
+            }
+            if (bias) {
+                float b = 0.0f;
+#pragma unroll 8
+                for (int s = 0; s < kTileS; ++s) b += X[8 * s + u];
+                S.bias[tile * 8 + u] = b;
+            }
+        }
+        __syncthreads();
+        // the tiles' sums in order
+        if (t < 64)
+            for (int i = 0; i < nt; ++i) g += S.part[i * 64 + t];
+        else if (t < 72)
+            for (int i = 0; i < nt; ++i) gb += S.bias[i * 8 + t - 64];
+    }
+    if (t >= 64) g = gb;
+    if (i_par >= 0)
+        adam_step(i_par, g, par, theta, m1, m2, wbf, lr, beta1, beta2, eps, bc1, bc2);
 }
 
 // ---------------------------------------------------------------------------
