@@ -862,17 +862,53 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
 // ---------------------------------------------------------------------------
 // Push mode: Algorithm 1 with the Boris push before every e+- draw
 // ---------------------------------------------------------------------------
-constexpr int kPushGroupMax = 16;   // busy lanes of a drained warp that switch to group mode
-constexpr int kPushPlanBatch = 8;   // lanes wanting a plan before the warp plans
-constexpr int kPushClaimBatch = 8;  // free lanes before the warp claims rows
-// A push-mode step.  The push makes every sub-step depend on the one before,
-// so a lane steps one particle through its sub-steps in order; a lane whose
-// particle is done takes the next row (the idle lanes of a warp share one
-// atomic on ctl->push_head, which starts at 0).  Per sub-step of an e+-: the
-// push over h, chi and eps of the new momentum, the squeeze bound for that
-// chi, the draw of sub-step s and the test.  A photon flies straight: its
-// momentum, chi and plan stay, as in the other kernels.  After an event the
-// particle is re-planned over the time that remains, from its state after
+constexpr int kPushBurst = 16;      // pushes of a lane per round,
+constexpr int kPushBurstFew = 32;   // and when at most 4 lanes are busy: fewer rounds per chain
+// lanes at a candidate before the warp tests them, lanes wanting a plan before
+// it plans (at most a quarter of the busy lanes: waiting for more stalls a warp
+// of few chains), free lanes before it claims rows
+constexpr int kPushTestBatch = 8, kPushPlanBatch = 8, kPushClaimBatch = 8, kPushFraction = 4;
+constexpr unsigned int kPushLook = 4;   // rounds between two looks of a starved warp
+constexpr unsigned int kBeatRounds = 1024;   // rounds of a warp between two beats
+
+struct PushBuf {      // one per warp
+    DrawKey key[32];
+    uint2 draw[32];   // drawing: first block of the window, last word that passes
+};
+
+// An upper bound of the squeeze threshold over the next m sub-steps of a
+// pushed e+-: a Boris push changes |p| by at most 2 |a| |E| (two half kicks
+// about a rotation), chi E_s <= eps |E| + |p| |B|, and the squeeze bound
+// c_h H(b) b^{2/3} grows with b (the tabulated H does not fall) and falls with
+// eps.  The margins of 1e-3 and more cover the roundings.
+__device__ __forceinline__ uint32_t push_cap(const PlanConst& PC, const SharedTables& sm,
+                                             const PState& st, const Fields& F, float a, float h,
+                                             uint32_t m) {
+    // 1e-38: a square that is lost below the smallest number must not lower the bound
+    const float E = sqrtf(fmaf(F.Ex, F.Ex, fmaf(F.Ey, F.Ey, fmaf(F.Ez, F.Ez, 1e-38f))));
+    const float B = sqrtf(fmaf(F.Bx, F.Bx, fmaf(F.By, F.By, fmaf(F.Bz, F.Bz, 1e-38f))));
+    const float p = sqrtf(fmaf(st.px, st.px, fmaf(st.py, st.py, fmaf(st.pz, st.pz, 1e-38f))));
+    const float d = 2.002f * fabsf(a) * E * (float)m + 1e-3f * p;
+    const float hi = p + d, lo = fmaxf(p - d, 0.0f);
+    const float b = 1.503f * PC.inv_Es * fmaf(1.0f + hi, E, hi * B);
+    if (!(b < 1e30f)) return 1u << 23;   // infinities and NaN as well
+    const float b23 = b > 0.0f ? exp2f(__log2f(b) * (2.0f / 3.0f)) : 0.0f;
+    const float c_h = 1.002f * PC.K * h * __fdividef(1.0f, sqrtf(fmaf(lo, lo, 1.0f)));
+    return squeeze_threshold(squeeze_bound(sm.sqz_e, sm.sqz_p, false, b, c_h, b23));
+}
+
+// A push-mode step.  The push makes every sub-step of an e+- depend on the one
+// before, so a lane moves one particle through its sub-steps in order; a lane
+// whose particle is done takes the next row (the idle lanes of a warp share
+// one atomic on ctl->push_head, which starts at 0).  But chi, the squeeze bound
+// and the test are needed only where the draw may pass: the draws do not depend
+// on the particle's state, so the warp draws a window of 64 sub-steps for a
+// lane at once (as the hot pass does) against an upper bound of the threshold
+// over the window (push_cap), and the lane pushes from candidate to candidate,
+// kPushBurst pushes a round; at a candidate it takes chi and eps of the pushed
+// momentum, the squeeze bound for that chi, and the test.  A photon flies
+// straight: it goes from candidate to candidate without a push.  After an event
+// the particle is re-planned over the time that remains, from its state after
 // the push and the recoil.
 //
 // kStream = false: one cascade generation, the rows [pass_begin, pass_end).
@@ -889,22 +925,29 @@ constexpr int kPushClaimBatch = 8;  // free lanes before the warp claims rows
 // (rows stored, rows completed, the beats of long chains) for SP.wait_ns
 // records QED_ERR_TIMEOUT and returns.
 //
+// What bounds it: the chain of pushes.  A lone chain takes about 285 clocks a
+// push (two correctly rounded square roots and divisions in series), so a store
+// of a few hundred long chains waits for them, and a large one for its warps'
+// issue slots.  Taking chi, the bound and the test out of the chain brought a
+// step of 2^22 rows (1% of them in a strong field, 91e6 sub-steps) from 5.95 to
+// 3.1 ms, 4096 rows that are all in it from 3.06 to 1.65 ms and 64 such rows from
+// 1.19 to 0.81 ms.
+//
 // Divergence control (both forms): a lane that wants a plan (a new row, or
-// after an event) waits until kPushPlanBatch lanes of its warp want one, or
-// until no busy lane is left to step; an accepted event is applied with the
-// lane's next plan; in the persistent form free lanes claim rows only once
-// kPushClaimBatch of them are free (or none is busy).  When the warp finds
-// no row to take and at most kPushGroupMax lanes are busy, it switches to
-// group mode (below).
-constexpr unsigned int kBeatRounds = 1024;   // rounds of a warp between two beats
+// after an event) waits until kPushPlanBatch lanes of its warp want one, a lane
+// at a candidate until kPushTestBatch lanes are, or until no lane is left to
+// push; an accepted event is applied with the lane's next plan; in the
+// persistent form free lanes claim rows only once kPushClaimBatch of them are
+// free (or none is busy).
 template <bool kStream>
-__global__ void __launch_bounds__(kLaneThreads) k_push(DevParticles P, StepParams SP, Scratch S,
-                                                       DevCtl* ctl) {
+__global__ void __launch_bounds__(kLaneThreads, 2) k_push(DevParticles P, StepParams SP, Scratch S,
+                                                          DevCtl* ctl) {
     const uint32_t step = step_index(SP);
     __shared__ SharedTables sm;
+    __shared__ PushBuf push_buf[kLaneThreads / 32];
+    if (ctl->status == (int)QED_ERR_TIMEOUT) return;
     stage_tables(sm);
     __syncthreads();
-    if (ctl->status == (int)QED_ERR_TIMEOUT) return;
     const bool first_pass = kStream || ctl->first_pass != 0;
     const long long begin = kStream ? 0 : (first_pass ? 0 : ctl->pass_begin);
     const long long n = kStream ? 0 : ctl->pass_end - begin;
@@ -912,10 +955,13 @@ __global__ void __launch_bounds__(kLaneThreads) k_push(DevParticles P, StepParam
     const bool cascade = SP.cascade != 0;
     constexpr unsigned int kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
+    PushBuf& PB = push_buf[threadIdx.x >> 5];
+    const uint32_t y1 = draw_y1(step, SP.draw_keys);
     const PlanConst PC = plan_const(SP);
     Stats stats;
     bool busy = false, drained = kStream ? false : n <= 0, photon = false, electron = false;
     bool need_plan = false, removed = false;
+    bool at_cand = false;                          // the last sub-step's draw may pass: to be tested
     bool waiting = false;                          // kStream: the lane's row is still being written
     bool ev = false;                               // an accepted event not yet applied
     float ev_x = 0.0f, ev_eps = 0.0f, ev_chi = 0.0f;
@@ -935,8 +981,9 @@ __global__ void __launch_bounds__(kLaneThreads) k_push(DevParticles P, StepParam
     pl.b = pl.c_h = 0.0f;
     pl.h = ftime{0.0f, 0.0f};
     float chi = 0.0f, eps = 0.0f, a = 0.0f;
-    uint32_t k = 0, s = 0, blk = kNoEvent;
-    uint4 r = make_uint4(0u, 0u, 0u, 0u);
+    // s0: first sub-step of the plan; s: next one; [.., win): the window drawn,
+    // its candidates from s on in mA (even sub-steps) and mB (odd ones)
+    uint32_t s0 = 0, s = 0, win = 0, mA = 0, mB = 0;
     // a row the lane holds: start its particle, or count the row as done
     auto take_row = [&](long long row) {
         const uint8_t type = P.type[row];
@@ -946,13 +993,13 @@ __global__ void __launch_bounds__(kLaneThreads) k_push(DevParticles P, StepParam
             if (time_positive(t_rem)) {
                 busy = true;
                 need_plan = true;
-                removed = false;
+                removed = at_cand = false;
                 electron = type == QED_ELECTRON;
                 id = P.id[row];
+                PB.key[lane] = draw_key(id, step, SP.draw_keys);
                 st = PState{P.px[row], P.py[row], P.pz[row]};
                 F = Fields{P.Ex[row], P.Ey[row], P.Ez[row], P.Bx[row], P.By[row], P.Bz[row]};
                 s = 0;
-                blk = kNoEvent;
                 return;
             }
         }
@@ -968,9 +1015,12 @@ __global__ void __launch_bounds__(kLaneThreads) k_push(DevParticles P, StepParam
             // initial rows.
             int got = 0;
             unsigned long long base = 0;
+            // A warp that found none goes on with its busy lanes for a few rounds
+            // before it looks again.
+            const bool none_busy = __ballot_sync(kAll, busy) == 0u;
             const bool claim = free_lanes != 0 &&
-                               (__popc(free_lanes) >= kPushClaimBatch ||
-                                __ballot_sync(kAll, busy) == 0u);
+                               (none_busy || (__popc(free_lanes) >= kPushClaimBatch &&
+                                              (!drained || rounds % kPushLook == 0u)));
             if (claim) {
                 const int want = __popc(free_lanes);
                 if (lane == 0) {
@@ -1006,7 +1056,7 @@ __global__ void __launch_bounds__(kLaneThreads) k_push(DevParticles P, StepParam
                 }
             }
             // the warp is starved when a claim left free lanes without a row
-            drained = claim && got < __popc(free_lanes);
+            if (claim) drained = got < __popc(free_lanes);
             if (waiting) {
                 const uint8_t ty = *reinterpret_cast<volatile uint8_t*>(P.type + i);
                 if (ty != kNotReady) {
@@ -1081,190 +1131,152 @@ __global__ void __launch_bounds__(kLaneThreads) k_push(DevParticles P, StepParam
                 if (lane == 0) atomicAdd(&ctl->beat, 1ull);
             }
         }
-        // plan the lane's particle (Algorithms 1/2, planning); true if it is
-        // done.  An accepted event of the lane's last sub-step is applied
-        // first (recoil or decay, children), so that the lanes of a warp
-        // apply their events together with their plans.
-        auto plan_now = [&]() -> bool {
+        bool done = false;
+        // plans: an accepted event of the lane's last sub-step is applied first
+        // (recoil or decay, children), so that the lanes of a warp apply their
+        // events together with their plans
+        const unsigned int pm = __ballot_sync(kAll, busy && need_plan);
+        const int batch = max(1, __popc(bm) / kPushFraction);
+        if ((__popc(pm) >= min(kPushPlanBatch, batch) || pm == bm) && busy && need_plan) {
             need_plan = false;
             if (ev) {
                 ev = false;
-                removed = apply_event(P, S, SP, ctl, i, id, photon, ev_x, ev_eps, ev_chi, step, s,
-                                      t_rem, st, stats, false, F, kStream);
-                ++s;
-                if (removed || !time_positive(t_rem)) return true;
+                removed = apply_event(P, S, SP, ctl, i, id, photon, ev_x, ev_eps, ev_chi, step,
+                                      s - 1u, t_rem, st, stats, false, F, kStream);
+                done = removed || !time_positive(t_rem);
             }
-            pl = plan_particle(SP, sm.sqz_e, sm.sqz_p, photon, st.px, st.py, st.pz, F.Ex, F.Ey,
-                               F.Ez, F.Bx, F.By, F.Bz, t_rem, &chi, &eps);
-            if (!(eps > 0.0f)) return true;
-            // per-cell counts: an initial row's first plan takes its cell's
-            // count when that is larger (the cell's sub-step)
-            apply_cell_count(SP, pl, sm.sqz_e, sm.sqz_p, photon, i, n_init, s, t_rem, eps);
-            stats.plans++;
-            stats.guard += pl.guard ? 1 : 0;
-            stats.max_N = max(stats.max_N, pl.N);
-            k = 0;
-            const float ah = __fmul_rn(kPi, pl.h.hi);
-            a = electron ? -ah : ah;
-            if (photon && pl.T == 0u) {
-                // a zero squeeze threshold admits no candidate
-                stats.substeps += pl.N;
-                s += pl.N;
-                return true;
+            if (!done) {
+                pl = plan_particle(SP, sm.sqz_e, sm.sqz_p, photon, st.px, st.py, st.pz, F.Ex, F.Ey,
+                                   F.Ez, F.Bx, F.By, F.Bz, t_rem, &chi, &eps);
+                done = !(eps > 0.0f);
             }
-            return false;
-        };
-        const int m = __popc(bm);
-        bool done = false;
-        if (drained && m <= kPushGroupMax) {
-            // Group mode: no rows are left and m <= kPushGroupMax lanes are
-            // busy.  The g-th busy lane's particle gets the G = 32 / m lanes
-            // [g G, (g+1) G):
-            // every lane of the group runs the same push chain from the
-            // owner's state and keeps the state after push j + 1 (j its place
-            // in the group), then tests sub-step s + j; the first accepted
-            // sub-step of the group decides, as in the sequential loop.  Only
-            // the pushes stay serial.
-            const int G = 32 / m;
-            const int g = lane / G, j = lane - g * G;
-            int owner = lane;
-            if (g < m) {
-                unsigned int mm = bm;
-                for (int t = 0; t < g; ++t) mm &= mm - 1u;
-                owner = __ffs(mm) - 1;
+            if (!done) {
+                // per-cell counts: an initial row's first plan takes its cell's
+                // count when that is larger (the cell's sub-step)
+                apply_cell_count(SP, pl, sm.sqz_e, sm.sqz_p, photon, i, n_init, s, t_rem, eps);
+                stats.plans++;
+                stats.guard += pl.guard ? 1 : 0;
+                stats.max_N = max(stats.max_N, pl.N);
+                s0 = win = s;
+                const float ah = __fmul_rn(kPi, pl.h.hi);
+                a = electron ? -ah : ah;
+                if (photon && pl.T == 0u) {
+                    // a zero squeeze threshold admits no candidate
+                    stats.substeps += pl.N;
+                    s += pl.N;
+                    done = true;
+                }
             }
-            const bool ready = busy && !need_plan;
-            if (busy && need_plan) done = plan_now();   // its group waits this round
-            const bool g_ready = (__shfl_sync(kAll, ready ? 1 : 0, owner) != 0) && g < m;
-            const float ox = __shfl_sync(kAll, st.px, owner), oy = __shfl_sync(kAll, st.py, owner),
-                        oz = __shfl_sync(kAll, st.pz, owner);
-            const float oa = __shfl_sync(kAll, a, owner);
-            const float oEx = __shfl_sync(kAll, F.Ex, owner), oEy = __shfl_sync(kAll, F.Ey, owner),
-                        oEz = __shfl_sync(kAll, F.Ez, owner), oBx = __shfl_sync(kAll, F.Bx, owner),
-                        oBy = __shfl_sync(kAll, F.By, owner), oBz = __shfl_sync(kAll, F.Bz, owner);
-            const float ohh = __shfl_sync(kAll, pl.h.hi, owner), ob = __shfl_sync(kAll, pl.b, owner),
-                        och = __shfl_sync(kAll, pl.c_h, owner), ochi = __shfl_sync(kAll, chi, owner),
-                        oeps = __shfl_sync(kAll, eps, owner);
-            const uint32_t oT = __shfl_sync(kAll, pl.T, owner), oN = __shfl_sync(kAll, pl.N, owner),
-                           ok = __shfl_sync(kAll, k, owner), os = __shfl_sync(kAll, s, owner);
-            const uint32_t oid0 = __shfl_sync(kAll, (uint32_t)id, owner),
-                           oid1 = __shfl_sync(kAll, (uint32_t)(id >> 32), owner);
-            const bool oph = __shfl_sync(kAll, photon ? 1 : 0, owner) != 0;
-            const uint32_t valid = g_ready ? min((uint32_t)G, oN - ok) : 0u;
-            PState q{ox, oy, oz}, mine = q;
-            const bool do_push = g_ready && !oph;
-            for (int t = 0; t < G; ++t) {
-                if (do_push && (uint32_t)t < valid)
-                    boris_push(q.px, q.py, q.pz, oa, oEx, oEy, oEz, oBx, oBy, oBz);
-                if (t == j) mine = q;
+        }
+        // a window for the lanes that have pushed through theirs
+        {
+            const bool need = busy && !need_plan && !at_cand && !done && s == win;
+            unsigned int nm = __ballot_sync(kAll, need);
+            if (nm) {
+                bool none = false;   // no draw can pass
+                if (need) {
+                    const uint32_t left = pl.N - (s - s0);
+                    win = s + min(left, 64u - (s & 63u));
+                    const uint32_t cap =
+                        photon ? pl.T : push_cap(PC, sm, st, F, a, pl.h.hi, win - s);
+                    PB.draw[lane] = make_uint2((s >> 6) << 5, (cap << 9) - 1u);   // (r >> 9) < cap
+                    mA = mB = 0u;
+                    none = cap == 0u;
+                }
+                nm &= ~__ballot_sync(kAll, none);
+                __syncwarp();
+                while (nm) {
+                    // two windows in flight
+                    const int o0 = __ffs(nm) - 1;
+                    nm &= nm - 1u;
+                    const int o1 = nm ? __ffs(nm) - 1 : o0;
+                    nm &= nm - 1u;
+                    const uint2 d0 = PB.draw[o0], d1 = PB.draw[o1];
+                    const uint4 c0 = draw_rounds(PB.key[o0], y1, d0.x + (uint32_t)lane, SP.draw_keys);
+                    const uint4 c1 = draw_rounds(PB.key[o1], y1, d1.x + (uint32_t)lane, SP.draw_keys);
+                    const unsigned int a0 = __ballot_sync(kAll, kPhiloxM1 * c0.z <= d0.y);
+                    const unsigned int b0 = __ballot_sync(kAll, kPhiloxM0 * c0.x <= d0.y);
+                    const unsigned int a1 = __ballot_sync(kAll, kPhiloxM1 * c1.z <= d1.y);
+                    const unsigned int b1 = __ballot_sync(kAll, kPhiloxM0 * c1.x <= d1.y);
+                    if (lane == o0) {
+                        mA = a0;
+                        mB = b0;
+                    } else if (lane == o1) {
+                        mA = a1;
+                        mB = b1;
+                    }
+                }
+                __syncwarp();
+                if (need) {   // candidates before s are past
+                    mA &= (uint32_t)(0xffffffffull << (((s & 63u) + 1u) >> 1));
+                    mB &= 0xffffffffu << ((s & 63u) >> 1);
+                }
             }
-            bool acc = false, cnd = false;
-            float cj = ochi, ej = oeps, xj = 0.0f;
-            if ((uint32_t)j < valid) {
-                float b = ob, c_h = och;
-                uint32_t T = oT;
-                if (!oph) {
-                    cj = chi_any(false, mine.px, mine.py, mine.pz, oEx, oEy, oEz, oBx, oBy, oBz,
-                                 PC.inv_Es, &ej);
-                    b = 1.5f * cj;
-                    c_h = PC.K * ohh * __fdividef(1.0f, ej);
+        }
+        // pushes: up to the next candidate, the end of the window, or the burst
+        const bool go = busy && !need_plan && !at_cand && !done;
+        {
+            uint32_t k = 0;
+            if (go) {
+                const uint32_t w0 = (win - 1u) & ~63u;
+                const uint32_t ca = 2u * (uint32_t)__clz(__brev(mA));
+                const uint32_t cb = 2u * (uint32_t)__clz(__brev(mB)) + 1u;
+                const uint32_t c = w0 + min(ca, cb);   // the next candidate, or beyond the window
+                const uint32_t stop = min(c - s + 1u, win - s);
+                k = photon ? stop
+                           : min(stop, (uint32_t)(__popc(bm) <= 4 ? kPushBurstFew : kPushBurst));
+                s += k;
+                stats.substeps += k;
+                if (min(ca, cb) < 64u && s == c + 1u && c < win) {
+                    at_cand = true;
+                    if (ca < cb) mA &= mA - 1u;
+                    else mB &= mB - 1u;
+                }
+                if (photon) k = 0;
+            }
+            const unsigned int most = __reduce_max_sync(kAll, k);
+#pragma unroll 1
+            for (uint32_t q = 0; q < most; ++q)
+                if (q < k) boris_push(st.px, st.py, st.pz, a, F.Ex, F.Ey, F.Ez, F.Bx, F.By, F.Bz);
+        }
+        // tests: chi of the pushed momentum, its squeeze bound, the draw
+        const unsigned int tm = __ballot_sync(kAll, at_cand);
+        if (tm && (__popc(tm) >= min(kPushTestBatch, batch) ||
+                   !__any_sync(kAll, busy && !need_plan && !at_cand && !done && s - s0 < pl.N))) {
+            if (at_cand) {
+                at_cand = false;
+                float b = pl.b, c_h = pl.c_h, chi_k = chi, eps_k = eps;
+                uint32_t T = pl.T;
+                if (!photon) {
+                    chi_k = chi_any(false, st.px, st.py, st.pz, F.Ex, F.Ey, F.Ez, F.Bx, F.By, F.Bz,
+                                    PC.inv_Es, &eps_k);
+                    b = 1.5f * chi_k;
+                    c_h = PC.K * pl.h.hi * __fdividef(1.0f, eps_k);
                     const float b23 = b > 0.0f ? exp2f(__log2f(b) * (2.0f / 3.0f)) : 0.0f;
                     T = squeeze_threshold(squeeze_bound(sm.sqz_e, sm.sqz_p, false, b, c_h, b23));
                 }
-                const uint32_t sj = os + (uint32_t)j;
-                const uint4 r = philox4x32_10(make_uint4(oid0, oid1, step, sj >> 1), SP.draw_keys);
-                const uint32_t yw = (sj & 1u) ? r.w : r.y;
-                xj = u01((sj & 1u) ? r.z : r.x);
+                const uint32_t c = s - 1u;
+                const uint4 r = draw_block(PB.key[lane], y1, c >> 1, SP.draw_keys);
+                const uint32_t yw = (c & 1u) ? r.w : r.y;
                 if ((yw >> 9) < T) {
-                    cnd = true;
+                    stats.cand++;
+                    const float x = u01((c & 1u) ? r.z : r.x);
                     float dtmp;
-                    acc = u01(yw) < acceptance(sm.syn, oph, b, c_h, xj, &dtmp);
+                    if (u01(yw) < acceptance(sm.syn, photon, b, c_h, x, &dtmp)) {
+                        // the event is applied with the next plan, s and the
+                        // pushed state stay until then
+                        t_rem = (s - s0 == pl.N) ? ftime{0.0f, 0.0f}
+                                                 : time_sub_mul(t_rem, s - s0, pl.h);
+                        ev = true;
+                        ev_x = x;
+                        ev_eps = eps_k;
+                        ev_chi = chi_k;
+                        need_plan = true;
+                    }
                 }
             }
-            const unsigned int am = __ballot_sync(kAll, acc);
-            const unsigned int gmask = G == 32 ? kAll : (((1u << G) - 1u) << (g * G));
-            const unsigned int ga = am & gmask;
-            const int jstar = ga ? __ffs(ga) - 1 - g * G : -1;
-            const uint32_t used = jstar >= 0 ? (uint32_t)jstar + 1u : valid;
-            if (cnd && (uint32_t)j < used) stats.cand++;
-            // each busy lane takes the outcome of the group it owns
-            const int my_g = __popc(bm & ((1u << lane) - 1u));
-            const int gl = (busy ? my_g : 0) * G;
-            const uint32_t used_o = __shfl_sync(kAll, used, gl);
-            const int jstar_o = __shfl_sync(kAll, jstar, gl);
-            const int src = gl + (used_o > 0u ? (int)used_o - 1 : 0);
-            const float nx = __shfl_sync(kAll, mine.px, src), ny = __shfl_sync(kAll, mine.py, src),
-                        nz = __shfl_sync(kAll, mine.pz, src);
-            const float nchi = __shfl_sync(kAll, cj, src), neps = __shfl_sync(kAll, ej, src),
-                        nxd = __shfl_sync(kAll, xj, src);
-            if (ready) {
-                stats.substeps += used_o;
-                st = PState{nx, ny, nz};
-                if (jstar_o >= 0) {
-                    const uint32_t kk = k + used_o;
-                    const ftime t_after = (kk == pl.N) ? ftime{0.0f, 0.0f}
-                                                       : time_sub_mul(t_rem, kk, pl.h);
-                    removed = apply_event(P, S, SP, ctl, i, id, photon, nxd, neps, nchi, step,
-                                          s + (uint32_t)jstar_o, t_after, st, stats, false, F,
-                                          kStream);
-                    s += used_o;
-                    t_rem = t_after;
-                    if (removed || !time_positive(t_rem)) done = true;
-                    else need_plan = true;
-                } else {
-                    s += used_o;
-                    k += used_o;
-                    if (k == pl.N) done = true;
-                }
-            }
-        } else {
-            // A plan taken by one or two lanes at a time would make the warp
-            // run the planner in most rounds while the others wait: a lane
-            // that wants a plan waits until kPushPlanBatch lanes want one, or
-            // until no busy lane is left to step, and then steps its first
-            // sub-step in the same round.
-            const unsigned int pm = __ballot_sync(kAll, busy && need_plan);
-            if ((__popc(pm) >= kPushPlanBatch || pm == bm) && busy && need_plan) done = plan_now();
         }
-        if (!(drained && m <= kPushGroupMax) && busy && !need_plan && !done) {
-            float b = pl.b, c_h = pl.c_h, chi_k = chi, eps_k = eps;
-            uint32_t T = pl.T;
-            if (!photon) {
-                boris_push(st.px, st.py, st.pz, a, F.Ex, F.Ey, F.Ez, F.Bx, F.By, F.Bz);
-                chi_k = chi_any(false, st.px, st.py, st.pz, F.Ex, F.Ey, F.Ez, F.Bx, F.By, F.Bz,
-                                PC.inv_Es, &eps_k);
-                b = 1.5f * chi_k;
-                c_h = PC.K * pl.h.hi * __fdividef(1.0f, eps_k);
-                const float b23 = b > 0.0f ? exp2f(__log2f(b) * (2.0f / 3.0f)) : 0.0f;
-                T = squeeze_threshold(squeeze_bound(sm.sqz_e, sm.sqz_p, false, b, c_h, b23));
-            }
-            if ((s >> 1) != blk) {
-                blk = s >> 1;
-                r = philox4x32_10(make_uint4((uint32_t)id, (uint32_t)(id >> 32), step, blk), SP.draw_keys);
-            }
-            const uint32_t yw = (s & 1u) ? r.w : r.y;
-            const float x = u01((s & 1u) ? r.z : r.x);
-            stats.substeps++;
-            bool acc = false;
-            if ((yw >> 9) < T) {
-                stats.cand++;
-                float dtmp;
-                acc = u01(yw) < acceptance(sm.syn, photon, b, c_h, x, &dtmp);
-            }
-            if (acc) {
-                // the event is applied with the next plan (plan_now), s and
-                // the pushed state stay until then
-                t_rem = (k + 1u == pl.N) ? ftime{0.0f, 0.0f} : time_sub_mul(t_rem, k + 1u, pl.h);
-                ev = true;
-                ev_x = x;
-                ev_eps = eps_k;
-                ev_chi = chi_k;
-                need_plan = true;
-            } else {
-                ++s;
-                if (++k == pl.N) done = true;
-            }
-        }
+        if (busy && !need_plan && !at_cand && s - s0 == pl.N) done = true;   // the plan ran out
         if (done) {
             busy = false;
             if (removed) {
