@@ -212,9 +212,9 @@ qed_status qed_plan_cells(qed_ctx* ctx, const qed_particles* p, int64_t n, const
  * Philox4x32-10 draws keyed by (id, step_index, sub-step), emits photons /
  * decays (photons are marked removed, type 3), recoils, and is re-planned
  * after every event over the remaining time.  Children are appended at rows
- * count.. and, if cascade_in_step, processed in the same step: generation by
- * generation while the generations are large, then (qed_set_tail) the rest
- * in one tail pass.  If out != NULL the call synchronises the stream and fills *out; if NULL it
+ * count.. and, if cascade_in_step, processed in the same step: in one
+ * persistent pass, or, with a learned sampler, generation by generation while
+ * the generations are large and the rest in one tail pass (qed_set_tail).  If out != NULL the call synchronises the stream and fills *out; if NULL it
  * returns without waiting (statistics readable with qed_read_stats).
  * Capacity: if the children do not fit, status QED_ERR_CAPACITY is returned
  * (in *out and as the return value when out != NULL) with the rows needed;
@@ -422,8 +422,11 @@ qed_status qed_set_launch(qed_ctx* ctx, uint32_t hot_min, uint32_t long_min,
                           int cold_blocks_per_sm, int hot_blocks_per_sm);
 
 /* Tail pass of the cascade (Sec. 2: the events of one step form a cascade
- * whose generations shrink).  Once a generation has fewer than tail_rows rows
- * the generations stop: one thread pass over that generation, then one
+ * whose generations shrink).  Without a learned sampler any tail_rows > 0 makes
+ * the whole step one thread pass and one persistent pass that takes every child
+ * as it is written (unless max_passes is below its default: then the
+ * generations are counted).  With one: once a generation has fewer than
+ * tail_rows rows the generations stop: one thread pass over that generation, then one
  * persistent kernel takes its queue and every child appended after it as
  * they come, so that the step is not bound by the longest chain of each
  * small generation in turn.  0 turns it off; default 131072 rows.  No

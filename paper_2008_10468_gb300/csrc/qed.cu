@@ -13,13 +13,17 @@
 //   k_hot_net              the same in sampler mode 1: long plans and the
 //                          sampler's particles one warp each, which evaluates
 //                          the network for its events
-//   k_advance              closes a cascade generation; below tail_rows rows
-//                          it hands the rest of the step to the tail pass
+//   k_stream               cascade step without a sampler: after the thread
+//                          pass over the initial rows one persistent launch
+//                          takes its queue and every child as it is written
+//   k_advance              closes a cascade generation (sampler modes, no
+//                          cascade, tail_rows 0); below tail_rows rows it
+//                          hands the rest of the step to the tail pass
 //   k_tail_begin / k_step / k_tail_end
-//                          tail pass: after one more thread pass, a persistent
-//                          kernel takes the queue and every child appended
-//                          later (no generations), children published by
-//                          their writers
+//                          tail pass of the sampler modes: after one more
+//                          thread pass, a persistent kernel takes the queue
+//                          and every child appended later, children published
+//                          by their writers
 //
 // Every sub-step draws (x, y) from Philox4x32-10 at counter
 // (id_lo, id_hi, step, s/2) under key = seed (even s: words 0,1; odd s:
@@ -55,6 +59,7 @@ constexpr uint32_t kSampLong = QED_SAMP_LONG;   // sampler: plans with N >= this
 #define QED_LONG_MIN 256
 #endif
 constexpr uint32_t kLongMinDefault = QED_LONG_MIN;  // ... and with N >= long_min to its warp mode
+constexpr int kMaxPassesDefault = 64;   // cascade generations per step
 constexpr long long kTailRowsDefault = 1ll << 17;   // generations below this go to the tail pass
 
 // Minimum resident blocks per SM requested from the register allocator:
@@ -79,8 +84,8 @@ struct DevCtl {
     int status;
     long long required;
     long long pass_begin, pass_end;
-    unsigned int hot_tail, hot_head;   // long plans: front of the queue array
-    unsigned int med_tail, med_head;   // medium plans: back of the queue array
+    unsigned int hot_tail;             // long plans: front of the queue array
+    unsigned int med_tail;             // medium plans: back of the queue array
     int more, passes;
     int first_pass;      // 1 until the first generation of the step is done
     int sticky;          // first error of a multi-step graph run: later steps do nothing
@@ -90,10 +95,10 @@ struct DevCtl {
     unsigned int hot_hw;            // long-plan queue entries written by this step's generations
     // tail pass (persistent kernel)
     long long n0;                   // first child row of the tail (rows before it are done)
+    long long n1;                   // rows in use when the last thread pass ended
+    unsigned int cold_done;         // its blocks that have ended
     unsigned long long child_head;  // next child row (from n0) to take
     unsigned long long finished;    // work units (queue entries, children) complete
-    unsigned int step_tail;         // long plans queued by the persistent kernel, stored
-                                    // after the thread pass's hot_tail entries
     int skip;                       // the tail pass does nothing
     unsigned long long push_head;   // push mode: next row of the generation to take
     // event-driven sampler, its queue of this generation: entries at the front
@@ -102,6 +107,13 @@ struct DevCtl {
     long long n_init;               // rows at the start of the step (the rest are children)
     unsigned long long beat;        // persistent passes: progress of long chains, so that
                                     // idle warps tell a long chain from a stalled step
+    // the queue's state, in a line of its own that idle warps poll with one load
+    struct alignas(128) Queue {
+        unsigned int hot_head, med_head;   // entries taken
+        unsigned int step_tail;            // entries queued by the persistent kernel, stored
+                                           // after the thread pass's hot_tail entries
+        unsigned int over;                 // every unit of the step is complete
+    } queue;
 };
 
 // Type byte of a child row that has been reserved but not yet written: in the
@@ -109,6 +121,7 @@ struct DevCtl {
 constexpr uint8_t kNotReady = 0xFF;
 // Row index of a long-plan queue entry that has not been written yet.
 constexpr uint32_t kNoItem = 0xFFFFFFFFu;
+constexpr uint32_t kVoidItem = 0xFFFFFFFEu;   // written, for a row that did not fit
 
 struct HotItem {
     uint32_t idx;
@@ -434,14 +447,14 @@ constexpr long long kReserveHere = -2;   // apply_event reserves the child rows 
 
 // Write the children of an accepted event into rows j.. (j < 0: they did not
 // fit) and the event into the log.  st: the parent before the event; the type
-// bytes come last.  kPublish: in a persistent pass another warp may be waiting
+// bytes come last.  Returns the child ids.  kPublish: in a persistent pass another warp may be waiting
 // for these rows: one fence for the event's children, then their type bytes.
 // kDeferred: the same, but fence and type bytes are the caller's.
 enum ChildMode { kPlain, kPublish, kDeferred };
 __device__ __forceinline__ uint8_t child_type(bool photon, int r) {
     return photon ? (r == 0 ? (uint8_t)QED_ELECTRON : (uint8_t)QED_POSITRON) : (uint8_t)QED_PHOTON;
 }
-__device__ __forceinline__ void write_children(const DevParticles& P, const Scratch& S,
+__device__ __forceinline__ ulonglong2 write_children(const DevParticles& P, const Scratch& S,
                                                const StepParams& SP, long long i, long long j,
                                                uint64_t id, bool photon, float x, float chi,
                                                uint32_t step, uint32_t s, ftime t_after,
@@ -480,6 +493,7 @@ __device__ __forceinline__ void write_children(const DevParticles& P, const Scra
             S.log[k] = r;
         }
     }
+    return make_ulonglong2(id0, id1);
 }
 
 // The parent after the event (recoil or decay).  True if it was removed.
@@ -854,6 +868,15 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
             P.px[i] = st.px;
             P.py[i] = st.py;
             P.pz[i] = st.pz;
+        }
+    }
+    // the last block to end notes the rows in use: the children so far (k_stream)
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&ctl->cold_done, 1u) == gridDim.x - 1u) {
+            ctl->n1 = (long long)stored_rows(P);
+            ctl->cold_done = 0u;
         }
     }
     flush_stats(stats, ctl);
@@ -2186,13 +2209,13 @@ __global__ void __launch_bounds__(kLaneThreads, QED_HOT_MIN_BLOCKS) k_hot(DevPar
                 if (lane == 0) {
                     if (more_long) {
                         const unsigned int k = (unsigned int)(first ? cap_long : room);
-                        base_l = atomicAdd(&ctl->hot_head, k);
+                        base_l = atomicAdd(&ctl->queue.hot_head, k);
                         got_l = base_l < n_long ? (int)min(k, n_long - base_l) : 0;
                         flags |= base_l + k >= n_long ? 1 : 0;
                     }
                     if (more_med && got_l < room) {
                         const unsigned int k = (unsigned int)(room - got_l);
-                        base_m = atomicAdd(&ctl->med_head, k);
+                        base_m = atomicAdd(&ctl->queue.med_head, k);
                         got_m = base_m < n_med ? (int)min(k, n_med - base_m) : 0;
                         flags |= base_m + k >= n_med ? 2 : 0;
                     }
@@ -2274,7 +2297,7 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_net(
         unsigned int wcand = 0;
         while (true) {
             unsigned int q = 0;
-            if (lane == 0) q = atomicAdd(&ctl->hot_head, 1u);
+            if (lane == 0) q = atomicAdd(&ctl->queue.hot_head, 1u);
             q = __shfl_sync(kAll, q, 0);
             if (q >= long_tail) break;
             warp_item<1>(P, S, SP, ctl, sm, dyn_smem, S.hot[q], step, k0, k1, wstats, wcand, false);
@@ -2303,7 +2326,7 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_net(
             const unsigned int idle = __ballot_sync(kAll, !active);
             if (idle) {
                 unsigned int base = 0;
-                if (lane == 0) base = atomicAdd(&ctl->med_head, (unsigned int)__popc(idle));
+                if (lane == 0) base = atomicAdd(&ctl->queue.med_head, (unsigned int)__popc(idle));
                 base = __shfl_sync(kAll, base, 0);
                 if (base + (unsigned int)__popc(idle) >= tail) more = false;
                 if (!active) {
@@ -2411,11 +2434,11 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_net(
 // queue and every child appended from then on (rows n0 and up) as they come.
 // As in the hot pass, a lane holds a particle, the warp draws the windows of
 // its lanes together, and lanes with an event or a new row plan together.  A
-// warp takes, in order, its share of the queue's long plans (each warp the
-// queue's length over the number of warps), child rows appended so far, then
-// the queue's medium plans.  With a learned sampler the long entries (the
-// sampler's particles among them) are stepped by a whole warp each
-// (warp_item), and so are the sampler's particles that appear later.
+// warp takes child rows appended so far, then its share of the queue's medium
+// plans (each warp the queue's length over the number of warps); the long
+// entries (the sampler's particles among them) are stepped by a whole warp each
+// (warp_item), and so are the sampler's particles that appear later.  (Without
+// a sampler the whole step is k_stream.)
 // A child row is published by its writer (type byte last, after a fence); a
 // lane that takes a row still being written waits for it.  Work units are the
 // thread pass's queue entries and the child rows; the pass ends when every
@@ -2459,7 +2482,7 @@ constexpr unsigned int kTailSpread = QED_TAIL_SPREAD;   // warps that share the 
 // Queue a long plan: the entry's row index is written last (readers wait for it).
 __device__ __forceinline__ void push_long(const Scratch& S, DevCtl* ctl, unsigned int cold_long,
                                           long long i, uint32_t s, ftime t_rem) {
-    const unsigned int k = cold_long + atomicAdd(&ctl->step_tail, 1u);
+    const unsigned int k = cold_long + atomicAdd(&ctl->queue.step_tail, 1u);
     HotItem* e = S.hot + k;
     e->s = s;
     e->t_rem = t_rem;
@@ -2467,7 +2490,7 @@ __device__ __forceinline__ void push_long(const Scratch& S, DevCtl* ctl, unsigne
     *reinterpret_cast<volatile uint32_t*>(&e->idx) = (uint32_t)i;
 }
 
-template <int kSampler, bool kCells = false>
+template <int kSampler>
 // Two resident blocks per SM (128 registers, no spills): the tail pass is
 // bound by latency, not by the number of warps.
 __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepParams SP,
@@ -2504,7 +2527,6 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
     const unsigned long long n0 = (unsigned long long)ctl->n0;
     const bool cascade = SP.cascade != 0;
     const unsigned int nwarps = blocks * (kLaneThreads / 32);
-    const unsigned int share_long = min(32u, (cold_long + nwarps - 1u) / nwarps);
     const unsigned int share_med = min(32u, (cold_med + nwarps - 1u) / nwarps);
     Stats stats;                 // per lane; the warp mode counts on lane 0
     unsigned int done = 0;       // units this lane completed, not yet added to ctl->finished
@@ -2518,23 +2540,23 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
     unsigned long long idle_ns = 0, seen = 0;
     unsigned int ticket = kNoItem;   // lane 0: long-queue entry taken, not yet pushed
     unsigned long long pend_lo = 0, pend_hi = 0;   // lane 0: child indices taken, not handed out
-    bool more_long = kSampler == 0 && cold_long != 0u, more_med = cold_med != 0u;   // lane 0
+    bool more_med = cold_med != 0u;   // lane 0
     bool timed_out = false;
     while (true) {
         // ---- 1. (sampler modes) a long plan, stepped by the whole warp.  Lane 0
         // takes a ticket with one atomic add when the queue looks non-empty; a
         // ticket past the tail is kept until its entry is pushed (void if the
         // step ends first).
-        if (kSampler != 0) {
+        {
             int got = 0;
             unsigned int q = 0;
             if (lane == 0) {
                 if (ticket == kNoItem &&
-                    *reinterpret_cast<volatile unsigned int*>(&ctl->hot_head) <
-                        cold_long + *reinterpret_cast<volatile unsigned int*>(&ctl->step_tail))
-                    ticket = atomicAdd(&ctl->hot_head, 1u);
+                    *reinterpret_cast<volatile unsigned int*>(&ctl->queue.hot_head) <
+                        cold_long + *reinterpret_cast<volatile unsigned int*>(&ctl->queue.step_tail))
+                    ticket = atomicAdd(&ctl->queue.hot_head, 1u);
                 if (ticket != kNoItem &&
-                    ticket < cold_long + *reinterpret_cast<volatile unsigned int*>(&ctl->step_tail)) {
+                    ticket < cold_long + *reinterpret_cast<volatile unsigned int*>(&ctl->queue.step_tail)) {
                     q = ticket;
                     ticket = kNoItem;
                     got = 1;
@@ -2565,7 +2587,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
                 it.t_rem.hi = __shfl_sync(kAll, it.t_rem.hi, 0);
                 it.t_rem.lo = __shfl_sync(kAll, it.t_rem.lo, 0);
                 const uint32_t k0 = (uint32_t)SP.seed, k1 = (uint32_t)(SP.seed >> 32);
-                warp_item<kSampler == 0 ? 1 : kSampler>(P, S, SP, ctl, sm, dyn_smem, it, step, k0,
+                warp_item<kSampler>(P, S, SP, ctl, sm, dyn_smem, it, step, k0,
                                                         k1, stats, stats.cand, true);
                 if (lane == 0) ++done;
                 idle = 0;
@@ -2589,59 +2611,47 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
             if (look || (free_lanes && __any_sync(kAll, lane == 0 && pend_lo < pend_hi))) {
                 const unsigned int want = (unsigned int)__popc(free_lanes);
                 unsigned long long base_c = 0;
-                unsigned int base_l = 0, base_m = 0;
-                int got_l = 0, got_c = 0, got_m = 0;
+                unsigned int base_m = 0;
+                int got_c = 0, got_m = 0;
                 if (lane == 0) {
                     // the control words are read at once, one round trip
-                    const unsigned int h_long =
-                        more_long ? *reinterpret_cast<volatile unsigned int*>(&ctl->hot_head) : 0u;
                     const unsigned int h_med =
-                        more_med ? *reinterpret_cast<volatile unsigned int*>(&ctl->med_head) : 0u;
+                        more_med ? *reinterpret_cast<volatile unsigned int*>(&ctl->queue.med_head) : 0u;
                     const unsigned long long ch =
                         *reinterpret_cast<volatile unsigned long long*>(&ctl->child_head);
                     const unsigned long long stored = cascade ? stored_rows(P) : n0;
-                    more_long = more_long && h_long < cold_long;
                     more_med = more_med && h_med < cold_med;
-                    if (more_long) {
-                        const unsigned int k = min(want, share_long);
-                        base_l = atomicAdd(&ctl->hot_head, k);
-                        got_l = base_l < cold_long ? (int)min(k, cold_long - base_l) : 0;
+                    if (pend_lo == pend_hi && ch < stored) {
+                        const unsigned long long k =
+                            min((unsigned long long)want,
+                                (stored - ch + kTailSpread - 1) / kTailSpread);
+                        pend_lo = atomicAdd(&ctl->child_head, k);
+                        pend_hi = pend_lo + k;
                     }
-                    if (got_l == 0) {
-                        if (pend_lo == pend_hi && ch < stored) {
-                            const unsigned long long k =
-                                min((unsigned long long)want,
-                                    (stored - ch + kTailSpread - 1) / kTailSpread);
-                            pend_lo = atomicAdd(&ctl->child_head, k);
-                            pend_hi = pend_lo + k;
-                        }
-                        if (pend_lo < pend_hi && pend_lo < stored) {
-                            got_c = (int)min((unsigned long long)want, min(pend_hi, stored) - pend_lo);
-                            base_c = pend_lo;
-                            pend_lo += (unsigned long long)got_c;
-                        }
+                    if (pend_lo < pend_hi && pend_lo < stored) {
+                        got_c = (int)min((unsigned long long)want, min(pend_hi, stored) - pend_lo);
+                        base_c = pend_lo;
+                        pend_lo += (unsigned long long)got_c;
                     }
-                    if (got_l == 0 && got_c == 0 && more_med) {
+                    if (got_c == 0 && more_med) {
                         const unsigned int k = min(want, share_med);
-                        base_m = atomicAdd(&ctl->med_head, k);
+                        base_m = atomicAdd(&ctl->queue.med_head, k);
                         got_m = base_m < cold_med ? (int)min(k, cold_med - base_m) : 0;
                     }
                 }
                 // one kind per claim
-                const int got = __shfl_sync(kAll, got_l + got_c + got_m, 0);
+                const int got = __shfl_sync(kAll, got_c + got_m, 0);
                 if (got) {
-                    const int kind = __shfl_sync(kAll, got_l ? 0 : (got_c ? 1 : 2), 0);
-                    const uint32_t base = __shfl_sync(
-                        kAll, got_l ? base_l : (got_c ? (uint32_t)base_c : base_m), 0);
+                    const bool kids = __shfl_sync(kAll, got_c != 0 ? 1 : 0, 0) != 0;
+                    const uint32_t base = __shfl_sync(kAll, got_c ? (uint32_t)base_c : base_m, 0);
                     const int rank = __popc(free_lanes & ((1u << lane) - 1u));
                     if (!L.active && !waiting && rank < got) {
                         // a child's row, or a queue entry's row, sub-step and time
-                        child = kind == 1;
+                        child = kids;
                         row = base + (uint32_t)rank;
                         waiting = true;
                         if (!child) {
-                            const HotItem it = S.hot[kind == 0 ? (long long)row
-                                                               : S.hot_cap - 1 - (long long)row];
+                            const HotItem it = S.hot[S.hot_cap - 1 - (long long)row];
                             row = it.idx;
                             L.s0 = it.s;
                             L.t_rem = it.t_rem;
@@ -2674,13 +2684,12 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
         bool fin = kids.mine && !L.need_plan;
         bool hand_over = false;
         if (L.need_plan) {
-            fin = lane_plan<kCells>(SP, sm, L, fld, ctl);
+            fin = lane_plan<false>(SP, sm, L, fld, ctl);
             if (!fin) {
                 stats.max_N = max(stats.max_N, L.pl.N);
-                hand_over = kSampler != 0 &&
-                            ((!L.photon && sampler_bin_ok(SP, L.chi)) ||
-                             (kSampler == 2 && L.photon && L.pl.N >= SP.hot_min &&
-                              pair_sampler_ok(SP, L.chi, L.pl.T)));
+                hand_over = (!L.photon && sampler_bin_ok(SP, L.chi)) ||
+                            (kSampler == 2 && L.photon && L.pl.N >= SP.hot_min &&
+                             pair_sampler_ok(SP, L.chi, L.pl.T));
                 if (!hand_over) fin = lane_count_plan(L, stats);
             }
         }
@@ -2772,6 +2781,362 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
     flush_stats(stats, ctl);
 }
 
+// ---------------------------------------------------------------------------
+// Cascade step without a sampler: the thread pass over the initial rows, then
+// one persistent launch that does the rest, whatever generation a particle
+// belongs to.  Its loop is the hot pass's; the queue goes on growing: a child
+// is written, then its queue entry (row, time left), then the entry's index,
+// and a lane that took an entry waits for that index.
+//
+// Launched generation by generation, every generation ends in its longest
+// chains with most of the GPU idle (11 of 16 warps resident on average) and
+// starts with a thread pass.  In one launch a step of 2^24 rows (1% in a strong
+// field, 1.0e9 sub-steps) takes 3.95 ms instead of 5.45, one of 2^20 rows with a
+// tenth in the field 2.05 instead of 3.68, and 4096 rows 0.28 instead of 0.35.
+// What bounds it is the issue rate of the warps' divergent parts (plans, tests)
+// and of the draws; children planned at birth by the warp that writes them cost
+// more than they saved, because the second copy of the plan's code did not fit
+// the instruction cache (2^24 rows: 4.3 ms).
+// ---------------------------------------------------------------------------
+constexpr int kStreamRefill = 8;             // idle lanes before a busy warp takes entries,
+constexpr unsigned int kStreamRounds = 8;    // and rounds between two looks at an empty queue
+constexpr unsigned int kStreamSpread = 16;   // warps that share the children on offer (256: 1.05
+                                             // instead of 0.98 ms at 2^20 rows)
+constexpr int kStreamLanes = 16;             // most particles of a warp, 32 when the queue holds
+constexpr unsigned int kStreamMany = 8;      // this many times the warps (always 16: 4.2 ms at 2^24)
+constexpr unsigned int kStreamNap = 4;       // idle warps poll every 256 ns << 0 ... 4
+
+// A warp's children.  Rows and entries are reserved at the start of a round,
+// written after its plans and published after its draws, so that the chains
+// that go on do not wait for the two atomics and the fence (65536 rows: 0.46
+// instead of 0.65 ms).
+struct StreamChildren {
+    bool mine = false, photon = false;   // this lane holds an event; its parent
+    int nq = 0, off_r = 0, off_q = 0;    // entries (0 or the children); offsets of rows, entries
+    unsigned long long base_r = 0;       // lane 0
+    unsigned int base_q = 0;             // lane 0
+    unsigned int n = 0;                  // events taken from the ring
+    uint32_t idx = kNoItem;              // written: the first child's index to publish
+    unsigned int entry = 0;
+};
+__device__ __forceinline__ StreamChildren stream_begin(const DevParticles& P, const StepParams& SP,
+                                                     DevCtl* ctl, const EventBuf& E, unsigned int n,
+                                                     unsigned int head) {
+    constexpr unsigned int kAll = 0xffffffffu;
+    const unsigned int lane = threadIdx.x & 31, below = (1u << lane) - 1u;
+    StreamChildren c;
+    c.n = min(n, 32u);
+    __syncwarp();
+    const unsigned int q = (head + lane) % kEventBuf;
+    c.mine = lane < c.n;
+    bool wanted = false;
+    if (c.mine) {
+        c.photon = E.x[q] < 0.0f;
+        wanted = time_positive(E.t_after[q]) && process_enabled(SP, !c.photon);
+    }
+    const unsigned int m1 = __ballot_sync(kAll, c.mine && !c.photon);
+    const unsigned int m2 = __ballot_sync(kAll, c.photon);
+    const unsigned int q1 = __ballot_sync(kAll, wanted && !c.photon);
+    const unsigned int q2 = __ballot_sync(kAll, wanted && c.photon);
+    c.off_r = __popc(m1 & below) + 2 * __popc(m2 & below);
+    c.off_q = __popc(q1 & below) + 2 * __popc(q2 & below);
+    c.nq = wanted ? (c.photon ? 2 : 1) : 0;
+    if (lane == 0) {
+        c.base_r = atomicAdd(reinterpret_cast<unsigned long long*>(P.count),
+                             (unsigned long long)(__popc(m1) + 2 * __popc(m2)));
+        if (q1 | q2)
+            c.base_q = atomicAdd(&ctl->queue.step_tail,
+                                 (unsigned int)(__popc(q1) + 2 * __popc(q2)));
+    }
+    return c;
+}
+__device__ __forceinline__ void stream_write(const DevParticles& P, const Scratch& S,
+                                            const StepParams& SP, DevCtl* ctl, const EventBuf& E,
+                                            unsigned int head, unsigned int cold_long,
+                                            StreamChildren& c, uint32_t step) {
+    constexpr unsigned int kAll = 0xffffffffu;
+    const unsigned long long base_r = __shfl_sync(kAll, c.base_r, 0);
+    c.entry = cold_long + __shfl_sync(kAll, c.base_q, 0) + (unsigned int)c.off_q;
+    if (c.mine) {
+        const unsigned int q = (head + (threadIdx.x & 31)) % kEventBuf;
+        const long long j = check_rows(P, ctl, (long long)base_r + c.off_r, c.photon ? 2 : 1);
+        write_children(P, S, SP, E.i[q], j, E.id[q], c.photon, fabsf(E.x[q]), E.chi[q], step,
+                       E.s[q], E.t_after[q], PState{E.px[q], E.py[q], E.pz[q]},
+                       Fields{E.f[0][q], E.f[1][q], E.f[2][q], E.f[3][q], E.f[4][q], E.f[5][q]},
+                       kPlain);
+        c.idx = j >= 0 ? (uint32_t)j : kVoidItem;
+        for (int k = 0; k < c.nq; ++k) {
+            S.hot[c.entry + k].s = 0u;
+            S.hot[c.entry + k].t_rem = E.t_after[q];
+        }
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ void stream_publish(const Scratch& S, const StreamChildren& c) {
+    if (c.nq) {
+        __threadfence();   // the children's rows and the entries before the indices
+        *reinterpret_cast<volatile uint32_t*>(&S.hot[c.entry].idx) = c.idx;
+        if (c.nq == 2)
+            *reinterpret_cast<volatile uint32_t*>(&S.hot[c.entry + 1].idx) =
+                c.idx == kVoidItem ? kVoidItem : c.idx + 1u;
+    }
+}
+
+// The queue's state, one load.
+__device__ __forceinline__ uint4 queue_state(const DevCtl* ctl) {
+    uint4 v;
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(&ctl->queue)
+                 : "memory");
+    return v;
+}
+
+template <bool kCells>
+__global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, StepParams SP, Scratch S,
+                                                            DevCtl* ctl) {
+    const uint32_t step = step_index(SP);
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    HotSmem& hs = *reinterpret_cast<HotSmem*>(dyn_smem);
+    SharedTables& sm = hs.tables;
+    LaneFields& fld = hs.fld;
+    // the thread pass's queue and children (fixed during this kernel)
+    const unsigned int cold_long = ctl->hot_tail, cold_med = ctl->med_tail;
+    const long long n0 = ctl->n0, n1 = ctl->n1;
+    const unsigned long long work = (unsigned long long)cold_long + cold_med + (unsigned long long)(n1 - n0);
+    const unsigned int blocks = (unsigned int)min(
+        (unsigned long long)gridDim.x, kTailMinBlocks + work * kTailWarps / (kLaneThreads / 32));
+    if (ctl->skip || ctl->status == (int)QED_ERR_TIMEOUT || blockIdx.x >= blocks) return;
+    stage_tables(sm);
+    __syncthreads();
+    constexpr unsigned int kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    ListBuf& B = hs.list[threadIdx.x >> 5];
+    EventBuf& E = hs.events[threadIdx.x >> 5];
+    unsigned int n_ev = 0, ev_head = 0;   // events whose children are not written yet
+    const uint32_t y1 = draw_y1(step, SP.draw_keys);
+    const unsigned int nwarps = blocks * (kLaneThreads / 32);
+    // units to complete: the thread pass's queue, each warp's part of its
+    // children, and every child queued so far
+    const unsigned long long units0 = (unsigned long long)cold_long + cold_med + nwarps;
+    const unsigned int share_long = max(1u, min(32u, (cold_long + nwarps - 1u) / nwarps));
+    const unsigned int share_med = max(1u, min(32u, (cold_med + nwarps - 1u) / nwarps));
+    Stats stats;                 // per lane
+    unsigned int done = 0;       // units this lane completed, not yet added to ctl->finished
+    Lane L;
+    L.pl.N = 0;
+    L.pl.T = 0;
+    L.pl.b = L.pl.c_h = 0.0f;
+    bool waiting = false;
+    unsigned int entry = 0;      // waiting: the queue entry,
+    bool from_med = false;       // counted from the back of the array
+    bool starved = false;        // the last look found the queue empty
+    bool pending = false;        // entries taken, not handed out
+    bool more_med = cold_med != 0u;                // lane 0
+    unsigned int pend_lo = 0, pend_hi = 0;         // lane 0: entries taken, not handed out
+    unsigned int idle = 0, rounds = 0;
+    unsigned long long idle_ns = 0, seen = 0;
+    bool timed_out = false, finish = false;
+    // ---- the thread pass's children
+    for (long long b = n0 + 32ll * (blockIdx.x * (kLaneThreads / 32) + (threadIdx.x >> 5)); b < n1;
+         b += 32ll * nwarps) {
+        const long long r = b + lane;
+        bool queue = r < n1;
+        ftime t{0.0f, 0.0f};
+        if (queue) {
+            const uint8_t type = P.type[r];
+            t = S.t_rem[r];
+            queue = type <= QED_PHOTON && process_enabled(SP, type == QED_PHOTON) && time_positive(t);
+        }
+        const unsigned int m = __ballot_sync(kAll, queue);
+        unsigned int q = 0;
+        if (lane == 0 && m) q = atomicAdd(&ctl->queue.step_tail, (unsigned int)__popc(m));
+        q = cold_long + __shfl_sync(kAll, q, 0) + (unsigned int)__popc(m & ((1u << lane) - 1u));
+        if (queue) {
+            S.hot[q].s = 0u;
+            S.hot[q].t_rem = t;
+            __threadfence();
+            *reinterpret_cast<volatile uint32_t*>(&S.hot[q].idx) = (uint32_t)r;
+        }
+    }
+    if (lane == 0) ++done;
+    while (true) {
+        // ---- 1. rows for the idle lanes
+        {
+            const unsigned int free_lanes = __ballot_sync(kAll, !L.active && !waiting);
+            const int n_free = __popc(free_lanes);
+            const bool look =
+                free_lanes == kAll ||
+                (n_free >= kStreamRefill && (!starved || rounds % kStreamRounds == 0u)) ||
+                (n_free != 0 && pending);
+            if (look) {
+                unsigned int base_l = 0, base_m = 0;
+                int got_l = 0, got_m = 0, dry = 0;
+                unsigned int over = 0;
+                if (lane == 0) {
+                    const uint4 qs = queue_state(ctl);
+                    const unsigned int h_long = qs.x, h_med = qs.y, tail = cold_long + qs.z;
+                    over = qs.w;
+                    more_med = more_med && h_med < cold_med;
+                    const unsigned int left = (h_long < tail ? tail - h_long : 0u) +
+                                              (more_med ? cold_med - h_med : 0u);
+                    const int room =
+                        n_free - (left >= kStreamMany * nwarps ? 0 : 32 - kStreamLanes);
+                    if (room > 0) {
+                        // the thread pass's long plans, its medium plans, then the
+                        // children: the chains left at the end are the shortest
+                        // (children first: 4.4 instead of 3.95 ms at 2^24 rows)
+                        if (pend_lo == pend_hi && h_long < (more_med ? min(tail, cold_long) : tail)) {
+                            const unsigned int k =
+                                h_long < cold_long
+                                    ? min((unsigned int)room, share_long)
+                                    : min((unsigned int)room,
+                                          (tail - h_long + kStreamSpread - 1) / kStreamSpread);
+                            pend_lo = atomicAdd(&ctl->queue.hot_head, k);
+                            pend_hi = pend_lo + k;
+                        }
+                        if (pend_lo < pend_hi && pend_lo < tail) {
+                            got_l = (int)min((unsigned int)room, min(pend_hi, tail) - pend_lo);
+                            base_l = pend_lo;
+                            pend_lo += (unsigned int)got_l;
+                        }
+                        if (more_med && got_l < room) {
+                            const unsigned int k = min((unsigned int)(room - got_l), share_med);
+                            base_m = atomicAdd(&ctl->queue.med_head, k);
+                            got_m = base_m < cold_med ? (int)min(k, cold_med - base_m) : 0;
+                        }
+                    }
+                    dry = (left <= (unsigned int)(got_l + got_m) ? 1 : 0) |
+                          (pend_lo < pend_hi ? 2 : 0);
+                }
+                got_l = __shfl_sync(kAll, got_l, 0);
+                got_m = __shfl_sync(kAll, got_m, 0);
+                base_l = __shfl_sync(kAll, base_l, 0);
+                base_m = __shfl_sync(kAll, base_m, 0);
+                dry = __shfl_sync(kAll, dry, 0);
+                starved = (dry & 1) != 0;
+                pending = (dry & 2) != 0;
+                finish = __shfl_sync(kAll, over, 0) != 0u;
+                const int rank = __popc(free_lanes & ((1u << lane) - 1u));
+                if (!L.active && !waiting && rank < got_l + got_m) {
+                    waiting = true;
+                    from_med = rank >= got_l;
+                    entry = from_med ? base_m + (unsigned int)(rank - got_l)
+                                     : base_l + (unsigned int)rank;
+                }
+            }
+        }
+        // ---- 2. lanes holding an entry: take its row once it is written
+        if (__any_sync(kAll, waiting)) {
+            uint32_t i = kNoItem;
+            const HotItem* e = S.hot + (from_med ? S.hot_cap - 1 - (long long)entry
+                                                 : (long long)entry);
+            if (waiting) i = *reinterpret_cast<const volatile uint32_t*>(&e->idx);
+            if (i != kNoItem) {
+                __threadfence();
+                const HotItem it = *e;
+                waiting = false;
+                if (i == kVoidItem) ++done;
+                else lane_take(P, SP, L, B, fld, step, i, P.type[i] == QED_PHOTON, it.s, it.t_rem);
+            }
+        }
+        // ---- 3. the events of the last round; they and new rows plan together
+        const bool had = L.active;
+        events_note(SP, L, E, fld, n_ev, ev_head, stats);
+        // the children: 32 events at a time, or at once when other warps may be
+        // waiting for them
+        const bool flush = n_ev != 0u && (starved || n_ev >= 32u || !__any_sync(kAll, L.active));
+        StreamChildren kids;
+        if (flush) kids = stream_begin(P, SP, ctl, E, n_ev, ev_head);
+        bool fin = had && !L.active;
+        if (L.need_plan) {
+            fin = lane_plan<kCells>(SP, sm, L, fld, ctl);
+            if (!fin) {
+                stats.max_N = max(stats.max_N, L.pl.N);
+                fin = lane_count_plan(L, stats);
+            }
+        }
+        if (fin) {
+            lane_finish(P, L);
+            ++done;
+        }
+        const bool on = __any_sync(kAll, L.active);
+        if (flush) {
+            stream_write(P, S, SP, ctl, E, ev_head, cold_long, kids, step);
+            n_ev -= kids.n;
+            ev_head += kids.n;
+        }
+        if (on) {
+            // ---- 4. the lists that have run out are drawn, the next candidates tested
+            idle = 0;
+            idle_ns = 0;
+            if (++rounds == kBeatRounds) {
+                rounds = 0;
+                if (lane == 0) atomicAdd(&ctl->beat, 1ull);
+            }
+            list_draw(B, L, y1, SP.draw_keys);
+            if (list_test(sm, B, L, y1, SP.draw_keys, stats.cand)) {
+                stats.substeps += L.pl.N;
+                lane_finish(P, L);
+                ++done;
+            }
+            if (flush) stream_publish(S, kids);
+            __syncwarp();   // the list buffer is reused by the next round
+            continue;
+        }
+        if (flush) stream_publish(S, kids);
+        // ---- 5. nothing to draw: wait for work, or finish.  The warp that
+        // completes the last unit sees as many units complete as are known, and
+        // says so in the word that idle warps poll.
+        if (n_ev) continue;
+        const bool hold = __any_sync(kAll, waiting);
+        if (!hold) {
+            const unsigned long long sum = warp_sum(done);
+            done = 0;
+            int again = 0;
+            if (lane == 0) {
+                if (sum) {
+                    __threadfence();   // this warp's entries before its completions
+                    const unsigned long long f = sum + atomicAdd(&ctl->finished, sum);
+                    const uint4 qs = queue_state(ctl);
+                    if (f == units0 + qs.z)
+                        *reinterpret_cast<volatile unsigned int*>(&ctl->queue.over) = 1u;
+                    again = 1;
+                }
+            }
+            if (__shfl_sync(kAll, again, 0) || !starved) continue;
+            if (finish) break;
+        }
+        // idle: back off from 256 ns to 4 us (64 ns while an entry is being
+        // written); the idle time counts from the last progress seen
+        const unsigned int nap = hold ? 64u : 256u << min(idle, kStreamNap);
+        ++idle;
+        idle_ns += nap;
+        if (idle_ns > SP.wait_ns && !hold) {
+            unsigned long long progress = 0;
+            if (lane == 0)
+                progress = *reinterpret_cast<volatile unsigned long long*>(&ctl->finished) +
+                           queue_state(ctl).z +
+                           *reinterpret_cast<volatile unsigned long long*>(&ctl->beat);
+            progress = __shfl_sync(kAll, progress, 0);
+            if (progress != seen && nap <= SP.wait_ns) {
+                seen = progress;
+                idle_ns = 0;
+            }
+        }
+        if (idle_ns > SP.wait_ns) {
+            timed_out = true;
+            break;
+        }
+        __nanosleep(nap);
+    }
+    if (timed_out && lane == 0) atomicExch(&ctl->status, (int)QED_ERR_TIMEOUT);
+    const unsigned long long sum = warp_sum(done);
+    if (lane == 0 && sum) atomicAdd(&ctl->finished, sum);
+    stats.warp_substeps = stats.substeps;
+    flush_stats(stats, ctl);
+}
+
 // Start a step.  keep_sticky: inside a multi-step graph, a step that follows
 // a failed step does nothing (its range is empty and it keeps the status).
 __global__ void k_step_init(DevCtl* ctl, long long* count, long long capacity, int keep_sticky) {
@@ -2811,8 +3176,9 @@ const void* hot_kernel(int mode, bool cells = false) {
 size_t hot_smem(int mode) { return mode == 1 ? kNetSmemBytes : sizeof(HotSmem); }
 // Their dynamic shared memory is above the default limit.
 cudaError_t allow_smem() {
-    const void* hot[] = {hot_kernel(1), hot_kernel(0), hot_kernel(0, true)};
-    for (int k = 0; k < 3; ++k) {
+    const void* hot[] = {hot_kernel(1), hot_kernel(0), hot_kernel(0, true),
+                         (const void*)k_stream<false>, (const void*)k_stream<true>};
+    for (int k = 0; k < 5; ++k) {
         const cudaError_t e = cudaFuncSetAttribute(
             hot[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hot_smem(k == 0 ? 1 : 0));
         if (e != cudaSuccess) return e;
@@ -2822,8 +3188,9 @@ cudaError_t allow_smem() {
 const void* step_kernel(int mode, bool cells = false) {
     return mode == 2 ? (const void*)k_step<2>
                      : mode ? (const void*)k_step<1>
-                            : cells ? (const void*)k_step<0, true> : (const void*)k_step<0>;
+                            : cells ? (const void*)k_stream<true> : (const void*)k_stream<false>;
 }
+size_t step_smem(int mode) { return mode ? kNetSmemBytes : sizeof(HotSmem); }
 
 // tail_rows > 0: a next generation of fewer rows goes to the tail pass
 // instead (ctl->tail set, the loop ends).
@@ -2838,9 +3205,9 @@ __global__ void k_advance(DevCtl* ctl, long long* count, long long capacity, int
     ctl->pass_begin = ctl->sticky ? 0 : ctl->pass_end;
     ctl->pass_end = ctl->sticky ? 0 : n;
     ctl->hot_hw = max(ctl->hot_hw, ctl->hot_tail);
-    ctl->hot_head = 0;
+    ctl->queue.hot_head = 0;
     ctl->hot_tail = 0;
-    ctl->med_head = 0;
+    ctl->queue.med_head = 0;
     ctl->med_tail = 0;
     ctl->samp_head = 0;
     ctl->samp_tail = 0;
@@ -2867,8 +3234,10 @@ __global__ void k_advance(DevCtl* ctl, long long* count, long long capacity, int
 // the generations wrote go back to "not written", so that a warp waiting for
 // an entry the persistent kernel pushes never reads an older one.  The thread
 // pass that follows runs over [pass_begin, pass_end) as one more generation.
-__global__ void k_tail_begin(DevParticles P, Scratch S, DevCtl* ctl) {
-    const bool on = ctl->tail != 0;
+// whole (k_stream): the step has no generations before it, and a child is
+// known by its queue entry, so no row is marked.
+__global__ void k_tail_begin(DevParticles P, Scratch S, DevCtl* ctl, int whole) {
+    const bool on = whole ? ctl->sticky == 0 : ctl->tail != 0;
     const long long n0 = ctl->pass_end;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -2877,9 +3246,10 @@ __global__ void k_tail_begin(DevParticles P, Scratch S, DevCtl* ctl) {
         ctl->n0 = n0;
         ctl->child_head = (unsigned long long)n0;
         ctl->finished = 0;
-        ctl->step_tail = 0;
+        ctl->queue.step_tail = 0;
+        if (whole) ctl->tail = on ? 1 : 0;
     }
-    if (!on) return;
+    if (!on || whole) return;
     for (long long r = n0 + t0; r < P.capacity; r += stride) P.type[r] = kNotReady;
     const long long used = min((long long)ctl->hot_hw, S.hot_cap);
     for (long long q = t0; q < used; q += stride) S.hot[q].idx = kNoItem;
@@ -2916,7 +3286,7 @@ __global__ void k_tail_end(DevParticles P, Scratch S, DevCtl* ctl) {
         }
     }
     const long long used =
-        min(max((long long)ctl->hot_hw, (long long)ctl->hot_tail + ctl->step_tail), S.hot_cap);
+        min(max((long long)ctl->hot_hw, (long long)ctl->hot_tail + ctl->queue.step_tail), S.hot_cap);
     for (long long q = t0; q < used; q += stride) S.hot[q].idx = kNoItem;
 }
 
@@ -3331,7 +3701,12 @@ qed_status ensure_samp(qed_ctx* ctx, long long cap, const StepParams& SP, Scratc
 int loop_hot_mode(const StepParams& SP) { return SP.sampler == 2 ? 0 : SP.sampler; }
 
 // Generations below this size go to the tail pass.
-long long tail_rows_for(const qed_ctx* ctx, const StepParams&) { return ctx->tail_rows; }
+// Without a sampler a cascade step is one thread pass and one persistent pass
+// (k_stream).  A limit on the generations below the default needs the
+// generations, and so does tail_rows 0.
+bool whole_step(int sampler, long long tail_rows, int max_passes) {
+    return sampler == 0 && tail_rows > 0 && max_passes >= kMaxPassesDefault;
+}
 
 // Bracket a launch with timing events when profiling is on; count it always.
 struct LaunchScope {
@@ -3453,7 +3828,7 @@ void qed_config_default(qed_config* c) {
     c->process_mask = QED_PROC_EMISSION | QED_PROC_PAIR;
     c->cascade_in_step = 1;
     c->recoil = 1;
-    c->max_passes = 64;
+    c->max_passes = kMaxPassesDefault;
     c->drain_chi = 0.0f;
     c->sampler_mode = 0;
     c->sampler_max_err = 1e-3f;
@@ -3469,7 +3844,7 @@ qed_status qed_init(qed_ctx** out, const qed_config* cfg, void* stream) {
     qed_ctx* ctx = new (std::nothrow) qed_ctx();
     if (!ctx) return QED_ERR_ARG;
     ctx->cfg = *cfg;
-    if (ctx->cfg.max_passes <= 0) ctx->cfg.max_passes = 64;
+    if (ctx->cfg.max_passes <= 0) ctx->cfg.max_passes = kMaxPassesDefault;
     ctx->stream = (cudaStream_t)stream;
     qed_status st = cuda_check(ctx, cudaGetDevice(&ctx->device), "cudaGetDevice");
     if (st == QED_OK)
@@ -3497,7 +3872,8 @@ qed_status qed_init(qed_ctx** out, const qed_config* cfg, void* stream) {
                                                       kNetSmemBytes);
         ctx->net_blocks = ctx->sms * (per_sm > 0 ? per_sm : 1);
         per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<0>, kLaneThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream<false>, kLaneThreads,
+                                                      step_smem(0));
         ctx->step_blocks = ctx->sms * (per_sm > 0 ? per_sm : 1);
         per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_plan, kColdThreads, 0);
@@ -3714,7 +4090,8 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
         LaunchScope ls(ctx, QED_KERNEL_CONTROL);
         k_step_init<<<1, 1, 0, ctx->stream>>>(ctx->d_ctl, D.count, D.capacity, 0);
     }
-    for (int pass = 0; pass < ctx->cfg.max_passes; ++pass) {
+    const int whole = cascade && whole_step(SP.sampler, ctx->tail_rows, ctx->cfg.max_passes) ? 1 : 0;
+    for (int pass = 0; !whole && pass < ctx->cfg.max_passes; ++pass) {
         {
             LaunchScope ls(ctx, QED_KERNEL_COLD);
             if (SP.N_cell) k_cold<true><<<ctx->cold_blocks, kColdThreads, 0, ctx->stream>>>(D, SP, S, ctx->d_ctl);
@@ -3740,7 +4117,7 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
         {
             LaunchScope ls(ctx, QED_KERNEL_CONTROL);
             k_advance<<<1, 1, 0, ctx->stream>>>(ctx->d_ctl, D.count, D.capacity, cascade ? 1 : 0,
-                                                ctx->cfg.max_passes, tail_rows_for(ctx, SP), 0ull,
+                                                ctx->cfg.max_passes, ctx->tail_rows, 0ull,
                                                 0);
         }
         QED_CUDA(ctx, cudaGetLastError());
@@ -3755,7 +4132,7 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
     S.samp = nullptr;
     {
         LaunchScope ls(ctx, QED_KERNEL_CONTROL);
-        k_tail_begin<<<ctx->sms * 8, 256, 0, ctx->stream>>>(D, S, ctx->d_ctl);
+        k_tail_begin<<<whole ? 1 : ctx->sms * 8, 256, 0, ctx->stream>>>(D, S, ctx->d_ctl, whole);
     }
     {
         LaunchScope ls(ctx, QED_KERNEL_COLD);
@@ -3771,8 +4148,8 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
         void* a[] = {&d, &sp, &sc, &c};
         QED_CUDA(ctx, cudaLaunchKernel(step_kernel(SP.sampler, SP.N_cell != nullptr),
                                        dim3(SP.sampler ? ctx->step_net_blocks : ctx->step_blocks),
-                                       dim3(kLaneThreads), a,
-                                       SP.sampler ? kNetSmemBytes : 0, ctx->stream));
+                                       dim3(kLaneThreads), a, step_smem(SP.sampler),
+                                       ctx->stream));
     }
     {
         LaunchScope ls(ctx, QED_KERNEL_CONTROL);
@@ -4033,12 +4410,57 @@ qed_status add_kernel(qed_ctx* ctx, cudaGraph_t g, cudaGraphNode_t* node, const 
                       "cudaGraphAddKernelNode");
 }
 
+// Adds a WHILE node after `dep`: one cascade generation per iteration (thread
+// pass, the event-driven sampler's pass, hot pass, generation control, which
+// sets the condition).
+qed_status add_generations(qed_ctx* ctx, cudaGraph_t g, cudaGraphNode_t dep, const DevParticles& Din,
+                           const StepParams& SPin, const Scratch& Sin, DevCtl* ctl_in,
+                           int more_allowed, cudaGraphNode_t* last) {
+    DevParticles D = Din;
+    StepParams SP = SPin;
+    Scratch S = Sin;
+    DevCtl* ctl = ctl_in;
+    long long* count = D.count;
+    long long capacity = D.capacity, tail_rows = ctx->tail_rows;
+    int max_passes = ctx->cfg.max_passes, use_handle = 1;
+    cudaGraphConditionalHandle h;
+    qed_status st =
+        cuda_check(ctx, cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault),
+                   "cudaGraphConditionalHandleCreate");
+    if (st != QED_OK) return st;
+    cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
+    memset(&cp.conditional, 0, sizeof cp.conditional);
+    cp.conditional.handle = h;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    st = cuda_check(ctx, cudaGraphAddNode(last, g, &dep, nullptr, 1, &cp), "cudaGraphAddNode");
+    if (st != QED_OK) return st;
+    cudaGraph_t body = cp.conditional.phGraph_out[0];
+    cudaGraphNode_t bc, bs, bh, ba;
+    void* a[] = {&D, &SP, &S, &ctl};
+    st = add_kernel(ctx, body, &bc, cold_kernel(SP.N_cell != nullptr), dim3(ctx->cold_blocks),
+                    dim3(kColdThreads), a, nullptr, 0);
+    bs = bc;
+    if (st == QED_OK && SP.sampler == 2)
+        st = add_kernel(ctx, body, &bs, (const void*)k_samp, dim3(ctx->samp_blocks),
+                        dim3(kLaneThreads), a, &bc, 1, kSampSmemBytes);
+    const int hm = loop_hot_mode(SP);
+    if (st == QED_OK)
+        st = add_kernel(ctx, body, &bh, hot_kernel(hm, SP.N_cell != nullptr),
+                        dim3(hm ? ctx->net_blocks : ctx->hot_blocks), dim3(kLaneThreads), a, &bs, 1,
+                        hot_smem(hm));
+    void* b[] = {&ctl, &count, &capacity, &more_allowed, &max_passes, &tail_rows, &h, &use_handle};
+    if (st == QED_OK)
+        st = add_kernel(ctx, body, &ba, (const void*)k_advance, dim3(1), dim3(1), b, &bh, 1);
+    return st;
+}
+
 // The tail pass after a step's generation loop (node `dep`): tail begin,
 // thread pass, persistent kernel, tail end (`last`).  Its kernels do nothing
 // when the generations ran to the end.
 qed_status add_tail_nodes(qed_ctx* ctx, cudaGraph_t g, cudaGraphNode_t dep, const DevParticles& Din,
                           const StepParams& SPin, const Scratch& Sin, DevCtl* ctl_in,
-                          cudaGraphNode_t* last) {
+                          int whole, cudaGraphNode_t* last) {
     DevParticles D = Din;
     StepParams SP = SPin;
     Scratch S = Sin;
@@ -4047,9 +4469,9 @@ qed_status add_tail_nodes(qed_ctx* ctx, cudaGraph_t g, cudaGraphNode_t dep, cons
     cudaGraphNode_t tb, tc, ts, te;
     qed_status st;
     {
-        void* a[] = {&D, &S, &ctl};
-        st = add_kernel(ctx, g, &tb, (const void*)k_tail_begin, dim3(ctx->sms * 8), dim3(256), a,
-                        &dep, 1);
+        void* a[] = {&D, &S, &ctl, &whole};
+        st = add_kernel(ctx, g, &tb, (const void*)k_tail_begin, dim3(whole ? 1 : ctx->sms * 8),
+                        dim3(256), a, &dep, 1);
     }
     if (st == QED_OK) {
         void* a[] = {&D, &SP, &S, &ctl};
@@ -4060,7 +4482,7 @@ qed_status add_tail_nodes(qed_ctx* ctx, cudaGraph_t g, cudaGraphNode_t dep, cons
         void* a[] = {&D, &SP, &S, &ctl};
         st = add_kernel(ctx, g, &ts, step_kernel(SP.sampler, SP.N_cell != nullptr),
                         dim3(SP.sampler ? ctx->step_net_blocks : ctx->step_blocks),
-                        dim3(kLaneThreads), a, &tc, 1, SP.sampler ? kNetSmemBytes : 0);
+                        dim3(kLaneThreads), a, &tc, 1, step_smem(SP.sampler));
     }
     if (st == QED_OK) {
         void* a[] = {&D, &S, &ctl};
@@ -4108,9 +4530,7 @@ qed_status qed_graph_capture(qed_ctx* ctx, const qed_particles* p, uint64_t firs
     DevCtl* ctl = ctx->d_ctl;
     long long* count = D.count;
     long long capacity = D.capacity;
-    int more_allowed = cascade_enabled(ctx->cfg) ? 1 : 0;
-    int max_passes = ctx->cfg.max_passes;
-    long long tail_rows = ctx->tail_rows;
+    const int more_allowed = cascade_enabled(ctx->cfg) ? 1 : 0;
     int keep_sticky = 1;
     float drain = ctx->cfg.drain_chi;
     double* hist = ctx->d_hist;
@@ -4139,47 +4559,13 @@ qed_status qed_graph_capture(qed_ctx* ctx, const qed_particles* p, uint64_t firs
             void* a[] = {&ctl, &count, &capacity, &keep_sticky};
             st = add_kernel(ctx, g, &init, (const void*)k_step_init, dim3(1), dim3(1), a, &prev, 1);
         }
-        // WHILE node: one cascade generation per iteration
-        cudaGraphConditionalHandle h;
-        if (st == QED_OK)
-            st = cuda_check(ctx, cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault),
-                            "cudaGraphConditionalHandleCreate");
-        if (st != QED_OK) break;
-        cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
-        memset(&cp.conditional, 0, sizeof cp.conditional);
-        cp.conditional.handle = h;
-        cp.conditional.type = cudaGraphCondTypeWhile;
-        cp.conditional.size = 1;
-        st = cuda_check(ctx, cudaGraphAddNode(&wnode, g, &init, nullptr, 1, &cp), "cudaGraphAddNode");
-        if (st != QED_OK) break;
-        cudaGraph_t body = cp.conditional.phGraph_out[0];
-        cudaGraphNode_t bc, bs, bh, ba;
-        int use_handle = 1;
-        {
-            void* a[] = {&D, &SP, &S, &ctl};
-            st = add_kernel(ctx, body, &bc, cold_kernel(SP.N_cell != nullptr), dim3(ctx->cold_blocks),
-                            dim3(kColdThreads), a, nullptr, 0);
-        }
-        bs = bc;
-        if (st == QED_OK && SP.sampler == 2) {
-            void* a[] = {&D, &SP, &S, &ctl};
-            st = add_kernel(ctx, body, &bs, (const void*)k_samp, dim3(ctx->samp_blocks),
-                            dim3(kLaneThreads), a, &bc, 1, kSampSmemBytes);
-        }
-        if (st == QED_OK) {
-            void* a[] = {&D, &SP, &S, &ctl};
-            const int hm = loop_hot_mode(SP);
-            st = add_kernel(ctx, body, &bh, hot_kernel(hm, SP.N_cell != nullptr),
-                            dim3(hm ? ctx->net_blocks : ctx->hot_blocks), dim3(kLaneThreads), a,
-                            &bs, 1, hot_smem(hm));
-        }
-        if (st == QED_OK) {
-            void* a[] = {&ctl,        &count, &capacity, &more_allowed, &max_passes,
-                         &tail_rows, &h,     &use_handle};
-            st = add_kernel(ctx, body, &ba, (const void*)k_advance, dim3(1), dim3(1), a, &bh, 1);
-        }
+        const int whole =
+            more_allowed && whole_step(SP.sampler, ctx->tail_rows, ctx->cfg.max_passes) ? 1 : 0;
+        wnode = init;
+        if (st == QED_OK && !whole)
+            st = add_generations(ctx, g, init, D, SP, S, ctl, more_allowed, &wnode);
         cudaGraphNode_t tend;
-        if (st == QED_OK) st = add_tail_nodes(ctx, g, wnode, D, SP, S, ctl, &tend);
+        if (st == QED_OK) st = add_tail_nodes(ctx, g, wnode, D, SP, S, ctl, whole, &tend);
         // compaction (and optional photon drain) after the cascade
         if (st == QED_OK) {
             void* a[] = {&D, &SP, &drain, &hist, &block_live};
@@ -4245,10 +4631,8 @@ qed_status qed_graph_read_stats(qed_ctx* ctx, qed_step_stats* out, int nsteps) {
 
 __global__ void k_set_step(uint32_t* p, uint32_t v) { *p = v; }
 
-// Build (when its key changed) and launch the one-step graph: step-init, then
-// a conditional WHILE node whose body is one cascade generation (thread
-// pass, hot pass, generation control; the control kernel sets the
-// condition).  The step index reaches the kernels through a device word
+// Build (when its key changed) and launch the one-step graph: step-init, the
+// generations (add_generations) unless the step is one pass, and the tail pass.  The step index reaches the kernels through a device word
 // written by a kernel launched just before the graph.
 static qed_status run_step_graph(qed_ctx* ctx, const DevParticles& Din, StepParams SPin,
                                  const Scratch& Sin, uint32_t step) {
@@ -4300,48 +4684,18 @@ static qed_status run_step_graph(qed_ctx* ctx, const DevParticles& Din, StepPara
         DevCtl* ctl = ctx->d_ctl;
         long long* count = D.count;
         long long capacity = D.capacity;
-        int keep_sticky = 0, more_allowed = 1, max_passes = ctx->cfg.max_passes, use_handle = 1;
-        long long tail_rows = tail_rows_for(ctx, SP);
-        cudaGraphNode_t init, wnode, bc, bs, bh, ba, tend;
+        int keep_sticky = 0;
+        const int whole = whole_step(SP.sampler, ctx->tail_rows, ctx->cfg.max_passes) ? 1 : 0;
+        cudaGraphNode_t init, wnode, tend;
         qed_status st;
         {
             void* a[] = {&ctl, &count, &capacity, &keep_sticky};
             st = add_kernel(ctx, g, &init, (const void*)k_step_init, dim3(1), dim3(1), a, nullptr, 0);
         }
-        cudaGraphConditionalHandle h;
-        if (st == QED_OK)
-            st = cuda_check(ctx, cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault),
-                            "cudaGraphConditionalHandleCreate");
-        cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
-        if (st == QED_OK) {
-            memset(&cp.conditional, 0, sizeof cp.conditional);
-            cp.conditional.handle = h;
-            cp.conditional.type = cudaGraphCondTypeWhile;
-            cp.conditional.size = 1;
-            st = cuda_check(ctx, cudaGraphAddNode(&wnode, g, &init, nullptr, 1, &cp),
-                            "cudaGraphAddNode");
-        }
-        if (st == QED_OK) {
-            cudaGraph_t body = cp.conditional.phGraph_out[0];
-            void* a[] = {&D, &SP, &S, &ctl};
-            st = add_kernel(ctx, body, &bc, cold_kernel(SP.N_cell != nullptr), dim3(ctx->cold_blocks),
-                            dim3(kColdThreads), a, nullptr, 0);
-            bs = bc;
-            if (st == QED_OK && SP.sampler == 2)
-                st = add_kernel(ctx, body, &bs, (const void*)k_samp, dim3(ctx->samp_blocks),
-                                dim3(kLaneThreads), a, &bc, 1, kSampSmemBytes);
-            const int hm = loop_hot_mode(SP);
-            if (st == QED_OK)
-                st = add_kernel(ctx, body, &bh, hot_kernel(hm, SP.N_cell != nullptr),
-                                dim3(hm ? ctx->net_blocks : ctx->hot_blocks), dim3(kLaneThreads),
-                                a, &bs, 1, hot_smem(hm));
-            if (st == QED_OK) {
-                void* b[] = {&ctl,        &count, &capacity, &more_allowed, &max_passes,
-                             &tail_rows, &h,     &use_handle};
-                st = add_kernel(ctx, body, &ba, (const void*)k_advance, dim3(1), dim3(1), b, &bh, 1);
-            }
-        }
-        if (st == QED_OK) st = add_tail_nodes(ctx, g, wnode, D, SP, S, ctl, &tend);
+        wnode = init;
+        if (st == QED_OK && !whole)
+            st = add_generations(ctx, g, init, D, SP, S, ctl, 1, &wnode);
+        if (st == QED_OK) st = add_tail_nodes(ctx, g, wnode, D, SP, S, ctl, whole, &tend);
         if (st == QED_OK)
             st = cuda_check(ctx, cudaGraphInstantiate(&ctx->step_exec, g, 0), "cudaGraphInstantiate");
         if (st != QED_OK) {
@@ -4998,7 +5352,7 @@ extern "C" qed_status qed_time_split(const float* t_hi, const float* t_lo, const
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr size_t kNoAllocCtlBytes = 256;
+constexpr size_t kNoAllocCtlBytes = 512;
 constexpr size_t kNoAllocTremOffset = kNoAllocCtlBytes;
 constexpr size_t kNoAllocHotOffset =
     kNoAllocTremOffset + sizeof(ftime) * (size_t)QED_NOALLOC_MAX_ROWS;
@@ -5033,8 +5387,8 @@ qed_status noalloc_setup(int dev, NoAllocDevice* out) {
                 cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_hot, k_hot<false>, kLaneThreads,
                                                           hot_smem(0)) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_step, k_step<0>, kLaneThreads, 0) !=
-                cudaSuccess)
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_step, k_stream<false>, kLaneThreads,
+                                                          step_smem(0)) != cudaSuccess)
             return QED_ERR_CUDA;
         // long-plan queue entries start "not written"; each step resets the ones it used
         if (cudaMemset(static_cast<unsigned char*>(ptr) + kNoAllocHotOffset, 0xFF,
@@ -5079,7 +5433,7 @@ extern "C" qed_status qed_event_step_noalloc(const qed_config* cfg, const qed_pa
     qed_status st = noalloc_setup(dev, &nd);
     if (st != QED_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    const int max_passes = cfg->max_passes > 0 ? cfg->max_passes : 64;
+    const int max_passes = cfg->max_passes > 0 ? cfg->max_passes : kMaxPassesDefault;
     const StepParams SP = make_params(*cfg, step_index);
     const DevParticles D = to_dev(p);
     DevCtl* ctl = reinterpret_cast<DevCtl*>(nd.base);
@@ -5097,7 +5451,8 @@ extern "C" qed_status qed_event_step_noalloc(const qed_config* cfg, const qed_pa
     // from an earlier call is read
     k_step_init<<<1, 1, 0, s>>>(ctl, D.count, D.capacity, 0);
     DevCtl h;
-    for (int pass = 0; pass < max_passes; ++pass) {
+    const int whole = cascade && whole_step(0, kTailRowsDefault, max_passes) ? 1 : 0;
+    for (int pass = 0; !whole && pass < max_passes; ++pass) {
         k_cold<false><<<nd.cold_blocks, kColdThreads, 0, s>>>(D, SP, S, ctl);
         k_hot<false><<<nd.hot_blocks, kLaneThreads, hot_smem(0), s>>>(D, SP, S, ctl);
         k_advance<<<1, 1, 0, s>>>(ctl, D.count, D.capacity, cascade ? 1 : 0, max_passes,
@@ -5110,9 +5465,9 @@ extern "C" qed_status qed_event_step_noalloc(const qed_config* cfg, const qed_pa
         if (!h.more) break;
     }
     // the tail pass (its kernels do nothing when the generations ran to the end)
-    k_tail_begin<<<nd.sms * 8, 256, 0, s>>>(D, S, ctl);
+    k_tail_begin<<<whole ? 1 : nd.sms * 8, 256, 0, s>>>(D, S, ctl, whole);
     k_cold<false><<<nd.cold_blocks, kColdThreads, 0, s>>>(D, SP, S, ctl);
-    k_step<0><<<nd.step_blocks, kLaneThreads, 0, s>>>(D, SP, S, ctl);
+    k_stream<false><<<nd.step_blocks, kLaneThreads, step_smem(0), s>>>(D, SP, S, ctl);
     k_tail_end<<<nd.sms * 8, 256, 0, s>>>(D, S, ctl);
     if (cudaGetLastError() != cudaSuccess) return noalloc_fail(dev, QED_ERR_CUDA);
     if (!out) return QED_OK;
