@@ -725,6 +725,61 @@ __device__ __forceinline__ float draw_x(const DrawKey& d, uint32_t y1, uint32_t 
     return u01((s & 1u) ? r.z : r.x);
 }
 
+// The hot pass and the event-driven sampler write their children 32 at a time: a round has a few events, and
+// the child ids, the reservation and the stores cost a warp the same for one
+// as for 32.  Nobody waits for them before the next generation.
+constexpr int kEventBuf = 64;
+struct __align__(16) EventBuf {   // one per warp, used as a ring
+    uint64_t id[kEventBuf];
+    ftime t_after[kEventBuf];
+    uint32_t i[kEventBuf], s[kEventBuf];
+    float x[kEventBuf];   // negative: the parent is a photon
+    float px[kEventBuf], py[kEventBuf], pz[kEventBuf], chi[kEventBuf];
+    float f[6][kEventBuf];   // E, B
+};
+__device__ __forceinline__ void note_event(EventBuf& E, unsigned int q, uint32_t i, uint64_t id,
+                                           bool photon, float x, float chi, uint32_t s,
+                                           ftime t_after, const PState& st, const Fields& F) {
+    E.id[q] = id;
+    E.t_after[q] = t_after;
+    E.i[q] = i;
+    E.s[q] = s;
+    E.x[q] = photon ? -x : x;
+    E.px[q] = st.px;
+    E.py[q] = st.py;
+    E.pz[q] = st.pz;
+    E.chi[q] = chi;
+    E.f[0][q] = F.Ex;
+    E.f[1][q] = F.Ey;
+    E.f[2][q] = F.Ez;
+    E.f[3][q] = F.Bx;
+    E.f[4][q] = F.By;
+    E.f[5][q] = F.Bz;
+}
+
+
+// The children of the ring's first min(n, 32) events.
+__device__ __forceinline__ void events_flush(const DevParticles& P, const Scratch& S,
+                                             const StepParams& SP, DevCtl* ctl, const EventBuf& E,
+                                             unsigned int& n, unsigned int& head, uint32_t step) {
+    const unsigned int lane = threadIdx.x & 31;
+    const unsigned int k = min(n, 32u);
+    __syncwarp();
+    if (lane < k) {
+        const unsigned int q = (head + lane) % kEventBuf;
+        const bool photon = E.x[q] < 0.0f;
+        const uint32_t i = E.i[q];
+        const long long j = reserve_rows(P, ctl, photon ? 2 : 1, true);
+        write_children(P, S, SP, i, j, E.id[q], photon, fabsf(E.x[q]), E.chi[q], step, E.s[q],
+                       E.t_after[q], PState{E.px[q], E.py[q], E.pz[q]},
+                       Fields{E.f[0][q], E.f[1][q], E.f[2][q], E.f[3][q], E.f[4][q], E.f[5][q]},
+                       kPlain);
+    }
+    __syncwarp();
+    n -= k;
+    head += k;
+}
+
 // Thread pass: one lane per row for planning and events, the warp's lanes
 // together for the draws (draw_round).  First generation of a step:
 // rows [0, pass_end) with the full step; later generations: rows
@@ -736,12 +791,15 @@ __device__ __forceinline__ float draw_x(const DrawKey& d, uint32_t y1, uint32_t 
 // takes its earliest accepted sub-step, the decision of testing its
 // sub-steps in order and stopping at the first acceptance.  Lanes with an
 // event apply it, re-plan the remaining time and join the next round.
-template <bool kCells = false>
+template <bool kCells, bool kLoop>
 __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevParticles P, StepParams SP, Scratch S,
                                                        DevCtl* ctl) {
     const uint32_t step = step_index(SP);
     __shared__ SharedTables sm;
     __shared__ DrawBuf draw_buf[kColdThreads / 32];
+    extern __shared__ __align__(16) unsigned char dyn_smem[];   // !kLoop: a ring per warp
+    EventBuf& E = reinterpret_cast<EventBuf*>(dyn_smem)[threadIdx.x >> 5];
+    unsigned int n_ev = 0, ev_head = 0;   // events whose children are not written yet
     stage_tables(sm);
     __syncthreads();
     if (ctl->status == (int)QED_ERR_TIMEOUT || ctl->skip) return;
@@ -784,7 +842,7 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
         pl.b = pl.c_h = 0.0f;
         float chi = 0.0f, eps = 0.0f;
         uint32_t s = 0;
-        bool need_plan = active;
+        bool need_plan = active, event = false;
         while (__any_sync(kAll, active)) {
             if (need_plan) {
                 need_plan = false;
@@ -850,16 +908,28 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
                     const float x = draw_x(B.key[lane], y1, s_ev, SP.draw_keys);
                     const ftime t_after = (k + 1u == pl.N) ? ftime{0.0f, 0.0f}
                                                            : time_sub_mul(t_rem, k + 1u, pl.h);
-                    removed = apply_event(P, S, SP, ctl, i, id, photon, x, eps, chi, step, s_ev,
-                                          t_after, st, stats, false,
-                                          Fields{Ex, Ey, Ez, Bx, By, Bz}, false);
                     changed = true;
                     s = s_ev + 1u;
                     t_rem = t_after;
-                    if (removed || !time_positive(t_rem)) active = false;
-                    else need_plan = true;
+                    if (kLoop) {
+                        removed = apply_event(P, S, SP, ctl, i, id, photon, x, eps, chi, step, s_ev,
+                                              t_after, st, stats, false,
+                                              Fields{Ex, Ey, Ez, Bx, By, Bz}, false);
+                        if (removed || !time_positive(t_rem)) active = false;
+                        else need_plan = true;
+                    } else {
+                        const unsigned int m = __activemask();
+                        note_event(E, (ev_head + n_ev + __popc(m & ((1u << lane) - 1u))) % kEventBuf,
+                                   (uint32_t)i, id, photon, x, chi, s_ev, t_after, st,
+                                   Fields{Ex, Ey, Ez, Bx, By, Bz});
+                        count_event(stats, photon);
+                        removed = event_recoil(SP, photon, x, eps, st);
+                        event = true;
+                        active = false;
+                    }
                 }
             }
+            if (!kLoop) break;
             __syncwarp();   // the draw buffer is reused by the next round
         }
         if (removed) {
@@ -869,7 +939,14 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
             P.py[i] = st.py;
             P.pz[i] = st.pz;
         }
+        if (!kLoop) {
+            // the parents go on in the hot pass
+            if (event && !removed && time_positive(t_rem)) push_hot(S, ctl, i, s, t_rem, false);
+            n_ev += (unsigned int)__popc(__ballot_sync(kAll, event));
+            if (n_ev >= 32u) events_flush(P, S, SP, ctl, E, n_ev, ev_head, step);
+        }
     }
+    if (!kLoop && n_ev) events_flush(P, S, SP, ctl, E, n_ev, ev_head, step);
     // the last block to end notes the rows in use: the children so far (k_stream)
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1504,61 +1581,6 @@ using LaneFields = float[6][kLaneThreads];
 __device__ __forceinline__ Fields lane_fields(const LaneFields& f) {
     const int t = threadIdx.x;
     return Fields{f[0][t], f[1][t], f[2][t], f[3][t], f[4][t], f[5][t]};
-}
-
-// The hot pass and the event-driven sampler write their children 32 at a time: a round has a few events, and
-// the child ids, the reservation and the stores cost a warp the same for one
-// as for 32.  Nobody waits for them before the next generation.
-constexpr int kEventBuf = 64;
-struct __align__(16) EventBuf {   // one per warp, used as a ring
-    uint64_t id[kEventBuf];
-    ftime t_after[kEventBuf];
-    uint32_t i[kEventBuf], s[kEventBuf];
-    float x[kEventBuf];   // negative: the parent is a photon
-    float px[kEventBuf], py[kEventBuf], pz[kEventBuf], chi[kEventBuf];
-    float f[6][kEventBuf];   // E, B
-};
-__device__ __forceinline__ void note_event(EventBuf& E, unsigned int q, uint32_t i, uint64_t id,
-                                           bool photon, float x, float chi, uint32_t s,
-                                           ftime t_after, const PState& st, const Fields& F) {
-    E.id[q] = id;
-    E.t_after[q] = t_after;
-    E.i[q] = i;
-    E.s[q] = s;
-    E.x[q] = photon ? -x : x;
-    E.px[q] = st.px;
-    E.py[q] = st.py;
-    E.pz[q] = st.pz;
-    E.chi[q] = chi;
-    E.f[0][q] = F.Ex;
-    E.f[1][q] = F.Ey;
-    E.f[2][q] = F.Ez;
-    E.f[3][q] = F.Bx;
-    E.f[4][q] = F.By;
-    E.f[5][q] = F.Bz;
-}
-
-
-// The children of the ring's first min(n, 32) events.
-__device__ __forceinline__ void events_flush(const DevParticles& P, const Scratch& S,
-                                             const StepParams& SP, DevCtl* ctl, const EventBuf& E,
-                                             unsigned int& n, unsigned int& head, uint32_t step) {
-    const unsigned int lane = threadIdx.x & 31;
-    const unsigned int k = min(n, 32u);
-    __syncwarp();
-    if (lane < k) {
-        const unsigned int q = (head + lane) % kEventBuf;
-        const bool photon = E.x[q] < 0.0f;
-        const uint32_t i = E.i[q];
-        const long long j = reserve_rows(P, ctl, photon ? 2 : 1, true);
-        write_children(P, S, SP, i, j, E.id[q], photon, fabsf(E.x[q]), E.chi[q], step, E.s[q],
-                       E.t_after[q], PState{E.px[q], E.py[q], E.pz[q]},
-                       Fields{E.f[0][q], E.f[1][q], E.f[2][q], E.f[3][q], E.f[4][q], E.f[5][q]},
-                       kPlain);
-    }
-    __syncwarp();
-    n -= k;
-    head += k;
 }
 
 #ifndef QED_SAMP_REFILL
@@ -3164,9 +3186,11 @@ __global__ void k_step_init(DevCtl* ctl, long long* count, long long capacity, i
 // cells: the step takes per-cell counts for the first plans (only without a
 // learned sampler); its kernels are separate instantiations, so that the
 // plain step carries none of that code.
-const void* cold_kernel(bool cells) {
-    return cells ? (const void*)k_cold<true> : (const void*)k_cold<false>;
+const void* cold_kernel(int mode, bool cells = false) {
+    return mode ? (const void*)k_cold<false, true>
+                : cells ? (const void*)k_cold<true, false> : (const void*)k_cold<false, false>;
 }
+size_t cold_smem(int mode) { return mode ? 0 : sizeof(EventBuf) * (kColdThreads / 32); }
 const void* hot_kernel(int mode, bool cells = false) {
     // sampler mode 2 runs its network in k_samp: the hot pass of its
     // generations is rejection's (loop_hot_mode)
@@ -3176,11 +3200,13 @@ const void* hot_kernel(int mode, bool cells = false) {
 size_t hot_smem(int mode) { return mode == 1 ? kNetSmemBytes : sizeof(HotSmem); }
 // Their dynamic shared memory is above the default limit.
 cudaError_t allow_smem() {
-    const void* hot[] = {hot_kernel(1), hot_kernel(0), hot_kernel(0, true),
-                         (const void*)k_stream<false>, (const void*)k_stream<true>};
-    for (int k = 0; k < 5; ++k) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            hot[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hot_smem(k == 0 ? 1 : 0));
+    const struct { const void* f; size_t bytes; } k[] = {
+        {hot_kernel(1), hot_smem(1)}, {hot_kernel(0), hot_smem(0)}, {hot_kernel(0, true), hot_smem(0)},
+        {(const void*)k_stream<false>, hot_smem(0)}, {(const void*)k_stream<true>, hot_smem(0)},
+        {cold_kernel(0), cold_smem(0)}, {cold_kernel(0, true), cold_smem(0)}};
+    for (const auto& q : k) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(q.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q.bytes);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -3857,10 +3883,11 @@ qed_status qed_init(qed_ctx** out, const qed_config* cfg, void* stream) {
     if (st == QED_OK) st = cuda_check(ctx, cudaMemset(ctx->d_ctl, 0, sizeof(DevCtl)), "memset");
     if (st == QED_OK) {
         int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cold<false>, kColdThreads, 0);
+        allow_smem();
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cold<false, false>,
+                                                      kColdThreads, cold_smem(0));
         ctx->cold_blocks = ctx->cold_blocks_max = ctx->sms * (per_sm > 0 ? per_sm : 1);
         per_sm = 0;
-        allow_smem();
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hot<false>, kLaneThreads,
                                                       hot_smem(0));
         ctx->hot_blocks = ctx->hot_blocks_max = ctx->sms * (per_sm > 0 ? per_sm : 1);
@@ -4055,6 +4082,13 @@ static qed_status cell_counts(qed_ctx* ctx, const DevParticles& D, StepParams* S
     return QED_OK;
 }
 
+static cudaError_t launch_cold(qed_ctx* ctx, DevParticles D, StepParams SP, Scratch S) {
+    DevCtl* ctl = ctx->d_ctl;
+    void* a[] = {&D, &SP, &S, &ctl};
+    return cudaLaunchKernel(cold_kernel(SP.sampler, SP.N_cell != nullptr), dim3(ctx->cold_blocks),
+                            dim3(kColdThreads), a, cold_smem(SP.sampler), ctx->stream);
+}
+
 // The event step, with per-cell first-plan counts when cell != NULL.
 static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step_index,
                              qed_step_stats* out, const uint32_t* cell, int64_t ncells) {
@@ -4094,8 +4128,7 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
     for (int pass = 0; !whole && pass < ctx->cfg.max_passes; ++pass) {
         {
             LaunchScope ls(ctx, QED_KERNEL_COLD);
-            if (SP.N_cell) k_cold<true><<<ctx->cold_blocks, kColdThreads, 0, ctx->stream>>>(D, SP, S, ctx->d_ctl);
-            else k_cold<false><<<ctx->cold_blocks, kColdThreads, 0, ctx->stream>>>(D, SP, S, ctx->d_ctl);
+            QED_CUDA(ctx, launch_cold(ctx, D, SP, S));
         }
         if (SP.sampler == 2) {
             LaunchScope ls(ctx, QED_KERNEL_SAMPLER);
@@ -4136,8 +4169,7 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
     }
     {
         LaunchScope ls(ctx, QED_KERNEL_COLD);
-        if (SP.N_cell) k_cold<true><<<ctx->cold_blocks, kColdThreads, 0, ctx->stream>>>(D, SP, S, ctx->d_ctl);
-        else k_cold<false><<<ctx->cold_blocks, kColdThreads, 0, ctx->stream>>>(D, SP, S, ctx->d_ctl);
+        QED_CUDA(ctx, launch_cold(ctx, D, SP, S));
     }
     {
         LaunchScope ls(ctx, QED_KERNEL_HOT);
@@ -4438,8 +4470,8 @@ qed_status add_generations(qed_ctx* ctx, cudaGraph_t g, cudaGraphNode_t dep, con
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     cudaGraphNode_t bc, bs, bh, ba;
     void* a[] = {&D, &SP, &S, &ctl};
-    st = add_kernel(ctx, body, &bc, cold_kernel(SP.N_cell != nullptr), dim3(ctx->cold_blocks),
-                    dim3(kColdThreads), a, nullptr, 0);
+    st = add_kernel(ctx, body, &bc, cold_kernel(SP.sampler, SP.N_cell != nullptr), dim3(ctx->cold_blocks),
+                    dim3(kColdThreads), a, nullptr, 0, cold_smem(SP.sampler));
     bs = bc;
     if (st == QED_OK && SP.sampler == 2)
         st = add_kernel(ctx, body, &bs, (const void*)k_samp, dim3(ctx->samp_blocks),
@@ -4475,8 +4507,8 @@ qed_status add_tail_nodes(qed_ctx* ctx, cudaGraph_t g, cudaGraphNode_t dep, cons
     }
     if (st == QED_OK) {
         void* a[] = {&D, &SP, &S, &ctl};
-        st = add_kernel(ctx, g, &tc, cold_kernel(SP.N_cell != nullptr), dim3(ctx->cold_blocks),
-                        dim3(kColdThreads), a, &tb, 1);
+        st = add_kernel(ctx, g, &tc, cold_kernel(SP.sampler, SP.N_cell != nullptr), dim3(ctx->cold_blocks),
+                        dim3(kColdThreads), a, &tb, 1, cold_smem(SP.sampler));
     }
     if (st == QED_OK) {
         void* a[] = {&D, &SP, &S, &ctl};
@@ -5383,7 +5415,8 @@ qed_status noalloc_setup(int dev, NoAllocDevice* out) {
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return QED_ERR_CUDA;
         if (allow_smem() != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_cold, k_cold<false>, kColdThreads, 0) !=
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_cold, k_cold<false, false>, kColdThreads,
+                                                          cold_smem(0)) !=
                 cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_hot, k_hot<false>, kLaneThreads,
                                                           hot_smem(0)) != cudaSuccess ||
@@ -5453,7 +5486,7 @@ extern "C" qed_status qed_event_step_noalloc(const qed_config* cfg, const qed_pa
     DevCtl h;
     const int whole = cascade && whole_step(0, kTailRowsDefault, max_passes) ? 1 : 0;
     for (int pass = 0; !whole && pass < max_passes; ++pass) {
-        k_cold<false><<<nd.cold_blocks, kColdThreads, 0, s>>>(D, SP, S, ctl);
+        k_cold<false, false><<<nd.cold_blocks, kColdThreads, cold_smem(0), s>>>(D, SP, S, ctl);
         k_hot<false><<<nd.hot_blocks, kLaneThreads, hot_smem(0), s>>>(D, SP, S, ctl);
         k_advance<<<1, 1, 0, s>>>(ctl, D.count, D.capacity, cascade ? 1 : 0, max_passes,
                                   kTailRowsDefault, 0ull, 0);
@@ -5466,7 +5499,7 @@ extern "C" qed_status qed_event_step_noalloc(const qed_config* cfg, const qed_pa
     }
     // the tail pass (its kernels do nothing when the generations ran to the end)
     k_tail_begin<<<whole ? 1 : nd.sms * 8, 256, 0, s>>>(D, S, ctl, whole);
-    k_cold<false><<<nd.cold_blocks, kColdThreads, 0, s>>>(D, SP, S, ctl);
+    k_cold<false, false><<<nd.cold_blocks, kColdThreads, cold_smem(0), s>>>(D, SP, S, ctl);
     k_stream<false><<<nd.step_blocks, kLaneThreads, step_smem(0), s>>>(D, SP, S, ctl);
     k_tail_end<<<nd.sms * 8, 256, 0, s>>>(D, S, ctl);
     if (cudaGetLastError() != cudaSuccess) return noalloc_fail(dev, QED_ERR_CUDA);
