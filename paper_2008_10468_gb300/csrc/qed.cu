@@ -466,12 +466,13 @@ __device__ __forceinline__ ulonglong2 write_children(const DevParticles& P, cons
     const float delta = photon ? x : x * x * x;
     if (j >= 0) {
         const float w = P.w[i];
-        write_child_fields(P, S, j, F, w, delta * st.px, delta * st.py, delta * st.pz, id0,
-                           t_after);
-        if (photon) {
-            const float omd = 1.0f - x;
-            write_child_fields(P, S, j + 1, F, w, omd * st.px, omd * st.py, omd * st.pz, id1,
-                               t_after);
+        float d = delta;
+        uint64_t cid_r = id0;
+#pragma unroll 1
+        for (int r = 0; r <= (photon ? 1 : 0); ++r) {
+            write_child_fields(P, S, j + r, F, w, d * st.px, d * st.py, d * st.pz, cid_r, t_after);
+            d = 1.0f - x;
+            cid_r = id1;
         }
         if (mode == kPublish) __threadfence();
         if (mode != kDeferred) {
@@ -1822,11 +1823,14 @@ __global__ void __launch_bounds__(kLaneThreads, QED_SAMP_BLOCKS) k_samp(DevParti
 #ifndef QED_WINDOWS
 #define QED_WINDOWS 8
 #endif
-#ifndef QED_DRAW_ILP
-#define QED_DRAW_ILP 4
+#ifndef QED_STREAM_ILP
+#define QED_STREAM_ILP 2
 #endif
 constexpr int kWindows = QED_WINDOWS;   // windows a lane draws at a time
-constexpr int kDrawIlp = QED_DRAW_ILP;  // windows in flight
+// Windows in flight.  In k_stream two: its loop is the longest and waits for
+// instructions; a second copy of two rounds costs more than it hides (cascade
+// of 4096 cells: 13.1 ms with four, 12.6 with two, 12.8 with one).
+constexpr int kHotIlp = 4, kStreamIlp = QED_STREAM_ILP;
 constexpr uint32_t kOwnMax = 8;      // plans of this many sub-steps are drawn by their lane
 struct ListBuf {                     // one per warp
     DrawKey key[32];
@@ -2004,6 +2008,7 @@ __device__ __forceinline__ bool lane_count_plan(Lane& L, Stats& stats) {
 // other, kDrawIlp at a time (a window's ten multiply rounds are one chain), by
 // all 32 lanes.  A lane whose plan ends within kOwnMax sub-steps draws its few
 // blocks by itself, at the same time as the other such lanes.
+template <int kDrawIlp>
 __device__ __forceinline__ void list_draw(ListBuf& B, Lane& L, uint32_t y1, const PhiloxKeys& K) {
     constexpr unsigned int kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -2276,7 +2281,7 @@ __global__ void __launch_bounds__(kLaneThreads, QED_HOT_MIN_BLOCKS) k_hot(DevPar
             if (!more_long && !more_med) break;
             continue;
         }
-        list_draw(B, L, y1, SP.draw_keys);
+        list_draw<kHotIlp>(B, L, y1, SP.draw_keys);
         if (list_test(sm, B, L, y1, SP.draw_keys, stats.cand)) {
             stats.substeps += L.pl.N;
             lane_finish(P, L);
@@ -2733,7 +2738,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
                 rounds = 0;
                 if (lane == 0) atomicAdd(&ctl->beat, 1ull);
             }
-            list_draw(B, L, y1, SP.draw_keys);
+            list_draw<kHotIlp>(B, L, y1, SP.draw_keys);
             if (list_test(sm, B, L, y1, SP.draw_keys, stats.cand)) {
                 stats.substeps += L.pl.N;
                 lane_finish(P, L);
@@ -3096,7 +3101,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
                 rounds = 0;
                 if (lane == 0) atomicAdd(&ctl->beat, 1ull);
             }
-            list_draw(B, L, y1, SP.draw_keys);
+            list_draw<kStreamIlp>(B, L, y1, SP.draw_keys);
             if (list_test(sm, B, L, y1, SP.draw_keys, stats.cand)) {
                 stats.substeps += L.pl.N;
                 lane_finish(P, L);
