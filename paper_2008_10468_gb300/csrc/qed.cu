@@ -993,7 +993,7 @@ __device__ __forceinline__ uint32_t push_cap(const PlanConst& PC, const SharedTa
     const float hi = p + d, lo = fmaxf(p - d, 0.0f);
     const float b = 1.503f * PC.inv_Es * fmaf(1.0f + hi, E, hi * B);
     if (!(b < 1e30f)) return 1u << 23;   // infinities and NaN as well
-    const float b23 = b > 0.0f ? exp2f(__log2f(b) * (2.0f / 3.0f)) : 0.0f;
+    const float b23 = b > 0.0f ? ex2_normal(__log2f(b) * (2.0f / 3.0f)) : 0.0f;
     const float c_h = 1.002f * PC.K * h * __fdividef(1.0f, sqrtf(fmaf(lo, lo, 1.0f)));
     return squeeze_threshold(squeeze_bound(sm.sqz_e, sm.sqz_p, false, b, c_h, b23));
 }
@@ -1353,7 +1353,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_push(DevParticles P, StepPa
                                     PC.inv_Es, &eps_k);
                     b = 1.5f * chi_k;
                     c_h = PC.K * pl.h.hi * __fdividef(1.0f, eps_k);
-                    const float b23 = b > 0.0f ? exp2f(__log2f(b) * (2.0f / 3.0f)) : 0.0f;
+                    const float b23 = b > 0.0f ? ex2_normal(__log2f(b) * (2.0f / 3.0f)) : 0.0f;
                     T = squeeze_threshold(squeeze_bound(sm.sqz_e, sm.sqz_p, false, b, c_h, b23));
                 }
                 const uint32_t c = s - 1u;

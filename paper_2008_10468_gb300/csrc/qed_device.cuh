@@ -383,7 +383,7 @@ __device__ __forceinline__ float bound_emission_l2(float b, float l2b, float c) 
     const bool p1 = b >= 0.1f, p2 = b >= 0.5f, p3 = b >= 10.0f;
     const float A = p3 ? 0.55f * kPi : (p2 ? 0.42f * kPi : (p1 ? 0.45f * kPi : 0.56f * kPi));
     const float e = p3 ? 2.0f / 3.0f : (p2 ? 19.0f / 24.0f : 11.0f / 12.0f);
-    const float v = p1 ? exp2f(l2b * e) : b;
+    const float v = p1 ? ex2_normal(l2b * e) : b;
     return c * fmaf(0.1f, b, __fmul_rn(A, v));
 }
 
@@ -583,7 +583,7 @@ __device__ __forceinline__ Plan make_plan(const PlanConst& P, const float* __res
                            : (b > 0.0f ? bound_emission_l2(b, l2b, c_rem) : 0.0f);
     const float q = f * P.inv_p_max;
     float b23 = 0.0f;
-    if (b > 0.0f) b23 = exp2f(l2b * (2.0f / 3.0f));
+    if (b > 0.0f) b23 = ex2_normal(l2b * (2.0f / 3.0f));
     const float graw = photon ? 0.0f : kSmallF * c_rem * b23;
     pl.guard = graw > fmaxf(1.0f, ceilf(q));   // ceil(graw) above max(1, ceil(q))
     // N = max(1, ceil(q), ceil(g)) is the ceiling of the larger one, monotone
@@ -724,7 +724,7 @@ __device__ __noinline__ Plan plan_slow(PlanConst P, const float* __restrict__ sq
     pl.safe = true;
     pl.h = time_div(T, pl.N);
     pl.c_h = P.K * pl.h.hi * __fdividef(1.0f, pl.eps);
-    const float b23 = pl.b > 0.0f ? exp2f(__log2f(pl.b) * (2.0f / 3.0f)) : 0.0f;
+    const float b23 = pl.b > 0.0f ? ex2_normal(__log2f(pl.b) * (2.0f / 3.0f)) : 0.0f;
     pl.T = squeeze_threshold(squeeze_bound(sqz_e, sqz_p, photon, pl.b, pl.c_h, b23));
     return pl;
 }
@@ -742,7 +742,7 @@ __device__ __forceinline__ Plan cell_count_plan(Plan pl, const float* __restrict
     pl.N = Nc;
     pl.h = time_div(T, Nc);
     pl.c_h = K * pl.h.hi * __fdividef(1.0f, eps);
-    const float b23 = pl.b > 0.0f ? exp2f(__log2f(pl.b) * (2.0f / 3.0f)) : 0.0f;
+    const float b23 = pl.b > 0.0f ? ex2_normal(__log2f(pl.b) * (2.0f / 3.0f)) : 0.0f;
     pl.T = squeeze_threshold(squeeze_bound(sqz_e, sqz_p, photon, pl.b, pl.c_h, b23));
     return pl;
 }

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(256) k_cdf_rows(float log10_lo, float log10_hi
     if (row >= nrows) return;
     const float l10 = log10_lo + (log10_hi - log10_lo) * (float)row / (float)(nrows - 1);
     const float b = 1.5f * exp10f(l10);
-    const float b23 = exp2f(__log2f(b) * (2.0f / 3.0f));
+    const float b23 = ex2_normal(__log2f(b) * (2.0f / 3.0f));
     const float dx = 1.0f / (float)M;
     if (threadIdx.x == 0) carry = 0.0;
     __syncthreads();
