@@ -51,26 +51,22 @@ namespace {
 // Defaults measured on the 2^24 clumped population (coordinate search over
 // hot_min 32..128 and long_min 128..2048)
 constexpr uint32_t kHotMinDefault = 32;    // plans with N >= hot_min go to the hot pass
-#ifndef QED_SAMP_LONG
-#define QED_SAMP_LONG 4096
-#endif
-constexpr uint32_t kSampLong = QED_SAMP_LONG;   // sampler: plans with N >= this are stepped first
-#ifndef QED_LONG_MIN
-#define QED_LONG_MIN 256
-#endif
-constexpr uint32_t kLongMinDefault = QED_LONG_MIN;  // ... and with N >= long_min to its warp mode
+constexpr uint32_t kLongMinDefault = 256;  // ... and with N >= long_min to its front (front_min)
+// Sampler: in a generation of at least kSampSplit rows, plans with N >= kSampLong
+// are stepped first, so that the last warps do not end on long chains (1e6
+// uniform-field electrons: 2.37 ms with the line at 3000, 2.44 at 4096, 2.95
+// without).  The children of a generation that the lanes hold at once start
+// together anyway, and the mixed order is faster (clumped 2^22: 4.54 against
+// 4.76 ms).
+constexpr uint32_t kSampLong = 3000;
+constexpr long long kSampSplit = 1 << 19;
 constexpr int kMaxPassesDefault = 64;   // cascade generations per step
 constexpr long long kTailRowsDefault = 1ll << 17;   // generations below this go to the tail pass
 
 // Minimum resident blocks per SM requested from the register allocator:
 // 3 x 256 threads hold the thread and hot passes at 80 registers (24 warps
 // per SM).
-#ifndef QED_COLD_MIN_BLOCKS
-#define QED_COLD_MIN_BLOCKS 3
-#endif
-#ifndef QED_LANES_MIN_BLOCKS
-#define QED_LANES_MIN_BLOCKS 3
-#endif
+constexpr int kColdMinBlocks = 3, kHotNetMinBlocks = 3;
 constexpr int kColdThreads = 256;
 constexpr int kLaneThreads = 256;
 constexpr int kSweepThreads = 256;
@@ -793,7 +789,7 @@ __device__ __forceinline__ void events_flush(const DevParticles& P, const Scratc
 // sub-steps in order and stopping at the first acceptance.  Lanes with an
 // event apply it, re-plan the remaining time and join the next round.
 template <bool kCells, bool kLoop>
-__global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevParticles P, StepParams SP, Scratch S,
+__global__ void __launch_bounds__(kColdThreads, kColdMinBlocks) k_cold(DevParticles P, StepParams SP, Scratch S,
                                                        DevCtl* ctl) {
     const uint32_t step = step_index(SP);
     __shared__ SharedTables sm;
@@ -808,6 +804,7 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
     const long long begin = first_pass ? 0 : ctl->pass_begin;
     const long long end = ctl->pass_end;
     const long long n_init = kCells ? ctl->n_init : 0;
+    const uint32_t samp_long = end - begin >= kSampSplit ? kSampLong : 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -873,7 +870,7 @@ __global__ void __launch_bounds__(kColdThreads, QED_COLD_MIN_BLOCKS) k_cold(DevP
                             it.idx = (uint32_t)i;
                             it.s = s;
                             it.t_rem = t_rem;
-                            if (pl.N >= kSampLong)
+                            if (pl.N >= samp_long)
                                 S.samp[atomicAdd(&ctl->samp_tail, 1u)] = it;
                             else
                                 S.samp[S.samp_cap - 1 - (long long)atomicAdd(&ctl->samp_back, 1u)] = it;
@@ -1584,17 +1581,9 @@ __device__ __forceinline__ Fields lane_fields(const LaneFields& f) {
     return Fields{f[0][t], f[1][t], f[2][t], f[3][t], f[4][t], f[5][t]};
 }
 
-#ifndef QED_SAMP_REFILL
-#define QED_SAMP_REFILL 4
-#endif
-constexpr int kSampRefill = QED_SAMP_REFILL;   // idle lanes before a warp takes queue entries
-#ifndef QED_SAMP_LANES
-#define QED_SAMP_LANES 8
-#endif
-constexpr int kSampLanes = QED_SAMP_LANES;
-#ifndef QED_SAMP_BLOCKS
-#define QED_SAMP_BLOCKS 2
-#endif
+constexpr int kSampRefill = 1;   // idle lanes before a warp takes queue entries (1e6 uniform-field
+                                 // electrons: 2.44 ms; 2.48 with 4, 2.52 with 8)
+constexpr int kSampLanes = 8;    // half a tile of the network
 // Dynamic shared memory of k_samp: the networks, then a ring per warp.
 constexpr size_t kSampSmemBytes = kMmaSmemBytes + sizeof(EventBuf) * (kLaneThreads / 32);
 static_assert(kMmaSmemBytes % 16 == 0, "ring alignment");
@@ -1614,7 +1603,7 @@ static_assert(kMmaSmemBytes % 16 == 0, "ring alignment");
 // sampler's usable bins continues with rejection: its state goes back to the
 // store and it joins the hot pass's queue (the hot pass runs after this
 // kernel).  Idle lanes take queue entries, one atomic per warp.  Persistent.
-__global__ void __launch_bounds__(kLaneThreads, QED_SAMP_BLOCKS) k_samp(DevParticles P, StepParams SP, Scratch S,
+__global__ void __launch_bounds__(kLaneThreads, 2) k_samp(DevParticles P, StepParams SP, Scratch S,
                                                        DevCtl* ctl) {
     const uint32_t step = step_index(SP);
     __shared__ SharedTables sm;
@@ -1820,17 +1809,12 @@ __global__ void __launch_bounds__(kLaneThreads, QED_SAMP_BLOCKS) k_samp(DevParti
 // bulk, a window to 32 lanes (the two ballots are the masks) and none of them
 // twice, and what is left on the chain from one event to the next is one
 // evaluation of the next candidates, the recoil and the plan.
-#ifndef QED_WINDOWS
-#define QED_WINDOWS 8
-#endif
-#ifndef QED_STREAM_ILP
-#define QED_STREAM_ILP 2
-#endif
-constexpr int kWindows = QED_WINDOWS;   // windows a lane draws at a time
+constexpr int kWindows = 8;   // windows a lane draws at a time (1e5 uniform-field electrons, 1e3
+                              // sub-steps each: 0.90 ms; 0.95 with 4)
 // Windows in flight.  In k_stream two: its loop is the longest and waits for
 // instructions; a second copy of two rounds costs more than it hides (cascade
 // of 4096 cells: 13.1 ms with four, 12.6 with two, 12.8 with one).
-constexpr int kHotIlp = 4, kStreamIlp = QED_STREAM_ILP;
+constexpr int kHotIlp = 4, kStreamIlp = 2;
 constexpr uint32_t kOwnMax = 8;      // plans of this many sub-steps are drawn by their lane
 struct ListBuf {                     // one per warp
     DrawKey key[32];
@@ -2165,21 +2149,7 @@ __device__ __forceinline__ bool list_test(const SharedTables& sm, ListBuf& B, La
     return L.active && t - L.s0 == L.pl.N;
 }
 
-#ifndef QED_HOT_LANES
-#define QED_HOT_LANES 16
-#endif
-#ifndef QED_HOT_MANY
-#define QED_HOT_MANY 256
-#endif
-#ifndef QED_HOT_REFILL
-#define QED_HOT_REFILL 8
-#endif
-#ifndef QED_HOT_MIN_BLOCKS
-#define QED_HOT_MIN_BLOCKS 2
-#endif
-constexpr unsigned int kHotLanes = QED_HOT_LANES;   // most particles a warp of the hot pass holds,
-constexpr int kHotMany = QED_HOT_MANY;       // 32 with a queue of this many times the warps
-constexpr int kHotRefill = QED_HOT_REFILL;   // idle lanes before it takes queue entries
+constexpr int kHotRefill = 8;      // idle lanes before a warp takes queue entries
 constexpr uint32_t kWindow = 64;             // mode 1's medium plans: sub-steps per lane and round
 
 // Hot pass (rejection).  One particle per lane.  A round applies the events
@@ -2199,7 +2169,7 @@ struct HotSmem {
 };
 
 template <bool kCells>
-__global__ void __launch_bounds__(kLaneThreads, QED_HOT_MIN_BLOCKS) k_hot(DevParticles P, StepParams SP,
+__global__ void __launch_bounds__(kLaneThreads, 2) k_hot(DevParticles P, StepParams SP,
                                                                  Scratch S, DevCtl* ctl) {
     const uint32_t step = step_index(SP);
     extern __shared__ __align__(16) unsigned char dyn_smem[];
@@ -2217,9 +2187,8 @@ __global__ void __launch_bounds__(kLaneThreads, QED_HOT_MIN_BLOCKS) k_hot(DevPar
     unsigned int n_ev = 0, ev_head = 0;   // events whose children are not written yet
     const uint32_t y1 = draw_y1(step, SP.draw_keys);
     const unsigned int nwarps = gridDim.x * (kLaneThreads / 32);
-    const unsigned int most = (n_long + n_med) / nwarps >= (unsigned int)kHotMany ? 32u : kHotLanes;
-    const int cap_long = (int)min(most, (n_long + nwarps - 1u) / nwarps);
-    const int cap = (int)min(most, (n_long + n_med + nwarps - 1u) / nwarps);
+    const int cap_long = (int)min(32u, (n_long + nwarps - 1u) / nwarps);
+    const int cap = (int)min(32u, (n_long + n_med + nwarps - 1u) / nwarps);
     bool more_long = n_long != 0u, more_med = n_med != 0u, first = true;   // warp-uniform
     Stats stats;
     Lane L;
@@ -2299,7 +2268,7 @@ __global__ void __launch_bounds__(kLaneThreads, QED_HOT_MIN_BLOCKS) k_hot(DevPar
 // plans (back of the queue), one lane each, with warp-shared draws over at
 // most kWindow sub-steps per lane and round.  Sampler mode 2 steps its
 // particles in k_samp and runs k_hot for the others.
-__global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_net(DevParticles P, StepParams SP,
+__global__ void __launch_bounds__(kLaneThreads, kHotNetMinBlocks) k_hot_net(DevParticles P, StepParams SP,
                                                                  Scratch S, DevCtl* ctl) {
     const uint32_t step = step_index(SP);
     __shared__ SharedTables sm;
@@ -2481,30 +2450,13 @@ __global__ void __launch_bounds__(kLaneThreads, QED_LANES_MIN_BLOCKS) k_hot_net(
 // returns.
 // ---------------------------------------------------------------------------
 constexpr unsigned long long kWaitNsDefault = 1000000000ull;   // idle time before giving up: 1 s
-#ifndef QED_TAIL_CLAIM
-#define QED_TAIL_CLAIM 8
-#endif
-#ifndef QED_TAIL_SPREAD
-#define QED_TAIL_SPREAD 256
-#endif
-#ifndef QED_TAIL_ROUNDS
-#define QED_TAIL_ROUNDS 8
-#endif
-#ifndef QED_TAIL_NAP
-#define QED_TAIL_NAP 4
-#endif
-#ifndef QED_TAIL_WARPS
-#define QED_TAIL_WARPS 8
-#endif
-#ifndef QED_TAIL_MINB
-#define QED_TAIL_MINB 8
-#endif
-constexpr unsigned int kTailMinBlocks = QED_TAIL_MINB;   // blocks that stay: these and
-constexpr unsigned int kTailWarps = QED_TAIL_WARPS;   // this many warps per queue entry (the
-                                         // polls of idle warps slow the others)
-constexpr int kTailClaim = QED_TAIL_CLAIM;   // idle lanes before a busy warp takes rows,
-constexpr unsigned int kTailRounds = QED_TAIL_ROUNDS;   // and rounds between two looks
-constexpr unsigned int kTailSpread = QED_TAIL_SPREAD;   // warps that share the rows on offer
+// Blocks that stay in a persistent pass: these and kTailWarps warps per queue
+// entry (the polls of idle warps slow the others).
+constexpr unsigned int kTailMinBlocks = 8, kTailWarps = 8;
+constexpr int kTailClaim = 8;              // idle lanes before a busy warp takes rows,
+constexpr unsigned int kTailRounds = 8;    // and rounds between two looks
+constexpr unsigned int kTailSpread = 256;  // warps that share the rows on offer
+constexpr unsigned int kTailNap = 4;       // idle warps poll every 256 ns << 0 ... 4
 
 // Queue a long plan: the entry's row index is written last (readers wait for it).
 __device__ __forceinline__ void push_long(const Scratch& S, DevCtl* ctl, unsigned int cold_long,
@@ -2789,7 +2741,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
                 seen = progress;
                 idle_ns = 0;
             }
-            const unsigned int nap = hold ? 64u : 256u << min(idle, (unsigned int)QED_TAIL_NAP);
+            const unsigned int nap = hold ? 64u : 256u << min(idle, kTailNap);
             ++idle;
             idle_ns += nap;
             if (idle_ns > SP.wait_ns) {
@@ -2831,7 +2783,6 @@ constexpr unsigned int kStreamSpread = 16;   // warps that share the children on
                                              // instead of 0.98 ms at 2^20 rows)
 constexpr int kStreamLanes = 16;             // most particles of a warp, 32 when the queue holds
 constexpr unsigned int kStreamMany = 8;      // this many times the warps (always 16: 4.2 ms at 2^24)
-constexpr unsigned int kStreamNap = 4;       // idle warps poll every 256 ns << 0 ... 4
 
 // A warp's children.  Rows and entries are reserved at the start of a round,
 // written after its plans and published after its draws, so that the chains
@@ -3136,7 +3087,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
         }
         // idle: back off from 256 ns to 4 us (64 ns while an entry is being
         // written); the idle time counts from the last progress seen
-        const unsigned int nap = hold ? 64u : 256u << min(idle, kStreamNap);
+        const unsigned int nap = hold ? 64u : 256u << min(idle, kTailNap);
         ++idle;
         idle_ns += nap;
         if (idle_ns > SP.wait_ns && !hold) {
