@@ -40,12 +40,11 @@ CASCADE_CELLS = 4096
 CASCADE_CAPACITY = 1 << 26
 CASCADE_DRAIN_CHI = 0.05
 # DRAM traffic of the hot pass is not reported per run: a capture of its
-# counters over whole steps of the full-size workload is larger than the
-# profiling rules allow, and at the 2^22 rows that may be captured the
-# children's writes stay in the 129 MB L2 (profiles/hot_pass_traffic_clumped_2p22.md).
-HOT_TRAFFIC_NOTE = ("null: a capture of the pass's launches at 2^22 rows reads 90 MB per step "
-                    "from DRAM while its writes (the children) stay in L2 at that size; a "
-                    "full-size capture of these counters is outside the profiling size rule")
+# counters on the full-size workload is larger than the profiling rules allow
+# (profiles/kernel_captures.md has it at 2^22 rows).
+HOT_TRAFFIC_NOTE = ("null: a capture of the pass at 2^22 rows reads 87 MB from DRAM and writes "
+                    "57 MB, part of its children staying in L2 at that size; a full-size "
+                    "capture of these counters is outside the profiling size rule")
 
 METRIC = "particle-steps/sec (sub-stepped)"
 UNIT = "substeps/s"
@@ -357,7 +356,7 @@ def run_gb300(args):
         t_launch = kern["hot"][0] / kern["hot"][1] / 1e3
         per_launch = 20.0 * pagg["substeps_warp"] / kern["hot"][1]
         achieved = per_launch / t_launch / 1e12
-        roof = {"kernel": "k_hot + k_step (hot pass)", "bound": "alu", "achieved": achieved,
+        roof = {"kernel": "k_stream (hot pass)", "bound": "alu", "achieved": achieved,
                 "peak": mul_peak, "unit": "T int32-mul/s", "frac": achieved / mul_peak,
                 "traffic": None, "traffic_note": HOT_TRAFFIC_NOTE,
                 "peak_kind": "measured: qed_peak_probe MUL32 (Philox multiplies) on this GPU"}
@@ -458,10 +457,9 @@ def run_sweep(ctx, dev, args, hbm_peak, peak_kind):
     del y, F1, F2
 
     # binary64 functions (the double-precision level of Table 1), same points:
-    # 8 B in + 16 B out per evaluation; the arithmetic is two degree-11
-    # polynomials (22 multiply-adds, 44 FP64 flops) plus exp for x >= 1/2, on
-    # the FP64 pipe (nominal 1.25 TFLOP/s dense on GB300; not in the measured
-    # peaks file)
+    # 8 B in + 16 B out per evaluation; the arithmetic is two degree-12
+    # polynomials and exp for x >= 1/2 in 64-bit fixed point, on the integer
+    # multiply pipe (the FP64 pipe is idle)
     y64 = torch.from_numpy(I.sweep_points(SWEEP_N, SEED_SWEEP).astype(np.float64)).to(dev)
     G1 = torch.empty_like(y64)
     G2 = torch.empty_like(y64)
@@ -475,11 +473,10 @@ def run_sweep(ctx, dev, args, hbm_peak, peak_kind):
     torch.cuda.synchronize()
     ms64 = e0.elapsed_time(e1) / reps
     del y64, G1, G2
-    tf64 = 44.0 * SWEEP_N / (ms64 / 1e3) / 1e12
-    f64 = {"evals_per_s": SWEEP_N / (ms64 / 1e3), "ms": ms64,
-           "hbm_gbs": 24.0 * SWEEP_N / (ms64 / 1e3) / 1e9,
-           "fp64": {"achieved": tf64, "peak": 1.25, "unit": "TFLOP/s", "frac": tf64 / 1.25,
-                    "peak_kind": "nominal (GB300 dense FP64)", "flops_per_eval": 44}}
+    gbs64 = 24.0 * SWEEP_N / (ms64 / 1e3) / 1e9
+    f64 = {"evals_per_s": SWEEP_N / (ms64 / 1e3), "ms": ms64, "hbm_gbs": gbs64,
+           "hbm": {"achieved": gbs64, "peak": hbm_peak, "unit": "GB/s", "frac": gbs64 / hbm_peak,
+                   "peak_kind": peak_kind, "bytes_per_eval": 24}}
     return {"n": SWEEP_N, "evals_per_s": evals, "ms": ms,
             "hbm": {"achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
                     "peak_kind": peak_kind, "bytes_per_eval": 12},

@@ -169,7 +169,7 @@ qed_status qed_synchrotron_F1F2(qed_ctx* ctx, const float* y, float* F1, float* 
 
 /* The same functions in binary64, at the double-precision accuracy level of
  * Sec. 3.2.1 (Table 1: 1e-14): relative error below 1e-15 for y in
- * (0, 512), from three polynomials of degree 11 per octave (no difference of
+ * (0, 512), from three polynomials of degree 12 per octave (no difference of
  * large terms is formed); 0 for y <= 0, y >= 512 (where F, G < 1e-220) and
  * NaN.  y, F1, F2 are device arrays of n doubles; F1 or F2 may be NULL (not
  * both when n > 0); n == 0 is a no-op.  No context: runs on `stream` (a
@@ -412,9 +412,9 @@ qed_status qed_sampler_load(qed_ctx* ctx, const float* params, int64_t n);
 qed_status qed_sampler_save(qed_ctx* ctx, float* params, int64_t n);
 
 /* Launch settings.  hot_min: plans of at least this many sub-steps leave the
- * thread pass for the hot pass (default 32); long_min: hot plans of at least
- * this many sub-steps are stepped by a whole warp each, the others one lane
- * each (default 256; the sampler mode steps every hot particle by a warp);
+ * thread pass for the hot pass (default 32); long_min orders the queue:
+ * plans of at least 4 long_min sub-steps (default 256) are stepped first, and
+ * in sampler mode 1 those of at least long_min by a whole warp each;
  * the resident blocks per SM of the thread and hot passes (default: the
  * occupancy maximum; larger values are clamped to it).  0 keeps a setting.
  * No setting changes a result.  Errors: QED_ERR_ARG. */

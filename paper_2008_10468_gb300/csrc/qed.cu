@@ -2156,11 +2156,14 @@ constexpr uint32_t kWindow = 64;             // mode 1's medium plans: sub-steps
 // the last one found, plans them and the rows just taken together, draws the
 // lists that have run out and tests the next candidates.  Persistent: the
 // grid is the resident block count.  A warp first takes its share of the long
-// plans (N >= long_min, front of the queue array), so that their chains start
+// plans (N >= front_min, front of the queue array), so that their chains start
 // early, then medium plans (back of the array); lanes whose particle is done
 // take further entries, kHotRefill at a time (one atomic per warp and queue).
 // The entries are spread evenly: a warp takes no more than the queue's length
-// over the number of warps.
+// over the number of warps.  Bound by the issue of the divergent parts (plans,
+// tests) and of the draws, and at the end by the longest chains: the 9.5e5
+// events of 1e5 uniform-field electrons take 830 us (1280 with a whole warp on
+// each particle, which planned in all its lanes).
 struct HotSmem {
     SharedTables tables;
     ListBuf list[kLaneThreads / 32];

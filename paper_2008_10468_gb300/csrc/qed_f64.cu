@@ -11,14 +11,15 @@
 // (F, G < 1e-220).
 //
 // The polynomial, exp(-x) and their product are 64-bit fixed-point integers,
-// not binary64: this GPU has 1/64 of the binary32 rate in binary64 (an FMA
-// pipe that 26 to 40 operations an evaluation kept 90% busy), but forms about
+// not binary64: this GPU has 1/64 of the binary32 rate in binary64 (a pipe that
+// the 22 multiply-adds and the exp of an evaluation kept 90% busy), but forms about
 // 30 wide 32 x 32 products per clock and SM.  A 64-bit step of the Horner
 // recurrence is three of them; the powers whose coefficients are below 2^-25
-// take one each in 32 bits.  Worst error against 40-digit values 1.3e-16 (half
-// a unit in the last place, the rounding of the result), where the binary64
-// evaluation had 7e-16.  2^24 log-uniform points in [1e-4, 50]: 1420 us in
-// binary64, see k_sweep64 for this form.
+// take one each in 32 bits.  Worst error against 40-digit values 1.8e-16
+// (little above half a unit in the last place, the rounding of the result),
+// where the binary64 evaluation of the same fit has 4.2e-16.  2^24 log-uniform
+// points in [1e-4, 50]: 1420 us in binary64, 291 us in this form.  Bound by the
+// issue of the 64-bit integer steps; the 24 bytes a point take 60 us of HBM.
 #include <cstdint>
 
 #include "qed.h"
