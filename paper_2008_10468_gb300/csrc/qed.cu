@@ -2783,9 +2783,12 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
 constexpr int kStreamRefill = 8;             // idle lanes before a busy warp takes entries,
 constexpr unsigned int kStreamRounds = 8;    // and rounds between two looks at an empty queue
 constexpr unsigned int kStreamSpread = 16;   // warps that share the children on offer (256: 1.05
-                                             // instead of 0.98 ms at 2^20 rows)
-constexpr int kStreamLanes = 16;             // most particles of a warp, 32 when the queue holds
-constexpr unsigned int kStreamMany = 8;      // this many times the warps (always 16: 4.2 ms at 2^24)
+                                             // instead of 0.96 ms at 2^20 rows)
+// Most particles of a warp: 16, and 32 when the queue holds kStreamMany times
+// the warps (128 times: 1.53 instead of 1.38 ms at 2^22 rows; always 32: 0.85
+// instead of 0.81 ms at 2^20 rows).
+constexpr int kStreamLanes = 16;
+constexpr unsigned int kStreamMany = 8;
 
 // A warp's children.  Rows and entries are reserved at the start of a round,
 // written after its plans and published after its draws, so that the chains
