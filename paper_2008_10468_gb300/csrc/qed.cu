@@ -1815,7 +1815,6 @@ constexpr int kWindows = 8;   // windows a lane draws at a time (1e5 uniform-fie
 // instructions; a second copy of two rounds costs more than it hides (cascade
 // of 4096 cells: 13.1 ms with four, 12.6 with two, 12.8 with one).
 constexpr int kHotIlp = 4, kStreamIlp = 2;
-constexpr uint32_t kOwnMax = 8;      // plans of this many sub-steps are drawn by their lane
 struct ListBuf {                     // one per warp
     DrawKey key[32];
     uint4 par[32];                   // evaluation: T, b, c_h
@@ -1990,8 +1989,10 @@ __device__ __forceinline__ bool lane_count_plan(Lane& L, Stats& stats) {
 // Draw the masks of the lanes that have walked through theirs and are not at
 // the end of their plan.  Their windows are listed and drawn one after the
 // other, kDrawIlp at a time (a window's ten multiply rounds are one chain), by
-// all 32 lanes.  A lane whose plan ends within kOwnMax sub-steps draws its few
-// blocks by itself, at the same time as the other such lanes.
+// all 32 lanes.  Also a plan of a few sub-steps takes a window: a second form in
+// which its lane drew its blocks by itself cost k_stream more in instruction
+// fetches than it saved (4096-cell cascade 12.4 against 12.0 ms, 2^24 rows 3.64
+// against 3.60) and gave the hot pass nothing.
 template <int kDrawIlp>
 __device__ __forceinline__ void list_draw(ListBuf& B, Lane& L, uint32_t y1, const PhiloxKeys& K) {
     constexpr unsigned int kAll = 0xffffffffu;
@@ -2001,25 +2002,11 @@ __device__ __forceinline__ void list_draw(ListBuf& B, Lane& L, uint32_t y1, cons
     if (!__any_sync(kAll, need)) return;
     const uint32_t last_word = (L.T_cap << 9) - 1u;   // (r >> 9) < T_cap, T_cap <= 2^23
     const uint32_t last = L.next + left - 1u;         // last sub-step of the plan
-    const bool own = need && left <= kOwnMax && (last >> 6) == (L.next >> 6);
     int nw = 0;
     if (need) {
         L.w0 = L.next >> 6;
-        nw = own ? 0 : (int)min((uint32_t)kWindows, (last >> 6) - L.w0 + 1u);
-        L.cov = own ? last + 1u : (L.w0 + (uint32_t)nw) << 6;
-    }
-    if (__any_sync(kAll, own)) {
-        unsigned int mA = 0, mB = 0;
-        uint32_t blk = L.next >> 1;
-        while (__any_sync(kAll, own && blk <= last >> 1)) {
-            if (own && blk <= last >> 1) {
-                const uint2 r = draw_yw(B.key[lane], y1, blk, K);
-                mA |= (r.x <= last_word ? 1u : 0u) << (blk & 31u);
-                mB |= (r.y <= last_word ? 1u : 0u) << (blk & 31u);
-                ++blk;
-            }
-        }
-        if (own) B.mask[0][lane] = make_uint2(mA, mB);
+        nw = (int)min((uint32_t)kWindows, (last >> 6) - L.w0 + 1u);
+        L.cov = (L.w0 + (uint32_t)nw) << 6;
     }
     int total = 0;
 #pragma unroll
@@ -2029,10 +2016,6 @@ __device__ __forceinline__ void list_draw(ListBuf& B, Lane& L, uint32_t y1, cons
         total += __popc(m);
     }
     if (nw) B.draw[lane] = make_uint2(L.w0 << 5, last_word);
-    if (!total) {
-        __syncwarp();
-        return;
-    }
     if (lane < kDrawIlp) B.item[total + lane] = (uint8_t)0;   // padding, overwritten below
     __syncwarp();
     if (lane < kDrawIlp) B.item[total + lane] = B.item[0];

@@ -1,5 +1,5 @@
 """The hot pass's and the tail pass's candidate masks at their edges, event by
-event against the oracle: plans so short that a lane draws them itself, plans
+event against the oracle: plans of a few sub-steps, plans
 that end inside, at and just past a window of 64 sub-steps, thresholds that
 admit most sub-steps (large p_max) and almost none, and queues that hold one
 particle per warp and many.  GPU only."""
