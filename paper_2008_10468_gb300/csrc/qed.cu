@@ -117,7 +117,6 @@ struct DevCtl {
 constexpr uint8_t kNotReady = 0xFF;
 // Row index of a long-plan queue entry that has not been written yet.
 constexpr uint32_t kNoItem = 0xFFFFFFFFu;
-constexpr uint32_t kVoidItem = 0xFFFFFFFEu;   // written, for a row that did not fit
 
 struct HotItem {
     uint32_t idx;
@@ -2750,8 +2749,8 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
 // Cascade step without a sampler: the thread pass over the initial rows, then
 // one persistent launch that does the rest, whatever generation a particle
 // belongs to.  Its loop is the hot pass's; the queue goes on growing: a child
-// is written, then its queue entry (row, time left), then the entry's index,
-// and a lane that took an entry waits for that index.
+// is written, then its row's index in its queue entry, and a lane that took an
+// entry waits for that index.
 //
 // Launched generation by generation, every generation ends in its longest
 // chains with most of the GPU idle (11 of 16 warps resident on average) and
@@ -2773,18 +2772,19 @@ constexpr unsigned int kStreamSpread = 16;   // warps that share the children on
 constexpr int kStreamLanes = 16;
 constexpr unsigned int kStreamMany = 8;
 
-// A warp's children.  Rows and entries are reserved at the start of a round,
-// written after its plans and published after its draws, so that the chains
-// that go on do not wait for the two atomics and the fence (65536 rows: 0.46
-// instead of 0.65 ms).
+// A warp's children.  Their rows are reserved at the start of a round; after its
+// plans they are written and the ones with time left take queue entries, which
+// are published after its draws, so that the chains that go on do not wait for
+// the two atomics and the fence (65536 rows: 0.46 instead of 0.65 ms).  Only a
+// row that exists takes an entry: parents go on emitting into a full store, and
+// the queue has room for the store's rows, not for all that is wanted.
 struct StreamChildren {
     bool mine = false, photon = false;   // this lane holds an event; its parent
     int nq = 0, off_r = 0, off_q = 0;    // entries (0 or the children); offsets of rows, entries
     unsigned long long base_r = 0;       // lane 0
     unsigned int base_q = 0;             // lane 0
     unsigned int n = 0;                  // events taken from the ring
-    uint32_t idx = kNoItem;              // written: the first child's index to publish
-    unsigned int entry = 0;
+    uint32_t idx = kNoItem;              // written: the first child's row
 };
 __device__ __forceinline__ StreamChildren stream_begin(const DevParticles& P, const StepParams& SP,
                                                      DevCtl* ctl, const EventBuf& E, unsigned int n,
@@ -2796,56 +2796,47 @@ __device__ __forceinline__ StreamChildren stream_begin(const DevParticles& P, co
     __syncwarp();
     const unsigned int q = (head + lane) % kEventBuf;
     c.mine = lane < c.n;
-    bool wanted = false;
-    if (c.mine) {
-        c.photon = E.x[q] < 0.0f;
-        wanted = time_positive(E.t_after[q]) && process_enabled(SP, !c.photon);
-    }
+    if (c.mine) c.photon = E.x[q] < 0.0f;
     const unsigned int m1 = __ballot_sync(kAll, c.mine && !c.photon);
     const unsigned int m2 = __ballot_sync(kAll, c.photon);
-    const unsigned int q1 = __ballot_sync(kAll, wanted && !c.photon);
-    const unsigned int q2 = __ballot_sync(kAll, wanted && c.photon);
     c.off_r = __popc(m1 & below) + 2 * __popc(m2 & below);
-    c.off_q = __popc(q1 & below) + 2 * __popc(q2 & below);
-    c.nq = wanted ? (c.photon ? 2 : 1) : 0;
-    if (lane == 0) {
+    if (lane == 0)
         c.base_r = atomicAdd(reinterpret_cast<unsigned long long*>(P.count),
                              (unsigned long long)(__popc(m1) + 2 * __popc(m2)));
-        if (q1 | q2)
-            c.base_q = atomicAdd(&ctl->queue.step_tail,
-                                 (unsigned int)(__popc(q1) + 2 * __popc(q2)));
-    }
     return c;
 }
 __device__ __forceinline__ void stream_write(const DevParticles& P, const Scratch& S,
                                             const StepParams& SP, DevCtl* ctl, const EventBuf& E,
-                                            unsigned int head, unsigned int cold_long,
-                                            StreamChildren& c, uint32_t step) {
+                                            unsigned int head, StreamChildren& c, uint32_t step) {
     constexpr unsigned int kAll = 0xffffffffu;
+    const unsigned int lane = threadIdx.x & 31, below = (1u << lane) - 1u;
     const unsigned long long base_r = __shfl_sync(kAll, c.base_r, 0);
-    c.entry = cold_long + __shfl_sync(kAll, c.base_q, 0) + (unsigned int)c.off_q;
     if (c.mine) {
-        const unsigned int q = (head + (threadIdx.x & 31)) % kEventBuf;
-        const long long j = check_rows(P, ctl, (long long)base_r + c.off_r, c.photon ? 2 : 1);
+        const unsigned int q = (head + lane) % kEventBuf;
+        const int n = c.photon ? 2 : 1;
+        const long long j = check_rows(P, ctl, (long long)base_r + c.off_r, n);
         write_children(P, S, SP, E.i[q], j, E.id[q], c.photon, fabsf(E.x[q]), E.chi[q], step,
                        E.s[q], E.t_after[q], PState{E.px[q], E.py[q], E.pz[q]},
                        Fields{E.f[0][q], E.f[1][q], E.f[2][q], E.f[3][q], E.f[4][q], E.f[5][q]},
                        kPlain);
-        c.idx = j >= 0 ? (uint32_t)j : kVoidItem;
-        for (int k = 0; k < c.nq; ++k) {
-            S.hot[c.entry + k].s = 0u;
-            S.hot[c.entry + k].t_rem = E.t_after[q];
-        }
+        c.idx = (uint32_t)j;
+        c.nq = j >= 0 && time_positive(E.t_after[q]) ? n : 0;   // a cascade has both processes on
     }
-    __syncwarp();
+    const unsigned int q1 = __ballot_sync(kAll, c.nq == 1), q2 = __ballot_sync(kAll, c.nq == 2);
+    c.off_q = __popc(q1 & below) + 2 * __popc(q2 & below);
+    if (lane == 0 && (q1 | q2))
+        c.base_q = atomicAdd(&ctl->queue.step_tail, (unsigned int)(__popc(q1) + 2 * __popc(q2)));
+    __syncwarp();   // the ring's entries are reused
 }
-__device__ __forceinline__ void stream_publish(const Scratch& S, const StreamChildren& c) {
+// All lanes of the warp.  A child's entry is its row; the rest of the entry (the
+// first sub-step, the time left) is the row's.
+__device__ __forceinline__ void stream_publish(const Scratch& S, unsigned int cold_long,
+                                               const StreamChildren& c) {
+    const unsigned int entry = cold_long + __shfl_sync(0xffffffffu, c.base_q, 0) + (unsigned int)c.off_q;
     if (c.nq) {
-        __threadfence();   // the children's rows and the entries before the indices
-        *reinterpret_cast<volatile uint32_t*>(&S.hot[c.entry].idx) = c.idx;
-        if (c.nq == 2)
-            *reinterpret_cast<volatile uint32_t*>(&S.hot[c.entry + 1].idx) =
-                c.idx == kVoidItem ? kVoidItem : c.idx + 1u;
+        __threadfence();   // the children's rows before the indices
+        *reinterpret_cast<volatile uint32_t*>(&S.hot[entry].idx) = c.idx;
+        if (c.nq == 2) *reinterpret_cast<volatile uint32_t*>(&S.hot[entry + 1].idx) = c.idx + 1u;
     }
 }
 
@@ -2920,9 +2911,6 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
         if (lane == 0 && m) q = atomicAdd(&ctl->queue.step_tail, (unsigned int)__popc(m));
         q = cold_long + __shfl_sync(kAll, q, 0) + (unsigned int)__popc(m & ((1u << lane) - 1u));
         if (queue) {
-            S.hot[q].s = 0u;
-            S.hot[q].t_rem = t;
-            __threadfence();
             *reinterpret_cast<volatile uint32_t*>(&S.hot[q].idx) = (uint32_t)r;
         }
     }
@@ -3001,10 +2989,11 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
             if (waiting) i = *reinterpret_cast<const volatile uint32_t*>(&e->idx);
             if (i != kNoItem) {
                 __threadfence();
-                const HotItem it = *e;
+                const bool child = !from_med && entry >= cold_long;
+                const uint32_t s = child ? 0u : e->s;
+                const ftime t = child ? S.t_rem[i] : e->t_rem;
                 waiting = false;
-                if (i == kVoidItem) ++done;
-                else lane_take(P, SP, L, B, fld, step, i, P.type[i] == QED_PHOTON, it.s, it.t_rem);
+                lane_take(P, SP, L, B, fld, step, i, P.type[i] == QED_PHOTON, s, t);
             }
         }
         // ---- 3. the events of the last round; they and new rows plan together
@@ -3029,7 +3018,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
         }
         const bool on = __any_sync(kAll, L.active);
         if (flush) {
-            stream_write(P, S, SP, ctl, E, ev_head, cold_long, kids, step);
+            stream_write(P, S, SP, ctl, E, ev_head, kids, step);
             n_ev -= kids.n;
             ev_head += kids.n;
         }
@@ -3047,11 +3036,11 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
                 lane_finish(P, L);
                 ++done;
             }
-            if (flush) stream_publish(S, kids);
+            if (flush) stream_publish(S, cold_long, kids);
             __syncwarp();   // the list buffer is reused by the next round
             continue;
         }
-        if (flush) stream_publish(S, kids);
+        if (flush) stream_publish(S, cold_long, kids);
         // ---- 5. nothing to draw: wait for work, or finish.  The warp that
         // completes the last unit sees as many units complete as are known, and
         // says so in the word that idle warps poll.
@@ -3639,11 +3628,12 @@ qed_status ensure_scratch(qed_ctx* ctx, long long cap) {
     ctx->d_hot = nullptr;
     ctx->scratch_cap = 0;
     QED_CUDA(ctx, cudaMalloc(&ctx->d_trem, sizeof(ftime) * cap));
-    // queue: long plans from the front, medium plans from the back.  Every
-    // entry belongs to a row and a row has at most two entries per generation
-    // (in the tail pass a medium plan may come back as a long plan), so 2 cap
-    // entries never let the ends meet.  Long-plan entries start "not written"
-    // (row index all ones) and each step resets the ones it used.
+    // queue: long plans (and k_stream's children) from the front, medium plans
+    // from the back.  Every entry belongs to a row of the store and a row has at
+    // most two entries per generation (in the tail pass a medium plan may come
+    // back as a long plan; k_stream: one, a child that did not fit has none), so
+    // 2 cap entries never let the ends meet.  Entries at the front start "not
+    // written" (row index all ones) and each step resets the ones it used.
     QED_CUDA(ctx, cudaMalloc(&ctx->d_hot, sizeof(HotItem) * 2 * cap));
     QED_CUDA(ctx, cudaMemset(ctx->d_hot, 0xFF, sizeof(HotItem) * 2 * cap));
     ctx->scratch_cap = cap;
