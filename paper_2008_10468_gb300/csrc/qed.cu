@@ -839,7 +839,8 @@ __global__ void __launch_bounds__(kColdThreads, kColdMinBlocks) k_cold(DevPartic
         pl.b = pl.c_h = 0.0f;
         float chi = 0.0f, eps = 0.0f;
         uint32_t s = 0;
-        bool need_plan = active, event = false;
+        bool need_plan = active;
+        unsigned int events = 0;   // !kLoop: the warp's lanes with an event
         while (__any_sync(kAll, active)) {
             if (need_plan) {
                 need_plan = false;
@@ -893,6 +894,9 @@ __global__ void __launch_bounds__(kColdThreads, kColdMinBlocks) k_cold(DevPartic
             const uint32_t s_end = active ? s + pl.N : 0u;
             draw_round(sm, B, active, s, s_end, pl.T, pl.b, pl.c_h, photon, y1, SP.draw_keys,
                        stats.cand);
+            // the lanes with an event, by all lanes of the warp: their places in
+            // the ring (the lanes of a branch need not run it together)
+            if (!kLoop) events = __ballot_sync(kAll, active && B.facc[lane] != kNoEvent);
             if (active) {
                 const uint32_t s_ev = B.facc[lane];
                 if (s_ev == kNoEvent) {
@@ -915,13 +919,12 @@ __global__ void __launch_bounds__(kColdThreads, kColdMinBlocks) k_cold(DevPartic
                         if (removed || !time_positive(t_rem)) active = false;
                         else need_plan = true;
                     } else {
-                        const unsigned int m = __activemask();
-                        note_event(E, (ev_head + n_ev + __popc(m & ((1u << lane) - 1u))) % kEventBuf,
+                        note_event(E,
+                                   (ev_head + n_ev + __popc(events & ((1u << lane) - 1u))) % kEventBuf,
                                    (uint32_t)i, id, photon, x, chi, s_ev, t_after, st,
                                    Fields{Ex, Ey, Ez, Bx, By, Bz});
                         count_event(stats, photon);
                         removed = event_recoil(SP, photon, x, eps, st);
-                        event = true;
                         active = false;
                     }
                 }
@@ -938,8 +941,9 @@ __global__ void __launch_bounds__(kColdThreads, kColdMinBlocks) k_cold(DevPartic
         }
         if (!kLoop) {
             // the parents go on in the hot pass
-            if (event && !removed && time_positive(t_rem)) push_hot(S, ctl, i, s, t_rem, false);
-            n_ev += (unsigned int)__popc(__ballot_sync(kAll, event));
+            if ((events >> lane & 1u) && !removed && time_positive(t_rem))
+                push_hot(S, ctl, i, s, t_rem, false);
+            n_ev += (unsigned int)__popc(events);
             if (n_ev >= 32u) events_flush(P, S, SP, ctl, E, n_ev, ev_head, step);
         }
     }
