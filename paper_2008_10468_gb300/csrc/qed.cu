@@ -2865,10 +2865,14 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
     // the thread pass's queue and children (fixed during this kernel)
     const unsigned int cold_long = ctl->hot_tail, cold_med = ctl->med_tail;
     const long long n0 = ctl->n0, n1 = ctl->n1;
-    const unsigned long long work = (unsigned long long)cold_long + cold_med + (unsigned long long)(n1 - n0);
+    const unsigned int cold_kids = (unsigned int)(n1 - n0);
+    // units to complete: these, and every child queued so far.  No unit belongs
+    // to a certain warp: next to another stream's kernels some of the blocks may
+    // not be resident, and the others must be able to end the step without them
+    const unsigned long long units0 = (unsigned long long)cold_long + cold_med + cold_kids;
     const unsigned int blocks = (unsigned int)min(
-        (unsigned long long)gridDim.x, kTailMinBlocks + work * kTailWarps / (kLaneThreads / 32));
-    if (ctl->skip || ctl->status == (int)QED_ERR_TIMEOUT || blockIdx.x >= blocks) return;
+        (unsigned long long)gridDim.x, kTailMinBlocks + units0 * kTailWarps / (kLaneThreads / 32));
+    if (ctl->skip || ctl->status == (int)QED_ERR_TIMEOUT || units0 == 0 || blockIdx.x >= blocks) return;
     stage_tables(sm);
     __syncthreads();
     constexpr unsigned int kAll = 0xffffffffu;
@@ -2878,9 +2882,9 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
     unsigned int n_ev = 0, ev_head = 0;   // events whose children are not written yet
     const uint32_t y1 = draw_y1(step, SP.draw_keys);
     const unsigned int nwarps = blocks * (kLaneThreads / 32);
-    // units to complete: the thread pass's queue, each warp's part of its
-    // children, and every child queued so far
-    const unsigned long long units0 = (unsigned long long)cold_long + cold_med + nwarps;
+    // entries in the order they are taken: the thread pass's long plans, its
+    // children (by their rows, nothing in the array), the children queued here
+    const unsigned int first_new = cold_long + cold_kids;
     const unsigned int share_long = max(1u, min(32u, (cold_long + nwarps - 1u) / nwarps));
     const unsigned int share_med = max(1u, min(32u, (cold_med + nwarps - 1u) / nwarps));
     Stats stats;                 // per lane
@@ -2899,26 +2903,6 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
     unsigned int idle = 0, rounds = 0;
     unsigned long long idle_ns = 0, seen = 0;
     bool timed_out = false, finish = false;
-    // ---- the thread pass's children
-    for (long long b = n0 + 32ll * (blockIdx.x * (kLaneThreads / 32) + (threadIdx.x >> 5)); b < n1;
-         b += 32ll * nwarps) {
-        const long long r = b + lane;
-        bool queue = r < n1;
-        ftime t{0.0f, 0.0f};
-        if (queue) {
-            const uint8_t type = P.type[r];
-            t = S.t_rem[r];
-            queue = type <= QED_PHOTON && process_enabled(SP, type == QED_PHOTON) && time_positive(t);
-        }
-        const unsigned int m = __ballot_sync(kAll, queue);
-        unsigned int q = 0;
-        if (lane == 0 && m) q = atomicAdd(&ctl->queue.step_tail, (unsigned int)__popc(m));
-        q = cold_long + __shfl_sync(kAll, q, 0) + (unsigned int)__popc(m & ((1u << lane) - 1u));
-        if (queue) {
-            *reinterpret_cast<volatile uint32_t*>(&S.hot[q].idx) = (uint32_t)r;
-        }
-    }
-    if (lane == 0) ++done;
     while (true) {
         // ---- 1. rows for the idle lanes
         {
@@ -2934,7 +2918,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
                 unsigned int over = 0;
                 if (lane == 0) {
                     const uint4 qs = queue_state(ctl);
-                    const unsigned int h_long = qs.x, h_med = qs.y, tail = cold_long + qs.z;
+                    const unsigned int h_long = qs.x, h_med = qs.y, tail = first_new + qs.z;
                     over = qs.w;
                     more_med = more_med && h_med < cold_med;
                     const unsigned int left = (h_long < tail ? tail - h_long : 0u) +
@@ -2988,16 +2972,23 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
         // ---- 2. lanes holding an entry: take its row once it is written
         if (__any_sync(kAll, waiting)) {
             uint32_t i = kNoItem;
+            const bool child = !from_med && entry >= cold_long;
             const HotItem* e = S.hot + (from_med ? S.hot_cap - 1 - (long long)entry
-                                                 : (long long)entry);
-            if (waiting) i = *reinterpret_cast<const volatile uint32_t*>(&e->idx);
+                                                 : (long long)entry - (child ? cold_kids : 0u));
+            if (waiting)
+                i = child && entry < first_new ? (uint32_t)n0 + (entry - cold_long)
+                                               : *reinterpret_cast<const volatile uint32_t*>(&e->idx);
             if (i != kNoItem) {
                 __threadfence();
-                const bool child = !from_med && entry >= cold_long;
+                waiting = false;
+                const uint8_t type = P.type[i];
                 const uint32_t s = child ? 0u : e->s;
                 const ftime t = child ? S.t_rem[i] : e->t_rem;
-                waiting = false;
-                lane_take(P, SP, L, B, fld, step, i, P.type[i] == QED_PHOTON, s, t);
+                // not so for some of the thread pass's children only
+                if (type <= QED_PHOTON && time_positive(t))
+                    lane_take(P, SP, L, B, fld, step, i, type == QED_PHOTON, s, t);
+                else
+                    ++done;
             }
         }
         // ---- 3. the events of the last round; they and new rows plan together
