@@ -414,7 +414,8 @@ qed_status qed_sampler_save(qed_ctx* ctx, float* params, int64_t n);
 /* Launch settings.  hot_min: plans of at least this many sub-steps leave the
  * thread pass for the hot pass (default 32); long_min orders the queue:
  * plans of at least 4 long_min sub-steps (default 256) are stepped first, and
- * in sampler mode 1 those of at least long_min by a whole warp each;
+ * those of at least long_min by a whole warp each in sampler mode 1 and in the
+ * sampler modes' tail pass;
  * the resident blocks per SM of the thread and hot passes (default: the
  * occupancy maximum; larger values are clamped to it).  0 keeps a setting.
  * No setting changes a result.  Errors: QED_ERR_ARG. */

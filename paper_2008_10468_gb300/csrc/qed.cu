@@ -444,8 +444,7 @@ constexpr long long kReserveHere = -2;   // apply_event reserves the child rows 
 // fit) and the event into the log.  st: the parent before the event; the type
 // bytes come last.  Returns the child ids.  kPublish: in a persistent pass another warp may be waiting
 // for these rows: one fence for the event's children, then their type bytes.
-// kDeferred: the same, but fence and type bytes are the caller's.
-enum ChildMode { kPlain, kPublish, kDeferred };
+enum ChildMode { kPlain, kPublish };
 __device__ __forceinline__ uint8_t child_type(bool photon, int r) {
     return photon ? (r == 0 ? (uint8_t)QED_ELECTRON : (uint8_t)QED_POSITRON) : (uint8_t)QED_PHOTON;
 }
@@ -470,10 +469,8 @@ __device__ __forceinline__ ulonglong2 write_children(const DevParticles& P, cons
             cid_r = id1;
         }
         if (mode == kPublish) __threadfence();
-        if (mode != kDeferred) {
-            *reinterpret_cast<volatile uint8_t*>(P.type + j) = child_type(photon, 0);
-            if (photon) *reinterpret_cast<volatile uint8_t*>(P.type + j + 1) = child_type(true, 1);
-        }
+        *reinterpret_cast<volatile uint8_t*>(P.type + j) = child_type(photon, 0);
+        if (photon) *reinterpret_cast<volatile uint8_t*>(P.type + j + 1) = child_type(true, 1);
     }
     if (S.log) {
         const long long k = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(S.log_count), 1ull);
@@ -1527,8 +1524,8 @@ __device__ __forceinline__ void warp_item(const DevParticles& P, const Scratch& 
             }
             const unsigned int m0 = __ballot_sync(0xffffffffu, a0);
             const unsigned int m1 = __ballot_sync(0xffffffffu, a1);
-            cand += (unsigned)c0 + (unsigned)c1;
             if ((m0 | m1) == 0u) {
+                cand += (unsigned)c0 + (unsigned)c1;
                 const uint32_t chunk_end = min(sa + 64u, lim);
                 if (lane == 0) stats.substeps += chunk_end - sb;
                 kdone += chunk_end - sb;
@@ -1543,6 +1540,9 @@ __device__ __forceinline__ void warp_item(const DevParticles& P, const Scratch& 
             const int p1 = m1 ? 2 * (__ffs(m1) - 1) + 1 : 1 << 30;
             const int pos = min(p0, p1);
             const uint32_t s_ev = sa + (uint32_t)pos;
+            // mode 1 counts its window's candidates past the event too
+            cand += (unsigned)(c0 && (kSampler == 1 || s0 <= s_ev)) +
+                    (unsigned)(c1 && (kSampler == 1 || s0 + 1u <= s_ev));
             const float xo = (pos & 1) ? u01(r.z) : u01(r.x);
             float x = __shfl_sync(0xffffffffu, xo, pos >> 1);
             if (kSampler == 1 && use_net) {
@@ -1880,46 +1880,6 @@ __device__ __forceinline__ void lane_finish(const DevParticles& P, Lane& L) {
     L.active = L.need_plan = false;
 }
 
-// Children of the warp's events: rows reserved, not yet written.
-struct PendingChildren {
-    bool mine = false;               // this lane has some
-    int offset = 0;
-    unsigned long long base = 0;     // on the leader
-    int leader = 0;
-    PState st{0.0f, 0.0f, 0.0f};     // the parent before the event
-};
-
-// First half of the lanes' events: the child rows are reserved (one atomic for
-// the warp, not waited for) and the parents recoil.
-__device__ __forceinline__ PendingChildren events_begin(const DevParticles& P, const StepParams& SP,
-                                                        Lane& L, Stats& stats) {
-    constexpr unsigned int kAll = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    PendingChildren c;
-    const unsigned int m1 = __ballot_sync(kAll, L.event && !L.photon);
-    const unsigned int m2 = __ballot_sync(kAll, L.event && L.photon);
-    if ((m1 | m2) == 0u) return c;
-    c.leader = __ffs(m1 | m2) - 1;
-    if (lane == c.leader)
-        c.base = atomicAdd(reinterpret_cast<unsigned long long*>(P.count),
-                           (unsigned long long)(__popc(m1) + 2 * __popc(m2)));
-    if (L.event) {
-        const unsigned int below = (1u << lane) - 1u;
-        c.mine = true;
-        c.offset = __popc(m1 & below) + 2 * __popc(m2 & below);
-        c.st = L.st;
-        const uint32_t k = L.s_ev - L.s0;
-        stats.substeps += k + 1u;
-        count_event(stats, L.photon);
-        L.t_rem = (k + 1u == L.pl.N) ? ftime{0.0f, 0.0f} : time_sub_mul(L.t_rem, k + 1u, L.pl.h);
-        L.removed = event_recoil(SP, L.photon, L.x_ev, L.eps, L.st);
-        L.changed = true;
-        L.s0 = L.next = L.s_ev + 1u;
-        L.need_plan = !L.removed && time_positive(L.t_rem);
-    }
-    return c;
-}
-
 // The lanes' events: noted for their children, the parents recoil.  n, head:
 // the ring's entries (warp-uniform).
 __device__ __forceinline__ void events_note(const StepParams& SP, Lane& L, EventBuf& E,
@@ -1944,25 +1904,7 @@ __device__ __forceinline__ void events_note(const StepParams& SP, Lane& L, Event
     n += (unsigned int)__popc(m);
 }
 
-// Second half: the children are written (their chi is the parent's before the
-// event, for the log).  Returns the first child's row, or -1.
-__device__ __forceinline__ long long events_end(const DevParticles& P, const Scratch& S,
-                                                const StepParams& SP, DevCtl* ctl, Lane& L,
-                                                const PendingChildren& c, ftime t_after, float chi,
-                                                const LaneFields& f, uint32_t step, ChildMode mode) {
-    const unsigned long long base = __shfl_sync(0xffffffffu, c.base, c.leader);
-    if (!c.mine) return -1;
-    const long long j =
-        check_rows(P, ctl, (long long)(base + (unsigned long long)c.offset), L.photon ? 2 : 1);
-    write_children(P, S, SP, L.i, j, L.id, L.photon, L.x_ev, chi, step, L.s_ev, t_after, c.st,
-                   lane_fields(f), mode);
-    L.event = false;
-    return j;
-}
-
-// Plan the time that is left; true if the particle is done with it: no energy,
-// or no candidate admitted (a zero squeeze threshold: the sub-steps pass
-// without an event).  hand_over (sampler modes): the particle goes elsewhere.
+// Plan the time that is left; true if the particle has no energy to go on with.
 template <bool kCells>
 __device__ __forceinline__ bool lane_plan(const StepParams& SP, const SharedTables& sm, Lane& L,
                                           const LaneFields& f, const DevCtl* ctl) {
@@ -1975,6 +1917,8 @@ __device__ __forceinline__ bool lane_plan(const StepParams& SP, const SharedTabl
                          L.eps);
     return !(L.eps > 0.0f);
 }
+// Count the plan; true if it admits no candidate (a zero squeeze threshold): its
+// sub-steps pass without an event.
 __device__ __forceinline__ bool lane_count_plan(Lane& L, Stats& stats) {
     stats.plans++;
     stats.guard += L.pl.guard ? 1 : 0;
@@ -2417,13 +2361,17 @@ __global__ void __launch_bounds__(kLaneThreads, kHotNetMinBlocks) k_hot_net(DevP
 // generations stop: a thread pass (k_cold) over that generation, then one
 // launch of this persistent kernel finishes the step, taking the thread pass's
 // queue and every child appended from then on (rows n0 and up) as they come.
-// As in the hot pass, a lane holds a particle, the warp draws the windows of
-// its lanes together, and lanes with an event or a new row plan together.  A
-// warp takes child rows appended so far, then its share of the queue's medium
-// plans (each warp the queue's length over the number of warps); the long
-// entries (the sampler's particles among them) are stepped by a whole warp each
-// (warp_item), and so are the sampler's particles that appear later.  (Without
-// a sampler the whole step is k_stream.)
+// Each warp takes, in order,
+//   1. a long plan from the queue (N >= long_min, or a sampler particle), stepped
+//      by the whole warp (warp_item);
+//   2. for its idle lanes, child rows appended so far, then the thread pass's
+//      medium plans, one lane each, with warp-shared draws (draw_round) in
+//      windows of kWindow sub-steps.
+// Only for the sampler modes: without a sampler the whole step is k_stream.  Its
+// form, a particle to each lane also for long plans, was no help here, where the
+// sampler's particles take a whole warp for the network anyway: clumped rows
+// (1% in a strong field) of the event-driven sampler, 46768 / 200000 / 1.4e6 of
+// them, 0.79 / 1.28 / 3.05 ms a step against 0.72 / 1.15 / 2.48 in this form.
 // A child row is published by its writer (type byte last, after a fence); a
 // lane that takes a row still being written waits for it.  Work units are the
 // thread pass's queue entries and the child rows; the pass ends when every
@@ -2442,9 +2390,6 @@ constexpr unsigned long long kWaitNsDefault = 1000000000ull;   // idle time befo
 // Blocks that stay in a persistent pass: these and kTailWarps warps per queue
 // entry (the polls of idle warps slow the others).
 constexpr unsigned int kTailMinBlocks = 8, kTailWarps = 8;
-constexpr int kTailClaim = 8;              // idle lanes before a busy warp takes rows,
-constexpr unsigned int kTailRounds = 8;    // and rounds between two looks
-constexpr unsigned int kTailSpread = 256;  // warps that share the rows on offer
 constexpr unsigned int kTailNap = 4;       // idle warps poll every 256 ns << 0 ... 4
 
 // Queue a long plan: the entry's row index is written last (readers wait for it).
@@ -2458,15 +2403,21 @@ __device__ __forceinline__ void push_long(const Scratch& S, DevCtl* ctl, unsigne
     *reinterpret_cast<volatile uint32_t*>(&e->idx) = (uint32_t)i;
 }
 
-template <int kSampler>
-// Two resident blocks per SM (128 registers, no spills): the tail pass is
-// bound by latency, not by the number of warps.
-__global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepParams SP,
-                                                            Scratch S, DevCtl* ctl) {
+// kBlocks resident blocks per SM.  With two a thread has 128 registers and mode 2
+// keeps 0.7 KB of them in local memory; with one nothing is spilled and a chain
+// is shorter (4096 / 46768 / 200000 rows as above: 0.42 / 0.68 / 1.07 ms instead
+// of 0.48 / 0.72 / 1.15), but there are half as many warps (1.4e6 rows, a tail
+// of 77000: 2.89 instead of 2.48; mode 1 with a tail of 40000: 1.44 instead of
+// 1.28).  Both are launched; the one whose tail it is not returns at once.
+constexpr long long kTailSmall = 1 << 14;   // rows of the tail's first generation below which one block is faster
+template <int kSampler, int kBlocks>
+__global__ void __launch_bounds__(kLaneThreads, kBlocks) k_step(DevParticles P, StepParams SP,
+                                                                Scratch S, DevCtl* ctl) {
+    if ((ctl->pass_end - ctl->pass_begin < kTailSmall) != (kBlocks == 1)) return;
     const uint32_t step = step_index(SP);
     __shared__ SharedTables sm;
-    __shared__ ListBuf list_buf[kLaneThreads / 32];
-    __shared__ LaneFields fld;
+    __shared__ DrawBuf draw_buf[kLaneThreads / 32];
+    __shared__ LaneFields fld;   // E, B at the lane's row (read at plans and events)
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     // the thread pass's queue (fixed during this kernel)
     const unsigned int cold_long = ctl->hot_tail, cold_med = ctl->med_tail;
@@ -2490,31 +2441,34 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
     __syncthreads();
     constexpr unsigned int kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    ListBuf& B = list_buf[threadIdx.x >> 5];
+    DrawBuf& B = draw_buf[threadIdx.x >> 5];
     const uint32_t y1 = draw_y1(step, SP.draw_keys);
+    const uint32_t k0 = (uint32_t)SP.seed, k1 = (uint32_t)(SP.seed >> 32);
     const unsigned long long n0 = (unsigned long long)ctl->n0;
     const bool cascade = SP.cascade != 0;
-    const unsigned int nwarps = blocks * (kLaneThreads / 32);
-    const unsigned int share_med = min(32u, (cold_med + nwarps - 1u) / nwarps);
     Stats stats;                 // per lane; the warp mode counts on lane 0
     unsigned int done = 0;       // units this lane completed, not yet added to ctl->finished
-    bool waiting = false, child = false;
-    uint32_t row = 0;            // waiting: a child's row, or a queue entry's position
-    Lane L;
-    L.pl.N = 0;
-    L.pl.T = 0;
-    L.pl.b = L.pl.c_h = 0.0f;
+    bool active = false, waiting = false, child = false;
+    bool photon = false, changed = false, removed = false;
+    uint32_t i = 0;
+    uint64_t id = 0;
+    PState st{0.0f, 0.0f, 0.0f};
+    ftime t_rem{0.0f, 0.0f};
+    uint32_t s = 0, k_done = 0;
+    Plan pl;
+    pl.N = 0;
+    pl.T = 0;
+    pl.b = pl.c_h = 0.0f;
+    float chi = 0.0f, eps = 0.0f;
     unsigned int idle = 0, rounds = 0;
     unsigned long long idle_ns = 0, seen = 0;
     unsigned int ticket = kNoItem;   // lane 0: long-queue entry taken, not yet pushed
     unsigned long long pend_lo = 0, pend_hi = 0;   // lane 0: child indices taken, not handed out
-    bool more_med = cold_med != 0u;   // lane 0
     bool timed_out = false;
     while (true) {
-        // ---- 1. (sampler modes) a long plan, stepped by the whole warp.  Lane 0
-        // takes a ticket with one atomic add when the queue looks non-empty; a
-        // ticket past the tail is kept until its entry is pushed (void if the
-        // step ends first).
+        // ---- 1. a long plan, stepped by the whole warp.  Lane 0 takes a ticket
+        // with one atomic add when the queue looks non-empty; a ticket past the
+        // tail is kept until its entry is pushed (void if the step ends first).
         {
             int got = 0;
             unsigned int q = 0;
@@ -2554,150 +2508,188 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
                 it.s = __shfl_sync(kAll, it.s, 0);
                 it.t_rem.hi = __shfl_sync(kAll, it.t_rem.hi, 0);
                 it.t_rem.lo = __shfl_sync(kAll, it.t_rem.lo, 0);
-                const uint32_t k0 = (uint32_t)SP.seed, k1 = (uint32_t)(SP.seed >> 32);
-                warp_item<kSampler>(P, S, SP, ctl, sm, dyn_smem, it, step, k0,
-                                                        k1, stats, stats.cand, true);
+                warp_item<kSampler>(P, S, SP, ctl, sm, dyn_smem, it, step, k0, k1, stats, stats.cand,
+                                    true);
                 if (lane == 0) ++done;
                 idle = 0;
                 idle_ns = 0;
                 continue;
             }
         }
-        // ---- 2. rows for the idle lanes: the queue's long plans, children, the
-        // queue's medium plans.  Lane 0 takes child indices with one atomic add
-        // into a pending range and hands a lane only an index whose row is
-        // reserved already (the rest stay pending; indices never reserved are
-        // void when the step ends); queue entries come the same way, an index
-        // past their count is dropped.  A warp takes a share of what is on
-        // offer (a round's time grows with the particles it steps, and other
-        // warps are idle when there is little), and a busy warp looks only when
-        // kTailClaim of its lanes are free, and not in every round.
+        // ---- 2. rows for the idle lanes: children first, then the medium plans.
+        // Lane 0 takes child indices with one atomic add into a pending range
+        // and hands a lane only an index whose row is reserved already (the
+        // rest stay pending; indices never reserved are void when the step
+        // ends); medium plans come the same way, an index past their count is
+        // dropped.
         {
-            const unsigned int free_lanes = __ballot_sync(kAll, !L.active && !waiting);
-            const bool look = free_lanes == kAll ||
-                              (__popc(free_lanes) >= kTailClaim && rounds % kTailRounds == 0u);
-            if (look || (free_lanes && __any_sync(kAll, lane == 0 && pend_lo < pend_hi))) {
-                const unsigned int want = (unsigned int)__popc(free_lanes);
+            const unsigned int free_lanes = __ballot_sync(kAll, !active && !waiting);
+            if (free_lanes) {
+                const int want = __popc(free_lanes);
                 unsigned long long base_c = 0;
                 unsigned int base_m = 0;
                 int got_c = 0, got_m = 0;
                 if (lane == 0) {
-                    // the control words are read at once, one round trip
-                    const unsigned int h_med =
-                        more_med ? *reinterpret_cast<volatile unsigned int*>(&ctl->queue.med_head) : 0u;
-                    const unsigned long long ch =
-                        *reinterpret_cast<volatile unsigned long long*>(&ctl->child_head);
-                    const unsigned long long stored = cascade ? stored_rows(P) : n0;
-                    more_med = more_med && h_med < cold_med;
-                    if (pend_lo == pend_hi && ch < stored) {
-                        const unsigned long long k =
-                            min((unsigned long long)want,
-                                (stored - ch + kTailSpread - 1) / kTailSpread);
-                        pend_lo = atomicAdd(&ctl->child_head, k);
-                        pend_hi = pend_lo + k;
+                    if (cascade) {
+                        const unsigned long long stored = stored_rows(P);
+                        if (pend_lo == pend_hi) {
+                            const unsigned long long ch =
+                                *reinterpret_cast<volatile unsigned long long*>(&ctl->child_head);
+                            if (ch < stored) {
+                                const unsigned long long k =
+                                    min((unsigned long long)want, stored - ch);
+                                pend_lo = atomicAdd(&ctl->child_head, k);
+                                pend_hi = pend_lo + k;
+                            }
+                        }
+                        if (pend_lo < pend_hi && pend_lo < stored) {
+                            got_c = (int)min((unsigned long long)want, min(pend_hi, stored) - pend_lo);
+                            base_c = pend_lo;
+                            pend_lo += (unsigned long long)got_c;
+                        }
                     }
-                    if (pend_lo < pend_hi && pend_lo < stored) {
-                        got_c = (int)min((unsigned long long)want, min(pend_hi, stored) - pend_lo);
-                        base_c = pend_lo;
-                        pend_lo += (unsigned long long)got_c;
-                    }
-                    if (got_c == 0 && more_med) {
-                        const unsigned int k = min(want, share_med);
+                    if (got_c < want &&
+                        *reinterpret_cast<volatile unsigned int*>(&ctl->queue.med_head) < cold_med) {
+                        const unsigned int k = (unsigned int)(want - got_c);
                         base_m = atomicAdd(&ctl->queue.med_head, k);
                         got_m = base_m < cold_med ? (int)min(k, cold_med - base_m) : 0;
                     }
                 }
-                // one kind per claim
-                const int got = __shfl_sync(kAll, got_c + got_m, 0);
-                if (got) {
-                    const bool kids = __shfl_sync(kAll, got_c != 0 ? 1 : 0, 0) != 0;
-                    const uint32_t base = __shfl_sync(kAll, got_c ? (uint32_t)base_c : base_m, 0);
+                got_c = __shfl_sync(kAll, got_c, 0);
+                got_m = __shfl_sync(kAll, got_m, 0);
+                if (got_c + got_m) {
+                    base_c = __shfl_sync(kAll, base_c, 0);
+                    base_m = __shfl_sync(kAll, base_m, 0);
                     const int rank = __popc(free_lanes & ((1u << lane) - 1u));
-                    if (!L.active && !waiting && rank < got) {
-                        // a child's row, or a queue entry's row, sub-step and time
-                        child = kids;
-                        row = base + (uint32_t)rank;
+                    if (!active && !waiting && rank < got_c + got_m) {
+                        // a child's row, or a medium plan's row, sub-step and time
+                        child = rank < got_c;
                         waiting = true;
-                        if (!child) {
-                            const HotItem it = S.hot[S.hot_cap - 1 - (long long)row];
-                            row = it.idx;
-                            L.s0 = it.s;
-                            L.t_rem = it.t_rem;
+                        s = 0;
+                        if (child) {
+                            i = (uint32_t)base_c + (uint32_t)rank;
+                        } else {
+                            const HotItem it =
+                                S.hot[S.hot_cap - 1 - ((long long)base_m + rank - got_c)];
+                            i = it.idx;
+                            s = it.s;
+                            t_rem = it.t_rem;
                         }
                     }
                 }
             }
         }
         // ---- 3. lanes holding a row: load it once it is written
+        bool plan = false;   // a new row or an event in the last round
         if (waiting) {
-            const uint8_t ty = *reinterpret_cast<volatile uint8_t*>(P.type + row);
+            const uint8_t ty = *reinterpret_cast<volatile uint8_t*>(P.type + i);
             if (!child || ty != kNotReady) {
                 if (child) {
                     __threadfence();
-                    L.t_rem = S.t_rem[row];
-                    L.s0 = 0;
+                    t_rem = S.t_rem[i];
                 }
                 waiting = false;
-                const bool photon = ty == QED_PHOTON;
-                if (ty <= QED_PHOTON && process_enabled(SP, photon) && time_positive(L.t_rem))
-                    lane_take(P, SP, L, B, fld, step, row, photon, L.s0, L.t_rem);
-                else
+                photon = ty == QED_PHOTON;
+                if (ty <= QED_PHOTON && process_enabled(SP, photon) && time_positive(t_rem)) {
+                    id = P.id[i];
+                    B.key[lane] = draw_key(id, step, SP.draw_keys);
+                    st = PState{P.px[i], P.py[i], P.pz[i]};
+                    fld[0][threadIdx.x] = P.Ex[i];
+                    fld[1][threadIdx.x] = P.Ey[i];
+                    fld[2][threadIdx.x] = P.Ez[i];
+                    fld[3][threadIdx.x] = P.Bx[i];
+                    fld[4][threadIdx.x] = P.By[i];
+                    fld[5][threadIdx.x] = P.Bz[i];
+                    changed = removed = false;
+                    plan = true;
+                } else {
                     ++done;
+                }
             }
         }
-        // ---- 4. the events of the last round; they and new rows plan together
-        const PendingChildren kids = events_begin(P, SP, L, stats);
-        const ftime t_kids = L.t_rem;
-        const float chi_kids = L.chi;
-        bool fin = kids.mine && !L.need_plan;
-        bool hand_over = false;
-        if (L.need_plan) {
-            fin = lane_plan<false>(SP, sm, L, fld, ctl);
-            if (!fin) {
-                stats.max_N = max(stats.max_N, L.pl.N);
-                hand_over = (!L.photon && sampler_bin_ok(SP, L.chi)) ||
-                            (kSampler == 2 && L.photon && L.pl.N >= SP.hot_min &&
-                             pair_sampler_ok(SP, L.chi, L.pl.T));
-                if (!hand_over) fin = lane_count_plan(L, stats);
+        bool fin = false;
+        auto plan_lane = [&]() {
+            const Fields F = lane_fields(fld);
+            pl = plan_particle(SP, sm.sqz_e, sm.sqz_p, photon, st.px, st.py, st.pz, F.Ex, F.Ey, F.Ez,
+                               F.Bx, F.By, F.Bz, t_rem, &chi, &eps);
+            k_done = 0;
+            active = eps > 0.0f;
+            fin = !active;
+            if (active) {
+                stats.max_N = max(stats.max_N, pl.N);
+                if (pl.N >= SP.long_min || (!photon && sampler_bin_ok(SP, chi)) ||
+                    (kSampler == 2 && photon && pl.N >= SP.hot_min &&
+                     pair_sampler_ok(SP, chi, pl.T))) {
+                    // to the warp mode, which plans again; its state goes with the row
+                    if (changed) {
+                        P.px[i] = st.px;
+                        P.py[i] = st.py;
+                        P.pz[i] = st.pz;
+                    }
+                    push_long(S, ctl, cold_long, i, s, t_rem);
+                    active = false;
+                } else {
+                    stats.plans++;
+                    stats.guard += pl.guard ? 1 : 0;
+                    if (pl.T == 0u) {   // no candidates: the plan passes without an event
+                        stats.substeps += pl.N;
+                        fin = true;
+                    }
+                }
             }
-        }
-        const long long j_kids =
-            events_end(P, S, SP, ctl, L, kids, t_kids, chi_kids, fld, step, kDeferred);
-        if (hand_over) {   // the warp mode plans again; the particle's state goes with the row
-            lane_finish(P, L);
-            push_long(S, ctl, cold_long, L.i, L.s0, L.t_rem);
-        } else if (fin) {
-            lane_finish(P, L);
+        };
+        auto finish_lane = [&]() {
+            if (removed) {
+                P.type[i] = QED_REMOVED;
+            } else if (changed) {
+                P.px[i] = st.px;
+                P.py[i] = st.py;
+                P.pz[i] = st.pz;
+            }
+            active = false;
             ++done;
-        }
-        const unsigned int on = __ballot_sync(kAll, L.active);
+        };
+        if (plan) plan_lane();
+        if (fin) finish_lane();
+        fin = false;
+        const unsigned int on = __ballot_sync(kAll, active);
         if (on) {
-            // ---- 5. the lists that have run out are drawn, the next candidates tested
+            // ---- 4. one round of warp-shared draws for the active lanes
             idle = 0;
             idle_ns = 0;
             if (++rounds == kBeatRounds) {
                 rounds = 0;
                 if (lane == 0) atomicAdd(&ctl->beat, 1ull);
             }
-            list_draw<kHotIlp>(B, L, y1, SP.draw_keys);
-            if (list_test(sm, B, L, y1, SP.draw_keys, stats.cand)) {
-                stats.substeps += L.pl.N;
-                lane_finish(P, L);
-                ++done;
+            const uint32_t n_win = active ? min(kWindow, pl.N - k_done) : 0u;
+            const uint32_t s_end = s + n_win;
+            draw_round(sm, B, active, s, s_end, pl.T, pl.b, pl.c_h, photon, y1, SP.draw_keys, stats.cand);
+            if (active) {
+                const uint32_t s_ev = B.facc[lane];
+                if (s_ev == kNoEvent) {
+                    stats.substeps += n_win;
+                    s = s_end;
+                    k_done += n_win;
+                    fin = k_done == pl.N;   // the plan ran out without an event
+                } else {
+                    const uint32_t k = k_done + (s_ev - s);
+                    stats.substeps += s_ev - s + 1u;
+                    const float x = draw_x(B.key[lane], y1, s_ev, SP.draw_keys);
+                    const ftime t_after = (k + 1u == pl.N) ? ftime{0.0f, 0.0f}
+                                                           : time_sub_mul(t_rem, k + 1u, pl.h);
+                    removed = apply_event(P, S, SP, ctl, i, id, photon, x, eps, chi, step, s_ev,
+                                          t_after, st, stats, false, lane_fields(fld), true);
+                    changed = true;
+                    s = s_ev + 1u;
+                    t_rem = t_after;
+                    fin = removed || !time_positive(t_rem);
+                    if (!fin) plan_lane();
+                }
+                if (fin) finish_lane();
             }
+            __syncwarp();   // the draw buffer is reused by the next round
         }
-        // the children's rows have been written since the last fence: publish
-        // them (after the draws, so that the fence finds the stores done)
-        if (__any_sync(kAll, kids.mine)) {
-            __threadfence();
-            if (j_kids >= 0) {
-                // kids.mine: the lane's photon flag is still the parent's
-                *reinterpret_cast<volatile uint8_t*>(P.type + j_kids) = child_type(L.photon, 0);
-                if (L.photon)
-                    *reinterpret_cast<volatile uint8_t*>(P.type + j_kids + 1) = child_type(true, 1);
-            }
-        }
-        // ---- 6. nothing to draw: wait for work, or finish
+        // ---- 5. nothing to draw: wait for work, or finish
         if (!on) {
             // lanes waiting for a row still being written hold the warp
             const bool hold = __any_sync(kAll, waiting);
@@ -2738,9 +2730,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_step(DevParticles P, StepPa
                 break;
             }
             __nanosleep(nap);
-            continue;
         }
-        __syncwarp();   // the list buffer is reused by the next round
     }
     if (timed_out && lane == 0) atomicExch(&ctl->status, (int)QED_ERR_TIMEOUT);
     const unsigned long long sum = warp_sum(done);
@@ -3140,9 +3130,10 @@ cudaError_t allow_smem() {
     }
     return cudaSuccess;
 }
-const void* step_kernel(int mode, bool cells = false) {
-    return mode == 2 ? (const void*)k_step<2>
-                     : mode ? (const void*)k_step<1>
+// small (sampler modes): the form for tails below kTailSmall rows.
+const void* step_kernel(int mode, bool cells = false, bool small = false) {
+    return mode == 2 ? (small ? (const void*)k_step<2, 1> : (const void*)k_step<2, 2>)
+           : mode    ? (small ? (const void*)k_step<1, 1> : (const void*)k_step<1, 2>)
                             : cells ? (const void*)k_stream<true> : (const void*)k_stream<false>;
 }
 size_t step_smem(int mode) { return mode ? kNetSmemBytes : sizeof(HotSmem); }
@@ -3581,6 +3572,7 @@ StepParams make_params(const qed_config& c, uint64_t step) {
     P.step_base = nullptr;
     P.hot_min = kHotMinDefault;
     P.front_min = front_min(kLongMinDefault, 0);
+    P.long_min = kLongMinDefault;
     P.sampler = 0;
     P.net_rows = 0;
     P.net_bins = 0;
@@ -3823,8 +3815,9 @@ qed_status qed_init(qed_ctx** out, const qed_config* cfg, void* stream) {
         ctx->hot_blocks = ctx->hot_blocks_max = ctx->sms * (per_sm > 0 ? per_sm : 1);
         per_sm = 0;
         for (int m = 1; m <= 2; ++m)
-            cudaFuncSetAttribute(step_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kNetSmemBytes);
+            for (bool small : {false, true})
+                cudaFuncSetAttribute(step_kernel(m, false, small),
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNetSmemBytes);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hot_net, kLaneThreads,
                                                       kNetSmemBytes);
         ctx->net_blocks = ctx->sms * (per_sm > 0 ? per_sm : 1);
@@ -3836,7 +3829,7 @@ qed_status qed_init(qed_ctx** out, const qed_config* cfg, void* stream) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_plan, kColdThreads, 0);
         ctx->plan_blocks = ctx->sms * (per_sm > 0 ? per_sm : 1);
         per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<1>, kLaneThreads,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<1, 2>, kLaneThreads,
                                                       kNetSmemBytes);
         ctx->step_net_blocks = ctx->sms * (per_sm > 0 ? per_sm : 1);
         per_sm = 0;
@@ -4027,6 +4020,7 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
     StepParams SP = make_params(ctx->cfg, step_index);
     SP.hot_min = ctx->hot_min;
     SP.front_min = front_min(ctx->long_min, ctx->cfg.sampler_mode);
+    SP.long_min = ctx->long_min;
     SP.wait_ns = ctx->wait_ns;
     st = sampler_params(ctx, &SP);
     if (st != QED_OK) return st;
@@ -4108,6 +4102,10 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
         Scratch sc = S;
         DevCtl* c = ctx->d_ctl;
         void* a[] = {&d, &sp, &sc, &c};
+        if (SP.sampler)
+            QED_CUDA(ctx, cudaLaunchKernel(step_kernel(SP.sampler, false, true), dim3(ctx->sms),
+                                           dim3(kLaneThreads), a, step_smem(SP.sampler),
+                                           ctx->stream));
         QED_CUDA(ctx, cudaLaunchKernel(step_kernel(SP.sampler, SP.N_cell != nullptr),
                                        dim3(SP.sampler ? ctx->step_net_blocks : ctx->step_blocks),
                                        dim3(kLaneThreads), a, step_smem(SP.sampler),
@@ -4442,6 +4440,13 @@ qed_status add_tail_nodes(qed_ctx* ctx, cudaGraph_t g, cudaGraphNode_t dep, cons
     }
     if (st == QED_OK) {
         void* a[] = {&D, &SP, &S, &ctl};
+        if (SP.sampler) {
+            cudaGraphNode_t small;
+            st = add_kernel(ctx, g, &small, step_kernel(SP.sampler, false, true), dim3(ctx->sms),
+                            dim3(kLaneThreads), a, &tc, 1, step_smem(SP.sampler));
+            if (st != QED_OK) return st;
+            tc = small;
+        }
         st = add_kernel(ctx, g, &ts, step_kernel(SP.sampler, SP.N_cell != nullptr),
                         dim3(SP.sampler ? ctx->step_net_blocks : ctx->step_blocks),
                         dim3(kLaneThreads), a, &tc, 1, step_smem(SP.sampler));
@@ -4512,6 +4517,7 @@ qed_status qed_graph_capture(qed_ctx* ctx, const qed_particles* p, uint64_t firs
         SP.step_base = step_base;
         SP.hot_min = ctx->hot_min;
         SP.front_min = front_min(ctx->long_min, ctx->cfg.sampler_mode);
+    SP.long_min = ctx->long_min;
         SP.wait_ns = ctx->wait_ns;
         st = sampler_params(ctx, &SP);
         if (st != QED_OK) break;
@@ -4620,7 +4626,7 @@ static qed_status run_step_graph(qed_ctx* ctx, const DevParticles& Din, StepPara
     { uint64_t b; memcpy(&b, &SPin.dt, 8); put(b); }
     putf(SPin.K); putf(SPin.inv_Es); putf(SPin.p_max); putf(SPin.inv_p_max); putf(SPin.pair_coeff);
     putf(SPin.t_step.hi); putf(SPin.t_step.lo);
-    put(SPin.hot_min); put(SPin.front_min); put((uint64_t)SPin.sampler); put((uint64_t)SPin.net_rows);
+    put(SPin.hot_min); put(SPin.front_min); put(SPin.long_min); put((uint64_t)SPin.sampler); put((uint64_t)SPin.net_rows);
     put(SPin.net_bins); putp(SPin.net_w); putp(SPin.net_wtot); put(SPin.process_mask);
     put(SPin.pnet_bins); putp(SPin.pnet_w); putp(SPin.pnet_wtot);
     put((uint64_t)SPin.recoil); put((uint64_t)SPin.cascade); put(SPin.wait_ns);

@@ -489,6 +489,7 @@ struct StepParams {
     const uint32_t* step_base;  // graph runs: device step base added to `step`
     uint32_t hot_min;           // plans with at least this many sub-steps go to the hot pass
     uint32_t front_min;         // ... and with at least this many to the front of its queue
+    uint32_t long_min;          // sampler modes' tail pass: ... to a whole warp
     int sampler;                // learned sampler on (e+- in usable bins)
     int net_rows;               // rows of the total-probability table
     unsigned long long net_bins;  // usable bins (64, uniform in log10 chi over [-2, 2))
