@@ -2950,6 +2950,10 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
                 starved = (dry & 1) != 0;
                 pending = (dry & 2) != 0;
                 finish = __shfl_sync(kAll, over, 0) != 0u;
+                if (got_l + got_m) {   // the wait for an entry to be written is a new one
+                    idle = 0;
+                    idle_ns = 0;
+                }
                 const int rank = __popc(free_lanes & ((1u << lane) - 1u));
                 if (!L.active && !waiting && rank < got_l + got_m) {
                     waiting = true;
@@ -3053,7 +3057,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
         const unsigned int nap = hold ? 64u : 256u << min(idle, kTailNap);
         ++idle;
         idle_ns += nap;
-        if (idle_ns > SP.wait_ns && !hold) {
+        if (idle_ns > SP.wait_ns) {
             unsigned long long progress = 0;
             if (lane == 0)
                 progress = *reinterpret_cast<volatile unsigned long long*>(&ctl->finished) +
