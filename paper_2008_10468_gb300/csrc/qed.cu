@@ -726,10 +726,13 @@ struct __align__(16) EventBuf {   // one per warp, used as a ring
     uint64_t id[kEventBuf];
     ftime t_after[kEventBuf];
     uint32_t i[kEventBuf], s[kEventBuf];
-    float x[kEventBuf];   // negative: the parent is a photon
+    float x[kEventBuf];   // sign bit set (also that of 0): the parent is a photon
     float px[kEventBuf], py[kEventBuf], pz[kEventBuf], chi[kEventBuf];
     float f[6][kEventBuf];   // E, B
 };
+__device__ __forceinline__ bool noted_photon(const EventBuf& E, unsigned int q) {
+    return __float_as_int(E.x[q]) < 0;
+}
 __device__ __forceinline__ void note_event(EventBuf& E, unsigned int q, uint32_t i, uint64_t id,
                                            bool photon, float x, float chi, uint32_t s,
                                            ftime t_after, const PState& st, const Fields& F) {
@@ -760,7 +763,7 @@ __device__ __forceinline__ void events_flush(const DevParticles& P, const Scratc
     __syncwarp();
     if (lane < k) {
         const unsigned int q = (head + lane) % kEventBuf;
-        const bool photon = E.x[q] < 0.0f;
+        const bool photon = noted_photon(E, q);
         const uint32_t i = E.i[q];
         const long long j = reserve_rows(P, ctl, photon ? 2 : 1, true);
         write_children(P, S, SP, i, j, E.id[q], photon, fabsf(E.x[q]), E.chi[q], step, E.s[q],
@@ -2790,7 +2793,7 @@ __device__ __forceinline__ StreamChildren stream_begin(const DevParticles& P, co
     __syncwarp();
     const unsigned int q = (head + lane) % kEventBuf;
     c.mine = lane < c.n;
-    if (c.mine) c.photon = E.x[q] < 0.0f;
+    c.photon = c.mine && noted_photon(E, q);
     const unsigned int m1 = __ballot_sync(kAll, c.mine && !c.photon);
     const unsigned int m2 = __ballot_sync(kAll, c.photon);
     c.off_r = __popc(m1 & below) + 2 * __popc(m2 & below);
