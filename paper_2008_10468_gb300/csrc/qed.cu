@@ -3504,6 +3504,7 @@ struct qed_ctx {
     float* d_batch;            // training inputs (2 per sample), targets and weights,
                                // or the two-kernel step's arrays (train_floats)
     size_t batch_cap;          // floats
+    bool train_three;          // the large-batch kernels for every batch (tests compare the two)
     float* d_loss;
     // multi-step graph
     cudaGraph_t graph;
@@ -4721,7 +4722,9 @@ cudaError_t launch_chained(void (*f)(P...), int blocks, int threads, size_t smem
 
 // Batches whose tiles have a block of k_mlp_grad each are trained by k_train_fwd
 // and k_train_update; larger ones fill the GPU with k_mlp_grad.
-bool two_kernel_step(const qed_ctx* ctx, int ntiles) { return ntiles <= ctx->sms * 2; }
+bool two_kernel_step(const qed_ctx* ctx, int ntiles) {
+    return ntiles <= ctx->sms * 2 && !ctx->train_three;
+}
 
 qed_status sampler_alloc(qed_ctx* ctx, int max_batch) {
     if (!cur_net(ctx).d_theta) {
@@ -5018,6 +5021,14 @@ qed_status qed_sampler_train(qed_ctx* ctx, uint64_t seed, int64_t samples, int b
                                       ctx->stream));
     }
     QED_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    return QED_OK;
+}
+
+// Not part of the interface (not in qed.h): lets a test train one batch size by
+// the two-kernel step and by the kernels of large batches.
+qed_status qed_test_train_three(qed_ctx* ctx, int on) {
+    if (!ctx) return QED_ERR_ARG;
+    ctx->train_three = on != 0;
     return QED_OK;
 }
 
