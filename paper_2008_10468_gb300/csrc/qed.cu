@@ -103,11 +103,12 @@ struct DevCtl {
     long long n_init;               // rows at the start of the step (the rest are children)
     unsigned long long beat;        // persistent passes: progress of long chains, so that
                                     // idle warps tell a long chain from a stalled step
-    // the queue's state, in a line of its own that idle warps poll with one load
+    // the queue's state, in a line of its own that idle warps poll (k_stream: with one
+    // load, and the store's count with another)
     struct alignas(128) Queue {
         unsigned int hot_head, med_head;   // entries taken
-        unsigned int step_tail;            // entries queued by the persistent kernel, stored
-                                           // after the thread pass's hot_tail entries
+        unsigned int step_tail;            // k_step: entries queued by it, stored after the
+                                           // thread pass's hot_tail entries
         unsigned int over;                 // every unit of the step is complete
     } queue;
 };
@@ -2769,19 +2770,16 @@ constexpr unsigned int kStreamSpread = 16;   // warps that share the children on
 constexpr int kStreamLanes = 16;
 constexpr unsigned int kStreamMany = 8;
 
-// A warp's children.  Their rows are reserved at the start of a round; after its
-// plans they are written and the ones with time left take queue entries, which
-// are published after its draws, so that the chains that go on do not wait for
-// the two atomics and the fence (65536 rows: 0.46 instead of 0.65 ms).  Only a
-// row that exists takes an entry: parents go on emitting into a full store, and
-// the queue has room for the store's rows, not for all that is wanted.
+// A warp's children.  Their rows are reserved at the start of a round, written
+// after its plans and published after its draws, so that the chains that go on do
+// not wait for the atomic and the fence (65536 rows: 0.46 instead of 0.65 ms).  A
+// row is its own queue entry: the queue has room for the store's rows, and a child
+// that does not fit (parents go on emitting into a full store) has none.
 struct StreamChildren {
     bool mine = false, photon = false;   // this lane holds an event; its parent
-    int nq = 0, off_r = 0, off_q = 0;    // entries (0 or the children); offsets of rows, entries
-    unsigned long long base_r = 0;       // lane 0
-    unsigned int base_q = 0;             // lane 0
+    int offset = 0;                      // its children's rows, from the warp's first
+    unsigned long long base = 0;         // lane 0
     unsigned int n = 0;                  // events taken from the ring
-    uint32_t idx = kNoItem;              // written: the first child's row
 };
 __device__ __forceinline__ StreamChildren stream_begin(const DevParticles& P, const StepParams& SP,
                                                      DevCtl* ctl, const EventBuf& E, unsigned int n,
@@ -2796,44 +2794,36 @@ __device__ __forceinline__ StreamChildren stream_begin(const DevParticles& P, co
     c.photon = c.mine && noted_photon(E, q);
     const unsigned int m1 = __ballot_sync(kAll, c.mine && !c.photon);
     const unsigned int m2 = __ballot_sync(kAll, c.photon);
-    c.off_r = __popc(m1 & below) + 2 * __popc(m2 & below);
+    c.offset = __popc(m1 & below) + 2 * __popc(m2 & below);
     if (lane == 0)
-        c.base_r = atomicAdd(reinterpret_cast<unsigned long long*>(P.count),
+        c.base = atomicAdd(reinterpret_cast<unsigned long long*>(P.count),
                              (unsigned long long)(__popc(m1) + 2 * __popc(m2)));
     return c;
 }
 __device__ __forceinline__ void stream_write(const DevParticles& P, const Scratch& S,
                                             const StepParams& SP, DevCtl* ctl, const EventBuf& E,
                                             unsigned int head, StreamChildren& c, uint32_t step) {
-    constexpr unsigned int kAll = 0xffffffffu;
-    const unsigned int lane = threadIdx.x & 31, below = (1u << lane) - 1u;
-    const unsigned long long base_r = __shfl_sync(kAll, c.base_r, 0);
+    c.base = __shfl_sync(0xffffffffu, c.base, 0) + (unsigned long long)c.offset;   // this lane's
     if (c.mine) {
-        const unsigned int q = (head + lane) % kEventBuf;
-        const int n = c.photon ? 2 : 1;
-        const long long j = check_rows(P, ctl, (long long)base_r + c.off_r, n);
+        const unsigned int q = (head + (threadIdx.x & 31)) % kEventBuf;
+        const long long j = check_rows(P, ctl, (long long)c.base, c.photon ? 2 : 1);
         write_children(P, S, SP, E.i[q], j, E.id[q], c.photon, fabsf(E.x[q]), E.chi[q], step,
                        E.s[q], E.t_after[q], PState{E.px[q], E.py[q], E.pz[q]},
                        Fields{E.f[0][q], E.f[1][q], E.f[2][q], E.f[3][q], E.f[4][q], E.f[5][q]},
                        kPlain);
-        c.idx = (uint32_t)j;
-        c.nq = j >= 0 && time_positive(E.t_after[q]) ? n : 0;   // a cascade has both processes on
     }
-    const unsigned int q1 = __ballot_sync(kAll, c.nq == 1), q2 = __ballot_sync(kAll, c.nq == 2);
-    c.off_q = __popc(q1 & below) + 2 * __popc(q2 & below);
-    if (lane == 0 && (q1 | q2))
-        c.base_q = atomicAdd(&ctl->queue.step_tail, (unsigned int)(__popc(q1) + 2 * __popc(q2)));
     __syncwarp();   // the ring's entries are reused
 }
-// All lanes of the warp.  A child's entry is its row; the rest of the entry (the
-// first sub-step, the time left) is the row's.
-__device__ __forceinline__ void stream_publish(const Scratch& S, unsigned int cold_long,
+// entries: where the entry of row 0 would be.
+__device__ __forceinline__ void stream_publish(const DevParticles& P, HotItem* entries,
                                                const StreamChildren& c) {
-    const unsigned int entry = cold_long + __shfl_sync(0xffffffffu, c.base_q, 0) + (unsigned int)c.off_q;
-    if (c.nq) {
-        __threadfence();   // the children's rows before the indices
-        *reinterpret_cast<volatile uint32_t*>(&S.hot[entry].idx) = c.idx;
-        if (c.nq == 2) *reinterpret_cast<volatile uint32_t*>(&S.hot[entry + 1].idx) = c.idx + 1u;
+    if (c.mine) {
+        __threadfence();   // the children's rows before their entries
+        const long long r = (long long)c.base;
+        if (r < P.capacity)
+            *reinterpret_cast<volatile uint32_t*>(&entries[r].idx) = (uint32_t)r;
+        if (c.photon && r + 1 < P.capacity)
+            *reinterpret_cast<volatile uint32_t*>(&entries[r + 1].idx) = (uint32_t)r + 1u;
     }
 }
 
@@ -2875,9 +2865,11 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
     unsigned int n_ev = 0, ev_head = 0;   // events whose children are not written yet
     const uint32_t y1 = draw_y1(step, SP.draw_keys);
     const unsigned int nwarps = blocks * (kLaneThreads / 32);
-    // entries in the order they are taken: the thread pass's long plans, its
-    // children (by their rows, nothing in the array), the children queued here
+    // entries in the order they are taken: the thread pass's long plans, then the
+    // rows from n0 on: its children (nothing in the array), the children of this
+    // kernel (their entries in the array follow the long plans')
     const unsigned int first_new = cold_long + cold_kids;
+    HotItem* const entries = S.hot + (long long)cold_long - n1;
     const unsigned int share_long = max(1u, min(32u, (cold_long + nwarps - 1u) / nwarps));
     const unsigned int share_med = max(1u, min(32u, (cold_med + nwarps - 1u) / nwarps));
     Stats stats;                 // per lane
@@ -2911,7 +2903,8 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
                 unsigned int over = 0;
                 if (lane == 0) {
                     const uint4 qs = queue_state(ctl);
-                    const unsigned int h_long = qs.x, h_med = qs.y, tail = first_new + qs.z;
+                    const unsigned int h_long = qs.x, h_med = qs.y,
+                                       tail = cold_long + (unsigned int)(stored_rows(P) - n0);
                     over = qs.w;
                     more_med = more_med && h_med < cold_med;
                     const unsigned int left = (h_long < tail ? tail - h_long : 0u) +
@@ -2981,11 +2974,13 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
                 const uint8_t type = P.type[i];
                 const uint32_t s = child ? 0u : e->s;
                 const ftime t = child ? S.t_rem[i] : e->t_rem;
-                // not so for some of the thread pass's children only
-                if (type <= QED_PHOTON && time_positive(t))
-                    lane_take(P, SP, L, B, fld, step, i, type == QED_PHOTON, s, t);
-                else
+                // the row's loads do not wait for its type and time
+                lane_take(P, SP, L, B, fld, step, i, type == QED_PHOTON, s, t);
+                if (type > QED_PHOTON || !time_positive(t)) {
+                    // a child at the end of the step, or one that did not fit
+                    L.active = L.need_plan = false;
                     ++done;
+                }
             }
         }
         // ---- 3. the events of the last round; they and new rows plan together
@@ -3028,11 +3023,11 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
                 lane_finish(P, L);
                 ++done;
             }
-            if (flush) stream_publish(S, cold_long, kids);
+            if (flush) stream_publish(P, entries, kids);
             __syncwarp();   // the list buffer is reused by the next round
             continue;
         }
-        if (flush) stream_publish(S, cold_long, kids);
+        if (flush) stream_publish(P, entries, kids);
         // ---- 5. nothing to draw: wait for work, or finish.  The warp that
         // completes the last unit sees as many units complete as are known, and
         // says so in the word that idle warps poll.
@@ -3046,8 +3041,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
                 if (sum) {
                     __threadfence();   // this warp's entries before its completions
                     const unsigned long long f = sum + atomicAdd(&ctl->finished, sum);
-                    const uint4 qs = queue_state(ctl);
-                    if (f == units0 + qs.z)
+                    if (f == units0 + (stored_rows(P) - n1))
                         *reinterpret_cast<volatile unsigned int*>(&ctl->queue.over) = 1u;
                     again = 1;
                 }
@@ -3064,7 +3058,7 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
             unsigned long long progress = 0;
             if (lane == 0)
                 progress = *reinterpret_cast<volatile unsigned long long*>(&ctl->finished) +
-                           queue_state(ctl).z +
+                           *reinterpret_cast<volatile unsigned long long*>(P.count) +
                            *reinterpret_cast<volatile unsigned long long*>(&ctl->beat);
             progress = __shfl_sync(kAll, progress, 0);
             if (progress != seen && nap <= SP.wait_ns) {
@@ -3224,7 +3218,8 @@ __global__ void k_push_begin(DevParticles P, DevCtl* ctl) {
 // (children that did not fit were dropped and the status says so) and rows
 // past it go back to removed; in every step the long-plan queue entries used
 // go back to "not written".
-__global__ void k_tail_end(DevParticles P, Scratch S, DevCtl* ctl) {
+// stream: k_stream's entries, one for each row from n1 on.
+__global__ void k_tail_end(DevParticles P, Scratch S, DevCtl* ctl, int stream) {
     const bool on = ctl->tail != 0;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -3238,8 +3233,8 @@ __global__ void k_tail_end(DevParticles P, Scratch S, DevCtl* ctl) {
             ctl->passes += 1;
         }
     }
-    const long long used =
-        min(max((long long)ctl->hot_hw, (long long)ctl->hot_tail + ctl->queue.step_tail), S.hot_cap);
+    const long long tail = stream && on ? c - ctl->n1 : (long long)ctl->queue.step_tail;
+    const long long used = min(max((long long)ctl->hot_hw, (long long)ctl->hot_tail + tail), S.hot_cap);
     for (long long q = t0; q < used; q += stride) S.hot[q].idx = kNoItem;
 }
 
@@ -3626,8 +3621,7 @@ qed_status ensure_scratch(qed_ctx* ctx, long long cap) {
     // queue: long plans (and k_stream's children) from the front, medium plans
     // from the back.  Every entry belongs to a row of the store and a row has at
     // most two entries per generation (in the tail pass a medium plan may come
-    // back as a long plan; k_stream: one, a child that did not fit has none), so
-    // 2 cap entries never let the ends meet.  Entries at the front start "not
+    // back as a long plan; k_stream: one), so 2 cap entries never let the ends meet.  Entries at the front start "not
     // written" (row index all ones) and each step resets the ones it used.
     QED_CUDA(ctx, cudaMalloc(&ctx->d_hot, sizeof(HotItem) * 2 * cap));
     QED_CUDA(ctx, cudaMemset(ctx->d_hot, 0xFF, sizeof(HotItem) * 2 * cap));
@@ -4121,7 +4115,7 @@ static qed_status plain_step(qed_ctx* ctx, const qed_particles* p, uint64_t step
     }
     {
         LaunchScope ls(ctx, QED_KERNEL_CONTROL);
-        k_tail_end<<<ctx->sms * 8, 256, 0, ctx->stream>>>(D, S, ctx->d_ctl);
+        k_tail_end<<<ctx->sms * 8, 256, 0, ctx->stream>>>(D, S, ctx->d_ctl, SP.sampler == 0);
     }
     QED_CUDA(ctx, cudaGetLastError());
     if (out) return qed_read_stats(ctx, out);
@@ -4178,7 +4172,7 @@ static qed_status push_step(qed_ctx* ctx, const qed_particles* p, uint64_t step_
         }
         {
             LaunchScope ls(ctx, QED_KERNEL_CONTROL);
-            k_tail_end<<<ctx->sms * 8, 256, 0, ctx->stream>>>(D, S, ctx->d_ctl);
+            k_tail_end<<<ctx->sms * 8, 256, 0, ctx->stream>>>(D, S, ctx->d_ctl, 0);
         }
         QED_CUDA(ctx, cudaGetLastError());
         if (out) return qed_read_stats(ctx, out);
@@ -4460,7 +4454,8 @@ qed_status add_tail_nodes(qed_ctx* ctx, cudaGraph_t g, cudaGraphNode_t dep, cons
                         dim3(kLaneThreads), a, &tc, 1, step_smem(SP.sampler));
     }
     if (st == QED_OK) {
-        void* a[] = {&D, &S, &ctl};
+        int stream = SP.sampler == 0;
+        void* a[] = {&D, &S, &ctl, &stream};
         st = add_kernel(ctx, g, &te, (const void*)k_tail_end, dim3(ctx->sms * 8), dim3(256), a,
                         &ts, 1);
     }
@@ -5455,7 +5450,7 @@ extern "C" qed_status qed_event_step_noalloc(const qed_config* cfg, const qed_pa
     k_tail_begin<<<whole ? 1 : nd.sms * 8, 256, 0, s>>>(D, S, ctl, whole);
     k_cold<false, false><<<nd.cold_blocks, kColdThreads, cold_smem(0), s>>>(D, SP, S, ctl);
     k_stream<false><<<nd.step_blocks, kLaneThreads, step_smem(0), s>>>(D, SP, S, ctl);
-    k_tail_end<<<nd.sms * 8, 256, 0, s>>>(D, S, ctl);
+    k_tail_end<<<nd.sms * 8, 256, 0, s>>>(D, S, ctl, 1);
     if (cudaGetLastError() != cudaSuccess) return noalloc_fail(dev, QED_ERR_CUDA);
     if (!out) return QED_OK;
     if (cudaMemcpyAsync(&h, ctl, sizeof h, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
