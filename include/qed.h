@@ -121,7 +121,9 @@ typedef struct {
     int32_t status;            /* qed_status of the step                        */
     int64_t required_capacity; /* rows needed when status == QED_ERR_CAPACITY   */
     int64_t count;             /* rows in use after the step                    */
-    int32_t passes;            /* cascade generations processed                 */
+    int32_t passes;            /* cascade generations processed one by one, a
+                                  persistent pass over the rest counting as one (1
+                                  for a step that is one such pass)             */
     int32_t tail;              /* 1: the step's last generations ran as the tail pass */
     uint64_t substeps_warp;    /* of `substeps`, those run by the hot pass and the tail pass's persistent kernel */
     uint64_t sampler_events;   /* emissions whose energy came from the learned sampler */
@@ -214,10 +216,13 @@ qed_status qed_plan_cells(qed_ctx* ctx, const qed_particles* p, int64_t n, const
  * after every event over the remaining time.  Children are appended at rows
  * count.. and, if cascade_in_step, processed in the same step: in one
  * persistent pass, or, with a learned sampler, generation by generation while
- * the generations are large and the rest in one tail pass (qed_set_tail).  If out != NULL the call synchronises the stream and fills *out; if NULL it
+ * the generations are large and the rest in one tail pass (qed_set_tail).  If
+ * out != NULL the call synchronises the stream and fills *out; if NULL it
  * returns without waiting (statistics readable with qed_read_stats).
  * Capacity: if the children do not fit, status QED_ERR_CAPACITY is returned
- * (in *out and as the return value when out != NULL) with the rows needed;
+ * (in *out and as the return value when out != NULL) with the rows asked for
+ * so far (children that did not fit ask for none of their own, so a cascade may
+ * need more);
  * the step is then incomplete (parents that emitted a dropped child have
  * recoiled) and the caller must restore its own copy of the store.
  * Errors: QED_ERR_ARG, QED_ERR_CUDA, QED_ERR_CAPACITY, QED_ERR_TIMEOUT. */
@@ -425,7 +430,7 @@ qed_status qed_set_launch(qed_ctx* ctx, uint32_t hot_min, uint32_t long_min,
 /* Tail pass of the cascade (Sec. 2: the events of one step form a cascade
  * whose generations shrink).  Without a learned sampler any tail_rows > 0 makes
  * the whole step one thread pass and one persistent pass that takes every child
- * as it is written (unless max_passes is below its default: then the
+ * as it is written (unless max_passes is below its default of 64: then the
  * generations are counted).  With one: once a generation has fewer than
  * tail_rows rows the generations stop: one thread pass over that generation, then one
  * persistent kernel takes its queue and every child appended after it as
@@ -510,8 +515,9 @@ qed_status qed_time_split(const float* t_hi, const float* t_lo, const uint32_t* 
  *
  * Same arguments and results as qed_event_step (no event log, no learned
  * sampler: cfg->sampler_mode must be 0), on `stream` (a cudaStream_t, NULL:
- * the legacy default stream); with cfg->cascade_in_step it synchronises that
- * stream after every cascade generation, and if out != NULL at the end.
+ * the legacy default stream); it synchronises that stream if out != NULL, and
+ * with cfg->cascade_in_step and max_passes below its default after every cascade
+ * generation.
  * The first call on a device looks up the array and the launch geometry with
  * that device current; later calls on the device reuse them.  The array is shared by every call
  * and keeps the contents of the last one: each step starts by resetting what

@@ -786,8 +786,11 @@ __device__ __forceinline__ void events_flush(const DevParticles& P, const Scratc
 // draws every remaining planned sub-step of the warp's rows, so that a warp
 // whose particles plan 1 to 30 sub-steps keeps its lanes busy; each particle
 // takes its earliest accepted sub-step, the decision of testing its
-// sub-steps in order and stopping at the first acceptance.  Lanes with an
-// event apply it, re-plan the remaining time and join the next round.
+// sub-steps in order and stopping at the first acceptance.
+// kLoop = false (no sampler): one round; an event is noted for its children, which
+// are written 32 at a time, and its parent goes on in the hot pass's queue.
+// kLoop = true (sampler modes): lanes with an event apply it, re-plan the
+// remaining time and join the next round.
 template <bool kCells, bool kLoop>
 __global__ void __launch_bounds__(kColdThreads, kColdMinBlocks) k_cold(DevParticles P, StepParams SP, Scratch S,
                                                        DevCtl* ctl) {
@@ -1738,9 +1741,9 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_samp(DevParticles P, StepPa
         }
         // while there is work for all, the block's warps go through the network
         // together: its instructions do not fit the caches next to the warps,
-        // and together they are fetched once for all (3.3 against 3.1 ms on 1e6
-        // uniform-field electrons).  The first warp without more work ends it
-        // for all.
+        // and together they are fetched once for all (1e6 uniform-field electrons:
+        // 3.1 ms, 3.3 with each warp by itself).  The first warp without more work
+        // ends it for all.
         if (in_step) in_step = __syncthreads_and(more) != 0;
         // the sub-steps to the next event
         bool ev = false;
@@ -2753,12 +2756,14 @@ __global__ void __launch_bounds__(kLaneThreads, kBlocks) k_step(DevParticles P, 
 // Launched generation by generation, every generation ends in its longest
 // chains with most of the GPU idle (11 of 16 warps resident on average) and
 // starts with a thread pass.  In one launch a step of 2^24 rows (1% in a strong
-// field, 1.0e9 sub-steps) takes 3.95 ms instead of 5.45, one of 2^20 rows with a
-// tenth in the field 2.05 instead of 3.68, and 4096 rows 0.28 instead of 0.35.
+// field, 1.0e9 sub-steps) takes 3.5 ms instead of 5.45, one of 2^20 rows with a
+// tenth in the field 1.87 instead of 3.68, and 4096 rows 0.25 instead of 0.35.
 // What bounds it is the issue rate of the warps' divergent parts (plans, tests)
-// and of the draws; children planned at birth by the warp that writes them cost
-// more than they saved, because the second copy of the plan's code did not fit
-// the instruction cache (2^24 rows: 4.3 ms).
+// and of the draws, and fetching its code: children planned at birth by the warp
+// that writes them cost more than they saved, because the second copy of the
+// plan's code did not fit the instruction cache (4.3 instead of 3.95 ms at 2^24
+// rows), and the two stores of stream_publish are written out because a loop
+// around one cost 1% to 4% of every step.
 // ---------------------------------------------------------------------------
 constexpr int kStreamRefill = 8;             // idle lanes before a busy warp takes entries,
 constexpr unsigned int kStreamRounds = 8;    // and rounds between two looks at an empty queue

@@ -140,8 +140,8 @@ __device__ __forceinline__ void syn64(const Syn64Table& T, double x, double& F, 
 }
 
 // 13 KB of tables per block, a row of a power's (F, G) pairs read with one
-// 128-bit load (random pieces conflict about 2.5-fold).  2^24 points: see the
-// figures above the kernels' launch.
+// 128-bit load (random pieces conflict about 2.5-fold).  The figures
+// stand at the top of this file.
 template <bool W1, bool W2>
 __global__ void __launch_bounds__(kThreads64) k_sweep64(const double* __restrict__ y,
                                                         double* __restrict__ F1,
