@@ -957,6 +957,7 @@ __global__ void __launch_bounds__(kColdThreads, kColdMinBlocks) k_cold(DevPartic
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(&ctl->cold_done, 1u) == gridDim.x - 1u) {
+            __threadfence();   // the count after the other blocks' ends
             ctl->n1 = (long long)stored_rows(P);
             ctl->cold_done = 0u;
         }
@@ -3046,6 +3047,8 @@ __global__ void __launch_bounds__(kLaneThreads, 2) k_stream(DevParticles P, Step
                 if (sum) {
                     __threadfence();   // this warp's entries before its completions
                     const unsigned long long f = sum + atomicAdd(&ctl->finished, sum);
+                    __threadfence();   // the count after the completions: rows reserved before
+                                       // any of them are in it
                     if (f == units0 + (stored_rows(P) - n1))
                         *reinterpret_cast<volatile unsigned int*>(&ctl->queue.over) = 1u;
                     again = 1;
